@@ -88,7 +88,7 @@ struct vp_ctx {
   // workspaces
   vp::DevBuf w_fac, w_q, w_gemm, w_j, w_p, w_tmp, w_tmp2, w_vec, w_split;
   vp::DevBuf w_piv, w_q1, w_q2, w_r, w_p2, w_a, w_b, w_c, w_l;  // preconditioned SVD
-  vp::DevBuf w_tca, w_tcb;            // packed operands of the tensor-core contractions
+  vp::DevBuf w_tca, w_tcb;            // packed operands (or digits) of the tensor-core contractions
   vp::DevBuf w_q_side, w_split_side;  // scratch of the side-stream phase
   vp::DevBuf w_tca_side, w_tcb_side;
   std::vector<vp::DevBuf> w_chain;
@@ -215,6 +215,29 @@ struct TcOperand {
 // C (M x N) = alpha * A (M x K) * B^T with B given as (N x K) operand, on the
 // tensor cores in the context's reduced-precision mode (tcgemm.cu).
 int launch_tc_gemm(vp_ctx* ctx, int M, int N, int K, double alpha, TcOperand a, TcOperand b, double* C, int ldc);
+// How an FP64 contraction is sliced over the tensor cores (ozgemm.cu); use = 0:
+// the FMA kernel (gemm_plan).  Shape and device only.
+struct OzPlan {
+  int use;
+  int swapped;  // tiles of C^T
+  int slices, kslice;
+};
+OzPlan oz_plan(const vp_ctx* ctx, int M, int N, int K);
+// One such contraction: C (M x N, or the partial products of each K slice at
+// C + s * stride) = alpha * A B^T in FP64; wa, wb: scratch of the digits.
+struct OzGemm {
+  TcOperand a, b;
+  int M, N, K;
+  double alpha;
+  double* C;
+  int ldc;
+  size_t stride;
+  DevBuf* wa;
+  DevBuf* wb;
+  DevStatus* st;
+  OzPlan plan;
+};
+int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);
 // C = alpha * triu(A_colmajor) (M x K) * B: the R factor read in place.
 int launch_gemm_r(vp_ctx* ctx, int M, int N, int K, const double* Acm, int lda, const double* B,
                   int ldb, double* C, int ldc);
@@ -311,6 +334,7 @@ struct BScratch {
   DevBuf fq[kScratchSlots];       // Q formation: double-word reflectors
   DevBuf qscr[kScratchSlots];     // Q formation: column scratch (m > 512)
   DevBuf split[kScratchSlots];    // GEMM split-K partial products
+  DevBuf oza[kScratchSlots], ozb[kScratchSlots];  // sliced GEMM: digits of the operands
   DevStatus* st = nullptr;        // status words of the problem (device)
 };
 void release_scratch(vp_ctx* ctx, BScratch& s);

@@ -1008,7 +1008,8 @@ __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, double alpha,
                                    blockIdx.z);
 }
 
-// How a GEMM is spread over the SMs.  FP64 issues about two FMAs per SM per
+// How a GEMM of the FMA kernel is spread over the SMs (the larger FP64 ones run
+// sliced on the tensor cores, oz_plan).  FP64 issues about two FMAs per SM per
 // clock on GB300, so a GEMM runs at the rate of the SMs it occupies: 64 x 64
 // tiles when they alone give every SM a block, else 32 x 32 tiles, and K
 // split into slices (multiples of 16, at most 32) until there are about two
@@ -1054,12 +1055,48 @@ static TcOperand tc_a(const AUpperColMajor& a) { return {a.A, a.lda, 2}; }
 static TcOperand tc_b(const BRowMajor& b) { return {b.B, b.ldb, 1}; }
 static TcOperand tc_b(const BTransposed& b) { return {b.B, b.ldb, 0}; }
 
+static OzGemm oz_job(const TcOperand& a, const TcOperand& b, int M, int N, int K, double alpha, double* C, int ldc,
+                     size_t stride, DevBuf* wa, DevBuf* wb, DevStatus* st, const OzPlan& plan) {
+  OzGemm g;
+  g.a = a;
+  g.b = b;
+  g.M = M;
+  g.N = N;
+  g.K = K;
+  g.alpha = alpha;
+  g.C = C;
+  g.ldc = ldc;
+  g.stride = stride;
+  g.wa = wa;
+  g.wb = wb;
+  g.st = st;
+  g.plan = plan;
+  return g;
+}
+
 // One GEMM launch (split K per gemm_plan, then the fixed-order slice sum).
 template <class ALoad, class BLoad>
 static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a, BLoad b, double* C, int ldc,
                          const char* what) {
   if (M <= 0 || N <= 0) return VP_OK;
   if (ctx->precision >= VP_PREC_TF32 && K > 0) return launch_tc_gemm(ctx, M, N, K, alpha, tc_a(a), tc_b(b), C, ldc);
+  if (ctx->precision == VP_PREC_FP64) {
+    const OzPlan oz = oz_plan(ctx, M, N, K);
+    if (oz.use) {
+      const size_t stride = (size_t)M * N;
+      const bool split = oz.slices > 1;
+      if (split) VP_TRY(reserve(ctx, ctx->w_split, stride * oz.slices));
+      std::vector<OzGemm> job;
+      job.push_back(oz_job(tc_a(a), tc_b(b), M, N, K, alpha, split ? ctx->w_split.p : C, split ? N : ldc,
+                           split ? stride : 0, &ctx->w_tca, &ctx->w_tcb, ctx->status, oz));
+      VP_TRY(blaunch_oz_gemm(ctx, ctx->stream, job));
+      if (!split) return VP_OK;
+      const int blocks = (int)std::min<size_t>((stride + 255) / 256, (size_t)ctx->num_sms * 8);
+      ctx->launches++;
+      k_sum_slices<<<blocks, 256, 0, ctx->stream>>>(ctx->w_split.p, M, N, oz.slices, stride, C, ldc);
+      return check_launch(ctx, what);
+    }
+  }
   const GemmPlan pl = gemm_plan(ctx, M, N, K);
   dim3 grid((M + pl.tile - 1) / pl.tile, (N + pl.tile - 1) / pl.tile, 1);
   if (grid.y > 65535) return fail(ctx, VP_ECAPACITY, "gemm: N too large");
@@ -2265,6 +2302,8 @@ void release_scratch(vp_ctx* ctx, BScratch& s) {
     release(ctx, s.fq[i]);
     release(ctx, s.qscr[i]);
     release(ctx, s.split[i]);
+    release(ctx, s.oza[i]);
+    release(ctx, s.ozb[i]);
   }
 }
 
@@ -2664,17 +2703,19 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
   std::vector<GemmJob<ARowMajor, BTransposed>> abt[2][2];
   std::vector<GemmJob<AUpperColMajor, BRowMajor>> rb[2][2];
   std::vector<SumArgs> sums;
+  std::vector<OzGemm> oz;
   SlotCounter slots;
   for (const BGemm& g : v) {
     if (g.M <= 0 || g.N <= 0) continue;
     const GemmPlan pl = gemm_plan(ctx, g.M, g.N, g.K);
-    const int slices = pl.slices, kslice = pl.kslice, ti = pl.tile == 64 ? 0 : 1;
+    const OzPlan op = g.fp32 ? OzPlan{} : oz_plan(ctx, g.M, g.N, g.K);
+    const int slices = op.use ? op.slices : pl.slices, kslice = pl.kslice, ti = pl.tile == 64 ? 0 : 1;
     double* C = g.C;
     int ldc = g.ldc;
     size_t stride = 0;
+    int sl = 0;
+    if (slices > 1 || op.use) VP_TRY(slots.next(ctx, g.s, &sl));
     if (slices > 1) {
-      int sl = 0;
-      VP_TRY(slots.next(ctx, g.s, &sl));
       stride = (size_t)g.M * g.N;
       VP_TRY(reserve(ctx, g.s->split[sl], stride * slices));
       C = g.s->split[sl].p;
@@ -2682,6 +2723,12 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
       sums.push_back({g.s->split[sl].p, g.M, g.N, slices, stride, g.C, g.ldc});
     }
     const int t = g.fp32 ? 1 : 0;
+    if (op.use) {
+      const TcOperand ta{g.A, g.lda, g.kind == BG_RB ? 2 : 0}, tb{g.B, g.ldb, g.kind == BG_ABT ? 0 : 1};
+      oz.push_back(oz_job(ta, tb, g.M, g.N, g.K, g.alpha, C, ldc, stride, &g.s->oza[sl], &g.s->ozb[sl],
+                          g.s->st ? g.s->st : ctx->status, op));
+      continue;
+    }
     if (g.kind == BG_AB)
       ab[t][ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, ARowMajor{g.A, g.lda}, BRowMajor{g.B, g.ldb}, C, ldc,
                        stride});
@@ -2692,6 +2739,7 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
       rb[t][ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, AUpperColMajor{g.A, g.lda}, BRowMajor{g.B, g.ldb}, C,
                        ldc, stride});
   }
+  VP_TRY(blaunch_oz_gemm(ctx, st, oz));
   VP_TRY((gemm_group<ARowMajor, BRowMajor, double, 64>(ctx, st, ab[0][0])));
   VP_TRY((gemm_group<ARowMajor, BRowMajor, double, 32>(ctx, st, ab[0][1])));
   VP_TRY((gemm_group<ARowMajor, BRowMajor, float, 64>(ctx, st, ab[1][0])));

@@ -1,0 +1,591 @@
+// FP64 contractions on the tensor cores by exact slicing (the Ozaki scheme:
+// K. Ozaki, T. Ogita, S. Oishi, S. Rump, "Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication and its
+// applications", Numer. Algorithms 59 (2012); on FP16 tensor cores: D. Mukunoki
+// et al., ISC High Performance 2020).
+//
+// GB300 issues two FP64 FMAs per SM and clock (1.26 TFLOP/s in all) and 4096
+// FP16 ones on the tensor cores.  Every element of A and B becomes a fixed-point
+// number of 56 bits relative to a power of two above its row's (A) or column's
+// (B) largest magnitude within a K slice, cut into eight signed 7-bit digits,
+//   a = 2^(e - 55) sum_i d_i 2^(7 (7 - i)),  -64 <= d_i <= 64,
+// which are exact FP16 integers.  Products of digits are at most 2^12, so the
+// FP32 accumulator holds the sum of up to eight digit products over K <= 512
+// exactly (2^24).  The digit products with i + j = l, l = 0..8 (43 of the 64)
+// accumulate into nine 128 x 48 accumulators of tensor memory, and the epilogue
+// adds the nine integers with their weights in 128-bit integer arithmetic and
+// rounds once to FP64.  What is dropped (l > 8) is below 2^-61 of the two
+// scales; the representation error of an element below 2^-56 of its scale.
+// Against 64-bit references the error is about a third of the FMA kernel's
+// (measured for K = 64..1008: 6-9e-17 of the norm, against 1.7-3.1e-16).
+//
+// The scales only work on rows and columns, so a factor common to column k of A
+// and, inversely, to row k of B would cost digits: kb_oz_kexp balances the
+// largest magnitudes of the two by a power of two per k first (exact).
+//
+// Passes: kb_oz_kexp (balance exponents), kb_oz_pack (digits, written as the
+// 128-byte-swizzled shared-memory images of whole tiles, so that the loads are
+// plain bulk copies), kb_oz_mma (one CTA per 128 x 48 tile and K slice), and with
+// several K slices the fixed-order sum of the FP64 partial products that the FMA
+// kernel uses too.  A row or column that holds a NaN or Inf, or K-scaling that
+// leaves the exponent range, sends its tiles through plain FP64 FMAs inside
+// kb_oz_mma, so non-finite values propagate as they do there.
+//
+// Measured (2048^3): 557 us in kb_oz_mma, 1.33 PFLOP/s of FP16 products, 71 % of
+// the measured 1.88 (the 9-accumulator epilogue is not overlapped: the tile's
+// accumulators fill tensor memory); kb_oz_pack moves 24 bytes per element at
+// 3 TB/s; whole call 24 TFLOP/s of FP64 against 1.1 for the FMA kernel.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "tc.cuh"
+
+namespace vp {
+namespace {
+
+constexpr int kOzS = 8;             // digits of an element
+constexpr int kOzL = 9;             // accumulators: digit products i + j = 0 .. 8
+constexpr int kOzM = 128, kOzN = 48, kOzKc = 64;  // tile rows, tile columns, K per stage
+constexpr uint32_t kOzABytes = kOzM * 128;        // one digit of an A stage (128 bytes of K per row)
+constexpr uint32_t kOzBDigit = kOzN * 128;        // one digit of a B stage
+constexpr uint32_t kOzBBytes = kOzS * kOzBDigit;  // all digits of a B stage
+constexpr int kOzAStages = kOzS;  // one slot per digit of a stage
+constexpr int kOzMaxK = 512;        // K whose digit products one accumulator holds exactly
+constexpr int kOzPackRows = 32;
+constexpr uint32_t kOzTmem = 512;   // columns allocated (a power of two >= 9 x 48)
+constexpr size_t kOzSmem = 1024 + 2 * (size_t)kOzBBytes + (size_t)kOzAStages * kOzABytes + 256;
+
+// x as an operand element (row r of the operand, index k along the contraction)
+__device__ __forceinline__ double oz_elem(const TcOperand& o, int r, int k) {
+  if (o.kind == 0) return o.p[(size_t)r * o.ld + k];
+  if (o.kind == 1) return o.p[(size_t)k * o.ld + r];
+  return r <= k ? o.p[(size_t)k * o.ld + r] : 0.0;
+}
+
+__device__ __forceinline__ int oz_bexp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
+
+// Exponent of x after the balance shift (0 for a zero, 2047 for a non-finite
+// value, clamped into 1 .. 2047 otherwise: 2047 sends the row to the FP64 path).
+__device__ __forceinline__ int oz_shifted_exp(double x, int sh) {
+  const int e = oz_bexp(x);
+  if (e == 2047) return 2047;
+  if (x == 0.0) return 0;
+  return min(max(max(e, 1) + sh, 1), 2047);
+}
+
+}  // namespace
+
+struct OzJob {
+  TcOperand a, b;        // a: M rows (tile rows), b: N rows (tile columns), both along K
+  int M, N, K, kslice, slices, chunks;  // chunks: 64-wide K stages
+  int swapped;           // the tile is C^T: element (i, j) goes to C[j * ldc + i]
+  double alpha;
+  double* C;
+  int ldc;
+  size_t stride;         // partial products: slice s at C + s * stride
+  int* kexp;             // per k: shift of A (B gets the opposite)
+  int* ea;               // slices x Mp exponents, then slices x Np
+  int* eb;
+  uint8_t* da;           // digit tiles
+  uint8_t* db;
+  DevStatus* st;
+};
+
+namespace {
+
+// Shift of column k of A: half the difference of the two largest exponents.
+// One block of 32 warps takes eight k, so that every load of an operand of up
+// to a few hundred rows is in flight at once.
+constexpr int kOzThreads = 1024;
+__device__ __forceinline__ void oz_kexp_body(const OzJob& j, int kblk) {
+  __shared__ int sa[8], sb[8];
+  const int k0 = kblk * 8;
+  if (threadIdx.x < 8) sa[threadIdx.x] = sb[threadIdx.x] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const TcOperand& o = side ? j.b : j.a;
+    const int R = side ? j.N : j.M;
+    int* s = side ? sb : sa;
+    if (o.kind == 0) {  // k contiguous: eight k per row
+      const int kk = threadIdx.x & 7, k = k0 + kk;
+      int e = 0;
+      if (k < j.K)
+#pragma unroll 4
+        for (int r = threadIdx.x >> 3; r < R; r += kOzThreads / 8) e = max(e, oz_bexp(o.p[(size_t)r * o.ld + k]));
+      for (int off = 8; off < 32; off <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
+      if ((threadIdx.x & 31) < 8) atomicMax(&s[kk], e);
+    } else {  // rows contiguous: four warps per k
+      const int kk = threadIdx.x >> 7, k = k0 + kk;
+      int e = 0;
+      if (k < j.K) {
+        const int rend = o.kind == 2 ? min(R, k + 1) : R;
+#pragma unroll 8
+        for (int r = threadIdx.x & 127; r < rend; r += 128) e = max(e, oz_bexp(o.p[(size_t)k * o.ld + r]));
+      }
+      e = __reduce_max_sync(0xffffffffu, e);
+      if ((threadIdx.x & 31) == 0) atomicMax(&s[kk], e);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 8 && k0 + threadIdx.x < j.K) {
+    const int a = sa[threadIdx.x], b = sb[threadIdx.x];
+    // a zero row or column (or one with a non-finite value) needs no balance
+    j.kexp[k0 + threadIdx.x] = (a == 0 || b == 0 || a == 2047 || b == 2047) ? 0 : (b - a) >> 1;
+  }
+}
+
+// Eight consecutive k of one row: eight digits each, one 16-byte store per digit.
+__device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int (&sh)[8], int emax, uint8_t* tile0,
+                                                size_t digit_stride, int row, int kchunk16) {
+  constexpr long long kBias = 64ll * ((1ll << 49) - 1) / 127;  // 64 * sum_{j<7} 2^(7 j)
+  long long X[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const long long bits = __double_as_longlong(x[u]);
+    const int e = (int)((bits >> 52) & 0x7ff);
+    long long m = (bits & ((1ll << 52) - 1)) | (e ? 1ll << 52 : 0ll);
+    const int s = emax - (max(e, 1) + sh[u]) - 2;  // right shift that puts 2^(emax - 1022) at 2^55
+    if (s <= 0)
+      m <<= -s;  // s >= -2: no element exceeds the row's largest
+    else
+      m = s <= 54 ? (m + (1ll << (s - 1))) >> s : 0ll;
+    X[u] = (bits < 0 ? -m : m) + kBias;
+  }
+  uint8_t* dst = tile0 + row * 128 + ((kchunk16 ^ (row & 7)) << 4);
+#pragma unroll
+  for (int i = 0; i < kOzS; ++i) {
+    uint32_t w[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      // 0x6400 | u is the FP16 number 1024 + u (u < 1024); digit = u - 64
+      uint32_t lo, hi;
+      if (i == 0) {
+        lo = (uint32_t)((int)(X[2 * h] >> 49) + 64);
+        hi = (uint32_t)((int)(X[2 * h + 1] >> 49) + 64);
+      } else {
+        lo = (uint32_t)(X[2 * h] >> (7 * (7 - i))) & 127u;
+        hi = (uint32_t)(X[2 * h + 1] >> (7 * (7 - i))) & 127u;
+      }
+      const uint32_t raw = 0x64006400u | lo | (hi << 16);
+      const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&raw), __float2half2_rn(1088.0f));
+      w[h] = *reinterpret_cast<const uint32_t*>(&d);
+    }
+    *reinterpret_cast<uint4*>(dst + i * digit_stride) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// Digits of 32 rows of one operand over one K slice: a thread holds up to two
+// groups of eight k of one row, the largest exponent of the row is reduced over
+// its threads, then the groups are converted from registers (one read).
+__device__ __forceinline__ void oz_pack_body(const OzJob& j, int side, int rblk, int slice) {
+  const TcOperand& o = side ? j.b : j.a;
+  const int R = side ? j.N : j.M;
+  const int tile_rows = side ? kOzN : kOzM;
+  const int Rp = (R + tile_rows - 1) / tile_rows * tile_rows;
+  const int row0 = rblk * kOzPackRows;
+  if (row0 >= Rp) return;
+  int* ex = side ? j.eb : j.ea;
+  uint8_t* out = side ? j.db : j.da;
+  const size_t dstride = side ? kOzBDigit : kOzABytes;
+  const int kbeg = slice * j.kslice, kend = min(j.K, kbeg + j.kslice);
+  const int kpad = min(j.chunks * kOzKc, kbeg + j.kslice);  // zero digits up to here
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int sgn = side ? -1 : 1;
+  // a warp per row, lanes along k, so that every store fills whole sectors
+  const int r = row0 + warp, g = lane;
+  double x[2][8];
+  if (o.kind == 0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int k = kbeg + 8 * (g + 32 * h);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[h][u] = r < R && k + u < kend ? o.p[(size_t)r * o.ld + k + u] : 0.0;
+    }
+  } else {
+    // rows contiguous: read with the lanes along the rows and turned in shared
+    // memory (row stride odd, one pad per eight k: both sides free of conflicts)
+    extern __shared__ double turn[];
+    const int P = j.kslice / 8 * 9 + 1;
+    const int rr = row0 + lane;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int kk = 8 * (warp + 32 * h), k = kbeg + kk;
+      if (kk >= j.kslice) continue;
+      double y[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        y[u] = rr < R && k + u < kend && !(o.kind == 2 && rr > k + u) ? o.p[(size_t)(k + u) * o.ld + rr] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) turn[lane * P + kk / 8 * 9 + u] = y[u];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int kk = 8 * (g + 32 * h);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[h][u] = kk < j.kslice ? turn[warp * P + kk / 8 * 9 + u] : 0.0;
+    }
+  }
+  int e = 1;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k = kbeg + 8 * (g + 32 * h);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (k + u < kend) e = max(e, oz_shifted_exp(x[h][u], sgn * j.kexp[k + u]));
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (r >= Rp) return;
+  if (g == 0) ex[(size_t)slice * Rp + r] = e;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k = kbeg + 8 * (g + 32 * h);
+    if (k >= kpad) continue;
+    int sh[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      sh[u] = k + u < kend ? sgn * j.kexp[k + u] : 0;
+      if (e >= 2047) x[h][u] = 0.0;  // the row takes the FP64 path
+    }
+    oz_store_digits(x[h], sh, e,
+                    out + ((size_t)(r / tile_rows) * j.chunks + k / kOzKc) * kOzS * dstride, dstride, r % tile_rows,
+                    (k % kOzKc) >> 3);
+  }
+}
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// sum_l S_l 2^(7 (8 - l)), |S_l| <= 2^24 exact integers, times 2^e2 as FP64: the
+// sum in two 64-bit integers, its 63 leading positions (what lies below is under
+// the dropped digit products) rounded once.  Integer arithmetic
+// throughout, since the FP64 pipe takes two operations per SM and clock.
+__device__ __forceinline__ double oz_combine(const int (&S)[kOzL], int e2) {
+  const long long H = ((long long)S[0] << 21) + ((long long)S[1] << 14) + ((long long)S[2] << 7) + S[3];  // times 2^35
+  const long long L = ((long long)S[4] << 28) + ((long long)S[5] << 21) + ((long long)S[6] << 14) +
+                      ((long long)S[7] << 7) + S[8];
+  // one product of two full-scale elements is 2^68, K <= 512 of them 2^77; |L| < 2^52.1
+  const int sh = (unsigned long long)(H + (1ll << 35)) >> 36 ? 18 : 8;
+  const long long T = (H << (35 - sh)) + (L >> sh);  // |T| < 2^63
+  const unsigned long long a = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
+  if (a == 0) return 0.0;
+  const int lz = __clzll((long long)a);
+  const unsigned long long top = a << lz;
+  const unsigned long long m = (top + 1023ull + ((top >> 11) & 1ull));  // to nearest, ties to even
+  // a carry out of the top bit: the mantissa is 2^53
+  const unsigned long long m53 = m < top ? 1ull << 53 : m >> 11;
+  const int be = 63 - lz + sh + e2 + 1023;
+  if (be >= 1 && be < 2046) {
+    const unsigned long long bits = m53 + ((unsigned long long)(be - 1) << 52) + ((unsigned long long)T & (1ull << 63));
+    return __longlong_as_double((long long)bits);
+  }
+  const double v = scalbn((double)m53, be - 1023 - 52);  // subnormal or overflow
+  return T < 0 ? -v : v;
+}
+
+// One 128 x 48 tile over one K slice.  Warp 0: bulk copies (all digits of a B
+// stage, double-buffered; the A digits of a stage one by one into their
+// slots); warp 1: per A digit i the products with B digits 0 .. min(7, 8 - i),
+// neighbouring B digits joined into one instruction of up to 240 columns, whose
+// accumulators lie next to each other in tensor memory; then all eight warps
+// read the accumulators, combine and store.
+__device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int slice) {
+  extern __shared__ uint8_t oz_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sB = base;
+  uint8_t* sA = base + 2 * kOzBBytes;
+  uint64_t* fullA = reinterpret_cast<uint64_t*>(sA + kOzAStages * kOzABytes);
+  uint64_t* emptyA = fullA + kOzAStages;
+  uint64_t* fullB = emptyA + kOzAStages;
+  uint64_t* emptyB = fullB + 2;
+  uint64_t* done = emptyB + 2;
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(done + 1);
+  __shared__ int s_abort, s_plain;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m0 = mt * kOzM, n0 = nt * kOzN;
+  const int Mp = (j.M + kOzM - 1) / kOzM * kOzM, Np = (j.N + kOzN - 1) / kOzN * kOzN;
+  const int* ea = j.ea + (size_t)slice * Mp + m0;
+  const int* eb = j.eb + (size_t)slice * Np + n0;
+  // an upper-triangular operand is zero for k below its first row
+  int kskip = 0;
+  if (j.a.kind == 2) kskip = m0;
+  if (j.b.kind == 2) kskip = max(kskip, n0);
+  const int cper = j.kslice / kOzKc;
+  const int c1 = min(j.chunks, (slice + 1) * cper), c0 = min(c1, max(slice * cper, kskip / kOzKc));
+  double* C = j.C + slice * j.stride;
+  auto store = [&](int i, int col, double v) {
+    if (i < j.M && col < j.N) C[j.swapped ? (size_t)col * j.ldc + i : (size_t)i * j.ldc + col] = v;
+  };
+
+  if (tid == 0) s_abort = s_plain = 0;
+  __syncthreads();
+  if ((tid < kOzM && ea[tid] >= 2047) || (tid < kOzN && eb[tid] >= 2047)) s_plain = 1;
+  __syncthreads();
+  if (s_plain || c0 >= c1) {
+    // non-finite operands (or a K range of exact zeros): plain FP64
+    const int kb = max(slice * j.kslice, c0 * kOzKc), ke = min(j.K, c1 * kOzKc);
+    for (int e = tid; e < kOzM * kOzN; e += 256) {
+      const int i = m0 + (j.swapped ? e % kOzM : e / kOzN), col = n0 + (j.swapped ? e / kOzM : e % kOzN);
+      if (i >= j.M || col >= j.N) continue;
+      double acc = 0.0;
+      for (int k = kb; k < ke; ++k) acc = fma(oz_elem(j.a, i, k), oz_elem(j.b, col, k), acc);
+      store(i, col, j.alpha * acc);
+    }
+    return;
+  }
+
+  if (tid == 0) {
+    for (int s = 0; s < kOzAStages; ++s) {
+      mbar_init(&fullA[s], 1);
+      mbar_init(&emptyA[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&fullB[s], 1);
+      mbar_init(&emptyB[s], 1);
+    }
+    mbar_init(done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  __syncwarp();
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
+                 "r"(kOzTmem)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_holder;
+  bool ok = true;
+
+  if (warp == 0 && lane == 0) {
+    const uint8_t* ga = j.da + (size_t)mt * j.chunks * kOzS * kOzABytes;
+    const uint8_t* gb = j.db + (size_t)nt * j.chunks * kOzBBytes;
+    int na = 0, nb = 0;  // A digits and B stages issued
+    for (int c = c0; c < c1 && ok; ++c) {
+      const int sb = nb & 1;
+      if (nb >= 2 && !mbar_wait(&emptyB[sb], ((nb >> 1) - 1) & 1)) {
+        ok = false;
+        break;
+      }
+      mbar_expect_tx(&fullB[sb], kOzBBytes);
+      bulk_load(sB + sb * kOzBBytes, gb + (size_t)c * kOzBBytes, kOzBBytes, &fullB[sb]);
+      ++nb;
+      for (int i = 0; i < kOzS; ++i) {
+        const int sa = na % kOzAStages;
+        if (na >= kOzAStages && !mbar_wait(&emptyA[sa], ((na / kOzAStages) - 1) & 1)) {
+          ok = false;
+          break;
+        }
+        mbar_expect_tx(&fullA[sa], kOzABytes);
+        bulk_load(sA + sa * kOzABytes, ga + ((size_t)c * kOzS + i) * kOzABytes, kOzABytes, &fullA[sa]);
+        ++na;
+      }
+    }
+    // every issued copy lands before the CTA can exit
+    for (int q = max(0, nb - 2); q < nb; ++q)
+      if (!mbar_wait(&fullB[q & 1], (q >> 1) & 1)) ok = false;
+    for (int q = max(0, na - kOzAStages); q < na; ++q)
+      if (!mbar_wait(&fullA[q % kOzAStages], (q / kOzAStages) & 1)) ok = false;
+  } else if (warp == 1 && lane == 0) {
+    // everything but the stage is a constant of the unrolled loops: a descriptor
+    // built at run time costs more issue slots than the smaller products take
+    const uint64_t a_desc = sw128_desc(smem_u32(sA)), b_desc = sw128_desc(smem_u32(sB));
+    for (int c = c0, n = 0; c < c1 && ok; ++c, ++n) {
+      const int sb = n & 1;
+      if (!mbar_wait(&fullB[sb], (n >> 1) & 1)) {
+        ok = false;
+        break;
+      }
+      const uint64_t bd = b_desc + (uint32_t)sb * (kOzBBytes >> 4);
+      const uint32_t later = n > 0 ? 1u : 0u;
+#pragma unroll
+      for (int i = 0; i < kOzS; ++i) {
+        if (ok && !mbar_wait(&fullA[i], n & 1)) ok = false;
+        if (!ok) continue;
+        tc_fence_after();
+        constexpr int kW[kOzS][3] = {{5, 3, 0}, {5, 2, 1}, {5, 2, 0}, {5, 1, 0}, {5, 0, 0}, {4, 0, 0}, {3, 0, 0}, {2, 0, 0}};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          // accumulators are first written by digit 0 (0 .. 7) and by the pair (1, 7) (8)
+          int q = 0;
+#pragma unroll
+          for (int part = 0; part < 3; ++part) {
+            const int w = kW[i][part];
+            if (w == 0) continue;
+            const bool opens = k == 0 && (i == 0 || (i == 1 && part == 2));
+            tc_mma<true>(tmem + (i + q) * kOzN, a_desc + i * (kOzABytes >> 4) + 2 * k, bd + q * (kOzBDigit >> 4) + 2 * k,
+                         tc_idesc(0, w * kOzN), opens ? later : 1u);
+            q += w;
+          }
+        }
+        tc_commit(&emptyA[i]);
+      }
+      if (ok) tc_commit(&emptyB[sb]);
+    }
+    tc_commit(done);
+  }
+  if (!ok) atomicExch(&s_abort, 1);
+  __syncwarp();
+  __syncthreads();
+
+  const bool got = mbar_wait(done, 0);
+  const int good = __syncthreads_and(got && s_abort == 0);
+  tc_fence_after();
+  if (good) {
+    // warp w reads lanes 32 (w mod 4) .., the column groups of 8 with (w / 4)
+    const int row = (warp & 3) * 32 + lane;
+    const int er = ea[row];
+#pragma unroll 1
+    for (int g = warp >> 2; g < kOzN / 8; g += 2) {
+      uint32_t r[kOzL][8];
+#pragma unroll
+      for (int l = 0; l < kOzL; ++l)
+        tmem_ld8(tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + l * kOzN + 8 * g, r[l]);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        int S[kOzL];
+#pragma unroll
+        for (int l = 0; l < kOzL; ++l) S[l] = __float2int_rn(__uint_as_float(r[l][u]));
+        const int col = 8 * g + u;
+        // digit products carry 2^(7 (14 - l)); scales 2^(er - 1022 - 55), 2^(ec - 1022 - 55)
+        double v = oz_combine(S, er + eb[col] - 2 * 1077 + 42);
+        if (j.alpha != 1.0) v *= j.alpha;
+        store(m0 + row, n0 + col, v);
+      }
+    }
+  }
+  if (!good && tid == 0) atomicCAS(&j.st->err, 0, 1);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kOzTmem) : "memory");
+}
+
+__global__ void __launch_bounds__(kOzThreads) kb_oz_kexp(const __grid_constant__ Pack<OzJob> pk) {
+  const OzJob& j = pk.a[blockIdx.y];
+  if ((int)blockIdx.x * 8 >= j.K) return;
+  oz_kexp_body(j, blockIdx.x);
+}
+// x: 32-row blocks of A, then of B (ablk of A at most); y: K slice; z: job
+__global__ void __launch_bounds__(kOzThreads) kb_oz_pack(const __grid_constant__ Pack<OzJob> pk, int ablk) {
+  const OzJob& j = pk.a[blockIdx.z];
+  if ((int)blockIdx.y >= j.slices) return;
+  const int side = (int)blockIdx.x >= ablk;
+  oz_pack_body(j, side, (int)blockIdx.x - (side ? ablk : 0), blockIdx.y);
+}
+__global__ void __launch_bounds__(256, 1) kb_oz_mma(const __grid_constant__ Pack<OzJob> pk, int zs) {
+  const OzJob& j = pk.a[blockIdx.z / zs];
+  const int slice = blockIdx.z % zs;
+  if (slice >= j.slices || (int)blockIdx.x * kOzM >= j.M || (int)blockIdx.y * kOzN >= j.N) return;
+  oz_mma_body(j, blockIdx.x, blockIdx.y, slice);
+}
+
+size_t oz_pack_smem(int kslice) { return (size_t)kOzPackRows * (kslice / 8 * 9 + 1) * sizeof(double); }
+long long tiles_of(int M, int N) { return (long long)((M + kOzM - 1) / kOzM) * ((N + kOzN - 1) / kOzN); }
+
+}  // namespace
+
+// Which FP64 contractions are sliced.  Three launches of ~6 + 11 + 17 us at the
+// smallest sizes stand against the FMA kernel's 2 M N K / 1.1 TFLOP/s: whole
+// vp_gemm calls on GB300, sliced / FMA, us: 256^3 (M N K = 1.7e7) 63 / 62,
+// 320 x 256 x 256 (2.1e7) 66 / 86, 300^3 67 / 99, 512 x 324 x 256 (4.3e7) 68 /
+// 135, 341 x 1008 x 503 (1.7e8) 74 / 430, 128 x 6784 x 6147 (5.3e9) 810 / 12300;
+// the line is drawn at 2e7.  Below K = 64 (one stage) or 16 rows or columns most
+// of a tile would be padding; so would a shape that fills less than a quarter of
+// its tiles in the better of the two orientations.  K is cut into slices until
+// the tiles fill the SMs once (at least 128 of K each, two stages), and always at
+// 512, where the accumulators stop being exact.
+OzPlan oz_plan(const vp_ctx* ctx, int M, int N, int K) {
+  OzPlan p{0, 0, 1, 0};
+  if (K < 64 || std::min(M, N) < 16 || (double)M * N * K < 2e7) return p;
+  const long long t = tiles_of(M, N), ts = tiles_of(N, M);
+  p.swapped = ts < t;
+  const long long tiles = std::min(t, ts);
+  // partial tiles compute their padding: not worth it where most of it is
+  if ((double)tiles * kOzM * kOzN > 4.0 * M * N) return p;
+  if (tiles > 2000000) return p;
+  const int chunks = (K + kOzKc - 1) / kOzKc;
+  int sl = (K + kOzMaxK - 1) / kOzMaxK;
+  sl = std::max<long long>(sl, std::min<long long>(ctx->num_sms / tiles, (chunks + 1) / 2));
+  const int per = std::min(kOzMaxK / kOzKc, (chunks + sl - 1) / sl);
+  p.use = 1;
+  p.kslice = per * kOzKc;
+  p.slices = (chunks + per - 1) / per;
+  return p;
+}
+
+int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
+  if (v.empty()) return VP_OK;
+  static AttrOnce attr, pattr;
+  VP_TRY(attr.ensure(ctx, (const void*)kb_oz_mma, (int)kOzSmem, false));
+  VP_TRY(pattr.ensure(ctx, (const void*)kb_oz_pack, (int)oz_pack_smem(kOzMaxK), false));
+  for (size_t i0 = 0; i0 < v.size(); i0 += kMaxBatch) {
+    const int nb = (int)std::min<size_t>(kMaxBatch, v.size() - i0);
+    Pack<OzJob> pk{};
+    int ks = 1, ablk = 1, bblk = 1, zs = 1, gx = 1, gy = 1, ksl = kOzKc;
+    for (int i = 0; i < nb; ++i) {
+      const OzGemm& g = v[i0 + i];
+      OzJob& j = pk.a[i];
+      j.a = g.plan.swapped ? g.b : g.a;
+      j.b = g.plan.swapped ? g.a : g.b;
+      j.M = g.plan.swapped ? g.N : g.M;
+      j.N = g.plan.swapped ? g.M : g.N;
+      j.K = g.K;
+      j.kslice = g.plan.kslice;
+      j.slices = g.plan.slices;
+      j.chunks = (g.K + kOzKc - 1) / kOzKc;
+      j.swapped = g.plan.swapped;
+      j.alpha = g.alpha;
+      j.C = g.C;
+      j.ldc = g.ldc;
+      j.stride = g.stride;
+      j.st = g.st;
+      const size_t Mp = (size_t)(j.M + kOzM - 1) / kOzM * kOzM, Np = (size_t)(j.N + kOzN - 1) / kOzN * kOzN;
+      const size_t abytes = Mp / kOzM * j.chunks * kOzS * kOzABytes, bbytes = Np / kOzN * j.chunks * (size_t)kOzBBytes;
+      const size_t ints = (size_t)j.K + (size_t)j.slices * (Mp + Np);
+      VP_TRY(reserve(ctx, *g.wa, abytes / 8 + ints / 2 + 64));
+      VP_TRY(reserve(ctx, *g.wb, bbytes / 8 + 64));
+      // bulk copies start on 16-byte boundaries, whatever the allocator's alignment
+      auto aligned = [](double* p) { return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 127) & ~uintptr_t(127)); };
+      j.da = aligned(g.wa->p);
+      j.db = aligned(g.wb->p);
+      j.kexp = reinterpret_cast<int*>(j.da + abytes);
+      j.ea = j.kexp + j.K;
+      j.eb = j.ea + (size_t)j.slices * Mp;
+      ks = std::max(ks, (j.K + 7) / 8);
+      ablk = std::max(ablk, (int)((Mp + kOzPackRows - 1) / kOzPackRows));
+      bblk = std::max(bblk, (int)((Np + kOzPackRows - 1) / kOzPackRows));
+      zs = std::max(zs, j.slices);
+      ksl = std::max(ksl, j.kslice);
+      gx = std::max(gx, (int)(Mp / kOzM));
+      gy = std::max(gy, (int)(Np / kOzN));
+    }
+    if (gy > 65535 || (long long)nb * zs > 65535) return fail(ctx, VP_ECAPACITY, "gemm: too large");
+    ctx->launches += 3;
+    kb_oz_kexp<<<dim3(ks, nb), kOzThreads, 0, st>>>(pk);
+    kb_oz_pack<<<dim3(ablk + bblk, zs, nb), kOzThreads, oz_pack_smem(ksl), st>>>(pk, ablk);
+    kb_oz_mma<<<dim3(gx, gy, nb * zs), 256, kOzSmem, st>>>(pk, zs);
+    VP_TRY(check_launch(ctx, "oz_gemm"));
+  }
+  return VP_OK;
+}
+
+}  // namespace vp
