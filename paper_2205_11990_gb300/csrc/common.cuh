@@ -174,11 +174,28 @@ int launch_to_colmajor(vp_ctx* ctx, const double* A, int m, int n, double* out);
 // R in the upper triangle, reflectors below, tau[min(m,n)].
 int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* vbuf);
 // Kernel that factors an m x n matrix (shape and device only).
-enum { QR_NONE = 0, QR_WIDE, QR_CDW, QR_CL, QR_GRID };
+enum { QR_NONE = 0, QR_WIDE, QR_PANEL, QR_GRID };
+enum { PANEL_NONE = 0, PANEL_SOLO, PANEL_CLUSTER, PANEL_GRID };
+struct PanelPlan {
+  int kind;
+  int cs;  // CTAs per cluster (PANEL_CLUSTER)
+};
 struct QRPlan {
   int kind;
-  int cs;  // CTAs per cluster (QR_CDW, QR_CL)
+  PanelPlan panel;  // QR_PANEL
 };
+// Where the panel QR (qrpanel.cu) keeps an m x n factor; PANEL_NONE: too many rows.
+PanelPlan qr_panel_plan(const vp_ctx* ctx, int m, int n);
+struct PanelJob {
+  double* A;
+  int m, n;
+  double* tau;
+  PanelPlan plan;
+  DevBuf* scratch;  // block reflectors' T and the columns' exponents
+  DevBuf* cols;     // columns beyond shared memory (PANEL_GRID)
+  DevStatus* st;    // status words (PANEL_GRID)
+};
+int blaunch_qr_panel(vp_ctx* ctx, cudaStream_t st, const std::vector<PanelJob>& v);
 QRPlan qr_plan(const vp_ctx* ctx, int m, int n);
 // Q (m x p, p = min(m,n)) written row-major from the factored A.
 int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q);

@@ -348,361 +348,21 @@ __global__ void __launch_bounds__(kThreads) k_qr_factor_dw(double* A, int m, int
   qr_factor_dw_body(A, m, n, tau, V, T, gcols, gexp, st, gridDim.x, blockIdx.x);
 }
 
-// Cluster-resident double-word QR (small factors).  Column k lives in CTA
-// k % CS (slot k / CS) as double words, scaled by its own power of two as in
-// k_qr_factor_dw.  Step j: in the owner of column j+1, warp 0 applies H_j to
-// that column, forms reflector j+1 in place and pushes it (rows >= j+1,
-// leading 1) with its tau into every CTA's incoming buffer (j+1) % 2 through
-// distributed shared memory; the other warps, and every other CTA, apply H_j
-// (read from the local incoming buffer j % 2) to their columns right of j+1.
-// One hardware cluster barrier per step orders the pushes.
-__device__ __forceinline__ void k_qr_factor_cdw_body(double* A, int m, int n, double* tau) {
-  cg::cluster_group cl = cg::this_cluster();
-  const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int p = min(m, n);
-  const int nmax = (n + CS - 1) / CS;
-  const int nown = rank < n ? (n - rank + CS - 1) / CS : 0;
-  extern __shared__ double qsm_raw[];
-  dw* cols = reinterpret_cast<dw*>(qsm_raw);  // nmax columns of m
-  dw* vbuf = cols + (size_t)nmax * m;         // 2 x m incoming reflectors
-  dw* tbuf = vbuf + 2 * (size_t)m;            // 2 incoming taus
-  int* cexp = reinterpret_cast<int*>(tbuf + 2);
-  // a one-CTA cluster needs only the block barrier
-  auto csync = [&] {
-    if (CS == 1)
-      __syncthreads();
-    else
-      cl.sync();
-  };
-
-  for (int lc = warp; lc < nown; lc += kWarps) {
-    const double* a = A + (size_t)(rank + lc * CS) * m;
-    float mx = 0.f;
-    for (int i = lane; i < m; i += 32) mx = fmaxf(mx, fabsf(__double2float_rn(a[i])));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    int e = 0;
-    if (mx > 0.f) frexpf(mx, &e);
-    if (lane == 0) cexp[lc] = e;
-    const double sc = ldexp(1.0, -e);
-    dw* c = cols + (size_t)lc * m;
-    for (int i = lane; i < m; i += 32) c[i] = dw_from(a[i] * sc);
-  }
-
-  // H_j (from the local incoming buffer) applied to a local column, one warp
-  auto apply = [&](int j, dw* c) {
-    const dw* v = vbuf + (size_t)(j & 1) * m;
-    const dw t = tbuf[j & 1];
-    if (t.hi == 0.f) return;
-    dw_acc acc;
-    for (int i = j + lane; i < m; i += 32) dw_dot_step(acc, v[i], c[i]);
-    const dw w = dw_mul(dw_warp_sum(dw_acc_value(acc)), t);
-    if (w.hi == 0.f) return;
-    for (int i = j + lane; i < m; i += 32) c[i] = dw_add(c[i], dw_neg(dw_mul(w, v[i])));
-  };
-  // reflector j formed in place in local column c, pushed to every CTA
-  auto reflect_push = [&](int j, dw* c) {
-    float mx = 0.f;
-    for (int i = j + lane; i < m; i += 32) mx = fmaxf(mx, fabsf(c[i].hi));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    int e = 0;
-    if (mx > 0.f) frexpf(mx, &e);
-    dw_acc acc;
-    for (int i = j + 1 + lane; i < m; i += 32) {
-      const dw x = dw_ldexp(c[i], -e);
-      dw_dot_step(acc, x, x);
-    }
-    const dw s = dw_warp_sum(dw_acc_value(acc));
-    const dw x0 = dw_ldexp(c[j], -e);
-    dw t = {0.f, 0.f}, beta = x0, scale = {0.f, 0.f};
-    if (s.hi > 0.f) {
-      const dw nrm = dw_sqrt(dw_add(dw_mul(x0, x0), s));
-      beta = x0.hi >= 0.f ? dw_neg(nrm) : nrm;
-      t = dw_div(dw_add(beta, dw_neg(x0)), beta);
-      scale = dw_div({1.0f, 0.0f}, dw_add(x0, dw_neg(beta)));
-    }
-    for (int i = j + 1 + lane; i < m; i += 32) c[i] = dw_mul(dw_ldexp(c[i], -e), scale);
-    __syncwarp();
-    if (lane == 0) {
-      c[j] = dw_ldexp(beta, e);
-      tau[j] = dw_to(t);
-    }
-    for (int r = 0; r < CS; ++r) {
-      dw* dst = cl.map_shared_rank(vbuf + (size_t)(j & 1) * m, r);
-      for (int i = j + lane; i < m; i += 32) dst[i] = (i == j) ? dw{1.0f, 0.0f} : c[i];
-      if (lane == 0) *cl.map_shared_rank(tbuf + (j & 1), r) = t;
-    }
-  };
-
-  csync();  // every CTA resident before the first remote write
-  if (rank == 0 && warp == 0 && p > 0) reflect_push(0, cols);
-  csync();
-  for (int j = 0; j < p; ++j) {
-    const bool owner = j + 1 < p && rank == (j + 1) % CS;
-    if (owner && warp == 0) {
-      dw* c = cols + (size_t)((j + 1) / CS) * m;
-      apply(j, c);
-      __syncwarp();
-      reflect_push(j + 1, c);
-    } else {
-      const int wk = owner ? warp - 1 : warp, nwk = owner ? kWarps - 1 : kWarps;
-      const int lc0 = (j + 2 - rank + CS - 1) / CS > 0 ? (j + 2 - rank + CS - 1) / CS : 0;
-      for (int lc = lc0 + wk; lc < nown; lc += nwk) apply(j, cols + (size_t)lc * m);
-    }
-    csync();
-  }
-  for (int lc = warp; lc < nown; lc += kWarps) {
-    const int k = rank + lc * CS;
-    const double sc = ldexp(1.0, cexp[lc]);
-    const dw* c = cols + (size_t)lc * m;
-    double* a = A + (size_t)k * m;
-    for (int i = lane; i < m; i += 32) a[i] = (k < p && i > k) ? dw_to(c[i]) : dw_to(c[i]) * sc;
-  }
-}
-__global__ void __launch_bounds__(kThreads) k_qr_factor_cdw(double* A, int m, int n, double* tau) { k_qr_factor_cdw_body(A, m, n, tau); }
-
-// Cluster-resident double-word QR (factors up to a 16-CTA cluster's shared
-// memory).  Column k lives in CTA k % CS (slot k / CS) as double words scaled
-// by its own power of two.  Reflector j is formed in its column by the owner,
-// which also publishes it through L2: rows > j as double words in A's column
-// j, its tau in row j.  Step j: one cluster barrier makes reflector j visible,
-// every CTA loads it into its own buffer; then in the owner of column j+1 the
-// first CW warps apply H_j to that column and form reflector j+1 in place
-// (rows split over the CW warps, partial sums combined in a fixed order
-// behind a named barrier), while every other warp applies H_j to the columns
-// right of j+1.  A's columns are rewritten with the factor after the last
-// barrier.  The L2 copy replaced a pull of each reflector from the owner's
-// shared memory through DSMEM, where up to sixteen CTAs wait on one SM's
-// DSMEM bandwidth (measured on GB300, two problems per launch: 3.00 -> 2.13 ms
-// at 512 x 504 on 16 CTAs, 1.17 -> 0.91 ms at 1008 x 135 on 8, 0.35 -> 0.33 ms
-// at 240 x 90; bit-identical results).  The per-row arithmetic is that of
-// k_qr_factor_dw; only the order in which the critical column's partial sums
-// are added differs.
-template <int NT, int CW>
-__device__ __forceinline__ void k_qr_factor_cl_body(double* A, int m, int n, double* tau) {
-  constexpr int NW = NT / 32;
-  static_assert(CW >= 1 && CW < NW, "critical warps must leave bulk warps");
-  cg::cluster_group cl = cg::this_cluster();
-  const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int p = min(m, n);
-  const int nmax = (n + CS - 1) / CS;
-  const int nown = rank < n ? (n - rank + CS - 1) / CS : 0;
-  extern __shared__ double qsm_raw[];
-  dw* cols = reinterpret_cast<dw*>(qsm_raw);  // nmax columns of m
-  dw* vin = cols + (size_t)nmax * m;          // reflector of the step (m)
-  dw* tsl = vin + m;                          // tau of each owned reflector (nmax)
-  dw* tin = tsl + nmax;                       // tau of the step
-  int* cexp = reinterpret_cast<int*>(tin + 1);
-  __shared__ dw red[3][CW];                   // partial sums of the critical warps
-  __shared__ float redm[CW];
-
-  for (int lc = warp; lc < nown; lc += NW) {
-    const double* a = A + (size_t)(rank + lc * CS) * m;
-    float mx = 0.f;
-    for (int i = lane; i < m; i += 32) mx = fmaxf(mx, fabsf(__double2float_rn(a[i])));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    int e = 0;
-    if (mx > 0.f) frexpf(mx, &e);
-    if (lane == 0) cexp[lc] = e;
-    const double sc = ldexp(1.0, -e);
-    dw* c = cols + (size_t)lc * m;
-    for (int i = lane; i < m; i += 32) c[i] = dw_from(a[i] * sc);
-  }
-
-  // H_j applied to a bulk column by one warp
-  auto apply = [&](int j, dw* c) {
-    const dw t = *tin;
-    if (t.hi == 0.f) return;
-    dw_acc acc;
-    dw_dot_rows(acc, vin, c, j, m, lane);
-    const dw w = dw_mul(dw_warp_sum(dw_acc_value(acc)), t);
-    if (w.hi == 0.f) return;
-    dw_axpy_rows(c, vin, w, j, m, lane);
-  };
-  auto cbar = [] { asm volatile("bar.sync 1, %0;" ::"r"(CW * 32) : "memory"); };
-  // Critical warps (warp < CW): H_{j-1} applied to column j (when j > 0),
-  // then reflector j formed in place; warp w handles rows i with
-  // (i - j) / 32 = w mod CW.
-  auto critical = [&](int j, dw* c, int lc) {
-    const int r0 = j + 32 * warp + lane, rs = 32 * CW;
-    if (j > 0) {  // H_{j-1} acts on rows >= j - 1 (its leading 1 sits in row j - 1)
-      const int a0 = r0 - 1;
-      const dw t = *tin;
-      dw_acc acc;
-      for (int i = a0; i < m; i += rs) dw_dot_step(acc, vin[i], c[i]);
-      const dw part = dw_warp_sum(dw_acc_value(acc));
-      if (lane == 0) red[0][warp] = part;
-      cbar();
-      dw dot = red[0][0];
-      for (int w = 1; w < CW; ++w) dot = dw_add(dot, red[0][w]);
-      const dw wv = dw_mul(dot, t);
-      if (t.hi != 0.f && wv.hi != 0.f)
-        for (int i = a0; i < m; i += rs) c[i] = dw_add(c[i], dw_neg(dw_mul(wv, vin[i])));
-    }
-    float mx = 0.f;
-    for (int i = r0; i < m; i += rs) mx = fmaxf(mx, fabsf(c[i].hi));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) redm[warp] = mx;
-    cbar();
-    for (int w = 0; w < CW; ++w) mx = fmaxf(mx, redm[w]);
-    int e = 0;
-    if (mx > 0.f) frexpf(mx, &e);
-    const dw x0 = dw_ldexp(c[j], -e);
-    dw_acc acc;
-    for (int i = r0; i < m; i += rs)
-      if (i > j) {
-        const dw x = dw_ldexp(c[i], -e);
-        dw_dot_step(acc, x, x);
-      }
-    const dw part = dw_warp_sum(dw_acc_value(acc));
-    if (lane == 0) red[1][warp] = part;
-    cbar();  // every critical warp has read x0 and its partial sum is in
-    dw sq = red[1][0];
-    for (int w = 1; w < CW; ++w) sq = dw_add(sq, red[1][w]);
-    dw t = {0.f, 0.f}, beta = x0, scale = {0.f, 0.f};
-    if (sq.hi > 0.f) {
-      const dw nrm = dw_sqrt(dw_add(dw_mul(x0, x0), sq));
-      beta = x0.hi >= 0.f ? dw_neg(nrm) : nrm;
-      t = dw_div(dw_add(beta, dw_neg(x0)), beta);
-      scale = dw_div({1.0f, 0.0f}, dw_add(x0, dw_neg(beta)));
-    }
-    dw* gj = reinterpret_cast<dw*>(A + (size_t)j * m);
-    for (int i = r0; i < m; i += rs)
-      if (i > j) {
-        const dw v = dw_mul(dw_ldexp(c[i], -e), scale);
-        c[i] = v;
-        __stcg(reinterpret_cast<float2*>(gj + i), make_float2(v.hi, v.lo));
-      }
-    if (warp == 0 && lane == 0) {
-      c[j] = dw_ldexp(beta, e);
-      tsl[lc] = t;
-      tau[j] = dw_to(t);
-      __stcg(reinterpret_cast<float2*>(gj + j), make_float2(t.hi, t.lo));
-    }
-  };
-
-  __syncthreads();
-  if (rank == 0 && warp < CW && p > 0) critical(0, cols, 0);
-  for (int j = 0; j < p; ++j) {
-    cl.sync();  // reflector j formed; every CTA done with the previous step
-    {
-      // every load of the batch issued before any local store
-      constexpr int PB = 8;
-      const float2* g = reinterpret_cast<const float2*>(A + (size_t)j * m);
-      for (int i0 = j + tid; i0 < m; i0 += NT * PB) {
-        float2 tmp[PB];
-#pragma unroll
-        for (int u = 0; u < PB; ++u) {
-          const int i = i0 + u * NT;
-          if (i < m) tmp[u] = __ldcg(g + i);
-        }
-#pragma unroll
-        for (int u = 0; u < PB; ++u) {
-          const int i = i0 + u * NT;
-          if (i < m) vin[i] = (i == j) ? dw{1.0f, 0.0f} : dw{tmp[u].x, tmp[u].y};
-        }
-      }
-      if (tid == 0) {
-        const float2 tj = __ldcg(g + j);
-        *tin = {tj.x, tj.y};
-      }
-    }
-    __syncthreads();
-    const bool owner = j + 1 < p && rank == (j + 1) % CS;
-    if (owner && warp < CW) {
-      const int lc = (j + 1) / CS;
-      critical(j + 1, cols + (size_t)lc * m, lc);
-    } else {
-      const int wk = owner ? warp - CW : warp, nwk = owner ? NW - CW : NW;
-      const int lc0 = (j + 2 - rank + CS - 1) / CS > 0 ? (j + 2 - rank + CS - 1) / CS : 0;
-      for (int lc = lc0 + wk; lc < nown; lc += nwk) apply(j, cols + (size_t)lc * m);
-    }
-  }
-  cl.sync();  // every CTA is done with every published reflector
-  for (int lc = warp; lc < nown; lc += NW) {
-    const int k = rank + lc * CS;
-    const double sc = ldexp(1.0, cexp[lc]);
-    const dw* c = cols + (size_t)lc * m;
-    double* a = A + (size_t)k * m;
-    for (int i = lane; i < m; i += 32) a[i] = (k < p && i > k) ? dw_to(c[i]) : dw_to(c[i]) * sc;
-  }
-}
-template <int NT, int CW>
-__global__ void __launch_bounds__(NT) k_qr_factor_cl(double* A, int m, int n, double* tau) { k_qr_factor_cl_body<NT, CW>(A, m, n, tau); }
-
-static size_t qr_cl_smem(int m, int n, int CS) {
-  const size_t nmax = (size_t)(n + CS - 1) / CS;
-  return (nmax * m + (size_t)m + nmax + 1) * sizeof(dw) + nmax * sizeof(int);
-}
-
-template <int NT, int CW>
-static int launch_cl(vp_ctx* ctx, double* A, int m, int n, double* tau, int cs, size_t need) {
-  static AttrOnce cattr;
-  VP_TRY(cattr.ensure(ctx, (const void*)k_qr_factor_cl<NT, CW>, 200 * 1024, true));
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  cfg.gridDim = dim3(cs);
-  cfg.blockDim = dim3(NT);
-  cfg.dynamicSmemBytes = std::max<size_t>(need, 116 * 1024);  // one CTA of the cluster per SM
-  cfg.stream = ctx->stream;
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cs;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  ctx->launches++;
-  VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_qr_factor_cl<NT, CW>, A, m, n, tau));
-  return VP_OK;
-}
-
-int launch_qr_factor_cl(vp_ctx* ctx, double* A, int m, int n, double* tau, int cs) {
-  const size_t need = qr_cl_smem(m, n, cs);
-  if (need > 200 * 1024) return fail(ctx, VP_ECAPACITY, "qr_factor_cl: factor too large for the cluster");
-  return launch_cl<512, 4>(ctx, A, m, n, tau, cs, need);
-}
-
-static size_t qr_cdw_smem(int m, int n, int CS) {
-  const size_t nmax = (size_t)(n + CS - 1) / CS;
-  return (nmax * m + 2 * (size_t)m + 2) * sizeof(dw) + nmax * sizeof(int);
-}
-
-// Which kernel factors an m x n matrix.  Measured per column on GB300 (the
-// step's shapes): up to ~4e3 elements the small-factor kernel (one CTA up to
-// 32 columns, else two; ~2.3 us per column); above, the cluster kernel with
-// four critical warps on 16 CTAs (~3-5.5 us per column, against 3.7-17.7 for
-// the grid kernel); the grid kernel takes what no cluster's shared memory
-// holds.  Factors more
-// than twice as wide as tall: the m reflectors depend on the leading m
-// columns alone, so that square block (contiguous in the column-major layout)
-// is factored in place, Q is formed from its reflectors, and the rest of R is
-// one FP64 GEMM, R2 = Q^T A2 (stored as R2^T = A2^T Q, which is A2's
-// column-major layout), instead of applying every reflector to all n columns
-// one column step at a time.  The choice depends on the shape and the device
-// only, so that results do not depend on the context or on the batch.
+// Which kernel factors an m x n matrix.  Factors more than twice as wide as
+// tall: the m reflectors depend on the leading m columns alone, so that square
+// block (contiguous in the column-major layout) is factored in place, Q is
+// formed from its reflectors, and the rest of R is one FP64 GEMM, R2 = Q^T A2
+// (stored as R2^T = A2^T Q, which is A2's column-major layout), instead of
+// applying every reflector to all n columns.  Otherwise the panel QR; what has
+// more rows than its panel holds in registers goes to the grid kernel.  The
+// choice depends on the shape and the device only, so that results do not depend
+// on the context or on the batch.
 QRPlan qr_plan(const vp_ctx* ctx, int m, int n) {
-  if (std::min(m, n) <= 0) return {QR_NONE, 0};
-  if (n > 2 * m && m >= 2) return {QR_WIDE, 0};
-  if (ctx->cluster_size > 1 && (long long)m * n <= 4096) {
-    // one CTA up to 32 columns, else two (measured on GB300 for 2x2 .. 128x32
-    // and 50x50 .. 120x34: four CTAs were never faster; the result does not
-    // depend on the CTA count)
-    const int cs = n <= 32 ? 1 : 2;
-    if (qr_cdw_smem(m, n, cs) <= 200 * 1024) return {QR_CDW, cs};
-  }
-  if (ctx->cluster_size >= 8 && 2 * m >= n) {
-    // the largest cluster: with reflectors published through L2, 16 CTAs beat
-    // 8 by 10-21 % on every shape of the step (two problems per launch) and 4
-    // were never faster; the result does not depend on the CTA count
-    const int cs = ctx->cluster_size >= 16 ? 16 : 8;
-    if (qr_cl_smem(m, n, cs) <= 200 * 1024) return {QR_CL, cs};
-  }
-  return {QR_GRID, 0};
+  if (std::min(m, n) <= 0) return {QR_NONE, {}};
+  if (n > 2 * m && m >= 2) return {QR_WIDE, {}};
+  const PanelPlan pl = qr_panel_plan(ctx, m, n);
+  if (pl.kind != PANEL_NONE) return {QR_PANEL, pl};
+  return {QR_GRID, {}};
 }
 
 // The cooperative grid kernels, for factors beyond a cluster's shared memory:
@@ -758,27 +418,8 @@ int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* 
       VP_TRY(st);
       return launch_copy(ctx, ctx->w_wr.p, A + (size_t)m * m, rest);
     }
-    case QR_CDW: {
-      static AttrOnce cattr;
-      VP_TRY(cattr.ensure(ctx, (const void*)k_qr_factor_cdw, 200 * 1024, true));
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute at[1];
-      cfg.gridDim = dim3(pl.cs);
-      cfg.blockDim = dim3(kThreads);
-      cfg.dynamicSmemBytes = std::max<size_t>(qr_cdw_smem(m, n, pl.cs), 116 * 1024);  // one CTA of the cluster per SM
-      cfg.stream = ctx->stream;
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = pl.cs;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      ctx->launches++;
-      VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_qr_factor_cdw, A, m, n, tau));
-      return VP_OK;
-    }
-    case QR_CL:
-      return launch_qr_factor_cl(ctx, A, m, n, tau, pl.cs);
+    case QR_PANEL:
+      return blaunch_qr_panel(ctx, ctx->stream, {PanelJob{A, m, n, tau, pl.panel, &ctx->w_qrv, &ctx->w_qrc, ctx->status}});
     default:
       return qr_factor_grid(ctx, ctx->stream, ctx->status, ctx->w_qrv, ctx->w_qrc, A, m, n, tau, vbuf);
   }
@@ -2414,21 +2055,6 @@ int blaunch_to_colmajor(vp_ctx* ctx, cudaStream_t st, const std::vector<BColMajo
 }
 
 // --------------------------------------------------------------- QR
-struct QRArgs {
-  double* A;
-  int m, n;
-  double* tau;
-};
-__global__ void __launch_bounds__(kThreads) kb_qr_factor_cdw(const __grid_constant__ Pack<QRArgs> pk) {
-  const QRArgs& a = pk.a[blockIdx.y];
-  k_qr_factor_cdw_body(a.A, a.m, a.n, a.tau);
-}
-template <int NT, int CW>
-__global__ void __launch_bounds__(NT) kb_qr_factor_cl(const __grid_constant__ Pack<QRArgs> pk) {
-  const QRArgs& a = pk.a[blockIdx.y];
-  k_qr_factor_cl_body<NT, CW>(a.A, a.m, a.n, a.tau);
-}
-
 // Several grid factors in one cooperative launch: problem i owns blocks
 // first .. first + nblocks - 1 and runs k_qr_factor_dw's body on them as if
 // they were its whole grid (the result does not depend on the block count).
@@ -2491,29 +2117,17 @@ static int grid_qr_batch(vp_ctx* ctx, cudaStream_t st, const std::vector<const B
 int blaunch_qr_factor(vp_ctx* ctx, cudaStream_t st, const std::vector<BQR>& v) {
   std::vector<BQR> wide;
   std::vector<const BQR*> grid;
-  std::vector<QRArgs> cdw[17], cl[17];
-  size_t cdw_smem[17] = {}, cl_smem[17] = {};
-  // More than four cluster factors in one call: 8-CTA clusters where they fit,
-  // so that twice as many problems run side by side (the result does not
-  // depend on the CTA count).
-  int ncl = 0;
-  for (const BQR& q : v) ncl += qr_plan(ctx, q.m, q.n).kind == QR_CL;
+  std::vector<PanelJob> panel;
   for (const BQR& q : v) {
-    QRPlan pl = qr_plan(ctx, q.m, q.n);
-    if (pl.kind == QR_CL && ncl > 4 && pl.cs > 8 && qr_cl_smem(q.m, q.n, 8) <= 200 * 1024) pl.cs = 8;
+    const QRPlan pl = qr_plan(ctx, q.m, q.n);
     switch (pl.kind) {
       case QR_NONE:
         break;
       case QR_WIDE:
         wide.push_back(q);
         break;
-      case QR_CDW:
-        cdw[pl.cs].push_back({q.A, q.m, q.n, q.tau});
-        cdw_smem[pl.cs] = std::max(cdw_smem[pl.cs], qr_cdw_smem(q.m, q.n, pl.cs));
-        break;
-      case QR_CL:
-        cl[pl.cs].push_back({q.A, q.m, q.n, q.tau});
-        cl_smem[pl.cs] = std::max(cl_smem[pl.cs], qr_cl_smem(q.m, q.n, pl.cs));
+      case QR_PANEL:
+        panel.push_back({q.A, q.m, q.n, q.tau, pl.panel, &q.s->qrv, &q.s->qrc, q.s->st});
         break;
       default:
         if (!q.s || !q.s->st) return fail(ctx, VP_EINVAL, "batched QR: no status words for a grid factor");
@@ -2523,20 +2137,7 @@ int blaunch_qr_factor(vp_ctx* ctx, cudaStream_t st, const std::vector<BQR>& v) {
           VP_TRY(qr_factor_grid(ctx, st, q.s->st, q.s->qrv, q.s->qrc, q.A, q.m, q.n, q.tau, q.vbuf));
     }
   }
-  for (int cs = 1; cs <= 16; ++cs) {
-    if (!cdw[cs].empty()) {
-      static AttrOnce a;
-      VP_TRY(a.ensure(ctx, (const void*)kb_qr_factor_cdw, 200 * 1024, true));
-      VP_TRY(run_cluster_packs(ctx, st, cdw[cs], kb_qr_factor_cdw, cs, kThreads,
-                               std::max<size_t>(cdw_smem[cs], 116 * 1024)));
-    }
-    if (!cl[cs].empty()) {
-      static AttrOnce a;
-      VP_TRY(a.ensure(ctx, (const void*)kb_qr_factor_cl<512, 4>, 200 * 1024, true));
-      VP_TRY(run_cluster_packs(ctx, st, cl[cs], kb_qr_factor_cl<512, 4>, cs, 512,
-                               std::max<size_t>(cl_smem[cs], 116 * 1024)));
-    }
-  }
+  VP_TRY(blaunch_qr_panel(ctx, st, panel));
   if (!grid.empty()) VP_TRY(grid_qr_batch(ctx, st, grid));
   if (!wide.empty()) {  // the square block, its Q, R2^T = A2^T Q in FP64, copied back (see qr_plan)
     std::vector<BQR> sq;
