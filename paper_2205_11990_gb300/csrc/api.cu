@@ -340,15 +340,17 @@ static int qr_sweep(vp_ctx* ctx, mps_t* s, int kend) {
 // already right-canonical: M = core_k (r_k x 2 r_{k+1}); keep r singular
 // triplets (truncation rule of the truncation-error equation).
 //
-// The SVD is one-sided Jacobi on a preconditioned square factor.  With A = M
-// (tall) or M^T (wide), q = min(r_k, 2 r_{k+1}):  A Pi = Q1 R1 (columns
-// ordered by decreasing norm, Householder QR), R1^T = Q2 L^T (second QR),
-// then Jacobi on the rows of the lower-triangular L (graded, so it converges
-// in far fewer sweeps than on M itself).  L = U_L S V_L^T gives
-//   tall: M = Q1 U_L S (Pi Q2 V_L)^T  ->  core_{k-1} <- P Q1 U_L S,
-//         core_k <- (V_L^T Q2^T) with columns scattered back by Pi;
-//   wide: M = Pi Q2 V_L S (Q1 U_L)^T ->  core_k <- U_L^T Q1^T,
-//         core_{k-1} <- P Pi (Q2 V_L S).
+// M = U S V^T: core_k <- V^T, and core_{k-1} <- core_{k-1} U S with U S = M V.
+// V comes from a one-sided Jacobi SVD of the rows of a preconditioned square
+// factor X, q = min(r_k, 2 r_{k+1}), whose right singular vectors it shares up to
+// known orthogonal factors (columns ordered by decreasing norm before each QR):
+//   tall: M Pi = Q1 R1,  R1^T = Q2 L^T,  L Pi2 = Q3 X:  V^T = Pi (Q2 Pi2 V_X)^T;
+//   wide: M^T Pi = Q1 R1,  R1^T Pi2 = Q2 X:  V^T = (Q1 Pi2 V_X)^T, since V_X holds
+//         the left singular vectors of R1.
+// The last QR costs nothing afterwards (it acts on the left), and Jacobi on its
+// R needs about 0.6 of the sweeps on L (tall) and 0.75 (wide): over 24 factors of
+// 1024 x 1024 and 256 x 256 steps, 108 rows 12 -> 7, 56: 11 -> 6, 30: 8 -> 4, 64:
+// 9 -> 6.  Neither the rotations nor Q1 (tall) or Q2 (wide) are needed.
 static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* err_out, double* sig_out = nullptr) {
   const int m = s->r[k];
   const int c = 2 * s->r[k + 1];
@@ -356,67 +358,73 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
   const bool tall = m >= c;
   const int q = tall ? c : m;  // square factor size
   const int p = tall ? m : c;  // long side of A
-  VP_TRY(reserve(ctx, ctx->w_piv, (size_t)q / 2 + 8));
+  VP_TRY(reserve(ctx, ctx->w_piv, (size_t)q + 8));
   int* piv = (int*)ctx->w_piv.p;
+  int* piv2 = piv + q;
   VP_TRY(launch_norm_order(ctx, s->core[k].p, m, c, tall ? 1 : 0, piv));
-  // first QR: A Pi = Q1 R1
+  // first QR: A Pi = Q1 R1, A = M or M^T
   VP_TRY(reserve(ctx, ctx->w_fac, (size_t)p * q));
   VP_TRY(reserve(ctx, ctx->w_p, (size_t)2 * p + q + 8));
   VP_TRY(launch_gather_cm(ctx, s->core[k].p, m, c, piv, tall ? 1 : 0, ctx->w_fac.p));
   prof_begin(ctx, VP_K_QR);
   VP_TRY(launch_qr_factor(ctx, ctx->w_fac.p, p, q, ctx->w_p.p, ctx->w_p.p + q + 8));
   prof_end(ctx, VP_K_QR, qr_flops(p, q), p, q);
-  VP_TRY(reserve(ctx, ctx->w_q1, (size_t)p * q));
-  // second QR: R1^T = Q2 L^T (R1 row-major is R1^T column-major)
   VP_TRY(reserve(ctx, ctx->w_r, (size_t)q * q));
   VP_TRY(launch_qr_getr(ctx, ctx->w_fac.p, p, q, ctx->w_r.p));
   VP_TRY(reserve(ctx, ctx->w_p2, (size_t)3 * q + 8));
-  prof_begin(ctx, VP_K_QR);
-  VP_TRY(launch_qr_factor(ctx, ctx->w_r.p, q, q, ctx->w_p2.p, ctx->w_p2.p + q + 8));
-  prof_end(ctx, VP_K_QR, qr_flops(q, q), q, q);
-  VP_TRY(reserve(ctx, ctx->w_q2, (size_t)q * q));
-  // Q1, Q2 (and, tall, P Q1) only feed the outputs: form them on the side
-  // stream while the Jacobi SVD runs.  Their scratch is reserved up front so
-  // nothing is reallocated while the two streams run.
-  if (tall) VP_TRY(reserve(ctx, ctx->w_tmp2, (size_t)pl * q));
+  VP_TRY(reserve(ctx, ctx->w_p3, (size_t)3 * q + 8));
+  VP_TRY(reserve(ctx, ctx->w_x, (size_t)q * q));
+  double* fac = ctx->w_fac.p;  // factor whose Q the output needs
+  double* tau = ctx->w_p.p;
+  int qm = p;
+  if (tall) {  // second QR: R1^T = Q2 L^T (R1 row-major is R1^T column-major)
+    prof_begin(ctx, VP_K_QR);
+    VP_TRY(launch_qr_factor(ctx, ctx->w_r.p, q, q, ctx->w_p2.p, ctx->w_p2.p + q + 8));
+    prof_end(ctx, VP_K_QR, qr_flops(q, q), q, q);
+    fac = ctx->w_r.p;
+    tau = ctx->w_p2.p;
+    qm = q;
+  }
+  // the Q of the output only feeds the output: formed on the side stream while
+  // the preconditioning and the Jacobi SVD run
+  VP_TRY(reserve(ctx, ctx->w_q1, (size_t)qm * q));
   VP_TRY(ensure_side(ctx));
-  VP_TRY(reserve(ctx, ctx->w_q_side, (size_t)std::max(p, q) * q));
-  VP_TRY(reserve(ctx, ctx->w_split_side, (size_t)pl * q * 33));
   VP_CUDA(ctx, cudaEventRecord(ctx->ev_fork, ctx->stream));
   VP_CUDA(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+  int side_st = VP_OK;
   {
     SideScope side(ctx);
     prof_begin(ctx, VP_K_FORMQ);
-    VP_TRY(launch_qr_formq(ctx, ctx->w_fac.p, p, q, ctx->w_p.p, ctx->w_q1.p));
-    prof_end(ctx, VP_K_FORMQ, 4.0 * p * q * q - 4.0 / 3.0 * q * q * q, p, q);
-    prof_begin(ctx, VP_K_FORMQ);
-    VP_TRY(launch_qr_formq(ctx, ctx->w_r.p, q, q, ctx->w_p2.p, ctx->w_q2.p));
-    prof_end(ctx, VP_K_FORMQ, 8.0 / 3.0 * q * q * q, q, q);
-    if (tall) VP_TRY(launch_gemm(ctx, pl, q, m, 1.0, s->core[k - 1].p, m, ctx->w_q1.p, q, ctx->w_tmp2.p, q));
+    side_st = launch_qr_formq(ctx, fac, qm, q, tau, ctx->w_q1.p);
+    prof_end(ctx, VP_K_FORMQ, 4.0 * qm * q * q - 4.0 / 3.0 * q * q * q, qm, q);
   }
   VP_CUDA(ctx, cudaEventRecord(ctx->ev_join, ctx->side));
   // every exit from here on makes the context's stream wait for the side
-  // stream's products (the normal path joins before the outputs, again below)
+  // stream's product (the normal path joins before the outputs, again below)
   struct SideJoin {
     vp_ctx* c;
     ~SideJoin() { cudaStreamWaitEvent(c->stream, c->ev_join, 0); }
   } side_join{ctx};
-  VP_TRY(reserve(ctx, ctx->w_tmp, (size_t)q * q));
-  double* X = ctx->w_tmp.p;
-  VP_TRY(launch_lower_from_upper(ctx, ctx->w_r.p, q, X));
-  // Jacobi on the rows of L.  Tall case: no rotation accumulator; U_L S = L V_L
-  // is recovered afterwards from a saved copy of L.
-  double* Lsave = nullptr;
+  VP_TRY(side_st);
+  // last QR, from the left: its R (columns ordered) is what Jacobi diagonalises
   if (tall) {
     VP_TRY(reserve(ctx, ctx->w_l, (size_t)q * q));
-    VP_TRY(launch_copy(ctx, X, ctx->w_l.p, (size_t)q * q));
-    Lsave = ctx->w_l.p;
-  } else {
-    VP_TRY(reserve(ctx, ctx->w_j, (size_t)q * q));
+    VP_TRY(launch_lower_from_upper(ctx, ctx->w_r.p, q, ctx->w_l.p));
+    VP_TRY(launch_norm_order(ctx, ctx->w_l.p, q, q, 1, piv2));
+    VP_TRY(launch_gather_cm(ctx, ctx->w_l.p, q, q, piv2, 1, ctx->w_x.p));
+  } else {  // columns of R1^T are rows of R1
+    VP_TRY(launch_norm_order(ctx, ctx->w_r.p, q, q, 0, piv2));
+    VP_TRY(launch_gather_cm(ctx, ctx->w_r.p, q, q, piv2, 0, ctx->w_x.p));
   }
+  prof_begin(ctx, VP_K_QR);
+  VP_TRY(launch_qr_factor(ctx, ctx->w_x.p, q, q, ctx->w_p3.p, ctx->w_p3.p + q + 8));
+  prof_end(ctx, VP_K_QR, qr_flops(q, q), q, q);
+  VP_TRY(reserve(ctx, ctx->w_tmp, (size_t)q * q));
+  double* X = ctx->w_tmp.p;
+  VP_TRY(launch_qr_getr(ctx, ctx->w_x.p, q, q, X));
   VP_CUDA(ctx, cudaMemsetAsync(ctx->status->rot, 0, sizeof(ctx->status->rot), ctx->stream));
   prof_begin(ctx, VP_K_JACOBI);
-  VP_TRY(launch_jacobi_rows(ctx, X, q, q, tall ? nullptr : ctx->w_j.p, tol >= 1e-13));
+  VP_TRY(launch_jacobi_rows(ctx, X, q, q, tol >= 1e-13));
   prof_end(ctx, VP_K_JACOBI, 0.0, q, q);
   const size_t jac_mark = ctx->prof_on && !ctx->prof_marks.empty() ? ctx->prof_marks.size() - 1 : (size_t)-1;
   VP_TRY(reserve(ctx, ctx->w_vec, (size_t)2 * q + 8));
@@ -431,44 +439,40 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
   if (err_out) *err_out = err;
   if (g_entropy) g_entropy[k - 1] = ctx->h_smalld[1];
   if (sig_out) VP_TRY(launch_copy(ctx, sigma, sig_out, (size_t)r));
-  const double jac = q > 1 ? (double)ctx->h_small[61] * 0.5 * q * (q - 1) * (6.0 * q + (tall ? 0.0 : 4.0 * q)) : 0.0;
+  const double jac = q > 1 ? (double)ctx->h_small[61] * 0.5 * q * (q - 1) * 6.0 * q : 0.0;
   if (ctx->prof_on) ctx->prof_work[VP_K_JACOBI] += jac;
   if (jac_mark != (size_t)-1 && jac_mark < ctx->prof_marks.size()) ctx->prof_marks[jac_mark].k = ctx->h_small[61];
-  double gem = 0.0;
   VP_TRY(reserve(ctx, ctx->w_a, (size_t)r * q + 8));
-  VP_TRY(reserve(ctx, ctx->w_b, (size_t)q * r + 8));
+  VP_TRY(reserve(ctx, ctx->w_b, (size_t)m * r + 8));
+  VP_TRY(reserve(ctx, ctx->w_tmp2, (size_t)r * c));
+  VP_TRY(reserve(ctx, ctx->w_gemm, (size_t)pl * r));
   VP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
   prof_begin(ctx, VP_K_GEMM);
+  double* Vt = ctx->w_tmp2.p;  // the new core k (r x c)
+  VP_TRY(launch_svd_outputs(ctx, X, q, r, perm, sigma, piv2, ctx->w_a.p));
+  // V^T enters both cores: FP64 in every contraction mode
+  const int prec = ctx->precision;
+  ctx->precision = VP_PREC_FP64;
+  int st = VP_OK;
   if (tall) {
-    // P1 = P Q1 (pl x q); core_{k-1} <- P1 (U_L S); core_k <- scatter(V_L^T Q2^T)
-    VP_TRY(launch_svd_outputs(ctx, X, nullptr, q, q, r, perm, sigma, ctx->w_a.p, nullptr));
-    VP_TRY(launch_gemm_bt(ctx, q, r, q, Lsave, q, ctx->w_a.p, q, ctx->w_b.p, r));  // U_L S = L V_L
-    VP_TRY(reserve(ctx, ctx->w_gemm, (size_t)pl * r));
-    VP_TRY(launch_gemm(ctx, pl, r, q, 1.0, ctx->w_tmp2.p, q, ctx->w_b.p, r, ctx->w_gemm.p, r));
-    VP_TRY(reserve(ctx, ctx->w_c, (size_t)r * q));
-    VP_TRY(launch_gemm_bt(ctx, r, q, q, ctx->w_a.p, q, ctx->w_q2.p, q, ctx->w_c.p, q));
-    VP_TRY(reserve(ctx, s->core[k], (size_t)r * c));
-    VP_TRY(launch_scatter(ctx, ctx->w_c.p, r, q, piv, 1, s->core[k].p));
-    gem = 2.0 * pl * q * m + 2.0 * pl * r * q + 2.0 * r * q * q + 2.0 * q * q * r;
+    st = reserve(ctx, ctx->w_c, (size_t)r * q);
+    if (st == VP_OK) st = launch_gemm_bt(ctx, r, q, q, ctx->w_a.p, q, ctx->w_q1.p, q, ctx->w_c.p, q);
+    if (st == VP_OK) st = launch_scatter(ctx, ctx->w_c.p, r, q, piv, 1, Vt);
   } else {
-    // core_k <- U_L^T Q1^T (r x c); core_{k-1} <- P Pi (Q2 V_L S)
-    VP_TRY(launch_svd_outputs_wide(ctx, X, ctx->w_j.p, q, r, perm, ctx->w_a.p, ctx->w_b.p));
-    VP_TRY(reserve(ctx, s->core[k], (size_t)r * c));
-    VP_TRY(launch_gemm_bt(ctx, r, c, m, ctx->w_a.p, m, ctx->w_q1.p, m, s->core[k].p, c));
-    VP_TRY(reserve(ctx, ctx->w_c, (size_t)m * r));
-    VP_TRY(launch_gemm(ctx, m, r, m, 1.0, ctx->w_q2.p, m, ctx->w_b.p, r, ctx->w_c.p, r));
-    VP_TRY(reserve(ctx, ctx->w_tmp2, (size_t)m * r));
-    VP_TRY(launch_scatter(ctx, ctx->w_c.p, m, r, piv, 0, ctx->w_tmp2.p));
-    VP_TRY(reserve(ctx, ctx->w_gemm, (size_t)pl * r));
-    VP_TRY(launch_gemm(ctx, pl, r, m, 1.0, s->core[k - 1].p, m, ctx->w_tmp2.p, r, ctx->w_gemm.p, r));
-    gem = 2.0 * r * c * m + 2.0 * m * r * m + 2.0 * pl * r * m;
+    st = launch_gemm_bt(ctx, r, c, q, ctx->w_a.p, q, ctx->w_q1.p, q, Vt, c);
   }
+  ctx->precision = prec;
+  VP_TRY(st);
+  VP_TRY(launch_gemm_bt(ctx, m, r, c, s->core[k].p, c, Vt, c, ctx->w_b.p, r));  // U S = M V
+  VP_TRY(launch_gemm(ctx, pl, r, m, 1.0, s->core[k - 1].p, m, ctx->w_b.p, r, ctx->w_gemm.p, r));
+  const double gem = 2.0 * r * c * q + 2.0 * m * r * c + 2.0 * pl * r * m;
   prof_end(ctx, VP_K_GEMM, gem, q, r, pl);
+  std::swap(s->core[k], ctx->w_tmp2);
   std::swap(s->core[k - 1], ctx->w_gemm);
   s->r[k] = r;
   if (g_flops) {
-    g_flops->qr += qr_flops(p, q) + qr_flops(q, q);
-    g_flops->formq += 4.0 * p * q * q - 4.0 / 3.0 * q * q * q + 8.0 / 3.0 * q * q * q;
+    g_flops->qr += qr_flops(p, q) + (tall ? 2.0 : 1.0) * qr_flops(q, q);
+    g_flops->formq += 4.0 * qm * q * q - 4.0 / 3.0 * q * q * q;
     g_flops->jacobi += jac;
     g_flops->gemm += gem;
   }
@@ -841,8 +845,8 @@ int vp_ctx_create(void* cuda_stream, vp_alloc_fn alloc, vp_free_fn free_fn, void
 int vp_ctx_destroy(vp_ctx* c) {
   if (!c) return VP_EINVAL;
   cudaStreamSynchronize(c->stream);
-  for (DevBuf* b : {&c->w_fac, &c->w_q, &c->w_gemm, &c->w_j, &c->w_p, &c->w_tmp, &c->w_tmp2, &c->w_vec, &c->w_split,
-                    &c->w_piv, &c->w_q1, &c->w_q2, &c->w_r, &c->w_p2, &c->w_a, &c->w_b, &c->w_c, &c->w_l,
+  for (DevBuf* b : {&c->w_fac, &c->w_q, &c->w_gemm, &c->w_x, &c->w_p3, &c->w_p, &c->w_tmp, &c->w_tmp2, &c->w_vec, &c->w_split,
+                    &c->w_piv, &c->w_q1, &c->w_r, &c->w_p2, &c->w_a, &c->w_b, &c->w_c, &c->w_l,
                     &c->w_q_side, &c->w_split_side, &c->w_tca, &c->w_tcb, &c->w_tca_side, &c->w_tcb_side,
                     &c->w_qrv, &c->w_qrc, &c->w_fq, &c->w_fq_side, &c->w_fac_b, &c->w_p_b,
                     &c->w_sig, &c->w_wq, &c->w_wr})

@@ -86,8 +86,8 @@ struct vp_ctx {
   double prof_work[VP_K_COUNT] = {};
   int64_t prof_launches[VP_K_COUNT] = {};
   // workspaces
-  vp::DevBuf w_fac, w_q, w_gemm, w_j, w_p, w_tmp, w_tmp2, w_vec, w_split;
-  vp::DevBuf w_piv, w_q1, w_q2, w_r, w_p2, w_a, w_b, w_c, w_l;  // preconditioned SVD
+  vp::DevBuf w_fac, w_q, w_gemm, w_p, w_tmp, w_tmp2, w_vec, w_split;
+  vp::DevBuf w_piv, w_q1, w_r, w_p2, w_x, w_p3, w_a, w_b, w_c, w_l;  // preconditioned SVD
   vp::DevBuf w_tca, w_tcb;            // packed operands (or digits) of the tensor-core contractions
   vp::DevBuf w_q_side, w_split_side;  // scratch of the side-stream phase
   vp::DevBuf w_tca_side, w_tcb_side;
@@ -219,8 +219,6 @@ int launch_norm_order(vp_ctx* ctx, const double* M, int m, int c, int by_cols, i
 int launch_gather_cm(vp_ctx* ctx, const double* M, int m, int c, const int* piv, int tall, double* out);
 int launch_lower_from_upper(vp_ctx* ctx, const double* Rcm, int q, double* L);
 int launch_scatter(vp_ctx* ctx, const double* Y, int rows, int cols_n, const int* piv, int cols, double* out);
-int launch_svd_outputs_wide(vp_ctx* ctx, const double* X, const double* J, int b, int r, const int* perm,
-                            double* Urows, double* Wv);
 // Operand of a tensor-core contraction as (row, k) -> value: kind 0
 // p[r * ld + k]; kind 1 p[k * ld + r]; kind 2 the upper triangle of a
 // column-major factor, r <= k ? p[k * ld + r] : 0.
@@ -258,15 +256,13 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);
 // C = alpha * triu(A_colmajor) (M x K) * B: the R factor read in place.
 int launch_gemm_r(vp_ctx* ctx, int M, int N, int K, const double* Acm, int lda, const double* B,
                   int ldb, double* C, int ldc);
-// One-sided Jacobi on the b rows (length c) of X, rotations also applied to
-// the rows of J (b x b, set to the identity here).  Row-major, contiguous.
+// One-sided Jacobi on the b rows (length c) of X.  Row-major, contiguous.
 // floor_ok: the caller truncates every singular value below 1e-13 of the
 // largest (tol >= 1e-13), so the double-word kernel, which leaves rows under
 // 1e-15 of the largest unrotated, may be used.
-int launch_jacobi_rows(vp_ctx* ctx, double* X, int b, int c, double* J, bool floor_ok);
+int launch_jacobi_rows(vp_ctx* ctx, double* X, int b, int c, bool floor_ok);
 // The same on a given stream with given status words.
-int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* X, int b, int c, double* J,
-                   bool floor_ok);
+int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* X, int b, int c, bool floor_ok);
 // Largest cluster (16 or 8 CTAs, one per SM) the cluster-resident kernels
 // can use on this device; 0 if none.
 int probe_cluster_size();
@@ -274,9 +270,9 @@ int probe_cluster_size();
 // write perm/sigma/rank/truncation error into ctx scratch.  d_out[0] = rank.
 int launch_select(vp_ctx* ctx, const double* X, int b, int c, int chi, double tol, int* perm,
                   double* sigma, int* d_rank, double* d_err);
-// Vt (r x c) = X[perm[t]] / sigma[t];  W (b x r) = J[perm[t]][i] * sigma[t].
-int launch_svd_outputs(vp_ctx* ctx, const double* X, const double* J, int b, int c, int r,
-                       const int* perm, const double* sigma, double* Vt, double* W);
+// V (r x q), V[t][cperm[j]] = X[perm[t]][j] / sigma[t].
+int launch_svd_outputs(vp_ctx* ctx, const double* X, int q, int r, const int* perm, const double* sigma,
+                       const int* cperm, double* V);
 
 // ------------------------------------------------------------ kernels (mpsops.cu)
 // out = alpha*a + beta*(B b) on one site (a may be NULL: pure apply; B may be
@@ -375,12 +371,11 @@ struct BNormOrder { const double* M; int m, c, by_cols; int* piv; };
 struct BGather { const double* M; int m, c; const int* piv; int tall; double* out; };
 struct BLowerUpper { const double* R; int q; double* L; };
 struct BCopy { const double* src; double* dst; size_t n; };
-struct BJacobi { double* X; int b, c; double* J; DevStatus* st; };
+struct BJacobi { double* X; int b, c; DevStatus* st; };
 struct BSelect {
   const double* X; int b, c, chi; double tol; int* perm; double* sigma; int* d_rank; double* d_err; DevStatus* st;
 };
-struct BSvdOut { const double* X; const double* J; int b, c, r; const int* perm; const double* sigma; double* Vt; double* W; };
-struct BSvdOutWide { const double* X; const double* J; int b, r; const int* perm; double* U; double* Wv; };
+struct BSvdOut { const double* X; int q, r; const int* perm; const double* sigma; const int* cperm; double* V; };
 struct BScatter { const double* Y; int rows, cols_n; const int* piv; int cols; double* out; };
 
 int blaunch_to_colmajor(vp_ctx* ctx, cudaStream_t st, const std::vector<BColMajor>& v);
@@ -391,11 +386,13 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v);
 int blaunch_norm_order(vp_ctx* ctx, cudaStream_t st, const std::vector<BNormOrder>& v);
 int blaunch_gather_cm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGather>& v);
 int blaunch_lower_from_upper(vp_ctx* ctx, cudaStream_t st, const std::vector<BLowerUpper>& v);
-// Jacobi of truncating compressions (tol >= 1e-13: the double-word kernel).
+// Jacobi of truncating compressions (tol >= 1e-13: the double-word kernel of
+// jacobi.cu where the rows fit a cluster).
+bool jacobi_dw_fits(const vp_ctx* ctx, int b, int c);
+int blaunch_jacobi_dw(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v);
 int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v);
 int blaunch_select(vp_ctx* ctx, cudaStream_t st, const std::vector<BSelect>& v);
 int blaunch_svd_outputs(vp_ctx* ctx, cudaStream_t st, const std::vector<BSvdOut>& v);
-int blaunch_svd_outputs_wide(vp_ctx* ctx, cudaStream_t st, const std::vector<BSvdOutWide>& v);
 int blaunch_scatter(vp_ctx* ctx, cudaStream_t st, const std::vector<BScatter>& v);
 
 // mpsops.cu

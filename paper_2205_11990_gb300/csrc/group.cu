@@ -46,13 +46,13 @@ struct TaskDev {
 // Workspaces of one compression problem (device, grow-only).
 struct Work {
   DevBuf F[2], P[2], gemm;                                       // QR sweep
-  DevBuf piv, fac, p, q1, r, p2, q2, tmp, tmp2, l, j, vec, a, b, c;  // SVD site
+  DevBuf piv, fac, p, q1, r, p2, p3, x, tmp, tmp2, l, vec, a, b, c;  // SVD site
   BScratch main, side;                                           // scratch of the batched launchers
 };
 
 void release_work(vp_ctx* ctx, Work& w) {
-  for (DevBuf* b : {&w.F[0], &w.F[1], &w.P[0], &w.P[1], &w.gemm, &w.piv, &w.fac, &w.p, &w.q1, &w.r, &w.p2, &w.q2,
-                    &w.tmp, &w.tmp2, &w.l, &w.j, &w.vec, &w.a, &w.b, &w.c})
+  for (DevBuf* b : {&w.F[0], &w.F[1], &w.P[0], &w.P[1], &w.gemm, &w.piv, &w.fac, &w.p, &w.q1, &w.r, &w.p2, &w.p3,
+                    &w.x, &w.tmp, &w.tmp2, &w.l, &w.vec, &w.a, &w.b, &w.c})
     release(ctx, *b);
   release_scratch(ctx, w.main);
   release_scratch(ctx, w.side);
@@ -303,14 +303,12 @@ int svd_sweep(vp_group* g, const Tasks& all) {
     for (Task* t : all)
       if (t->s->n - 1 - jstep >= 1 && alive(g, t)) ts.push_back(t);
     if (ts.empty()) continue;
-    std::vector<BNormOrder> no;
-    std::vector<BGather> ga;
-    std::vector<BQR> qr1, qr2;
-    std::vector<BGetR> gr;
+    std::vector<BNormOrder> no, no2;
+    std::vector<BGather> ga, ga2;
+    std::vector<BQR> qr1, qr2, qr3;
+    std::vector<BGetR> gr, gx;
     std::vector<BFormQ> fq;
-    std::vector<BGemm> pq;
     std::vector<BLowerUpper> lu;
-    std::vector<BCopy> cp;
     std::vector<BJacobi> jc;
     std::vector<BSelect> se;
     for (Task* t : ts) {
@@ -325,53 +323,55 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       t->tall = t->m >= t->c;
       t->q = t->tall ? t->c : t->m;
       t->p = t->tall ? t->m : t->c;
-      const int q = t->q, p = t->p, m = t->m, c = t->c, pl = t->pl;
+      const int q = t->q, p = t->p, m = t->m, c = t->c;
       const bool inner = t->pairs && (k & 1);  // bond inside an IG pair
       const int chi = inner ? 1 << 30 : t->chi;
       const double tol = inner ? std::min(t->tol, kPairTolG) : t->tol;
-      VP_TRY(reserve(ctx, w.piv, (size_t)q / 2 + 8));
+      VP_TRY(reserve(ctx, w.piv, (size_t)q + 8));
       VP_TRY(reserve(ctx, w.fac, (size_t)p * q));
       VP_TRY(reserve(ctx, w.p, (size_t)2 * p + q + 8));
-      VP_TRY(reserve(ctx, w.q1, (size_t)p * q));
+      VP_TRY(reserve(ctx, w.q1, (size_t)(t->tall ? q : p) * q));
       VP_TRY(reserve(ctx, w.r, (size_t)q * q));
       VP_TRY(reserve(ctx, w.p2, (size_t)3 * q + 8));
-      VP_TRY(reserve(ctx, w.q2, (size_t)q * q));
-      if (t->tall) VP_TRY(reserve(ctx, w.tmp2, (size_t)pl * q));
+      VP_TRY(reserve(ctx, w.p3, (size_t)3 * q + 8));
+      VP_TRY(reserve(ctx, w.x, (size_t)q * q));
       VP_TRY(reserve(ctx, w.tmp, (size_t)q * q));
-      if (t->tall)
-        VP_TRY(reserve(ctx, w.l, (size_t)q * q));
-      else
-        VP_TRY(reserve(ctx, w.j, (size_t)q * q));
+      if (t->tall) VP_TRY(reserve(ctx, w.l, (size_t)q * q));
       VP_TRY(reserve(ctx, w.vec, (size_t)2 * q + 8));
       int* piv = (int*)w.piv.p;
+      int* piv2 = piv + q;
       no.push_back({s->core[k].p, m, c, t->tall ? 1 : 0, piv});
       ga.push_back({s->core[k].p, m, c, piv, t->tall ? 1 : 0, w.fac.p});
       qr1.push_back({w.fac.p, p, q, w.p.p, w.p.p + q + 8, &w.main});
       gr.push_back({w.fac.p, p, q, w.r.p});
-      qr2.push_back({w.r.p, q, q, w.p2.p, w.p2.p + q + 8, &w.main});
-      fq.push_back({w.fac.p, p, q, w.p.p, w.q1.p, &w.side});
-      fq.push_back({w.r.p, q, q, w.p2.p, w.q2.p, &w.side});
-      if (t->tall)
-        pq.push_back({BG_AB, t->fp32, pl, q, m, 1.0, s->core[k - 1].p, m, w.q1.p, q, w.tmp2.p, q, &w.side});
-      lu.push_back({w.r.p, q, w.tmp.p});
-      if (t->tall) cp.push_back({w.tmp.p, w.l.p, (size_t)q * q});
+      if (t->tall) {
+        qr2.push_back({w.r.p, q, q, w.p2.p, w.p2.p + q + 8, &w.main});
+        fq.push_back({w.r.p, q, q, w.p2.p, w.q1.p, &w.side});
+        lu.push_back({w.r.p, q, w.l.p});
+        no2.push_back({w.l.p, q, q, 1, piv2});
+        ga2.push_back({w.l.p, q, q, piv2, 1, w.x.p});
+      } else {
+        fq.push_back({w.fac.p, p, q, w.p.p, w.q1.p, &w.side});
+        no2.push_back({w.r.p, q, q, 0, piv2});
+        ga2.push_back({w.r.p, q, q, piv2, 0, w.x.p});
+      }
+      qr3.push_back({w.x.p, q, q, w.p3.p, w.p3.p + q + 8, &w.main});
+      gx.push_back({w.x.p, q, q, w.tmp.p});
       TaskDev* rec = g->d_task + t->slot;
-      jc.push_back({w.tmp.p, q, q, t->tall ? nullptr : w.j.p, &rec->st});
+      jc.push_back({w.tmp.p, q, q, &rec->st});
       int* perm = (int*)w.vec.p;
       double* sigma = w.vec.p + (q + 1) / 2 + 4;
       se.push_back({w.tmp.p, q, q, chi, tol, perm, sigma, &rec->rank, &rec->err, &rec->st});
     }
-    double wq = 0, wf = 0, wp = 0;
+    double wq = 0, wf = 0;
     for (Task* t : ts) {
-      const double p = t->p, q = t->q;
-      const double a = qr_flops(p, q) + qr_flops(q, q), f = 4.0 * p * q * q - 4.0 / 3.0 * q * q * q + 8.0 / 3.0 * q * q * q;
-      const double gm = t->tall ? 2.0 * t->pl * q * t->m : 0.0;
-      account(g, t, a, f, gm, 0.0);
+      const double p = t->p, q = t->q, qm = t->tall ? q : p;
+      const double a = qr_flops(p, q) + (t->tall ? 2.0 : 1.0) * qr_flops(q, q), f = 4.0 * qm * q * q - 4.0 / 3.0 * q * q * q;
+      account(g, t, a, f, 0.0, 0.0);
       wq += a;
       wf += f;
-      wp += gm;
     }
-    // A Pi = Q1 R1, R1^T = Q2 L^T
+    // A Pi = Q1 R1; tall: R1^T = Q2 L^T (see api.cu's svd_site)
     VP_TRY(blaunch_norm_order(ctx, ctx->stream, no));
     VP_TRY(blaunch_gather_cm(ctx, ctx->stream, ga));
     VP_TRY(timed(ctx, VP_K_QR, wq, [&] {
@@ -380,21 +380,24 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       if (st == VP_OK) st = blaunch_qr_factor(ctx, ctx->stream, qr2);
       return st;
     }));
-    // Q1, Q2 (and, tall, P Q1) on the side stream while the Jacobi SVD runs
+    // the Q of the output on the side stream, beside the last QR and the Jacobi SVD
     VP_CUDA(ctx, cudaEventRecord(g->ev_fork, ctx->stream));
     VP_CUDA(ctx, cudaStreamWaitEvent(g->side, g->ev_fork, 0));
     {
       OnSide side(ctx, &g->side);
       VP_TRY(timed(ctx, VP_K_FORMQ, wf, [&] { return blaunch_qr_formq(ctx, ctx->stream, fq); }));
-      VP_TRY(timed(ctx, VP_K_GEMM, wp, [&] { return blaunch_gemm(ctx, ctx->stream, pq); }));
       VP_CUDA(ctx, cudaEventRecord(g->ev_join, ctx->stream));
     }
     struct SideJoin {
       vp_group* g;
       ~SideJoin() { cudaStreamWaitEvent(g->ctx->stream, g->ev_join, 0); }
     } side_join{g};
+    // last QR, from the left: its R (columns ordered) is what Jacobi diagonalises
     VP_TRY(blaunch_lower_from_upper(ctx, ctx->stream, lu));
-    VP_TRY(blaunch_copy(ctx, ctx->stream, cp));
+    VP_TRY(blaunch_norm_order(ctx, ctx->stream, no2));
+    VP_TRY(blaunch_gather_cm(ctx, ctx->stream, ga2));
+    VP_TRY(timed(ctx, VP_K_QR, 0.0, [&] { return blaunch_qr_factor(ctx, ctx->stream, qr3); }));
+    VP_TRY(blaunch_qr_getr(ctx, ctx->stream, gx));
     const size_t jac_mark = ctx->prof_on ? ctx->prof_marks.size() : (size_t)-1;
     VP_TRY(timed(ctx, VP_K_JACOBI, 0.0, [&] { return blaunch_jacobi(ctx, ctx->stream, jc); }));
     VP_TRY(timed(ctx, VP_K_SELECT, 0.0, [&] { return blaunch_select(ctx, ctx->stream, se); }));
@@ -405,7 +408,7 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       double wj = 0.0;
       for (Task* t : ts) {
         const double q = t->q, sweeps = g->h_task[t->slot].st.pad2;
-        const double j = q > 1 ? sweeps * 0.5 * q * (q - 1) * (6.0 * q + (t->tall ? 0.0 : 4.0 * q)) : 0.0;
+        const double j = q > 1 ? sweeps * 0.5 * q * (q - 1) * 6.0 * q : 0.0;
         account(g, t, 0, 0, 0, j);
         wj += j;
       }
@@ -414,8 +417,7 @@ int svd_sweep(vp_group* g, const Tasks& all) {
     }
     ts = live(g, ts);
     std::vector<BSvdOut> so;
-    std::vector<BSvdOutWide> sw;
-    std::vector<BGemm> g2, g3, g5;
+    std::vector<BGemm> g2, g3, g4;
     std::vector<BScatter> sc;
     for (Task* t : ts) {
       mps_t* s = t->s;
@@ -426,52 +428,43 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       if (t->errs) t->errs[k - 1] = rec.err;
       if (t->ent) t->ent[k - 1] = rec.ent;
       VP_TRY(reserve(ctx, w.a, (size_t)r * q + 8));
-      VP_TRY(reserve(ctx, w.b, (size_t)q * r + 8));
+      VP_TRY(reserve(ctx, w.b, (size_t)m * r + 8));
+      VP_TRY(reserve(ctx, w.tmp2, (size_t)r * c));
+      VP_TRY(reserve(ctx, w.gemm, (size_t)pl * r));
       int* perm = (int*)w.vec.p;
       double* sigma = w.vec.p + (q + 1) / 2 + 4;
       const int* piv = (const int*)w.piv.p;
+      // core_k <- V^T (in tmp2, swapped in below; FP64 in every mode, as it enters
+      // both cores); core_{k-1} <- core_{k-1} (M V)
+      so.push_back({w.tmp.p, q, r, perm, sigma, piv + q, w.a.p});
       if (t->tall) {
-        // core_{k-1} <- (P Q1) (U_L S), U_L S = L V_L; core_k <- scatter(V_L^T Q2^T)
-        VP_TRY(reserve(ctx, w.gemm, (size_t)pl * r));
         VP_TRY(reserve(ctx, w.c, (size_t)r * q));
-        VP_TRY(reserve(ctx, s->core[k], (size_t)r * c));
-        so.push_back({w.tmp.p, nullptr, q, q, r, perm, sigma, w.a.p, nullptr});
-        g2.push_back({BG_ABT, t->fp32, q, r, q, 1.0, w.l.p, q, w.a.p, q, w.b.p, r, &w.main});
-        g2.push_back({BG_ABT, t->fp32, r, q, q, 1.0, w.a.p, q, w.q2.p, q, w.c.p, q, &w.main});
-        g3.push_back({BG_AB, t->fp32, pl, r, q, 1.0, w.tmp2.p, q, w.b.p, r, w.gemm.p, r, &w.main});
-        sc.push_back({w.c.p, r, q, piv, 1, s->core[k].p});
+        g2.push_back({BG_ABT, 0, r, q, q, 1.0, w.a.p, q, w.q1.p, q, w.c.p, q, &w.main});
+        sc.push_back({w.c.p, r, q, piv, 1, w.tmp2.p});
       } else {
-        // core_k <- U_L^T Q1^T; core_{k-1} <- P Pi (Q2 V_L S)
-        VP_TRY(reserve(ctx, s->core[k], (size_t)r * c));
-        VP_TRY(reserve(ctx, w.c, (size_t)m * r));
-        VP_TRY(reserve(ctx, w.tmp2, (size_t)m * r));
-        VP_TRY(reserve(ctx, w.gemm, (size_t)pl * r));
-        sw.push_back({w.tmp.p, w.j.p, q, r, perm, w.a.p, w.b.p});
-        g2.push_back({BG_ABT, t->fp32, r, c, m, 1.0, w.a.p, m, w.q1.p, m, s->core[k].p, c, &w.main});
-        g3.push_back({BG_AB, t->fp32, m, r, m, 1.0, w.q2.p, m, w.b.p, r, w.c.p, r, &w.main});
-        sc.push_back({w.c.p, m, r, piv, 0, w.tmp2.p});
-        g5.push_back({BG_AB, t->fp32, pl, r, m, 1.0, s->core[k - 1].p, m, w.tmp2.p, r, w.gemm.p, r, &w.main});
+        g2.push_back({BG_ABT, 0, r, c, q, 1.0, w.a.p, q, w.q1.p, q, w.tmp2.p, c, &w.main});
       }
+      g3.push_back({BG_ABT, t->fp32, m, r, c, 1.0, s->core[k].p, c, w.tmp2.p, c, w.b.p, r, &w.main});
+      g4.push_back({BG_AB, t->fp32, pl, r, m, 1.0, s->core[k - 1].p, m, w.b.p, r, w.gemm.p, r, &w.main});
     }
     double wo = 0.0;
-    for (const auto* v : {&g2, &g3, &g5})
+    for (const auto* v : {&g2, &g3, &g4})
       for (const BGemm& x : *v) wo += 2.0 * x.M * x.N * x.K;
     for (Task* t : ts) {
       const double q = t->q, r = t->r, m = t->m, c = t->c, pl = t->pl;
-      account(g, t, 0, 0, t->tall ? 2.0 * pl * r * q + 4.0 * r * q * q : 2.0 * r * c * m + 2.0 * m * r * m + 2.0 * pl * r * m,
-              0);
+      account(g, t, 0, 0, 2.0 * r * c * q + 2.0 * m * r * c + 2.0 * pl * r * m, 0);
     }
     VP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, g->ev_join, 0));
     VP_TRY(timed(ctx, VP_K_GEMM, wo, [&] {
       int st = blaunch_svd_outputs(ctx, ctx->stream, so);
-      if (st == VP_OK) st = blaunch_svd_outputs_wide(ctx, ctx->stream, sw);
       if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g2);
-      if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g3);
       if (st == VP_OK) st = blaunch_scatter(ctx, ctx->stream, sc);
-      if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g5);
+      if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g3);
+      if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g4);
       return st;
     }));
     for (Task* t : ts) {
+      std::swap(t->s->core[t->k], t->w->tmp2);
       std::swap(t->s->core[t->k - 1], t->w->gemm);
       t->s->r[t->k] = t->r;
     }

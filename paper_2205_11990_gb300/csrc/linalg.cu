@@ -780,8 +780,7 @@ int launch_gemm_r(vp_ctx* ctx, int M, int N, int K, const double* Acm, int lda, 
 
 // ------------------------------------------------------------ Jacobi SVD
 // One-sided (Hestenes) Jacobi on the rows of X: rotate row pairs until all
-// are mutually orthogonal; then X = diag(s) V^T and the accumulated rotation
-// G (rows of J) gives U = G^T.  Round-robin ("circle") ordering: b' - 1
+// are mutually orthogonal; then X = diag(s) V^T.  Round-robin ("circle") ordering: b' - 1
 // rounds of b'/2 disjoint pairs per sweep, one warp per pair, one grid
 // barrier per round.
 __device__ __forceinline__ int rr_index(int pos, int round, int bp) {
@@ -800,7 +799,7 @@ __device__ __forceinline__ void jacobi_rotation(double al, double be, double ga,
   sn = cs * t;
 }
 
-__global__ void __launch_bounds__(kThreads) k_jacobi_rows(double* X, int b, int c, double* J, double eps,
+__global__ void __launch_bounds__(kThreads) k_jacobi_rows(double* X, int b, int c, double eps,
                                                           int max_sweeps, DevStatus* st) {
   const int nb = gridDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -842,15 +841,6 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_rows(double* X, int b, int 
           __stcg(xi + q, cs * u - sn * v);
           __stcg(xj + q, sn * u + cs * v);
         }
-        if (J) {
-          double* ji = J + (size_t)i * b;
-          double* jj = J + (size_t)j * b;
-          for (int q = lane; q < b; q += 32) {
-            const double u = __ldcg(ji + q), v = __ldcg(jj + q);
-            __stcg(ji + q, cs * u - sn * v);
-            __stcg(jj + q, sn * u + cs * v);
-          }
-        }
         if (lane == 0) atomicAdd(cnt, 1u);
       }
       if (!gs.sync()) return;
@@ -867,20 +857,18 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_rows(double* X, int b, int 
   }
 }
 
-// Cluster-resident variant: the b rows of X (length c) and of the rotation
-// accumulator J (length b) live in the distributed shared memory of one
-// thread-block cluster (row x in CTA x % CS, slot x / CS, X and J parts
-// contiguous), one CTA per SM.  A pair is processed by one warp through
+// Cluster-resident variant: the b rows of X (length c) live in the distributed
+// shared memory of one thread-block cluster (row x in CTA x % CS, slot x / CS),
+// one CTA per SM.  A pair is processed by one warp through
 // DSMEM pointers; rounds are separated by the hardware cluster barrier
 // (about 0.2 us on GB300, against 2 us for a grid-wide software barrier).
-__global__ void __launch_bounds__(kThreads) k_jacobi_cluster(double* X, int b, int c, double* J, double eps,
+__global__ void __launch_bounds__(kThreads) k_jacobi_cluster(double* X, int b, int c, double eps,
                                                              int max_sweeps, DevStatus* st) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ double sm[];
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int jb = J ? b : 0;  // accumulate the rotations only when J is wanted
-  const int rpc = (b + CS - 1) / CS, stride = c + jb;
+  const int rpc = (b + CS - 1) / CS, stride = c;
   double* nrm = sm + (size_t)rpc * stride;                   // squared row norms, one per local row
   unsigned* cnt = reinterpret_cast<unsigned*>(nrm + rpc);
   for (int sl = 0; sl < rpc; ++sl) {
@@ -888,7 +876,6 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_cluster(double* X, int b, i
     if (x >= b) break;
     double* row = sm + (size_t)sl * stride;
     for (int q = tid; q < c; q += kThreads) row[q] = X[(size_t)x * c + q];
-    for (int q = tid; q < jb; q += kThreads) row[c + q] = (q == x) ? 1.0 : 0.0;
   }
   if (tid < 4) cnt[tid] = 0u;
   unsigned* c0 = cl.map_shared_rank(cnt, 0);
@@ -955,19 +942,12 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_cluster(double* X, int b, i
     if (x >= b) break;
     const double* row = sm + (size_t)sl * stride;
     for (int q = tid; q < c; q += kThreads) X[(size_t)x * c + q] = row[q];
-    for (int q = tid; q < jb; q += kThreads) J[(size_t)x * b + q] = row[c + q];
   }
   if (rank == 0 && tid == 0) {
     st->pad2 = sweep + 1;
     if (!converged) atomicCAS(&st->err, 0, 3);
   }
   cl.sync();  // keep every CTA's shared memory alive until all remote accesses are done
-}
-
-__global__ void k_identity(double* J, int b) {
-  const size_t total = (size_t)b * b;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x)
-    J[e] = (e / b == e % b) ? 1.0 : 0.0;
 }
 
 int probe_cluster_size() {
@@ -993,9 +973,9 @@ int probe_cluster_size() {
   return 0;
 }
 
-static size_t cluster_jacobi_smem(int b, int c, int CS, bool withJ) {
+static size_t cluster_jacobi_smem(int b, int c, int CS) {
   const size_t rpc = (size_t)(b + CS - 1) / CS;
-  return rpc * (size_t)(c + (withJ ? b : 0) + 1) * sizeof(double) + 4 * sizeof(unsigned);
+  return rpc * (size_t)(c + 1) * sizeof(double) + 4 * sizeof(unsigned);
 }
 
 // Block-local variant.  The b rows are split into 2 CS blocks of nb rows (nb
@@ -1016,8 +996,7 @@ static size_t cluster_jacobi_smem(int b, int c, int CS, bool withJ) {
 // x~_j <- x~_j + (t d_i / d_j) x~_i, d <- c d: two FMAs per element pair
 // instead of four operations, with the same rounding bound.  Each sweep
 // starts by folding d back into the rows and recomputing alpha exactly.
-// Row layout (stride c + jb + 2 doubles): x~ (c), accumulated rotation row
-// (jb, when J is wanted), alpha, d.
+// Row layout (stride c + 2 doubles): x~ (c), alpha, d.
 struct JacBlockCfg {
   int CS, nb, stride;
 };
@@ -1076,14 +1055,13 @@ __device__ __forceinline__ void jac_update(double* ri, double* rj, int w, int la
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_jacobi_block(double* X, int b, int c, double* J, double eps,
+__global__ void __launch_bounds__(kThreads) k_jacobi_block(double* X, int b, int c, double eps,
                                                            int max_sweeps, int nb, DevStatus* st) {
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ double sm[];
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int jb = J ? b : 0;
-  const int w = c + jb, stride = w + 2;
+  const int w = c, stride = w + 2;
   const size_t slot_sz = (size_t)nb * stride;
   // buffer set s, slot (0 top, 1 bottom), row r
   auto row = [&](int s, int slot, int r) { return sm + ((size_t)(s * 2 + slot)) * slot_sz + (size_t)r * stride; };
@@ -1124,7 +1102,6 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_block(double* X, int b, int
         double v = 0.0;
         if (x < b) {
           if (q < c) v = X[(size_t)x * c + q];
-          else if (q < w) v = (q - c == x) ? 1.0 : 0.0;
         }
         if (q == w + 1) v = 1.0;  // scale d
         d[q] = v;
@@ -1210,7 +1187,6 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_block(double* X, int b, int
       const double* d = row(cur, slot, r);
       const double sc = d[w + 1];
       for (int q = tid; q < c; q += kThreads) X[(size_t)x * c + q] = sc * d[q];
-      for (int q = tid; q < jb; q += kThreads) J[(size_t)x * b + q] = sc * d[c + q];
     }
   }
   if (rank == 0 && tid == 0) {
@@ -1220,291 +1196,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_block(double* X, int b, int
   cl.sync();  // keep every CTA's shared memory alive until all remote accesses are done
 }
 
-// Double-word variant of k_jacobi_block (the production path): the same
-// block-local circle schedule, with the rows held as double-word FP32 pairs
-// (dw.cuh), so that the dot products, rotation parameters and updates run on
-// the FP32 pipe.  The matrix is first scaled by a power of two common to the
-// whole cluster (exact) so that its largest entry is ~1; rows whose squared
-// norm falls below 1e-30 of that (singular values under 1e-15 of the
-// largest) are left alone.  A rotation uses the standard form
-// x_i <- c x_i - s x_j, x_j <- s x_i + c x_j with c = 1/sqrt(1 + t^2) and
-// s = c t computed to double-word accuracy from an FP32 tangent t: the angle
-// need not be the exact Jacobi angle, the rotation is orthogonal to ~1e-14
-// either way.  Pairs rotate while |gamma| > eps sqrt(alpha beta) with eps
-// above the ~1e-14 noise of a double-word dot product.  Row layout (stride
-// w + 1, w = c + jb, in double-word units): x (c), rotation row (jb), alpha.
-__device__ __forceinline__ void k_jacobi_dw_body(double* X, int b, int c, double* J, float eps,
-                                                        int max_sweeps, int nb, DevStatus* st) {
-  cg::cluster_group cl = cg::this_cluster();
-  extern __shared__ double smd[];
-  dw* sm = reinterpret_cast<dw*>(smd);
-  const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int jb = J ? b : 0;
-  const int w = c + jb, stride = w + 1;
-  const size_t slot_sz = (size_t)nb * stride;
-  auto row = [&](int s, int slot, int r) { return sm + ((size_t)(s * 2 + slot)) * slot_sz + (size_t)r * stride; };
-  dw* par = sm + 4 * slot_sz;  // per pair: flag, cos, sin
-  float* red = reinterpret_cast<float*>(par + 3 * nb);  // kWarps + 1 floats
-  unsigned* cnt = reinterpret_cast<unsigned*>(red + kWarps + 2);
-
-  // common power-of-two scale: largest |x| over the cluster's rows
-  float mx = 0.f;
-  for (int slot = 0; slot < 2; ++slot) {
-    const int blk = slot == 0 ? rank : 2 * CS - 1 - rank;
-    for (int r = 0; r < nb; ++r) {
-      const int x = blk * nb + r;
-      if (x >= b) continue;
-      for (int q = tid; q < c; q += kThreads) mx = fmaxf(mx, fabsf(__double2float_rn(X[(size_t)x * c + q])));
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) red[warp] = mx;
-  __syncthreads();
-  if (tid == 0) {
-    float m = 0.f;
-    for (int i = 0; i < kWarps; ++i) m = fmaxf(m, red[i]);
-    red[kWarps] = m;
-  }
-  if (tid < 4) cnt[tid] = 0u;
-  cl.sync();
-  float gmax = 0.f;
-  for (int r = 0; r < CS; ++r) gmax = fmaxf(gmax, *cl.map_shared_rank(red + kWarps, r));
-  int ex = 0;
-  if (gmax > 0.f) frexpf(gmax, &ex);
-  const double sc = ldexp(1.0, -ex), inv_sc = ldexp(1.0, ex);
-
-  // home placement: top = block rank, bottom = block 2 CS - 1 - rank
-  for (int slot = 0; slot < 2; ++slot) {
-    const int blk = slot == 0 ? rank : 2 * CS - 1 - rank;
-    for (int r = 0; r < nb; ++r) {
-      const int x = blk * nb + r;
-      dw* d = row(0, slot, r);
-      for (int q = tid; q < stride; q += kThreads) {
-        dw v = {0.f, 0.f};
-        if (x < b) {
-          if (q < c) v = dw_from(X[(size_t)x * c + q] * sc);
-          else if (q < w) v.hi = (q - c == x) ? 1.0f : 0.0f;
-        }
-        d[q] = v;
-      }
-    }
-  }
-  unsigned* c0 = cl.map_shared_rank(cnt, 0);
-  const float tiny = 1e-30f;
-
-  // Rotation parameters of one pair from gamma = <x_i, x_j> and the squared
-  // norms alpha, beta held after each row (false: the pair is left alone).
-  auto pair_params = [&](dw al, dw be, dw g, dw& cs, dw& sn, dw& tg) -> bool {
-    if (!(al.hi > tiny && be.hi > tiny && fabsf(g.hi) * rsqrtf(al.hi) * rsqrtf(be.hi) > eps)) return false;
-    // tangent in FP32 after an exact power-of-two scaling of d and gamma
-    // (their squares would leave the FP32 range for small rows)
-    const float d0 = 0.5f * dw_add(be, dw_neg(al)).hi;
-    int e2;
-    frexpf(fmaxf(fabsf(d0), fabsf(g.hi)), &e2);
-    const float d = ldexpf(d0, -e2), gs = ldexpf(g.hi, -e2);
-    const float t = copysignf(1.0f, d) * gs / (fabsf(d) + sqrtf(fmaf(d, d, gs * gs)));
-    if (t == 0.f) return false;
-    const dw t2 = two_prod(t, t);
-    cs = dw_rsqrt(dw_add({1.0f, 0.0f}, t2));
-    sn = dw_mul_f(cs, t);
-    tg = dw_mul_f(g, t);
-    return true;
-  };
-  // One inner round over nb disjoint pairs.  With at most one pair per warp
-  // (nb <= kWarps, the usual case) pair i belongs to the wpp = kWarps / nb
-  // warps i wpp .. i wpp + wpp - 1: each of them forms gamma and the
-  // rotation itself (the same operations, so the same bits), and rotates its
-  // share of the columns; one named barrier of the pair's warps orders the
-  // reads of alpha and beta before their update, and one block barrier ends
-  // the round.  With more pairs than warps the round runs in three phases:
-  // A dot products (a warp per pair), B rotation parameters (a lane per
-  // pair), C updates (a warp per pair), each ended by a block barrier.
-  auto inner_round = [&](auto pair_rows, unsigned& rotated) {
-    if (nb <= kWarps) {
-      const int wpp = kWarps / nb, pi = warp / wpp, part = warp % wpp;
-      if (pi < nb) {
-        dw *ri, *rj;
-        pair_rows(pi, ri, rj);
-        dw_acc acc;
-        dw_dot_rows(acc, ri, rj, 0, c, lane);
-        const dw g = dw_warp_sum(dw_acc_value(acc));
-        const dw al = ri[w], be = rj[w];
-        dw cs, sn, tg;
-        const bool rot = pair_params(al, be, g, cs, sn, tg);
-        // every warp of the pair has read alpha and beta before they change
-        if (wpp > 1)
-          asm volatile("bar.sync %0, %1;" ::"r"(1 + pi), "r"(32 * wpp) : "memory");
-        else
-          __syncwarp();
-        if (rot) {
-          if (part == 0 && lane == 0) {
-            ri[w] = dw_add(al, dw_neg(tg));
-            rj[w] = dw_add(be, tg);
-            ++rotated;
-          }
-          const int span = (w + wpp - 1) / wpp, q0 = part * span;
-          if (q0 < w) dw_rot_rows(ri + q0, rj + q0, cs, sn, min(span, w - q0), lane);
-        }
-      }
-      __syncthreads();
-      return;
-    }
-    for (int pi = warp; pi < nb; pi += kWarps) {
-      dw *ri, *rj;
-      pair_rows(pi, ri, rj);
-      dw_acc acc;
-      dw_dot_rows(acc, ri, rj, 0, c, lane);
-      const dw g = dw_warp_sum(dw_acc_value(acc));
-      if (lane == 0) par[3 * pi] = g;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      for (int pi = lane; pi < nb; pi += 32) {
-        dw *ri, *rj;
-        pair_rows(pi, ri, rj);
-        const dw al = ri[w], be = rj[w];
-        dw cs, sn, tg;
-        float flag = 0.f;
-        if (pair_params(al, be, par[3 * pi], cs, sn, tg)) {
-          ri[w] = dw_add(al, dw_neg(tg));
-          rj[w] = dw_add(be, tg);
-          par[3 * pi + 1] = cs;
-          par[3 * pi + 2] = sn;
-          flag = 1.f;
-          ++rotated;
-        }
-        par[3 * pi].hi = flag;
-      }
-    }
-    __syncthreads();
-    for (int pi = warp; pi < nb; pi += kWarps) {
-      if (par[3 * pi].hi == 0.f) continue;
-      dw *ri, *rj;
-      pair_rows(pi, ri, rj);
-      dw_rot_rows(ri, rj, par[3 * pi + 1], par[3 * pi + 2], w, lane);
-    }
-    __syncthreads();
-  };
-
-  // A pair that would rotate, counted without rotating (the test of
-  // inner_round on the same operands in the same order).
-  auto dry_pair = [&](const dw* ri, const dw* rj, unsigned& would) {
-    dw_acc acc;
-    dw_dot_rows(acc, ri, rj, 0, c, lane);
-    const dw g = dw_warp_sum(dw_acc_value(acc));
-    dw cs, sn, tg;
-    if (pair_params(ri[w], rj[w], g, cs, sn, tg) && lane == 0) ++would;
-  };
-
-  // Sweeps of the circle schedule until one rotates nothing.  After a sweep
-  // with few rotations (at most max(4, b/2)) the next pass is a dry sweep:
-  // every pair of the schedule is tested in the same order and orientation
-  // but nothing is rotated, so its pairs need no barriers between rounds.  If
-  // no pair would rotate, the plain sweep would have rotated nothing either
-  // (its operands never change) and the rows are final; otherwise nothing has
-  // changed and the plain sweep runs.  The result is the plain schedule's,
-  // bit for bit, without its last, rotation-free sweep.
-  int cur = 0, iter = 0, sweeps = 0;
-  bool converged = false, dry_failed = false;
-  unsigned last_rot = 0xffffffffu;
-  const unsigned dry_max = (unsigned)max(4, b / 2);
-  const int brounds = 2 * CS - 1;
-  for (; sweeps < max_sweeps; ++iter) {
-    const bool dry = last_rot <= dry_max && !dry_failed;
-    // exact squared norms of the local rows
-    __syncthreads();
-    for (int rr = warp; rr < 2 * nb; rr += kWarps) {
-      dw* d = row(cur, rr / nb, rr % nb);
-      dw_acc acc;
-      dw_dot_rows(acc, d, d, 0, c, lane);
-      const dw a = dw_warp_sum(dw_acc_value(acc));
-      if (lane == 0) d[w] = a;
-    }
-    if (rank == 0 && tid == 0) cnt[(iter + 1) % 3] = 0u;
-    cl.sync();
-    unsigned rotated = 0;
-    for (int br = 0; br < brounds; ++br) {
-      if (dry) {
-        if (br == 0)
-          for (int e = warp; e < (nb - 1) * nb; e += kWarps) {
-            const int ir = e / nb, pi = e % nb;
-            const int slot = pi / (nb / 2), pos = pi % (nb / 2);
-            dry_pair(row(cur, slot, rr_index(pos, ir, nb)), row(cur, slot, rr_index(nb - 1 - pos, ir, nb)), rotated);
-          }
-        for (int e = warp; e < nb * nb; e += kWarps) {
-          const int sh = e / nb, pi = e % nb;
-          dry_pair(row(cur, 0, pi), row(cur, 1, (pi + sh) % nb), rotated);
-        }
-      } else {
-        if (br == 0) {
-          for (int ir = 0; ir < nb - 1; ++ir)
-            inner_round(
-                [&](int pi, dw*& ri, dw*& rj) {
-                  const int slot = pi / (nb / 2), pos = pi % (nb / 2);
-                  ri = row(cur, slot, rr_index(pos, ir, nb));
-                  rj = row(cur, slot, rr_index(nb - 1 - pos, ir, nb));
-                },
-                rotated);
-        }
-        for (int sh = 0; sh < nb; ++sh)
-          inner_round(
-              [&](int pi, dw*& ri, dw*& rj) {
-                ri = row(cur, 0, pi);
-                rj = row(cur, 1, (pi + sh) % nb);
-              },
-              rotated);
-      }
-      if (br == brounds - 1) {
-        const unsigned tot = __reduce_add_sync(0xffffffffu, rotated);
-        if (lane == 0 && tot) atomicAdd(&c0[iter % 3], tot);
-      }
-      if (CS > 1) {
-        for (int slot = 0; slot < 2; ++slot) {
-          const int pos = slot == 0 ? rank : 2 * CS - 1 - rank;
-          const int np = jac_next_pos(pos, CS);
-          dw* dst = cl.map_shared_rank(row(cur ^ 1, jac_pos_slot(np, CS), 0), jac_pos_cta(np, CS));
-          const dw* src = row(cur, slot, 0);
-          for (size_t e = tid; e < slot_sz; e += kThreads) dst[e] = src[e];
-        }
-        cur ^= 1;
-      }
-      cl.sync();
-    }
-    const unsigned tot = *(volatile unsigned*)&c0[iter % 3];
-    if (tot == 0u) {
-      converged = true;
-      ++sweeps;
-      break;
-    }
-    dry_failed = dry;
-    if (!dry) {
-      ++sweeps;
-      last_rot = tot;
-    }
-  }
-  __syncthreads();
-  for (int slot = 0; slot < 2; ++slot) {
-    const int blk = slot == 0 ? rank : 2 * CS - 1 - rank;
-    for (int r = 0; r < nb; ++r) {
-      const int x = blk * nb + r;
-      if (x >= b) continue;
-      const dw* d = row(cur, slot, r);
-      for (int q = tid; q < c; q += kThreads) X[(size_t)x * c + q] = dw_to(d[q]) * inv_sc;
-      for (int q = tid; q < jb; q += kThreads) J[(size_t)x * b + q] = dw_to(d[c + q]);
-    }
-  }
-  if (rank == 0 && tid == 0) {
-    st->pad2 = converged ? sweeps : max_sweeps + 1;  // as the plain schedule counts them
-    if (!converged) atomicCAS(&st->err, 0, 3);
-  }
-  cl.sync();  // keep every CTA's shared memory alive until all remote accesses are done
-}
-__global__ void __launch_bounds__(kThreads) k_jacobi_dw(double* X, int b, int c, double* J, float eps,
-                                                        int max_sweeps, int nb, DevStatus* st) { k_jacobi_dw_body(X, b, c, J, eps, max_sweeps, nb, st); }
-
-static JacBlockCfg jac_block_cfg(int b, int c, bool withJ, int cs_max) {
+static JacBlockCfg jac_block_cfg(int b, int c, int cs_max) {
   JacBlockCfg g{1, 2, 0};
   int cs = 1;
   while (cs < 16 && cs < cs_max && cs * 8 < b) cs *= 2;
@@ -1513,50 +1205,19 @@ static JacBlockCfg jac_block_cfg(int b, int c, bool withJ, int cs_max) {
   if (nb < 2) nb = 2;
   g.CS = cs;
   g.nb = nb;
-  g.stride = c + (withJ ? b : 0) + 2;
+  g.stride = c + 2;
   return g;
-}
-
-static size_t jac_dw_smem(const JacBlockCfg& g) {
-  // rows (stride - 1 double words: no scale slot), pair parameters, reduction, counters
-  return (4 * (size_t)g.nb * (g.stride - 1) + 3 * (size_t)g.nb) * sizeof(dw) + (kWarps + 2) * sizeof(float) +
-         4 * sizeof(unsigned);
 }
 
 static size_t jac_block_smem(const JacBlockCfg& g) {
   return (4 * (size_t)g.nb * g.stride + 4 * (size_t)g.nb) * sizeof(double) + 4 * sizeof(unsigned);
 }
 
-int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* X, int b, int c, double* J,
-                   bool floor_ok) {
+int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* X, int b, int c, bool floor_ok) {
   if (b <= 0) return VP_OK;
   const int CS = ctx->cluster_size;
-  const JacBlockCfg bc = jac_block_cfg(b, c, J != nullptr, std::max(1, CS));
-  if (floor_ok && b > 1 && jac_dw_smem(bc) <= 200 * 1024) {
-    static AttrOnce dattr_done;
-    VP_TRY(dattr_done.ensure(ctx, (const void*)k_jacobi_dw, 200 * 1024, true));
-    const size_t smem = std::max<size_t>(jac_dw_smem(bc), 120 * 1024);
-    // rotate while |gamma| > eps sqrt(alpha beta); eps above the double-word
-    // dot-product noise, which grows like sqrt(c) u^2
-    float eps = (float)(4e-13 * std::sqrt((double)c));
-    int max_sweeps = 60;
-    int nb = bc.nb;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    cfg.gridDim = dim3(bc.CS);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = bc.CS;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    ctx->launches++;
-    VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_jacobi_dw, X, b, c, J, eps, max_sweeps, nb, status));
-    return VP_OK;
-  }
+  if (floor_ok && jacobi_dw_fits(ctx, b, c)) return blaunch_jacobi_dw(ctx, stream, {BJacobi{X, b, c, status}});
+  const JacBlockCfg bc = jac_block_cfg(b, c, std::max(1, CS));
   if (b > 1 && jac_block_smem(bc) <= 200 * 1024) {
     static AttrOnce battr_done;
     VP_TRY(battr_done.ensure(ctx, (const void*)k_jacobi_block, 200 * 1024, true));
@@ -1578,13 +1239,13 @@ int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* 
     cfg.attrs = at;
     cfg.numAttrs = 1;
     ctx->launches++;
-    VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_jacobi_block, X, b, c, J, eps, max_sweeps, nb, status));
+    VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_jacobi_block, X, b, c, eps, max_sweeps, nb, status));
     return VP_OK;
   }
-  if (CS > 0 && b > 1 && cluster_jacobi_smem(b, c, CS, J != nullptr) <= 200 * 1024) {
+  if (CS > 0 && b > 1 && cluster_jacobi_smem(b, c, CS) <= 200 * 1024) {
     static AttrOnce attr_done;
     // at least 120 KB per CTA, so no two CTAs of the cluster share an SM
-    const size_t smem = std::max<size_t>(cluster_jacobi_smem(b, c, CS, J != nullptr), 120 * 1024);
+    const size_t smem = std::max<size_t>(cluster_jacobi_smem(b, c, CS), 120 * 1024);
     VP_TRY(attr_done.ensure(ctx, (const void*)k_jacobi_cluster, 200 * 1024, true));
     double eps = 1e-15 * std::sqrt((double)c);
     int max_sweeps = 60;
@@ -1601,13 +1262,8 @@ int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* 
     cfg.attrs = at;
     cfg.numAttrs = 1;
     ctx->launches++;
-    VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_jacobi_cluster, X, b, c, J, eps, max_sweeps, status));
+    VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, k_jacobi_cluster, X, b, c, eps, max_sweeps, status));
     return VP_OK;
-  }
-  if (J) {
-    ctx->launches++;
-    k_identity<<<std::min(1024, (b * b + 255) / 256 + 1), 256, 0, stream>>>(J, b);
-    VP_TRY(check_launch(ctx, "identity"));
   }
   if (b == 1) return VP_OK;
   const int npairs = (b + 1) / 2;
@@ -1617,12 +1273,12 @@ int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* 
   double eps = 1e-15 * std::sqrt((double)c);
   int max_sweeps = 60;
   DevStatus* st = status;
-  void* args[] = {&X, &b, &c, &J, &eps, &max_sweeps, &st};
+  void* args[] = {&X, &b, &c, &eps, &max_sweeps, &st};
   return coop_launch(ctx, stream, (const void*)k_jacobi_rows, blocks, kThreads, args, 0, "jacobi_rows");
 }
 
-int launch_jacobi_rows(vp_ctx* ctx, double* X, int b, int c, double* J, bool floor_ok) {
-  return jacobi_rows_on(ctx, ctx->stream, ctx->status, X, b, c, J, floor_ok);
+int launch_jacobi_rows(vp_ctx* ctx, double* X, int b, int c, bool floor_ok) {
+  return jacobi_rows_on(ctx, ctx->stream, ctx->status, X, b, c, floor_ok);
 }
 
 // ------------------------------------------------------------ truncation
@@ -1766,32 +1422,26 @@ int launch_select(vp_ctx* ctx, const double* X, int b, int c, int chi, double to
   return check_launch(ctx, "select");
 }
 
-__device__ __forceinline__ void k_svd_outputs_body(const double* __restrict__ X, const double* __restrict__ J, int b, int c, int r,
-                              const int* __restrict__ perm, const double* __restrict__ sigma, double* Vt,
-                              double* W) {
-  const size_t nv = (size_t)r * c, nw = J ? (size_t)b * r : 0;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < nv + nw; e += (size_t)gridDim.x * blockDim.x) {
-    if (e < nv) {
-      const int t = (int)(e / c), q = (int)(e % c);
-      const double s = sigma[t];
-      Vt[e] = s > 0.0 ? X[(size_t)perm[t] * c + q] / s : 0.0;
-    } else {
-      const size_t f = e - nv;
-      const int i = (int)(f / r), t = (int)(f % r);
-      W[f] = J[(size_t)perm[t] * b + i] * sigma[t];
-    }
+__device__ __forceinline__ void k_svd_outputs_body(const double* __restrict__ X, int q, int r, const int* __restrict__ perm,
+                                                   const double* __restrict__ sigma, const int* __restrict__ cperm,
+                                                   double* __restrict__ V) {
+  const size_t total = (size_t)r * q;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+    const int t = (int)(e / q), j = (int)(e % q);
+    const double s = sigma[t];
+    V[(size_t)t * q + cperm[j]] = s > 0.0 ? X[(size_t)perm[t] * q + j] / s : 0.0;
   }
 }
-__global__ void k_svd_outputs(const double* __restrict__ X, const double* __restrict__ J, int b, int c, int r,
-                              const int* __restrict__ perm, const double* __restrict__ sigma, double* Vt,
-                              double* W) { k_svd_outputs_body(X, J, b, c, r, perm, sigma, Vt, W); }
+__global__ void k_svd_outputs(const double* __restrict__ X, int q, int r, const int* __restrict__ perm,
+                              const double* __restrict__ sigma, const int* __restrict__ cperm, double* __restrict__ V) {
+  k_svd_outputs_body(X, q, r, perm, sigma, cperm, V);
+}
 
-int launch_svd_outputs(vp_ctx* ctx, const double* X, const double* J, int b, int c, int r, const int* perm,
-                       const double* sigma, double* Vt, double* W) {
-  const size_t total = (size_t)r * c + (size_t)b * r;
-  const int blocks = (int)std::min<size_t>((total + 255) / 256, (size_t)ctx->num_sms * 8);
+int launch_svd_outputs(vp_ctx* ctx, const double* X, int q, int r, const int* perm, const double* sigma,
+                       const int* cperm, double* V) {
+  const int blocks = (int)std::min<size_t>(((size_t)r * q + 255) / 256, (size_t)ctx->num_sms * 8);
   ctx->launches++;
-  k_svd_outputs<<<std::max(1, blocks), 256, 0, ctx->stream>>>(X, J, b, c, r, perm, sigma, Vt, W);
+  k_svd_outputs<<<std::max(1, blocks), 256, 0, ctx->stream>>>(X, q, r, perm, sigma, cperm, V);
   return check_launch(ctx, "svd_outputs");
 }
 
@@ -1902,34 +1552,6 @@ int launch_scatter(vp_ctx* ctx, const double* Y, int rows, int cols_n, const int
   ctx->launches++;
   k_scatter<<<blocks, 256, 0, ctx->stream>>>(Y, rows, cols_n, piv, cols, out);
   return check_launch(ctx, "scatter");
-}
-
-// Wide-case outputs: Urows (r x b) = J[perm[t]] (rows of the accumulated
-// rotation), Wv (b x r) = X[perm[t]][i] (= V diag(s) of the factor).
-__device__ __forceinline__ void k_svd_outputs_wide_body(const double* __restrict__ X, const double* __restrict__ J, int b, int r,
-                                   const int* __restrict__ perm, double* Urows, double* Wv) {
-  const size_t nu = (size_t)r * b;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < 2 * nu; e += (size_t)gridDim.x * blockDim.x) {
-    if (e < nu) {
-      const int t = (int)(e / b), q = (int)(e % b);
-      Urows[e] = J[(size_t)perm[t] * b + q];
-    } else {
-      const size_t f = e - nu;
-      const int i = (int)(f / r), t = (int)(f % r);
-      Wv[f] = X[(size_t)perm[t] * b + i];
-    }
-  }
-}
-__global__ void k_svd_outputs_wide(const double* __restrict__ X, const double* __restrict__ J, int b, int r,
-                                   const int* __restrict__ perm, double* Urows, double* Wv) { k_svd_outputs_wide_body(X, J, b, r, perm, Urows, Wv); }
-
-int launch_svd_outputs_wide(vp_ctx* ctx, const double* X, const double* J, int b, int r, const int* perm,
-                            double* Urows, double* Wv) {
-  const size_t total = 2 * (size_t)r * b;
-  const int blocks = (int)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)ctx->num_sms * 8));
-  ctx->launches++;
-  k_svd_outputs_wide<<<blocks, 256, 0, ctx->stream>>>(X, J, b, r, perm, Urows, Wv);
-  return check_launch(ctx, "svd_outputs_wide");
 }
 
 // ====================================================== batched launches
@@ -2388,41 +2010,18 @@ int blaunch_lower_from_upper(vp_ctx* ctx, cudaStream_t st, const std::vector<BLo
                    "b_lower_from_upper");
 }
 
-struct JacArgs {
-  double* X;
-  int b, c;
-  double* J;
-  float eps;
-  int max_sweeps, nb;
-  DevStatus* st;
-};
-__global__ void __launch_bounds__(kThreads) kb_jacobi_dw(const __grid_constant__ Pack<JacArgs> pk) {
-  const JacArgs& a = pk.a[blockIdx.y];
-  k_jacobi_dw_body(a.X, a.b, a.c, a.J, a.eps, a.max_sweeps, a.nb, a.st);
-}
 int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v) {
-  const int CS = ctx->cluster_size;
-  std::vector<JacArgs> grp[17];
-  size_t smem[17] = {};
+  std::vector<BJacobi> fit;
   for (const BJacobi& j : v) {
     if (j.b <= 1) continue;  // nothing to rotate (as in the single launch)
-    const JacBlockCfg bc = jac_block_cfg(j.b, j.c, j.J != nullptr, std::max(1, CS));
-    if (jac_dw_smem(bc) <= 200 * 1024) {
-      // the thresholds of launch_jacobi_rows
-      grp[bc.CS].push_back({j.X, j.b, j.c, j.J, (float)(4e-13 * std::sqrt((double)j.c)), 60, bc.nb, j.st});
-      smem[bc.CS] = std::max(smem[bc.CS], jac_dw_smem(bc));
+    if (jacobi_dw_fits(ctx, j.b, j.c)) {
+      fit.push_back(j);
     } else {
       VP_CUDA(ctx, cudaMemsetAsync(j.st->rot, 0, sizeof(j.st->rot), st));
-      VP_TRY(jacobi_rows_on(ctx, st, j.st, j.X, j.b, j.c, j.J, true));
+      VP_TRY(jacobi_rows_on(ctx, st, j.st, j.X, j.b, j.c, true));
     }
   }
-  for (int cs = 1; cs <= 16; ++cs)
-    if (!grp[cs].empty()) {
-      static AttrOnce a;
-      VP_TRY(a.ensure(ctx, (const void*)kb_jacobi_dw, 200 * 1024, true));
-      VP_TRY(run_cluster_packs(ctx, st, grp[cs], kb_jacobi_dw, cs, kThreads, std::max<size_t>(smem[cs], 120 * 1024)));
-    }
-  return VP_OK;
+  return blaunch_jacobi_dw(ctx, st, fit);
 }
 
 __global__ void kb_select(const __grid_constant__ Pack<BSelect> pk) {
@@ -2439,23 +2038,11 @@ int blaunch_select(vp_ctx* ctx, cudaStream_t st, const std::vector<BSelect>& v) 
 }
 __global__ void kb_svd_outputs(const __grid_constant__ Pack<BSvdOut> pk) {
   const BSvdOut& a = pk.a[blockIdx.y];
-  k_svd_outputs_body(a.X, a.J, a.b, a.c, a.r, a.perm, a.sigma, a.Vt, a.W);
+  k_svd_outputs_body(a.X, a.q, a.r, a.perm, a.sigma, a.cperm, a.V);
 }
 int blaunch_svd_outputs(vp_ctx* ctx, cudaStream_t st, const std::vector<BSvdOut>& v) {
   return run_packs(ctx, st, v, kb_svd_outputs, 256, 0,
-                   [&](const BSvdOut& a) {
-                     return grid_stride_blocks(ctx, (size_t)a.r * a.c + (size_t)a.b * a.r, 8);
-                   },
-                   "b_svd_outputs");
-}
-__global__ void kb_svd_outputs_wide(const __grid_constant__ Pack<BSvdOutWide> pk) {
-  const BSvdOutWide& a = pk.a[blockIdx.y];
-  k_svd_outputs_wide_body(a.X, a.J, a.b, a.r, a.perm, a.U, a.Wv);
-}
-int blaunch_svd_outputs_wide(vp_ctx* ctx, cudaStream_t st, const std::vector<BSvdOutWide>& v) {
-  return run_packs(ctx, st, v, kb_svd_outputs_wide, 256, 0,
-                   [&](const BSvdOutWide& a) { return grid_stride_blocks(ctx, 2 * (size_t)a.r * a.b, 8); },
-                   "b_svd_outputs_wide");
+                   [&](const BSvdOut& a) { return grid_stride_blocks(ctx, (size_t)a.r * a.q, 8); }, "b_svd_outputs");
 }
 __global__ void kb_scatter(const __grid_constant__ Pack<BScatter> pk) {
   const BScatter& a = pk.a[blockIdx.y];
