@@ -201,7 +201,7 @@ QRPlan qr_plan(const vp_ctx* ctx, int m, int n);
 int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q);
 // Upper-trapezoidal R (p x n) of the factored A, written row-major.
 int launch_qr_getr(vp_ctx* ctx, const double* A, int m, int n, double* R);
-// Output tile and split-K of a GEMM (shape and device only).
+// Output tile and split-K of an FP32 contraction (shape and device only).
 struct GemmPlan {
   int tile;    // 64 or 32
   int slices;  // K slices (1: no split)
@@ -253,6 +253,8 @@ struct OzGemm {
   OzPlan plan;
 };
 int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);
+// The same on the FMA pipe (fgemm.cu; neither plan nor scratch are used).
+int blaunch_fma_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);
 // C = alpha * triu(A_colmajor) (M x K) * B: the R factor read in place.
 int launch_gemm_r(vp_ctx* ctx, int M, int N, int K, const double* Acm, int lda, const double* B,
                   int ldb, double* C, int ldc);

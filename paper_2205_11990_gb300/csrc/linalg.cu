@@ -558,11 +558,11 @@ int launch_qr_getr(vp_ctx* ctx, const double* A, int m, int n, double* R) {
 }
 
 // ------------------------------------------------------------------- GEMM
-// TILE x TILE output tile per block (64 or 32), K step 16, 256 threads with a
-// (TILE / 16)^2 register tile each.  FP64 FMA, row-major B and C.  ALoad
-// selects the A operand: row-major, or the column-major upper triangle of a
-// QR factor.  Each output is the sum over its K slice in ascending k, so the
-// tile size does not change the result; the K slicing does (gemm_plan).
+// The FP32 contraction mode: TILE x TILE output tile per block (64 or 32), K step
+// 16, 256 threads with a (TILE / 16)^2 register tile each, inputs rounded to FP32
+// and FP32 FMA (FP64 contractions: fgemm.cu, ozgemm.cu).  ALoad selects the A
+// operand: row-major, or the column-major upper triangle of a QR factor.  Each
+// output is the sum over its K slice in ascending k; the K slicing is gemm_plan's.
 // kfirst(row0): the first k that can be nonzero in rows >= row0.
 struct ARowMajor {
   const double* A;
@@ -591,10 +591,11 @@ struct BTransposed {
   __device__ double operator()(int k, int n) const { return B[(size_t)n * ldb + k]; }
 };
 
-template <class ALoad, class BLoad, class T, int TILE>
+template <class ALoad, class BLoad, int TILE>
 __device__ __forceinline__ void gemm_body(int M, int N, int K, double alpha, ALoad a, BLoad bl, double* __restrict__ C,
                                           int ldc, int kslice, size_t slice_stride, int bx, int by, int bz) {
   constexpr int R = TILE / 16;  // outputs per thread along each dimension
+  using T = float;
   __shared__ T As[16][TILE + 1];
   __shared__ T Bs[16][TILE];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -642,21 +643,18 @@ __device__ __forceinline__ void gemm_body(int M, int N, int K, double alpha, ALo
   }
 }
 
-template <class ALoad, class BLoad, class T, int TILE>
+template <class ALoad, class BLoad, int TILE>
 __global__ void __launch_bounds__(256) k_gemm(int M, int N, int K, double alpha, ALoad a, BLoad bl,
                                               double* __restrict__ C, int ldc, int kslice, size_t slice_stride) {
-  gemm_body<ALoad, BLoad, T, TILE>(M, N, K, alpha, a, bl, C, ldc, kslice, slice_stride, blockIdx.x, blockIdx.y,
+  gemm_body<ALoad, BLoad, TILE>(M, N, K, alpha, a, bl, C, ldc, kslice, slice_stride, blockIdx.x, blockIdx.y,
                                    blockIdx.z);
 }
 
-// How a GEMM of the FMA kernel is spread over the SMs (the larger FP64 ones run
-// sliced on the tensor cores, oz_plan).  FP64 issues about two FMAs per SM per
-// clock on GB300, so a GEMM runs at the rate of the SMs it occupies: 64 x 64
-// tiles when they alone give every SM a block, else 32 x 32 tiles, and K
-// split into slices (multiples of 16, at most 32) until there are about two
-// blocks per SM; the slices' partial products are summed in a fixed order.
-// The plan depends on the shape and the device only, so a GEMM gives the same
-// bits alone, in a batch or in a group.
+// How an FP32 contraction is spread over the SMs: 64 x 64 tiles when they alone
+// give every SM a block, else 32 x 32 tiles, and K split into slices (multiples of
+// 16, at most 32) until there are about two blocks per SM; the slices' partial
+// products are summed in a fixed order.  Shape and device only, so a GEMM gives
+// the same bits alone, in a batch or in a group.
 GemmPlan gemm_plan(const vp_ctx* ctx, int M, int N, int K) {
   GemmPlan g{64, 1, K};
   const int t64 = ((M + 63) / 64) * ((N + 63) / 64);
@@ -723,28 +721,25 @@ static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a
   if (ctx->precision >= VP_PREC_TF32 && K > 0) return launch_tc_gemm(ctx, M, N, K, alpha, tc_a(a), tc_b(b), C, ldc);
   if (ctx->precision == VP_PREC_FP64) {
     const OzPlan oz = oz_plan(ctx, M, N, K);
-    if (oz.use) {
-      const size_t stride = (size_t)M * N;
-      const bool split = oz.slices > 1;
-      if (split) VP_TRY(reserve(ctx, ctx->w_split, stride * oz.slices));
-      std::vector<OzGemm> job;
-      job.push_back(oz_job(tc_a(a), tc_b(b), M, N, K, alpha, split ? ctx->w_split.p : C, split ? N : ldc,
-                           split ? stride : 0, &ctx->w_tca, &ctx->w_tcb, ctx->status, oz));
-      VP_TRY(blaunch_oz_gemm(ctx, ctx->stream, job));
-      if (!split) return VP_OK;
-      const int blocks = (int)std::min<size_t>((stride + 255) / 256, (size_t)ctx->num_sms * 8);
-      ctx->launches++;
-      k_sum_slices<<<blocks, 256, 0, ctx->stream>>>(ctx->w_split.p, M, N, oz.slices, stride, C, ldc);
-      return check_launch(ctx, what);
-    }
+    const size_t stride = (size_t)M * N;
+    const bool split = oz.use && oz.slices > 1;
+    if (split) VP_TRY(reserve(ctx, ctx->w_split, stride * oz.slices));
+    std::vector<OzGemm> job;
+    job.push_back(oz_job(tc_a(a), tc_b(b), M, N, K, alpha, split ? ctx->w_split.p : C, split ? N : ldc,
+                         split ? stride : 0, &ctx->w_tca, &ctx->w_tcb, ctx->status, oz));
+    if (!oz.use) return blaunch_fma_gemm(ctx, ctx->stream, job);
+    VP_TRY(blaunch_oz_gemm(ctx, ctx->stream, job));
+    if (!split) return VP_OK;
+    const int blocks = (int)std::min<size_t>((stride + 255) / 256, (size_t)ctx->num_sms * 8);
+    ctx->launches++;
+    k_sum_slices<<<blocks, 256, 0, ctx->stream>>>(ctx->w_split.p, M, N, oz.slices, stride, C, ldc);
+    return check_launch(ctx, what);
   }
   const GemmPlan pl = gemm_plan(ctx, M, N, K);
   dim3 grid((M + pl.tile - 1) / pl.tile, (N + pl.tile - 1) / pl.tile, 1);
   if (grid.y > 65535) return fail(ctx, VP_ECAPACITY, "gemm: N too large");
   // FP32 contraction mode: inputs rounded to FP32, FP32 FMA and accumulation
-  const bool f32 = ctx->precision == VP_PREC_FP32_CONTRACT;
-  auto kern = pl.tile == 64 ? (f32 ? k_gemm<ALoad, BLoad, float, 64> : k_gemm<ALoad, BLoad, double, 64>)
-                            : (f32 ? k_gemm<ALoad, BLoad, float, 32> : k_gemm<ALoad, BLoad, double, 32>);
+  auto kern = pl.tile == 64 ? k_gemm<ALoad, BLoad, 64> : k_gemm<ALoad, BLoad, 32>;
   int slices = pl.slices;
   const int kslice = pl.kslice;
   if (slices <= 1) {
@@ -1877,12 +1872,12 @@ struct GemmJob {
   int ldc;
   size_t stride;
 };
-template <class ALoad, class BLoad, class T, int TILE>
+template <class ALoad, class BLoad, int TILE>
 __global__ void __launch_bounds__(256) kb_gemm(const __grid_constant__ Pack<GemmJob<ALoad, BLoad>> pk, int zs) {
   const GemmJob<ALoad, BLoad>& j = pk.a[blockIdx.z / zs];
   const int slice = blockIdx.z % zs;
   if (slice >= j.slices || (int)blockIdx.x * TILE >= j.M || (int)blockIdx.y * TILE >= j.N) return;
-  gemm_body<ALoad, BLoad, T, TILE>(j.M, j.N, j.K, j.alpha, j.a, j.b, j.C, j.ldc, j.kslice, j.stride, blockIdx.x,
+  gemm_body<ALoad, BLoad, TILE>(j.M, j.N, j.K, j.alpha, j.a, j.b, j.C, j.ldc, j.kslice, j.stride, blockIdx.x,
                                    blockIdx.y, slice);
 }
 struct SumArgs {
@@ -1898,7 +1893,7 @@ __global__ void kb_sum_slices(const __grid_constant__ Pack<SumArgs> pk) {
 }
 
 namespace {
-template <class ALoad, class BLoad, class T, int TILE>
+template <class ALoad, class BLoad, int TILE>
 int gemm_group(vp_ctx* ctx, cudaStream_t st, const std::vector<GemmJob<ALoad, BLoad>>& jobs) {
   for (size_t i0 = 0; i0 < jobs.size(); i0 += kMaxBatch) {
     const int nb = (int)std::min<size_t>(kMaxBatch, jobs.size() - i0);
@@ -1913,7 +1908,7 @@ int gemm_group(vp_ctx* ctx, cudaStream_t st, const std::vector<GemmJob<ALoad, BL
     }
     if (gy > 65535) return fail(ctx, VP_ECAPACITY, "gemm: N too large");
     ctx->launches++;
-    kb_gemm<ALoad, BLoad, T, TILE><<<dim3(gx, gy, nb * zs), 256, 0, st>>>(pk, zs);
+    kb_gemm<ALoad, BLoad, TILE><<<dim3(gx, gy, nb * zs), 256, 0, st>>>(pk, zs);
     VP_TRY(check_launch(ctx, "b_gemm"));
   }
   return VP_OK;
@@ -1921,18 +1916,18 @@ int gemm_group(vp_ctx* ctx, cudaStream_t st, const std::vector<GemmJob<ALoad, BL
 }  // namespace
 
 int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
-  // [FP32 contraction][tile 64 / 32]
-  std::vector<GemmJob<ARowMajor, BRowMajor>> ab[2][2];
-  std::vector<GemmJob<ARowMajor, BTransposed>> abt[2][2];
-  std::vector<GemmJob<AUpperColMajor, BRowMajor>> rb[2][2];
+  // FP32 contractions by tile (64 / 32)
+  std::vector<GemmJob<ARowMajor, BRowMajor>> ab[2];
+  std::vector<GemmJob<ARowMajor, BTransposed>> abt[2];
+  std::vector<GemmJob<AUpperColMajor, BRowMajor>> rb[2];
   std::vector<SumArgs> sums;
-  std::vector<OzGemm> oz;
+  std::vector<OzGemm> oz, fma;
   SlotCounter slots;
   for (const BGemm& g : v) {
     if (g.M <= 0 || g.N <= 0) continue;
     const GemmPlan pl = gemm_plan(ctx, g.M, g.N, g.K);
     const OzPlan op = g.fp32 ? OzPlan{} : oz_plan(ctx, g.M, g.N, g.K);
-    const int slices = op.use ? op.slices : pl.slices, kslice = pl.kslice, ti = pl.tile == 64 ? 0 : 1;
+    const int slices = g.fp32 ? pl.slices : op.use ? op.slices : 1, kslice = pl.kslice, ti = pl.tile == 64 ? 0 : 1;
     double* C = g.C;
     int ldc = g.ldc;
     size_t stride = 0;
@@ -1945,36 +1940,30 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
       ldc = g.N;
       sums.push_back({g.s->split[sl].p, g.M, g.N, slices, stride, g.C, g.ldc});
     }
-    const int t = g.fp32 ? 1 : 0;
-    if (op.use) {
+    if (!g.fp32) {
       const TcOperand ta{g.A, g.lda, g.kind == BG_RB ? 2 : 0}, tb{g.B, g.ldb, g.kind == BG_ABT ? 0 : 1};
-      oz.push_back(oz_job(ta, tb, g.M, g.N, g.K, g.alpha, C, ldc, stride, &g.s->oza[sl], &g.s->ozb[sl],
-                          g.s->st ? g.s->st : ctx->status, op));
+      (op.use ? oz : fma).push_back(oz_job(ta, tb, g.M, g.N, g.K, g.alpha, C, ldc, stride, g.s ? &g.s->oza[sl] : nullptr,
+                                           g.s ? &g.s->ozb[sl] : nullptr, g.s && g.s->st ? g.s->st : ctx->status, op));
       continue;
     }
     if (g.kind == BG_AB)
-      ab[t][ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, ARowMajor{g.A, g.lda}, BRowMajor{g.B, g.ldb}, C, ldc,
-                       stride});
+      ab[ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, ARowMajor{g.A, g.lda}, BRowMajor{g.B, g.ldb}, C, ldc,
+                        stride});
     else if (g.kind == BG_ABT)
-      abt[t][ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, ARowMajor{g.A, g.lda}, BTransposed{g.B, g.ldb}, C,
-                        ldc, stride});
+      abt[ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, ARowMajor{g.A, g.lda}, BTransposed{g.B, g.ldb}, C, ldc,
+                         stride});
     else
-      rb[t][ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, AUpperColMajor{g.A, g.lda}, BRowMajor{g.B, g.ldb}, C,
-                       ldc, stride});
+      rb[ti].push_back({g.M, g.N, g.K, kslice, slices, g.alpha, AUpperColMajor{g.A, g.lda}, BRowMajor{g.B, g.ldb}, C,
+                        ldc, stride});
   }
   VP_TRY(blaunch_oz_gemm(ctx, st, oz));
-  VP_TRY((gemm_group<ARowMajor, BRowMajor, double, 64>(ctx, st, ab[0][0])));
-  VP_TRY((gemm_group<ARowMajor, BRowMajor, double, 32>(ctx, st, ab[0][1])));
-  VP_TRY((gemm_group<ARowMajor, BRowMajor, float, 64>(ctx, st, ab[1][0])));
-  VP_TRY((gemm_group<ARowMajor, BRowMajor, float, 32>(ctx, st, ab[1][1])));
-  VP_TRY((gemm_group<ARowMajor, BTransposed, double, 64>(ctx, st, abt[0][0])));
-  VP_TRY((gemm_group<ARowMajor, BTransposed, double, 32>(ctx, st, abt[0][1])));
-  VP_TRY((gemm_group<ARowMajor, BTransposed, float, 64>(ctx, st, abt[1][0])));
-  VP_TRY((gemm_group<ARowMajor, BTransposed, float, 32>(ctx, st, abt[1][1])));
-  VP_TRY((gemm_group<AUpperColMajor, BRowMajor, double, 64>(ctx, st, rb[0][0])));
-  VP_TRY((gemm_group<AUpperColMajor, BRowMajor, double, 32>(ctx, st, rb[0][1])));
-  VP_TRY((gemm_group<AUpperColMajor, BRowMajor, float, 64>(ctx, st, rb[1][0])));
-  VP_TRY((gemm_group<AUpperColMajor, BRowMajor, float, 32>(ctx, st, rb[1][1])));
+  VP_TRY(blaunch_fma_gemm(ctx, st, fma));
+  VP_TRY((gemm_group<ARowMajor, BRowMajor, 64>(ctx, st, ab[0])));
+  VP_TRY((gemm_group<ARowMajor, BRowMajor, 32>(ctx, st, ab[1])));
+  VP_TRY((gemm_group<ARowMajor, BTransposed, 64>(ctx, st, abt[0])));
+  VP_TRY((gemm_group<ARowMajor, BTransposed, 32>(ctx, st, abt[1])));
+  VP_TRY((gemm_group<AUpperColMajor, BRowMajor, 64>(ctx, st, rb[0])));
+  VP_TRY((gemm_group<AUpperColMajor, BRowMajor, 32>(ctx, st, rb[1])));
   return run_packs(ctx, st, sums, kb_sum_slices, 256, 0,
                    [&](const SumArgs& a) { return grid_stride_blocks(ctx, a.stride, 8); }, "b_sum_slices");
 }
