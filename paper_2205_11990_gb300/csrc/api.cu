@@ -268,6 +268,15 @@ struct SideScope {
   }
 };
 
+// A row-major matrix with rows of n entries as the source of a QR.
+static QRSrc row_major(const double* p, int n) {
+  QRSrc s;
+  s.p = p;
+  s.rs = n;
+  s.cs = 1;
+  return s;
+}
+
 // QR sweep over sites 0..kend-1 (left-canonical form up to site kend): at
 // site k the Householder QR of the (2 r_{k-1} x r_k) reshape, R multiplied
 // into core k+1 on the context's stream, while Q (the new core k) is formed
@@ -302,9 +311,8 @@ static int qr_sweep(vp_ctx* ctx, mps_t* s, int kend) {
     VP_TRY(reserve(ctx, P, (size_t)2 * m + p + 8));
     double* tau = P.p;
     double* vbuf = P.p + p + 8;
-    VP_TRY(launch_to_colmajor(ctx, s->core[k].p, m, n, F.p));
     prof_begin(ctx, VP_K_QR);
-    VP_TRY(launch_qr_factor(ctx, F.p, m, n, tau, vbuf));
+    VP_TRY(launch_qr_factor(ctx, F.p, m, n, tau, vbuf, row_major(s->core[k].p, n)));
     prof_end(ctx, VP_K_QR, qr_flops(m, n), m, n);
     VP_CUDA(ctx, cudaEventRecord(ctx->ev_qf[b], ctx->stream));
     {
@@ -361,25 +369,30 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
   VP_TRY(reserve(ctx, ctx->w_piv, (size_t)q + 8));
   int* piv = (int*)ctx->w_piv.p;
   int* piv2 = piv + q;
-  VP_TRY(launch_norm_order(ctx, s->core[k].p, m, c, tall ? 1 : 0, piv));
+  VP_TRY(launch_norm_order(ctx, s->core[k].p, c, m, c, tall ? 1 : 0, 0, piv));
   // first QR: A Pi = Q1 R1, A = M or M^T
   VP_TRY(reserve(ctx, ctx->w_fac, (size_t)p * q));
   VP_TRY(reserve(ctx, ctx->w_p, (size_t)2 * p + q + 8));
-  VP_TRY(launch_gather_cm(ctx, s->core[k].p, m, c, piv, tall ? 1 : 0, ctx->w_fac.p));
+  QRSrc src1;
+  src1.p = s->core[k].p;
+  (tall ? src1.rs : src1.cs) = c;
+  (tall ? src1.cs : src1.rs) = 1;
+  src1.perm = piv;
   prof_begin(ctx, VP_K_QR);
-  VP_TRY(launch_qr_factor(ctx, ctx->w_fac.p, p, q, ctx->w_p.p, ctx->w_p.p + q + 8));
+  VP_TRY(launch_qr_factor(ctx, ctx->w_fac.p, p, q, ctx->w_p.p, ctx->w_p.p + q + 8, src1));
   prof_end(ctx, VP_K_QR, qr_flops(p, q), p, q);
   VP_TRY(reserve(ctx, ctx->w_r, (size_t)q * q));
-  VP_TRY(launch_qr_getr(ctx, ctx->w_fac.p, p, q, ctx->w_r.p));
   VP_TRY(reserve(ctx, ctx->w_p2, (size_t)3 * q + 8));
   VP_TRY(reserve(ctx, ctx->w_p3, (size_t)3 * q + 8));
   VP_TRY(reserve(ctx, ctx->w_x, (size_t)q * q));
-  double* fac = ctx->w_fac.p;  // factor whose Q the output needs
-  double* tau = ctx->w_p.p;
+  const double* fac = ctx->w_fac.p;  // factor whose Q the output needs
+  const double* tau = ctx->w_p.p;
   int qm = p;
-  if (tall) {  // second QR: R1^T = Q2 L^T (R1 row-major is R1^T column-major)
+  if (tall) {  // second QR: R1^T = Q2 L^T
+    QRSrc src2 = row_major(ctx->w_fac.p, p);  // R1, read as its transpose
+    src2.lower = 1;
     prof_begin(ctx, VP_K_QR);
-    VP_TRY(launch_qr_factor(ctx, ctx->w_r.p, q, q, ctx->w_p2.p, ctx->w_p2.p + q + 8));
+    VP_TRY(launch_qr_factor(ctx, ctx->w_r.p, q, q, ctx->w_p2.p, ctx->w_p2.p + q + 8, src2));
     prof_end(ctx, VP_K_QR, qr_flops(q, q), q, q);
     fac = ctx->w_r.p;
     tau = ctx->w_p2.p;
@@ -395,7 +408,7 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
   {
     SideScope side(ctx);
     prof_begin(ctx, VP_K_FORMQ);
-    side_st = launch_qr_formq(ctx, fac, qm, q, tau, ctx->w_q1.p);
+    side_st = launch_qr_formq(ctx, fac, qm, q, tau, ctx->w_q1.p, tall ? piv : nullptr);  // tall: Pi Q2
     prof_end(ctx, VP_K_FORMQ, 4.0 * qm * q * q - 4.0 / 3.0 * q * q * q, qm, q);
   }
   VP_CUDA(ctx, cudaEventRecord(ctx->ev_join, ctx->side));
@@ -406,32 +419,30 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
     ~SideJoin() { cudaStreamWaitEvent(c->stream, c->ev_join, 0); }
   } side_join{ctx};
   VP_TRY(side_st);
-  // last QR, from the left: its R (columns ordered) is what Jacobi diagonalises
-  if (tall) {
-    VP_TRY(reserve(ctx, ctx->w_l, (size_t)q * q));
-    VP_TRY(launch_lower_from_upper(ctx, ctx->w_r.p, q, ctx->w_l.p));
-    VP_TRY(launch_norm_order(ctx, ctx->w_l.p, q, q, 1, piv2));
-    VP_TRY(launch_gather_cm(ctx, ctx->w_l.p, q, q, piv2, 1, ctx->w_x.p));
-  } else {  // columns of R1^T are rows of R1
-    VP_TRY(launch_norm_order(ctx, ctx->w_r.p, q, q, 0, piv2));
-    VP_TRY(launch_gather_cm(ctx, ctx->w_r.p, q, q, piv2, 0, ctx->w_x.p));
-  }
+  // last QR, from the left, of L or R1^T (the transpose of the factor's upper
+  // triangle), columns ordered: its R is what Jacobi diagonalises
+  VP_TRY(launch_norm_order(ctx, fac, qm, q, q, 1, 1, piv2));
+  QRSrc src3 = row_major(fac, qm);
+  src3.perm = piv2;
+  src3.lower = 1;
   prof_begin(ctx, VP_K_QR);
-  VP_TRY(launch_qr_factor(ctx, ctx->w_x.p, q, q, ctx->w_p3.p, ctx->w_p3.p + q + 8));
+  VP_TRY(launch_qr_factor(ctx, ctx->w_x.p, q, q, ctx->w_p3.p, ctx->w_p3.p + q + 8, src3));
   prof_end(ctx, VP_K_QR, qr_flops(q, q), q, q);
-  VP_TRY(reserve(ctx, ctx->w_tmp, (size_t)q * q));
+  VP_TRY(reserve(ctx, ctx->w_tmp, (size_t)q * q + q));
   double* X = ctx->w_tmp.p;
-  VP_TRY(launch_qr_getr(ctx, ctx->w_x.p, q, q, X));
+  double* norms = X + (size_t)q * q;
+  bool have_norms = false;
   VP_CUDA(ctx, cudaMemsetAsync(ctx->status->rot, 0, sizeof(ctx->status->rot), ctx->stream));
   prof_begin(ctx, VP_K_JACOBI);
-  VP_TRY(launch_jacobi_rows(ctx, X, q, q, tol >= 1e-13));
+  VP_TRY(launch_jacobi_rows(ctx, ctx->w_x.p, X, q, norms, tol >= 1e-13, &have_norms));
   prof_end(ctx, VP_K_JACOBI, 0.0, q, q);
   const size_t jac_mark = ctx->prof_on && !ctx->prof_marks.empty() ? ctx->prof_marks.size() - 1 : (size_t)-1;
   VP_TRY(reserve(ctx, ctx->w_vec, (size_t)2 * q + 8));
   int* perm = (int*)ctx->w_vec.p;
   double* sigma = ctx->w_vec.p + (q + 1) / 2 + 4;
   prof_begin(ctx, VP_K_SELECT);
-  VP_TRY(launch_select(ctx, X, q, q, chi, tol, perm, sigma, ctx->d_small, ctx->d_smalld));
+  VP_TRY(launch_select(ctx, X, have_norms ? norms : nullptr, q, q, chi, tol, g_entropy != nullptr, perm, sigma, ctx->d_small,
+                       ctx->d_smalld));
   prof_end(ctx, VP_K_SELECT, 0.0, q, q);
   int r = 1;
   double err = 0.0;
@@ -453,14 +464,7 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
   // V^T enters both cores: FP64 in every contraction mode
   const int prec = ctx->precision;
   ctx->precision = VP_PREC_FP64;
-  int st = VP_OK;
-  if (tall) {
-    st = reserve(ctx, ctx->w_c, (size_t)r * q);
-    if (st == VP_OK) st = launch_gemm_bt(ctx, r, q, q, ctx->w_a.p, q, ctx->w_q1.p, q, ctx->w_c.p, q);
-    if (st == VP_OK) st = launch_scatter(ctx, ctx->w_c.p, r, q, piv, 1, Vt);
-  } else {
-    st = launch_gemm_bt(ctx, r, c, q, ctx->w_a.p, q, ctx->w_q1.p, q, Vt, c);
-  }
+  const int st = launch_gemm_bt(ctx, r, c, q, ctx->w_a.p, q, ctx->w_q1.p, q, Vt, c);
   ctx->precision = prec;
   VP_TRY(st);
   VP_TRY(launch_gemm_bt(ctx, m, r, c, s->core[k].p, c, Vt, c, ctx->w_b.p, r));  // U S = M V
@@ -503,10 +507,12 @@ static int lq_site(vp_ctx* ctx, mps_t* s, int k) {
   const int rows = 2 * s->r[k - 1];
   VP_TRY(reserve(ctx, ctx->w_fac, (size_t)m * n));
   VP_TRY(reserve(ctx, ctx->w_p, (size_t)2 * m + p + 8));
-  VP_TRY(launch_copy(ctx, s->core[k].p, ctx->w_fac.p, (size_t)m * n));
+  QRSrc src;
+  src.p = s->core[k].p;
+  src.cs = m;
   double* tau = ctx->w_p.p;
   prof_begin(ctx, VP_K_QR);
-  VP_TRY(launch_qr_factor(ctx, ctx->w_fac.p, m, n, tau, ctx->w_p.p + p + 8));
+  VP_TRY(launch_qr_factor(ctx, ctx->w_fac.p, m, n, tau, ctx->w_p.p + p + 8, src));
   prof_end(ctx, VP_K_QR, qr_flops(m, n), m, n);
   VP_TRY(reserve(ctx, ctx->w_q1, (size_t)m * p));
   prof_begin(ctx, VP_K_FORMQ);
@@ -615,8 +621,7 @@ static int from_vector(vp_ctx* ctx, mps_t* s, int n, const double* vec, int chi,
     const int nc = (int)cols, p = (int)std::min<size_t>(m, cols);
     VP_TRY(reserve(ctx, ctx->w_fac, (size_t)m * nc));
     VP_TRY(reserve(ctx, ctx->w_p, (size_t)2 * m + p + 8));
-    VP_TRY(launch_to_colmajor(ctx, rem.p, m, nc, ctx->w_fac.p));
-    VP_TRY(launch_qr_factor(ctx, ctx->w_fac.p, m, nc, ctx->w_p.p, ctx->w_p.p + p + 8));
+    VP_TRY(launch_qr_factor(ctx, ctx->w_fac.p, m, nc, ctx->w_p.p, ctx->w_p.p + p + 8, row_major(rem.p, nc)));
     VP_TRY(reserve(ctx, s->core[k], (size_t)m * p));
     VP_TRY(launch_qr_formq(ctx, ctx->w_fac.p, m, nc, ctx->w_p.p, s->core[k].p));
     VP_TRY(launch_qr_getr(ctx, ctx->w_fac.p, m, nc, rem.p));
@@ -846,7 +851,7 @@ int vp_ctx_destroy(vp_ctx* c) {
   if (!c) return VP_EINVAL;
   cudaStreamSynchronize(c->stream);
   for (DevBuf* b : {&c->w_fac, &c->w_q, &c->w_gemm, &c->w_x, &c->w_p3, &c->w_p, &c->w_tmp, &c->w_tmp2, &c->w_vec, &c->w_split,
-                    &c->w_piv, &c->w_q1, &c->w_r, &c->w_p2, &c->w_a, &c->w_b, &c->w_c, &c->w_l,
+                    &c->w_piv, &c->w_q1, &c->w_r, &c->w_p2, &c->w_a, &c->w_b,
                     &c->w_q_side, &c->w_split_side, &c->w_tca, &c->w_tcb, &c->w_tca_side, &c->w_tcb_side,
                     &c->w_qrv, &c->w_qrc, &c->w_fq, &c->w_fq_side, &c->w_fac_b, &c->w_p_b,
                     &c->w_sig, &c->w_wq, &c->w_wr})

@@ -87,7 +87,7 @@ struct vp_ctx {
   int64_t prof_launches[VP_K_COUNT] = {};
   // workspaces
   vp::DevBuf w_fac, w_q, w_gemm, w_p, w_tmp, w_tmp2, w_vec, w_split;
-  vp::DevBuf w_piv, w_q1, w_r, w_p2, w_x, w_p3, w_a, w_b, w_c, w_l;  // preconditioned SVD
+  vp::DevBuf w_piv, w_q1, w_r, w_p2, w_x, w_p3, w_a, w_b;  // preconditioned SVD
   vp::DevBuf w_tca, w_tcb;            // packed operands (or digits) of the tensor-core contractions
   vp::DevBuf w_q_side, w_split_side;  // scratch of the side-stream phase
   vp::DevBuf w_tca_side, w_tcb_side;
@@ -170,9 +170,18 @@ struct AttrOnce {
 // ------------------------------------------------------------ kernels (linalg.cu)
 // Row-major (m x n) -> column-major copy.
 int launch_to_colmajor(vp_ctx* ctx, const double* A, int m, int n, double* out);
-// In-place Householder QR of the column-major m x n matrix A (lda = m):
-// R in the upper triangle, reflectors below, tau[min(m,n)].
-int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* vbuf);
+// Where the entries of a factor come from: entry (i, k) at p[i rs + c cs], c =
+// perm[k] (k without perm); lower: zero above the diagonal, i < c.  p NULL: the
+// factor's own column-major buffer.
+struct QRSrc {
+  const double* p = nullptr;
+  long long rs = 1, cs = 0;
+  const int* perm = nullptr;
+  int lower = 0;
+};
+// Householder QR of an m x n matrix into the column-major buffer A (lda = m): R in
+// the upper triangle, reflectors below, tau[min(m,n)].
+int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* vbuf, const QRSrc& src = QRSrc());
 // Kernel that factors an m x n matrix (shape and device only).
 enum { QR_NONE = 0, QR_WIDE, QR_PANEL, QR_GRID };
 enum { PANEL_NONE = 0, PANEL_SOLO, PANEL_CLUSTER, PANEL_GRID };
@@ -191,14 +200,16 @@ struct PanelJob {
   int m, n;
   double* tau;
   PanelPlan plan;
-  DevBuf* scratch;  // block reflectors' T and the columns' exponents
+  QRSrc src;
+  DevBuf* scratch;  // the panels' products and the columns' exponents
   DevBuf* cols;     // columns beyond shared memory (PANEL_GRID)
   DevStatus* st;    // status words (PANEL_GRID)
 };
 int blaunch_qr_panel(vp_ctx* ctx, cudaStream_t st, const std::vector<PanelJob>& v);
 QRPlan qr_plan(const vp_ctx* ctx, int m, int n);
-// Q (m x p, p = min(m,n)) written row-major from the factored A.
-int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q);
+// Q (m x p, p = min(m,n)) written row-major from the factored A, its row i in row
+// rows[i] of the output (NULL: i).
+int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q, const int* rows = nullptr);
 // Upper-trapezoidal R (p x n) of the factored A, written row-major.
 int launch_qr_getr(vp_ctx* ctx, const double* A, int m, int n, double* R);
 // Output tile and split-K of an FP32 contraction (shape and device only).
@@ -214,11 +225,9 @@ int launch_gemm(vp_ctx* ctx, int M, int N, int K, double alpha, const double* A,
 // C (M x N) = A (M x K) * Bt^T, Bt given row-major (N x K).
 int launch_gemm_bt(vp_ctx* ctx, int M, int N, int K, const double* A, int lda, const double* Bt, int ldbt,
                    double* C, int ldc);
-// SVD preconditioning helpers (static pivoting by norm, see linalg.cu).
-int launch_norm_order(vp_ctx* ctx, const double* M, int m, int c, int by_cols, int* piv);
-int launch_gather_cm(vp_ctx* ctx, const double* M, int m, int c, const int* piv, int tall, double* out);
-int launch_lower_from_upper(vp_ctx* ctx, const double* Rcm, int q, double* L);
-int launch_scatter(vp_ctx* ctx, const double* Y, int rows, int cols_n, const int* piv, int cols, double* out);
+// Decreasing order of the column (by_cols) or row norms of a row-major m x c matrix
+// (row stride ld; lower: entries right of the diagonal count as zero).
+int launch_norm_order(vp_ctx* ctx, const double* M, int ld, int m, int c, int by_cols, int lower, int* piv);
 // Operand of a tensor-core contraction as (row, k) -> value: kind 0
 // p[r * ld + k]; kind 1 p[k * ld + r]; kind 2 the upper triangle of a
 // column-major factor, r <= k ? p[k * ld + r] : 0.
@@ -258,20 +267,24 @@ int blaunch_fma_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v)
 // C = alpha * triu(A_colmajor) (M x K) * B: the R factor read in place.
 int launch_gemm_r(vp_ctx* ctx, int M, int N, int K, const double* Acm, int lda, const double* B,
                   int ldb, double* C, int ldc);
-// One-sided Jacobi on the b rows (length c) of X.  Row-major, contiguous.
-// floor_ok: the caller truncates every singular value below 1e-13 of the
+// One-sided Jacobi on the rows of X (b x b, row-major), starting from the upper
+// triangle R of a column-major factor (the rest of its entries ignored).
+// norms: receives the row norms where the double-word kernel ran, which *have_norms
+// tells.  floor_ok: the caller truncates every singular value below 1e-13 of the
 // largest (tol >= 1e-13), so the double-word kernel, which leaves rows under
 // 1e-15 of the largest unrotated, may be used.
-int launch_jacobi_rows(vp_ctx* ctx, double* X, int b, int c, bool floor_ok);
+int launch_jacobi_rows(vp_ctx* ctx, const double* R, double* X, int b, double* norms, bool floor_ok, bool* have_norms);
 // The same on a given stream with given status words.
-int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* X, int b, int c, bool floor_ok);
+int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, const double* R, double* X, int b, double* norms,
+                   bool floor_ok, bool* have_norms);
 // Largest cluster (16 or 8 CTAs, one per SM) the cluster-resident kernels
 // can use on this device; 0 if none.
 int probe_cluster_size();
 // Sort row norms of X descending, choose the kept rank (chi, tol, ties),
 // write perm/sigma/rank/truncation error into ctx scratch.  d_out[0] = rank.
-int launch_select(vp_ctx* ctx, const double* X, int b, int c, int chi, double tol, int* perm,
-                  double* sigma, int* d_rank, double* d_err);
+// norms: the row norms, or NULL; the entropy is formed only if want_ent.
+int launch_select(vp_ctx* ctx, const double* X, const double* norms, int b, int c, int chi, double tol, bool want_ent,
+                  int* perm, double* sigma, int* d_rank, double* d_err);
 // V (r x q), V[t][cperm[j]] = X[perm[t]][j] / sigma[t].
 int launch_svd_outputs(vp_ctx* ctx, const double* X, int q, int r, const int* perm, const double* sigma,
                        const int* cperm, double* V);
@@ -354,9 +367,8 @@ struct BScratch {
 };
 void release_scratch(vp_ctx* ctx, BScratch& s);
 
-struct BColMajor { const double* A; int m, n; double* out; };
-struct BQR { double* A; int m, n; double* tau; double* vbuf; BScratch* s; };
-struct BFormQ { const double* A; int m, n; const double* tau; double* Q; BScratch* s; };
+struct BQR { double* A; int m, n; double* tau; double* vbuf; BScratch* s; QRSrc src = QRSrc(); };
+struct BFormQ { const double* A; int m, n; const double* tau; double* Q; BScratch* s; const int* rows = nullptr; };
 struct BGetR { const double* A; int m, n; double* R; };
 enum { BG_AB = 0, BG_ABT = 1, BG_RB = 2 };  // A row-major x B row-major / B^T given / triu(A col-major) x B
 struct BGemm {
@@ -369,33 +381,29 @@ struct BGemm {
   double* C; int ldc;
   BScratch* s;
 };
-struct BNormOrder { const double* M; int m, c, by_cols; int* piv; };
-struct BGather { const double* M; int m, c; const int* piv; int tall; double* out; };
-struct BLowerUpper { const double* R; int q; double* L; };
+struct BNormOrder { const double* M; int ld, m, c, by_cols, lower; int* piv; };
+struct BGather { QRSrc src; int m, n; double* A; };
 struct BCopy { const double* src; double* dst; size_t n; };
-struct BJacobi { double* X; int b, c; DevStatus* st; };
+struct BJacobi { const double* R; double* X; int b; double* norms; DevStatus* st; };
 struct BSelect {
-  const double* X; int b, c, chi; double tol; int* perm; double* sigma; int* d_rank; double* d_err; DevStatus* st;
+  const double* X; const double* norms; int b, c, chi; double tol; int want_ent; int* perm; double* sigma; int* d_rank;
+  double* d_err; DevStatus* st;
 };
 struct BSvdOut { const double* X; int q, r; const int* perm; const double* sigma; const int* cperm; double* V; };
-struct BScatter { const double* Y; int rows, cols_n; const int* piv; int cols; double* out; };
 
-int blaunch_to_colmajor(vp_ctx* ctx, cudaStream_t st, const std::vector<BColMajor>& v);
 int blaunch_qr_factor(vp_ctx* ctx, cudaStream_t st, const std::vector<BQR>& v);
 int blaunch_qr_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<BFormQ>& v);
 int blaunch_qr_getr(vp_ctx* ctx, cudaStream_t st, const std::vector<BGetR>& v);
 int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v);
 int blaunch_norm_order(vp_ctx* ctx, cudaStream_t st, const std::vector<BNormOrder>& v);
-int blaunch_gather_cm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGather>& v);
-int blaunch_lower_from_upper(vp_ctx* ctx, cudaStream_t st, const std::vector<BLowerUpper>& v);
-// Jacobi of truncating compressions (tol >= 1e-13: the double-word kernel of
-// jacobi.cu where the rows fit a cluster).
-bool jacobi_dw_fits(const vp_ctx* ctx, int b, int c);
+// Jacobi of truncating compressions (tol >= 1e-13): the double-word kernel of
+// jacobi.cu where the rows fit a cluster.
+bool jacobi_dw_fits(const vp_ctx* ctx, int b);
 int blaunch_jacobi_dw(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v);
-int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v);
+// have_norms[i]: problem i's norms were written.
+int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v, std::vector<char>& have_norms);
 int blaunch_select(vp_ctx* ctx, cudaStream_t st, const std::vector<BSelect>& v);
 int blaunch_svd_outputs(vp_ctx* ctx, cudaStream_t st, const std::vector<BSvdOut>& v);
-int blaunch_scatter(vp_ctx* ctx, cudaStream_t st, const std::vector<BScatter>& v);
 
 // mpsops.cu
 struct BSiteSum { SiteSum s; double* out; int ol, orr; };

@@ -87,6 +87,45 @@ __device__ __forceinline__ dw dw_from(double x) {
 }
 __device__ __forceinline__ double dw_to(dw x) { return (double)x.hi + (double)x.lo; }
 
+// The same through integer and FP32 operations: a conversion, product or sum on the
+// FP64 pipe costs one of the two slots an SM has per clock, and a split or a
+// recombination four of them.  x 2^-e split to hi = RN24, lo = RN24 of the rest
+// (|x 2^-e| below 2^127; what lies below the FP32 range becomes zero).
+__device__ __forceinline__ float pow2f(int e) { return e < -126 ? 0.0f : __int_as_float((e + 127) << 23); }
+__device__ __forceinline__ dw dw_from_scaled(double x, int e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)(b >> 52) & 0x7ff;
+  if (ex == 0) return {0.f, 0.f};  // zero (or far below any column's scale)
+  if (ex == 2047) return {__int_as_float(0x7fc00000), 0.f};  // not finite: NaN
+  const unsigned long long m = (b & ((1ull << 52) - 1)) | (1ull << 52);
+  const unsigned rest = (unsigned)m & ((1u << 29) - 1);
+  unsigned top = (unsigned)(m >> 29);
+  const unsigned up = (rest + (1u << 28) - 1 + (top & 1u)) >> 29;  // to nearest, ties to even
+  top += up;
+  const int s = ex - 1075 - e;  // x 2^-e = m 2^s
+  const float sg = (b >> 63) ? -1.0f : 1.0f;
+  return {sg * __uint2float_rn(top) * pow2f(s + 29), sg * __int2float_rn((int)rest - (int)(up << 29)) * pow2f(s)};
+}
+// (hi + lo) 2^e as FP64, rounded to nearest.
+__device__ __forceinline__ double dw_to_scaled(dw v, int e) {
+  const int bh = __float_as_int(v.hi), eh = (bh >> 23) & 255;
+  const int bl = __float_as_int(v.lo), el = (bl >> 23) & 255;
+  const int d = eh - max(el, 1) - 38;  // > -31: a low word below 2^-7 of the high one
+  if (eh == 0 || eh == 255 || d < -31) return ldexp((double)v.hi + (double)v.lo, e);
+  // in units of 2^(eh - 150 - 38): hi is mh 2^38, lo its bits d places further right,
+  // the last of them standing for all that fall off
+  const long long mh = (long long)((bh & 0x7fffff) | 0x800000) << 38;
+  long long ml = (long long)((bl & 0x7fffff) | (el ? 0x800000 : 0));
+  ml = d <= 0 ? ml << -d : d < 25 ? (ml >> d) | ((ml & ((1ll << d) - 1)) != 0) : (long long)(ml != 0);
+  unsigned long long m = (unsigned long long)(mh + (((bh ^ bl) < 0) ? -ml : ml));
+  const int lz = __clzll((long long)m);                      // 1 .. 3: leading bit at 63 - lz
+  m <<= lz - 1;                                              // to bit 62
+  const unsigned long long r = (m + 511 + ((m >> 10) & 1)) >> 10;  // 53 bits, to nearest even
+  const int be = eh - 127 + 2 - lz + e + 1023;               // exponent of the leading bit: bit 61 was 2^(eh - 127)
+  if (be < 1 || be > 2045) return ldexp((double)v.hi + (double)v.lo, e);
+  return __longlong_as_double((long long)(r + ((unsigned long long)(be - 1) << 52)) | ((long long)(bh & 0x80000000) << 32));
+}
+
 // Compensated dot-product accumulator (Dot2): s + c approximates the sum.
 struct dw_acc {
   float s = 0.f, c = 0.f;

@@ -46,13 +46,13 @@ struct TaskDev {
 // Workspaces of one compression problem (device, grow-only).
 struct Work {
   DevBuf F[2], P[2], gemm;                                       // QR sweep
-  DevBuf piv, fac, p, q1, r, p2, p3, x, tmp, tmp2, l, vec, a, b, c;  // SVD site
+  DevBuf piv, fac, p, q1, r, p2, p3, x, tmp, tmp2, vec, a, b;  // SVD site
   BScratch main, side;                                           // scratch of the batched launchers
 };
 
 void release_work(vp_ctx* ctx, Work& w) {
   for (DevBuf* b : {&w.F[0], &w.F[1], &w.P[0], &w.P[1], &w.gemm, &w.piv, &w.fac, &w.p, &w.q1, &w.r, &w.p2, &w.p3,
-                    &w.x, &w.tmp, &w.tmp2, &w.l, &w.vec, &w.a, &w.b, &w.c})
+                    &w.x, &w.tmp, &w.tmp2, &w.vec, &w.a, &w.b})
     release(ctx, *b);
   release_scratch(ctx, w.main);
   release_scratch(ctx, w.side);
@@ -207,6 +207,15 @@ int reset_records(vp_group* g) {
   return VP_OK;
 }
 
+// A row-major matrix with rows of n entries as the source of a QR.
+QRSrc row_major(const double* p, int n) {
+  QRSrc s;
+  s.p = p;
+  s.rs = n;
+  s.cs = 1;
+  return s;
+}
+
 // ------------------------------------------------------------ QR sweep
 // The lockstep form of api.cu's qr_sweep: at site k of every problem with a
 // site k + 1, the Householder QR of the (2 r_{k-1} x r_k) reshape, R
@@ -234,7 +243,6 @@ int qr_sweep(vp_group* g, const Tasks& all) {
       VP_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, g->ev_qd[b], 0));
       join.busy[b] = false;
     }
-    std::vector<BColMajor> cm;
     std::vector<BQR> qr;
     std::vector<BFormQ> fq;
     std::vector<BGemm> gr;
@@ -248,8 +256,7 @@ int qr_sweep(vp_group* g, const Tasks& all) {
       VP_TRY(reserve(ctx, w.P[b], (size_t)2 * m + p + 8));
       VP_TRY(reserve(ctx, w.gemm, (size_t)p * nn));
       double* tau = w.P[b].p;
-      cm.push_back({s->core[k].p, m, n, w.F[b].p});
-      qr.push_back({w.F[b].p, m, n, tau, w.P[b].p + p + 8, &w.main});
+      qr.push_back({w.F[b].p, m, n, tau, w.P[b].p + p + 8, &w.main, row_major(s->core[k].p, n)});
       fq.push_back({w.F[b].p, m, n, tau, s->core[k].p, &w.side});
       gr.push_back({BG_RB, t->fp32, p, nn, n, 1.0, w.F[b].p, m, s->core[k + 1].p, nn, w.gemm.p, nn, &w.main});
       pv.push_back(p);
@@ -263,7 +270,6 @@ int qr_sweep(vp_group* g, const Tasks& all) {
       wf += f;
       wg += gm;
     }
-    VP_TRY(blaunch_to_colmajor(ctx, ctx->stream, cm));
     VP_TRY(timed(ctx, VP_K_QR, wq, [&] { return blaunch_qr_factor(ctx, ctx->stream, qr); }));
     VP_CUDA(ctx, cudaEventRecord(g->ev_qf[b], ctx->stream));
     {
@@ -304,11 +310,8 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       if (t->s->n - 1 - jstep >= 1 && alive(g, t)) ts.push_back(t);
     if (ts.empty()) continue;
     std::vector<BNormOrder> no, no2;
-    std::vector<BGather> ga, ga2;
     std::vector<BQR> qr1, qr2, qr3;
-    std::vector<BGetR> gr, gx;
     std::vector<BFormQ> fq;
-    std::vector<BLowerUpper> lu;
     std::vector<BJacobi> jc;
     std::vector<BSelect> se;
     for (Task* t : ts) {
@@ -335,33 +338,39 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       VP_TRY(reserve(ctx, w.p2, (size_t)3 * q + 8));
       VP_TRY(reserve(ctx, w.p3, (size_t)3 * q + 8));
       VP_TRY(reserve(ctx, w.x, (size_t)q * q));
-      VP_TRY(reserve(ctx, w.tmp, (size_t)q * q));
-      if (t->tall) VP_TRY(reserve(ctx, w.l, (size_t)q * q));
+      VP_TRY(reserve(ctx, w.tmp, (size_t)q * q + q));
       VP_TRY(reserve(ctx, w.vec, (size_t)2 * q + 8));
       int* piv = (int*)w.piv.p;
       int* piv2 = piv + q;
-      no.push_back({s->core[k].p, m, c, t->tall ? 1 : 0, piv});
-      ga.push_back({s->core[k].p, m, c, piv, t->tall ? 1 : 0, w.fac.p});
-      qr1.push_back({w.fac.p, p, q, w.p.p, w.p.p + q + 8, &w.main});
-      gr.push_back({w.fac.p, p, q, w.r.p});
+      // (the sources and factors of api.cu's svd_site)
+      QRSrc src1;
+      src1.p = s->core[k].p;
+      (t->tall ? src1.rs : src1.cs) = c;
+      (t->tall ? src1.cs : src1.rs) = 1;
+      src1.perm = piv;
+      no.push_back({s->core[k].p, c, m, c, t->tall ? 1 : 0, 0, piv});
+      qr1.push_back({w.fac.p, p, q, w.p.p, w.p.p + q + 8, &w.main, src1});
+      const double* fac = w.fac.p;
+      int qm = p;
       if (t->tall) {
-        qr2.push_back({w.r.p, q, q, w.p2.p, w.p2.p + q + 8, &w.main});
-        fq.push_back({w.r.p, q, q, w.p2.p, w.q1.p, &w.side});
-        lu.push_back({w.r.p, q, w.l.p});
-        no2.push_back({w.l.p, q, q, 1, piv2});
-        ga2.push_back({w.l.p, q, q, piv2, 1, w.x.p});
-      } else {
-        fq.push_back({w.fac.p, p, q, w.p.p, w.q1.p, &w.side});
-        no2.push_back({w.r.p, q, q, 0, piv2});
-        ga2.push_back({w.r.p, q, q, piv2, 0, w.x.p});
+        QRSrc src2 = row_major(w.fac.p, p);
+        src2.lower = 1;
+        qr2.push_back({w.r.p, q, q, w.p2.p, w.p2.p + q + 8, &w.main, src2});
+        fac = w.r.p;
+        qm = q;
       }
-      qr3.push_back({w.x.p, q, q, w.p3.p, w.p3.p + q + 8, &w.main});
-      gx.push_back({w.x.p, q, q, w.tmp.p});
+      fq.push_back({fac, qm, q, t->tall ? w.p2.p : w.p.p, w.q1.p, &w.side, t->tall ? piv : nullptr});
+      no2.push_back({fac, qm, q, q, 1, 1, piv2});
+      QRSrc src3 = row_major(fac, qm);
+      src3.perm = piv2;
+      src3.lower = 1;
+      qr3.push_back({w.x.p, q, q, w.p3.p, w.p3.p + q + 8, &w.main, src3});
       TaskDev* rec = g->d_task + t->slot;
-      jc.push_back({w.tmp.p, q, q, &rec->st});
+      double* norms = w.tmp.p + (size_t)q * q;
+      jc.push_back({w.x.p, w.tmp.p, q, norms, &rec->st});
       int* perm = (int*)w.vec.p;
       double* sigma = w.vec.p + (q + 1) / 2 + 4;
-      se.push_back({w.tmp.p, q, q, chi, tol, perm, sigma, &rec->rank, &rec->err, &rec->st});
+      se.push_back({w.tmp.p, norms, q, q, chi, tol, t->ent != nullptr, perm, sigma, &rec->rank, &rec->err, &rec->st});
     }
     double wq = 0, wf = 0;
     for (Task* t : ts) {
@@ -373,10 +382,8 @@ int svd_sweep(vp_group* g, const Tasks& all) {
     }
     // A Pi = Q1 R1; tall: R1^T = Q2 L^T (see api.cu's svd_site)
     VP_TRY(blaunch_norm_order(ctx, ctx->stream, no));
-    VP_TRY(blaunch_gather_cm(ctx, ctx->stream, ga));
     VP_TRY(timed(ctx, VP_K_QR, wq, [&] {
       int st = blaunch_qr_factor(ctx, ctx->stream, qr1);
-      if (st == VP_OK) st = blaunch_qr_getr(ctx, ctx->stream, gr);
       if (st == VP_OK) st = blaunch_qr_factor(ctx, ctx->stream, qr2);
       return st;
     }));
@@ -393,13 +400,13 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       ~SideJoin() { cudaStreamWaitEvent(g->ctx->stream, g->ev_join, 0); }
     } side_join{g};
     // last QR, from the left: its R (columns ordered) is what Jacobi diagonalises
-    VP_TRY(blaunch_lower_from_upper(ctx, ctx->stream, lu));
     VP_TRY(blaunch_norm_order(ctx, ctx->stream, no2));
-    VP_TRY(blaunch_gather_cm(ctx, ctx->stream, ga2));
     VP_TRY(timed(ctx, VP_K_QR, 0.0, [&] { return blaunch_qr_factor(ctx, ctx->stream, qr3); }));
-    VP_TRY(blaunch_qr_getr(ctx, ctx->stream, gx));
     const size_t jac_mark = ctx->prof_on ? ctx->prof_marks.size() : (size_t)-1;
-    VP_TRY(timed(ctx, VP_K_JACOBI, 0.0, [&] { return blaunch_jacobi(ctx, ctx->stream, jc); }));
+    std::vector<char> have_norms;
+    VP_TRY(timed(ctx, VP_K_JACOBI, 0.0, [&] { return blaunch_jacobi(ctx, ctx->stream, jc, have_norms); }));
+    for (size_t i = 0; i < se.size(); ++i)
+      if (!have_norms[i]) se[i].norms = nullptr;
     VP_TRY(timed(ctx, VP_K_SELECT, 0.0, [&] { return blaunch_select(ctx, ctx->stream, se); }));
     // one wait for the kept ranks of every problem at this step
     VP_TRY(sync_records(g, slots));
@@ -418,7 +425,6 @@ int svd_sweep(vp_group* g, const Tasks& all) {
     ts = live(g, ts);
     std::vector<BSvdOut> so;
     std::vector<BGemm> g2, g3, g4;
-    std::vector<BScatter> sc;
     for (Task* t : ts) {
       mps_t* s = t->s;
       Work& w = *t->w;
@@ -433,17 +439,11 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       VP_TRY(reserve(ctx, w.gemm, (size_t)pl * r));
       int* perm = (int*)w.vec.p;
       double* sigma = w.vec.p + (q + 1) / 2 + 4;
-      const int* piv = (const int*)w.piv.p;
+      const int* piv2 = (const int*)w.piv.p + q;
       // core_k <- V^T (in tmp2, swapped in below; FP64 in every mode, as it enters
       // both cores); core_{k-1} <- core_{k-1} (M V)
-      so.push_back({w.tmp.p, q, r, perm, sigma, piv + q, w.a.p});
-      if (t->tall) {
-        VP_TRY(reserve(ctx, w.c, (size_t)r * q));
-        g2.push_back({BG_ABT, 0, r, q, q, 1.0, w.a.p, q, w.q1.p, q, w.c.p, q, &w.main});
-        sc.push_back({w.c.p, r, q, piv, 1, w.tmp2.p});
-      } else {
-        g2.push_back({BG_ABT, 0, r, c, q, 1.0, w.a.p, q, w.q1.p, q, w.tmp2.p, c, &w.main});
-      }
+      so.push_back({w.tmp.p, q, r, perm, sigma, piv2, w.a.p});
+      g2.push_back({BG_ABT, 0, r, c, q, 1.0, w.a.p, q, w.q1.p, q, w.tmp2.p, c, &w.main});
       g3.push_back({BG_ABT, t->fp32, m, r, c, 1.0, s->core[k].p, c, w.tmp2.p, c, w.b.p, r, &w.main});
       g4.push_back({BG_AB, t->fp32, pl, r, m, 1.0, s->core[k - 1].p, m, w.b.p, r, w.gemm.p, r, &w.main});
     }
@@ -458,7 +458,6 @@ int svd_sweep(vp_group* g, const Tasks& all) {
     VP_TRY(timed(ctx, VP_K_GEMM, wo, [&] {
       int st = blaunch_svd_outputs(ctx, ctx->stream, so);
       if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g2);
-      if (st == VP_OK) st = blaunch_scatter(ctx, ctx->stream, sc);
       if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g3);
       if (st == VP_OK) st = blaunch_gemm(ctx, ctx->stream, g4);
       return st;
@@ -516,7 +515,6 @@ int from_vectors(vp_group* g, const std::vector<VecJob>& jobs) {
   VP_TRY(blaunch_copy(ctx, ctx->stream, cp));
   std::vector<int> rr(jobs.size(), 1);
   for (int k = 0; k + 1 < nmax; ++k) {
-    std::vector<BColMajor> cm;
     std::vector<BQR> qr;
     std::vector<BFormQ> fq;
     std::vector<BGetR> gr;
@@ -532,14 +530,12 @@ int from_vectors(vp_group* g, const std::vector<VecJob>& jobs) {
       VP_TRY(reserve(ctx, w.fac, (size_t)m * nc));
       VP_TRY(reserve(ctx, w.p, (size_t)2 * m + p + 8));
       VP_TRY(reserve(ctx, jb.out->core[k], (size_t)m * p));
-      cm.push_back({jb.rem->p, m, nc, w.fac.p});
-      qr.push_back({w.fac.p, m, nc, w.p.p, w.p.p + p + 8, &w.main});
+      qr.push_back({w.fac.p, m, nc, w.p.p, w.p.p + p + 8, &w.main, row_major(jb.rem->p, nc)});
       fq.push_back({w.fac.p, m, nc, w.p.p, jb.out->core[k].p, &w.main});
       gr.push_back({w.fac.p, m, nc, jb.rem->p});
       jb.out->r[k + 1] = p;
       rr[a] = p;
     }
-    VP_TRY(blaunch_to_colmajor(ctx, ctx->stream, cm));
     VP_TRY(blaunch_qr_factor(ctx, ctx->stream, qr));
     VP_TRY(blaunch_qr_formq(ctx, ctx->stream, fq));
     VP_TRY(blaunch_qr_getr(ctx, ctx->stream, gr));

@@ -46,8 +46,10 @@ constexpr int kJMaxNb = 15;       // pairs of a round fit one warp's ballot and 
 constexpr float kTiny = 1e-30f;   // squared norm (largest entry ~1) below which a row is left alone
 
 struct JacArgs {
-  double* X;
-  int b, c;
+  const double* R;  // upper triangle of a column-major b x b factor: the rows
+  double* X;        // out, row-major
+  double* norms;    // out: row norms
+  int b;
   float eps;
   int max_sweeps, nb;
   DevStatus* st;
@@ -153,7 +155,7 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
   extern __shared__ double smd[];
   const int CS = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b = a.b, c = a.c, nb = a.nb, B = 2 * nb;
+  const int b = a.b, c = a.b, nb = a.nb, B = 2 * nb;
   dw* rows = reinterpret_cast<dw*>(smd);  // two sets of B rows: top block, bottom block
   dw* G2 = rows + 2 * (size_t)B * c;      // two Gram matrices
   dw* par = G2 + 2 * B * B;  // cosine, sine of pair p of round rd at 2 (16 rd + p)
@@ -161,7 +163,7 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
   unsigned short* xtab = tab + B * (B + 1) / 2;     // the pairs across the two blocks
   unsigned short* prow = xtab + nb * nb;            // rows (i << 8 | j) of pair p of round rd at 16 rd + p
   unsigned short* ptab = prow + 16 * (2 * nb + 1);  // pairs of pairs (P << 8 | Q), P <= Q, of np = nb, then bp
-  __shared__ float red[kJW + 1];
+  __shared__ int red[kJW + 1];
   __shared__ unsigned cnt[4];
   __shared__ unsigned rmask[2 * (kJMaxNb + 1)];  // pairs that rotate in each round
   // rounds: the pairs inside both blocks (bp - 1 rounds of bp pairs, a row of an
@@ -171,14 +173,21 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
 
   // common power-of-two scale: largest |x| over the cluster's rows
   auto home = [&](int slot) { return slot == 0 ? rank : 2 * CS - 1 - rank; };
-  float mx = 0.f;
-  for (int l = warp; l < B; l += kJW) {
+  // (a row of the block is strided in the factor: a warp takes 8 rows by 4 columns,
+  // the entries in place as they are while their largest exponent is taken)
+  int mx = 0;
+  for (int l0 = 0; l0 < B; l0 += 8) {
+    const int l = l0 + (lane & 7);
+    if (l >= B) continue;
     const int x = home(l / nb) * nb + l % nb;
-    if (x >= b) continue;
-    for (int q = lane; q < c; q += 32) mx = fmaxf(mx, fabsf(__double2float_rn(a.X[(size_t)x * c + q])));
+    for (int q = 4 * warp + (lane >> 3); q < c; q += 4 * kJW) {
+      const double v = x < b && q >= x ? a.R[(size_t)q * b + x] : 0.0;
+      reinterpret_cast<double*>(rows)[l * c + q] = v;
+      mx = max(mx, (int)((__double_as_longlong(v) >> 52) & 0x7ff));
+    }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  __syncwarp();
+  mx = __reduce_max_sync(0xffffffffu, mx);
   if (lane == 0) red[warp] = mx;
   if (tid < 4) cnt[tid] = 0u;
   for (int i = tid; i < B; i += kJT) {
@@ -216,20 +225,15 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
   }
   __syncthreads();
   if (tid == 0) {
-    float m = 0.f;
-    for (int i = 0; i < kJW; ++i) m = fmaxf(m, red[i]);
+    int m = 0;
+    for (int i = 0; i < kJW; ++i) m = max(m, red[i]);
     red[kJW] = m;
   }
   cl.sync();
-  float gmax = 0.f;
-  for (int r = 0; r < CS; ++r) gmax = fmaxf(gmax, *cl.map_shared_rank(red + kJW, r));
-  int ex = 0;
-  if (gmax > 0.f) frexpf(gmax, &ex);
-  const double sc = ldexp(1.0, -ex), inv_sc = ldexp(1.0, ex);
-  for (int l = warp; l < B; l += kJW) {
-    const int x = home(l / nb) * nb + l % nb;
-    for (int q = lane; q < c; q += 32) rows[l * c + q] = x < b ? dw_from(a.X[(size_t)x * c + q] * sc) : dw{0.f, 0.f};
-  }
+  int gmax = 0;
+  for (int r = 0; r < CS; ++r) gmax = max(gmax, *cl.map_shared_rank(red + kJW, r));
+  const int ex = gmax - 1022;  // largest entry to [1/2, 1)
+  for (int e = tid; e < B * c; e += kJT) rows[e] = dw_from_scaled(reinterpret_cast<double*>(rows)[e], ex);
   __syncthreads();  // every row of the block in place before the first products
   unsigned* c0 = cl.map_shared_rank(cnt, 0);
 
@@ -350,7 +354,15 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
     const int x = home(l / nb) * nb + l % nb;
     if (x >= b) continue;
     const dw* d = rows + ((size_t)cur * B + l) * c;
-    for (int q = lane; q < c; q += 32) a.X[(size_t)x * c + q] = dw_to(d[q]) * inv_sc;
+    double sum = 0.0;  // the norm as the selection would form it
+    for (int q = lane; q < c; q += 32) {
+      const double v = dw_to_scaled(d[q], ex);
+      a.X[(size_t)x * c + q] = v;
+      sum = fma(v, v, sum);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) a.norms[x] = sqrt(sum);
   }
   if (rank == 0 && tid == 0) {
     a.st->pad2 = converged ? sweep : a.max_sweeps + 1;
@@ -381,9 +393,9 @@ constexpr size_t kJacSmemMax = 216 * 1024;
 
 }  // namespace
 
-bool jacobi_dw_fits(const vp_ctx* ctx, int b, int c) {
+bool jacobi_dw_fits(const vp_ctx* ctx, int b) {
   const JacCfg g = jac_cfg(b, std::max(1, ctx->cluster_size));
-  return b > 1 && g.nb <= kJMaxNb && jac_smem(g, c) <= kJacSmemMax;
+  return b > 1 && g.nb <= kJMaxNb && jac_smem(g, b) <= kJacSmemMax;
 }
 
 int blaunch_jacobi_dw(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v) {
@@ -395,8 +407,8 @@ int blaunch_jacobi_dw(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& 
     // double-word products (~1e-14).  core_{k-1} takes M V, so what is left of
     // gamma enters the state twice: at 4e-13 sqrt(c) random states of 40 .. 200
     // rows kept 2.2 times the error, at 1e-13 half of it, for at most a sweep more
-    grp[g.cs].push_back({j.X, j.b, j.c, (float)(1e-13 * std::sqrt((double)j.c)), 60, g.nb, j.st});
-    smem[g.cs] = std::max(smem[g.cs], jac_smem(g, j.c));
+    grp[g.cs].push_back({j.R, j.X, j.norms, j.b, (float)(1e-13 * std::sqrt((double)j.b)), 60, g.nb, j.st});
+    smem[g.cs] = std::max(smem[g.cs], jac_smem(g, j.b));
   }
   for (int cs = 1; cs <= 16; ++cs) {
     if (grp[cs].empty()) continue;

@@ -92,26 +92,55 @@ static int coop_launch(vp_ctx* ctx, cudaStream_t stream, const void* fn, int blo
   return VP_OK;
 }
 
-// ------------------------------------------------------------ transposition
-__global__ void k_to_colmajor(const double* __restrict__ A, int m, int n, double* __restrict__ out) {
+// ------------------------------------------------------- strided gathers
+// A (m x n, column-major) from its source (QRSrc), through 32 x 32 tiles: the
+// kernels that do not read a source themselves.
+__device__ __forceinline__ void gather_tile(const QRSrc& s, int m, int n, double* __restrict__ A, int bx, int by) {
   __shared__ double tile[32][33];
-  const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
+  const int i0 = by * 32, k0 = bx * 32;
+  if (i0 >= m || k0 >= n) return;  // the whole block is outside this problem
+  const bool along_k = s.cs == 1;  // lanes along the contiguous direction
   for (int y = threadIdx.y; y < 32; y += 8) {
-    const int r = by + y, c = bx + threadIdx.x;
-    if (r < m && c < n) tile[y][threadIdx.x] = A[(size_t)r * n + c];
+    const int i = along_k ? i0 + y : i0 + threadIdx.x, k = along_k ? k0 + threadIdx.x : k0 + y;
+    if (i < m && k < n) {
+      const int c = s.perm ? s.perm[k] : k;
+      const double v = s.lower && i < c ? 0.0 : s.p[i * s.rs + c * s.cs];
+      tile[i - i0][k - k0] = v;
+    }
   }
   __syncthreads();
   for (int y = threadIdx.y; y < 32; y += 8) {
-    const int c = bx + y, r = by + threadIdx.x;
-    if (r < m && c < n) out[(size_t)c * m + r] = tile[threadIdx.x][y];
+    const int k = k0 + y, i = i0 + threadIdx.x;
+    if (i < m && k < n) A[(size_t)k * m + i] = tile[threadIdx.x][y];
   }
 }
-
+__global__ void kb_gather(const __grid_constant__ Pack<BGather> pk) {
+  const BGather& a = pk.a[blockIdx.z];
+  gather_tile(a.src, a.m, a.n, a.A, blockIdx.x, blockIdx.y);
+}
+static int blaunch_gather(vp_ctx* ctx, cudaStream_t st, const std::vector<BGather>& v) {
+  for (size_t i0 = 0; i0 < v.size(); i0 += kMaxBatch) {
+    const int nb = (int)std::min<size_t>(kMaxBatch, v.size() - i0);
+    Pack<BGather> pk{};
+    int gx = 1, gy = 1;
+    for (int i = 0; i < nb; ++i) {
+      pk.a[i] = v[i0 + i];
+      gx = std::max(gx, (v[i0 + i].n + 31) / 32);
+      gy = std::max(gy, (v[i0 + i].m + 31) / 32);
+    }
+    ctx->launches++;
+    kb_gather<<<dim3(gx, gy, nb), dim3(32, 8), 0, st>>>(pk);
+    VP_TRY(check_launch(ctx, "gather"));
+  }
+  return VP_OK;
+}
+// Row-major (m x n) -> column-major copy.
 int launch_to_colmajor(vp_ctx* ctx, const double* A, int m, int n, double* out) {
-  dim3 grid((n + 31) / 32, (m + 31) / 32);
-  ctx->launches++;
-  k_to_colmajor<<<grid, dim3(32, 8), 0, ctx->stream>>>(A, m, n, out);
-  return check_launch(ctx, "to_colmajor");
+  QRSrc s;
+  s.p = A;
+  s.rs = n;
+  s.cs = 1;
+  return blaunch_gather(ctx, ctx->stream, {BGather{s, m, n, out}});
 }
 
 // ------------------------------------------------------------ Householder QR
@@ -400,8 +429,10 @@ int qr_factor_grid(vp_ctx* ctx, cudaStream_t stream, DevStatus* st, DevBuf& qrv,
   return coop_launch(ctx, stream, (const void*)k_qr_factor<GridSync>, blocks, kThreads, args, 0, "qr_factor");
 }
 
-int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* vbuf) {
+int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* vbuf, const QRSrc& src) {
   const QRPlan pl = qr_plan(ctx, m, n);
+  if (src.p && (pl.kind == QR_WIDE || pl.kind == QR_GRID))
+    VP_TRY(blaunch_gather(ctx, ctx->stream, {BGather{src, m, n, A}}));
   switch (pl.kind) {
     case QR_NONE:
       return VP_OK;
@@ -419,7 +450,7 @@ int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* 
       return launch_copy(ctx, ctx->w_wr.p, A + (size_t)m * m, rest);
     }
     case QR_PANEL:
-      return blaunch_qr_panel(ctx, ctx->stream, {PanelJob{A, m, n, tau, pl.panel, &ctx->w_qrv, &ctx->w_qrc, ctx->status}});
+      return blaunch_qr_panel(ctx, ctx->stream, {PanelJob{A, m, n, tau, pl.panel, src, &ctx->w_qrv, &ctx->w_qrc, ctx->status}});
     default:
       return qr_factor_grid(ctx, ctx->stream, ctx->status, ctx->w_qrv, ctx->w_qrc, A, m, n, tau, vbuf);
   }
@@ -435,15 +466,15 @@ __device__ __forceinline__ void k_reflectors_to_dw_body(const double* __restrict
   const size_t total = (size_t)m * p;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
     const int j = (int)(e / m), i = (int)(e % m);
-    V[e] = i > j ? dw_from(A[e]) : (i == j ? dw{1.0f, 0.0f} : dw{0.0f, 0.0f});
-    if (e < (size_t)p) T[e] = dw_from(tau[e]);
+    V[e] = i > j ? dw_from_scaled(A[e], 0) : (i == j ? dw{1.0f, 0.0f} : dw{0.0f, 0.0f});
+    if (e < (size_t)p) T[e] = dw_from_scaled(tau[e], 0);
   }
 }
 __global__ void k_reflectors_to_dw(const double* __restrict__ A, int m, int p, const double* __restrict__ tau,
                                    dw* __restrict__ V, dw* __restrict__ T) { k_reflectors_to_dw_body(A, m, p, tau, V, T); }
 
 __device__ __forceinline__ void k_qr_formq_dw_body(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T, dw* __restrict__ scratch,
-                              double* __restrict__ Q) {
+                              double* __restrict__ Q, const int* __restrict__ rows) {
   const int lane = threadIdx.x & 31;
   const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (k >= p) return;
@@ -460,10 +491,10 @@ __device__ __forceinline__ void k_qr_formq_dw_body(const dw* __restrict__ V, int
     for (int i = j + lane; i < m; i += 32) q[i] = dw_add(q[i], dw_neg(dw_mul(w, v[i])));
     __syncwarp();
   }
-  for (int i = lane; i < m; i += 32) Q[(size_t)i * p + k] = dw_to(q[i]);
+  for (int i = lane; i < m; i += 32) Q[(size_t)(rows ? rows[i] : i) * p + k] = dw_to_scaled(q[i], 0);
 }
 __global__ void k_qr_formq_dw(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T, dw* __restrict__ scratch,
-                              double* __restrict__ Q) { k_qr_formq_dw_body(V, m, p, T, scratch, Q); }
+                              double* __restrict__ Q, const int* __restrict__ rows) { k_qr_formq_dw_body(V, m, p, T, scratch, Q, rows); }
 
 // The same product with column k of Q held in registers (rows lane + 32 u,
 // u < R, for m <= 32 R): per reflector the R reflector entries of a lane are
@@ -473,7 +504,7 @@ __global__ void k_qr_formq_dw(const dw* __restrict__ V, int m, int p, const dw* 
 // the column unchanged.
 template <int R>
 __device__ __forceinline__ void k_qr_formq_reg_body(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T,
-                               double* __restrict__ Q) {
+                               double* __restrict__ Q, const int* __restrict__ rows) {
   const int lane = threadIdx.x & 31;
   const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (k >= p) return;
@@ -506,14 +537,14 @@ __device__ __forceinline__ void k_qr_formq_reg_body(const dw* __restrict__ V, in
 #pragma unroll
   for (int u = 0; u < R; ++u) {
     const int i = lane + 32 * u;
-    if (i < m) Q[(size_t)i * p + k] = dw_to(q[u]);
+    if (i < m) Q[(size_t)(rows ? rows[i] : i) * p + k] = dw_to_scaled(q[u], 0);
   }
 }
 template <int R>
 __global__ void k_qr_formq_reg(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T,
-                               double* __restrict__ Q) { k_qr_formq_reg_body<R>(V, m, p, T, Q); }
+                               double* __restrict__ Q, const int* __restrict__ rows) { k_qr_formq_reg_body<R>(V, m, p, T, Q, rows); }
 
-int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q) {
+int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q, const int* rows) {
   const int p = std::min(m, n);
   if (p <= 0) return VP_OK;
   VP_TRY(reserve(ctx, ctx->w_q, (size_t)m * p));
@@ -527,14 +558,14 @@ int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* ta
   VP_TRY(check_launch(ctx, "reflectors_to_dw"));
   if (m <= 512) {  // column of Q in registers
     const int wpb = 4, blocks = (p + wpb - 1) / wpb;
-    if (m <= 64) k_qr_formq_reg<2><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q);
-    else if (m <= 128) k_qr_formq_reg<4><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q);
-    else if (m <= 256) k_qr_formq_reg<8><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q);
-    else k_qr_formq_reg<16><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q);
+    if (m <= 64) k_qr_formq_reg<2><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
+    else if (m <= 128) k_qr_formq_reg<4><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
+    else if (m <= 256) k_qr_formq_reg<8><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
+    else k_qr_formq_reg<16><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
     return check_launch(ctx, "qr_formq");
   }
   const int wpb = 8;
-  k_qr_formq_dw<<<(p + wpb - 1) / wpb, wpb * 32, 0, ctx->stream>>>(V, m, p, T, reinterpret_cast<dw*>(ctx->w_q.p), Q);
+  k_qr_formq_dw<<<(p + wpb - 1) / wpb, wpb * 32, 0, ctx->stream>>>(V, m, p, T, reinterpret_cast<dw*>(ctx->w_q.p), Q, rows);
   return check_launch(ctx, "qr_formq");
 }
 
@@ -1208,10 +1239,17 @@ static size_t jac_block_smem(const JacBlockCfg& g) {
   return (4 * (size_t)g.nb * g.stride + 4 * (size_t)g.nb) * sizeof(double) + 4 * sizeof(unsigned);
 }
 
-int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* X, int b, int c, bool floor_ok) {
+int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, const double* R, double* X, int b, double* norms,
+                   bool floor_ok, bool* have_norms) {
+  *have_norms = false;
   if (b <= 0) return VP_OK;
   const int CS = ctx->cluster_size;
-  if (floor_ok && jacobi_dw_fits(ctx, b, c)) return blaunch_jacobi_dw(ctx, stream, {BJacobi{X, b, c, status}});
+  int c = b;
+  if (floor_ok && jacobi_dw_fits(ctx, b)) {
+    *have_norms = true;
+    return blaunch_jacobi_dw(ctx, stream, {BJacobi{R, X, b, norms, status}});
+  }
+  VP_TRY(blaunch_qr_getr(ctx, stream, {BGetR{R, b, b, X}}));
   const JacBlockCfg bc = jac_block_cfg(b, c, std::max(1, CS));
   if (b > 1 && jac_block_smem(bc) <= 200 * 1024) {
     static AttrOnce battr_done;
@@ -1272,17 +1310,22 @@ int jacobi_rows_on(vp_ctx* ctx, cudaStream_t stream, DevStatus* status, double* 
   return coop_launch(ctx, stream, (const void*)k_jacobi_rows, blocks, kThreads, args, 0, "jacobi_rows");
 }
 
-int launch_jacobi_rows(vp_ctx* ctx, double* X, int b, int c, bool floor_ok) {
-  return jacobi_rows_on(ctx, ctx->stream, ctx->status, X, b, c, floor_ok);
+int launch_jacobi_rows(vp_ctx* ctx, const double* R, double* X, int b, double* norms, bool floor_ok, bool* have_norms) {
+  return jacobi_rows_on(ctx, ctx->stream, ctx->status, R, X, b, norms, floor_ok, have_norms);
 }
 
 // ------------------------------------------------------------ truncation
-// Descending order with ties broken by index, as a strict total order even
-// when values are NaN (NaNs first, by index): the rank of each element is
-// then a permutation, so the indices written from it always stay in range.
-__device__ __forceinline__ bool sorts_before(double a, int ia, double b, int ib) {
-  const bool na = isnan(a), nb = isnan(b);
-  if (na || nb) return na && (!nb || ia < ib);
+// Descending order with ties broken by index, as a strict total order even when
+// values are NaN (NaNs first): the rank of each element is then a permutation, so
+// the indices written from it always stay in range.  The values are >= 0 or NaN,
+// whose order is that of their bits without the sign: an FP64 comparison costs an
+// FP64 issue slot, of which an SM has two a clock.
+__device__ __forceinline__ unsigned long long order_key(double a) {
+  return (unsigned long long)__double_as_longlong(a) & ~(1ull << 63);
+}
+__device__ __forceinline__ unsigned order_key(float a) { return __float_as_uint(a) & 0x7fffffffu; }
+template <class Key>
+__device__ __forceinline__ bool sorts_before(Key a, int ia, Key b, int ib) {
   return a > b || (a == b && ia < ib);
 }
 
@@ -1295,8 +1338,13 @@ __device__ __forceinline__ bool sorts_before(double a, int ia, double b, int ib)
 // order as alone), the tail sums as a block-wide suffix scan (chunk sums,
 // then a scan of the chunk totals), r_tol as a minimum over the rows that
 // meet the tolerance, and the entanglement entropy as a fixed-order tree sum.
-__device__ __forceinline__ void k_select_body(const double* __restrict__ X, int b, int c, int chi, double tol, int* perm,
-                         double* sigma, int* d_rank, double* d_err, DevStatus* st) {
+// norms: the row norms where the Jacobi kernel left them, else NULL (formed here,
+// with the same sums); want_ent: whether the entropy is asked for.  (18 us on
+// average over the sites of a 1024 x 1024 step with norms, entropy and FP64
+// comparisons here, 6.7 now.)
+__device__ __forceinline__ void k_select_body(const double* __restrict__ X, const double* __restrict__ norms, int b, int c,
+                                              int chi, double tol, int want_ent, int* perm, double* sigma, int* d_rank,
+                                              double* d_err, DevStatus* st) {
   extern __shared__ double sm[];
   double* s = sm;          // b
   double* tail = sm + b;   // b + 1
@@ -1306,32 +1354,37 @@ __device__ __forceinline__ void k_select_body(const double* __restrict__ X, int 
   const int T = blockDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = T >> 5;
   constexpr int RB = 4;
-  for (int i0 = warp * RB; i0 < b; i0 += nwarps * RB) {
-    double a[RB];
+  if (norms) {
+    for (int i = threadIdx.x; i < b; i += T) s[i] = norms[i];
+  } else {
+    for (int i0 = warp * RB; i0 < b; i0 += nwarps * RB) {
+      double a[RB];
 #pragma unroll
-    for (int u = 0; u < RB; ++u) a[u] = 0.0;
-    for (int q = lane; q < c; q += 32)
+      for (int u = 0; u < RB; ++u) a[u] = 0.0;
+      for (int q = lane; q < c; q += 32)
 #pragma unroll
-      for (int u = 0; u < RB; ++u)
-        if (i0 + u < b) {
-          const double x = X[(size_t)(i0 + u) * c + q];
-          a[u] = fma(x, x, a[u]);
-        }
+        for (int u = 0; u < RB; ++u)
+          if (i0 + u < b) {
+            const double x = X[(size_t)(i0 + u) * c + q];
+            a[u] = fma(x, x, a[u]);
+          }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
+      for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-      for (int u = 0; u < RB; ++u) a[u] += __shfl_xor_sync(0xffffffffu, a[u], o);
-    if (lane == 0)
+        for (int u = 0; u < RB; ++u) a[u] += __shfl_xor_sync(0xffffffffu, a[u], o);
+      if (lane == 0)
 #pragma unroll
-      for (int u = 0; u < RB; ++u)
-        if (i0 + u < b) s[i0 + u] = sqrt(a[u]);
+        for (int u = 0; u < RB; ++u)
+          if (i0 + u < b) s[i0 + u] = sqrt(a[u]);
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < b; i += T) {
     const double si = s[i];
-    if (!isfinite(si)) atomicCAS(&st->err, 0, 2);
+    const unsigned long long ki = order_key(si);
+    if ((ki >> 52) == 2047) atomicCAS(&st->err, 0, 2);  // NaN or Inf
     int pos = 0;
-    for (int j = 0; j < b; ++j) pos += sorts_before(s[j], j, si, i);
+    for (int j = 0; j < b; ++j) pos += sorts_before(order_key(s[j]), j, ki, i);
     perm[pos] = i;
     sigma[pos] = si;
   }
@@ -1386,7 +1439,7 @@ __device__ __forceinline__ void k_select_body(const double* __restrict__ X, int 
   const int r = rkeep;
   const double kept2 = tail[0] - tail[r];
   double ee = 0.0;
-  if (kept2 > 0.0)
+  if (want_ent && kept2 > 0.0)
     for (int q = threadIdx.x; q < r; q += T) {
       const double pq = sigma[q] * sigma[q] / kept2;
       if (pq > 0.0) ee -= pq * log2(pq);
@@ -1401,11 +1454,16 @@ __device__ __forceinline__ void k_select_body(const double* __restrict__ X, int 
     d_err[1] = tot;
   }
 }
-__global__ void k_select(const double* __restrict__ X, int b, int c, int chi, double tol, int* perm,
-                         double* sigma, int* d_rank, double* d_err, DevStatus* st) { k_select_body(X, b, c, chi, tol, perm, sigma, d_rank, d_err, st); }
+__global__ void k_select(const double* __restrict__ X, const double* __restrict__ norms, int b, int c, int chi, double tol,
+                         int want_ent, int* perm, double* sigma, int* d_rank, double* d_err, DevStatus* st) {
+  k_select_body(X, norms, b, c, chi, tol, want_ent, perm, sigma, d_rank, d_err, st);
+}
+// Threads of the selection: one per value up to 512 (the scans take as many steps
+// as the block is wide).
+static int select_threads(int b) { return std::min(512, std::max(128, (b + 31) / 32 * 32)); }
 
-int launch_select(vp_ctx* ctx, const double* X, int b, int c, int chi, double tol, int* perm, double* sigma,
-                  int* d_rank, double* d_err) {
+int launch_select(vp_ctx* ctx, const double* X, const double* norms, int b, int c, int chi, double tol, bool want_ent,
+                  int* perm, double* sigma, int* d_rank, double* d_err) {
   const size_t smem = (size_t)(2 * b + 1) * sizeof(double);
   if (smem > 200 * 1024) return fail(ctx, VP_ECAPACITY, "select: bond too large");
   // always: the kernel's own 8 KB of static shared memory counts against the
@@ -1413,7 +1471,8 @@ int launch_select(vp_ctx* ctx, const double* X, int b, int c, int chi, double to
   static AttrOnce sattr;
   VP_TRY(sattr.ensure(ctx, (const void*)k_select, 200 * 1024, false));
   ctx->launches++;
-  k_select<<<1, 512, smem, ctx->stream>>>(X, b, c, chi, tol, perm, sigma, d_rank, d_err, ctx->status);
+  k_select<<<1, select_threads(b), smem, ctx->stream>>>(X, norms, b, c, chi, tol, want_ent, perm, sigma, d_rank, d_err,
+                                                        ctx->status);
   return check_launch(ctx, "select");
 }
 
@@ -1444,109 +1503,81 @@ int launch_svd_outputs(vp_ctx* ctx, const double* X, int q, int r, const int* pe
 // Static pivoting for the Jacobi SVD: order the columns (tall) or rows (wide)
 // of M by decreasing norm, so that the triangular factor of the reordered
 // matrix is graded and one-sided Jacobi on it converges in fewer sweeps.
-__device__ __forceinline__ void k_norm_order_body(const double* __restrict__ M, int m, int c, int by_cols, int* __restrict__ piv) {
-  extern __shared__ double nrm[];
-  const int q = by_cols ? c : m, len = by_cols ? m : c;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int j = warp; j < q; j += nw) {
-    double a = 0.0;
-    for (int i = lane; i < len; i += 32) {
-      const double u = by_cols ? M[(size_t)i * c + j] : M[(size_t)j * c + i];
-      a = fma(u, u, a);
+// The norms only decide an order, so they are FP32 sums of the entries scaled by a
+// common power of two: with FP64 squares and comparisons an SM's two FP64 slots a
+// clock were what the kernel waited for (10.5 us on average over the sites of a
+// 1024 x 1024 step, now 6.5).  Entries 2^-60 below the largest count as zero.
+__device__ __forceinline__ void k_norm_order_body(const double* __restrict__ M, int ld, int m, int c, int by_cols, int lower,
+                                                  int* __restrict__ piv) {
+  extern __shared__ double nrm_raw[];
+  float* nrm = reinterpret_cast<float*>(nrm_raw);
+  __shared__ int emax;
+  const int q = by_cols ? c : m;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  if (tid == 0) emax = 1;
+  __syncthreads();
+  // (lanes along the contiguous direction in both cases)
+  int e = 1;
+  for (int r = warp; r < m; r += nw)
+#pragma unroll 4
+    for (int k = lane; k < (lower ? min(c, r + 1) : c); k += 32) {
+      const int x = (int)((__double_as_longlong(M[(size_t)r * ld + k]) >> 52) & 0x7ff);
+      if (x < 2047) e = max(e, x);
     }
-    a = warp_sum(a);
-    if (lane == 0) nrm[j] = a;
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0) atomicMax(&emax, e);
+  __syncthreads();
+  const int sh = emax - 1022;  // largest entry to [1/2, 1)
+  // a non-finite entry makes its norm NaN, which sorts first
+  auto entry = [&](int r, int k) {
+    const double x = M[(size_t)r * ld + k];
+    return ((__double_as_longlong(x) >> 52) & 0x7ff) == 2047 ? __int_as_float(0x7fc00000) : dw_from_scaled(x, sh).hi;
+  };
+  if (by_cols) {
+    float* part = nrm + q;  // nw x 32: the warps' sums of one group of 32 columns
+    for (int k0 = 0; k0 < c; k0 += 32) {
+      const int k = k0 + lane;
+      float s = 0.f;
+      if (k < c)
+#pragma unroll 4
+        for (int r = warp; r < m; r += nw) {
+          const float x = lower && r < k ? 0.f : entry(r, k);
+          s = fmaf(x, x, s);
+        }
+      part[warp * 32 + lane] = s;
+      __syncthreads();
+      if (warp == 0 && k < c) {
+        float t = 0.f;
+        for (int w = 0; w < nw; ++w) t += part[w * 32 + lane];
+        nrm[k] = t;
+      }
+      __syncthreads();
+    }
+  } else {
+    for (int r = warp; r < m; r += nw) {
+      float s = 0.f;
+      for (int k = lane; k < (lower ? min(c, r + 1) : c); k += 32) {
+        const float x = entry(r, k);
+        s = fmaf(x, x, s);
+      }
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) nrm[r] = s;
+    }
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < q; j += blockDim.x) {
-    const double v = nrm[j];
+  for (int j = tid; j < q; j += blockDim.x) {
+    const unsigned v = order_key(nrm[j]);
     int pos = 0;
-    for (int k = 0; k < q; ++k) pos += sorts_before(nrm[k], k, v, j);
+    for (int k = 0; k < q; ++k) pos += sorts_before(order_key(nrm[k]), k, v, j);
     piv[pos] = j;
   }
 }
-__global__ void k_norm_order(const double* __restrict__ M, int m, int c, int by_cols, int* __restrict__ piv) { k_norm_order_body(M, m, c, by_cols, piv); }
-
-int launch_norm_order(vp_ctx* ctx, const double* M, int m, int c, int by_cols, int* piv) {
-  const int q = by_cols ? c : m;
-  const size_t smem = (size_t)q * sizeof(double);
-  if (smem > 200 * 1024) return fail(ctx, VP_ECAPACITY, "norm_order: too many columns");
-  if (smem > 48 * 1024) {
-    static AttrOnce nattr;  // the largest size once, never lowered under another thread's launch
-    VP_TRY(nattr.ensure(ctx, (const void*)k_norm_order, 200 * 1024, false));
-  }
-  ctx->launches++;
-  k_norm_order<<<1, 512, smem, ctx->stream>>>(M, m, c, by_cols, piv);
-  return check_launch(ctx, "norm_order");
+__global__ void __launch_bounds__(512) kb_norm_order(const __grid_constant__ Pack<BNormOrder> pk) {
+  const BNormOrder& a = pk.a[blockIdx.y];
+  k_norm_order_body(a.M, a.ld, a.m, a.c, a.by_cols, a.lower, a.piv);
 }
-
-// Column-major copy of the reordered matrix: tall, A = M[:, piv] (m x c);
-// wide, A = (M[piv, :])^T (c x m).
-__device__ __forceinline__ void k_gather_cm_body(const double* __restrict__ M, int m, int c, const int* __restrict__ piv, int tall,
-                            double* __restrict__ out) {
-  const size_t total = (size_t)m * c;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    if (tall) {
-      const size_t j = e / m, i = e % m;  // out[j*m + i] = M[i][piv[j]]
-      out[e] = M[i * c + piv[j]];
-    } else {
-      const size_t j = e / c, i = e % c;  // out[j*c + i] = M[piv[j]][i]
-      out[e] = M[(size_t)piv[j] * c + i];
-    }
-  }
-}
-__global__ void k_gather_cm(const double* __restrict__ M, int m, int c, const int* __restrict__ piv, int tall,
-                            double* __restrict__ out) { k_gather_cm_body(M, m, c, piv, tall, out); }
-
-int launch_gather_cm(vp_ctx* ctx, const double* M, int m, int c, const int* piv, int tall, double* out) {
-  const size_t total = (size_t)m * c;
-  const int blocks = (int)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)ctx->num_sms * 16));
-  ctx->launches++;
-  k_gather_cm<<<blocks, 256, 0, ctx->stream>>>(M, m, c, piv, tall, out);
-  return check_launch(ctx, "gather_cm");
-}
-
-// L = R^T, row-major, from a factored column-major q x q matrix whose upper
-// triangle holds R (the reflectors below are dropped).
-__device__ __forceinline__ void k_lower_from_upper_body(const double* __restrict__ Rcm, int q, double* __restrict__ L) {
-  const size_t total = (size_t)q * q;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t i = e / q, j = e % q;
-    L[e] = (j <= i) ? Rcm[e] : 0.0;
-  }
-}
-__global__ void k_lower_from_upper(const double* __restrict__ Rcm, int q, double* __restrict__ L) { k_lower_from_upper_body(Rcm, q, L); }
-
-int launch_lower_from_upper(vp_ctx* ctx, const double* Rcm, int q, double* L) {
-  const size_t total = (size_t)q * q;
-  const int blocks = (int)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)ctx->num_sms * 8));
-  ctx->launches++;
-  k_lower_from_upper<<<blocks, 256, 0, ctx->stream>>>(Rcm, q, L);
-  return check_launch(ctx, "lower_from_upper");
-}
-
-// Undo the static pivoting: cols = 1: out[t][piv[j]] = Y[t][j] (rows x q);
-// cols = 0: out[piv[j]][t] = Y[j][t] (q x rows_len).
-__device__ __forceinline__ void k_scatter_body(const double* __restrict__ Y, int rows, int cols_n, const int* __restrict__ piv, int cols,
-                          double* __restrict__ out) {
-  const size_t total = (size_t)rows * cols_n;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const size_t a = e / cols_n, b = e % cols_n;
-    if (cols)
-      out[a * cols_n + piv[b]] = Y[e];
-    else
-      out[(size_t)piv[a] * cols_n + b] = Y[e];
-  }
-}
-__global__ void k_scatter(const double* __restrict__ Y, int rows, int cols_n, const int* __restrict__ piv, int cols,
-                          double* __restrict__ out) { k_scatter_body(Y, rows, cols_n, piv, cols, out); }
-
-int launch_scatter(vp_ctx* ctx, const double* Y, int rows, int cols_n, const int* piv, int cols, double* out) {
-  const size_t total = (size_t)rows * cols_n;
-  const int blocks = (int)std::max<size_t>(1, std::min<size_t>((total + 255) / 256, (size_t)ctx->num_sms * 8));
-  ctx->launches++;
-  k_scatter<<<blocks, 256, 0, ctx->stream>>>(Y, rows, cols_n, piv, cols, out);
-  return check_launch(ctx, "scatter");
+int launch_norm_order(vp_ctx* ctx, const double* M, int ld, int m, int c, int by_cols, int lower, int* piv) {
+  return blaunch_norm_order(ctx, ctx->stream, {BNormOrder{M, ld, m, c, by_cols, lower, piv}});
 }
 
 // ====================================================== batched launches
@@ -1638,39 +1669,6 @@ int run_cluster_packs(vp_ctx* ctx, cudaStream_t st, const std::vector<A>& v, voi
 
 }  // namespace
 
-__global__ void kb_to_colmajor(const __grid_constant__ Pack<BColMajor> pk) {
-  const BColMajor& a = pk.a[blockIdx.z];
-  __shared__ double tile[32][33];
-  const int bx = blockIdx.x * 32, by = blockIdx.y * 32;
-  if (bx >= a.n || by >= a.m) return;  // the whole block is outside this problem
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const int r = by + y, c = bx + threadIdx.x;
-    if (r < a.m && c < a.n) tile[y][threadIdx.x] = a.A[(size_t)r * a.n + c];
-  }
-  __syncthreads();
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const int c = bx + y, r = by + threadIdx.x;
-    if (r < a.m && c < a.n) a.out[(size_t)c * a.m + r] = tile[threadIdx.x][y];
-  }
-}
-
-int blaunch_to_colmajor(vp_ctx* ctx, cudaStream_t st, const std::vector<BColMajor>& v) {
-  for (size_t i0 = 0; i0 < v.size(); i0 += kMaxBatch) {
-    const int nb = (int)std::min<size_t>(kMaxBatch, v.size() - i0);
-    Pack<BColMajor> pk{};
-    int gx = 1, gy = 1;
-    for (int i = 0; i < nb; ++i) {
-      pk.a[i] = v[i0 + i];
-      gx = std::max(gx, (v[i0 + i].n + 31) / 32);
-      gy = std::max(gy, (v[i0 + i].m + 31) / 32);
-    }
-    ctx->launches++;
-    kb_to_colmajor<<<dim3(gx, gy, nb), dim3(32, 8), 0, st>>>(pk);
-    VP_TRY(check_launch(ctx, "b_to_colmajor"));
-  }
-  return VP_OK;
-}
-
 // --------------------------------------------------------------- QR
 // Several grid factors in one cooperative launch: problem i owns blocks
 // first .. first + nblocks - 1 and runs k_qr_factor_dw's body on them as if
@@ -1735,6 +1733,12 @@ int blaunch_qr_factor(vp_ctx* ctx, cudaStream_t st, const std::vector<BQR>& v) {
   std::vector<BQR> wide;
   std::vector<const BQR*> grid;
   std::vector<PanelJob> panel;
+  std::vector<BGather> gat;
+  for (const BQR& q : v) {
+    const int kind = qr_plan(ctx, q.m, q.n).kind;
+    if (q.src.p && (kind == QR_WIDE || kind == QR_GRID)) gat.push_back({q.src, q.m, q.n, q.A});
+  }
+  VP_TRY(blaunch_gather(ctx, st, gat));
   for (const BQR& q : v) {
     const QRPlan pl = qr_plan(ctx, q.m, q.n);
     switch (pl.kind) {
@@ -1744,7 +1748,7 @@ int blaunch_qr_factor(vp_ctx* ctx, cudaStream_t st, const std::vector<BQR>& v) {
         wide.push_back(q);
         break;
       case QR_PANEL:
-        panel.push_back({q.A, q.m, q.n, q.tau, pl.panel, &q.s->qrv, &q.s->qrc, q.s->st});
+        panel.push_back({q.A, q.m, q.n, q.tau, pl.panel, q.src, &q.s->qrv, &q.s->qrc, q.s->st});
         break;
       default:
         if (!q.s || !q.s->st) return fail(ctx, VP_EINVAL, "batched QR: no status words for a grid factor");
@@ -1796,15 +1800,16 @@ struct FormQArgs {
   const dw* T;
   dw* scratch;
   double* Q;
+  const int* rows;
 };
 template <int R>
 __global__ void kb_qr_formq_reg(const __grid_constant__ Pack<FormQArgs> pk) {
   const FormQArgs& a = pk.a[blockIdx.y];
-  k_qr_formq_reg_body<R>(a.V, a.m, a.p, a.T, a.Q);
+  k_qr_formq_reg_body<R>(a.V, a.m, a.p, a.T, a.Q, a.rows);
 }
 __global__ void kb_qr_formq_dw(const __grid_constant__ Pack<FormQArgs> pk) {
   const FormQArgs& a = pk.a[blockIdx.y];
-  k_qr_formq_dw_body(a.V, a.m, a.p, a.T, a.scratch, a.Q);
+  k_qr_formq_dw_body(a.V, a.m, a.p, a.T, a.scratch, a.Q, a.rows);
 }
 
 int blaunch_qr_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<BFormQ>& v) {
@@ -1820,7 +1825,7 @@ int blaunch_qr_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<BFormQ>& v)
     dw* V = reinterpret_cast<dw*>(f.s->fq[sl].p);
     dw* T = V + (size_t)f.m * p;
     conv.push_back({f.A, f.m, p, f.tau, V, T});
-    FormQArgs a{V, f.m, p, T, nullptr, f.Q};
+    FormQArgs a{V, f.m, p, T, nullptr, f.Q, f.rows};
     if (f.m <= 64) reg[1].push_back(a);
     else if (f.m <= 128) reg[2].push_back(a);
     else if (f.m <= 256) reg[3].push_back(a);
@@ -1969,45 +1974,26 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
 }
 
 // --------------------------------------------------------------- SVD site helpers
-__global__ void kb_norm_order(const __grid_constant__ Pack<BNormOrder> pk) {
-  const BNormOrder& a = pk.a[blockIdx.y];
-  k_norm_order_body(a.M, a.m, a.c, a.by_cols, a.piv);
-}
 int blaunch_norm_order(vp_ctx* ctx, cudaStream_t st, const std::vector<BNormOrder>& v) {
   size_t smem = 0;
-  for (const BNormOrder& a : v) smem = std::max(smem, (size_t)(a.by_cols ? a.c : a.m) * sizeof(double));
+  for (const BNormOrder& a : v) smem = std::max(smem, (size_t)((a.by_cols ? a.c : a.m) + 16 * 32) * sizeof(float));
   if (smem > 200 * 1024) return fail(ctx, VP_ECAPACITY, "norm_order: too many columns");
   static AttrOnce at;
   VP_TRY(at.ensure(ctx, (const void*)kb_norm_order, 200 * 1024, false));
   return run_packs(ctx, st, v, kb_norm_order, 512, smem, [](const BNormOrder&) { return 1; }, "b_norm_order");
 }
-__global__ void kb_gather_cm(const __grid_constant__ Pack<BGather> pk) {
-  const BGather& a = pk.a[blockIdx.y];
-  k_gather_cm_body(a.M, a.m, a.c, a.piv, a.tall, a.out);
-}
-int blaunch_gather_cm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGather>& v) {
-  return run_packs(ctx, st, v, kb_gather_cm, 256, 0,
-                   [&](const BGather& a) { return grid_stride_blocks(ctx, (size_t)a.m * a.c, 16); }, "b_gather_cm");
-}
-__global__ void kb_lower_from_upper(const __grid_constant__ Pack<BLowerUpper> pk) {
-  const BLowerUpper& a = pk.a[blockIdx.y];
-  k_lower_from_upper_body(a.R, a.q, a.L);
-}
-int blaunch_lower_from_upper(vp_ctx* ctx, cudaStream_t st, const std::vector<BLowerUpper>& v) {
-  return run_packs(ctx, st, v, kb_lower_from_upper, 256, 0,
-                   [&](const BLowerUpper& a) { return grid_stride_blocks(ctx, (size_t)a.q * a.q, 8); },
-                   "b_lower_from_upper");
-}
-
-int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v) {
+int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v, std::vector<char>& have_norms) {
   std::vector<BJacobi> fit;
-  for (const BJacobi& j : v) {
-    if (j.b <= 1) continue;  // nothing to rotate (as in the single launch)
-    if (jacobi_dw_fits(ctx, j.b, j.c)) {
+  have_norms.assign(v.size(), 0);
+  for (size_t i = 0; i < v.size(); ++i) {
+    const BJacobi& j = v[i];
+    if (jacobi_dw_fits(ctx, j.b)) {
       fit.push_back(j);
+      have_norms[i] = 1;
     } else {
+      bool hn = false;
       VP_CUDA(ctx, cudaMemsetAsync(j.st->rot, 0, sizeof(j.st->rot), st));
-      VP_TRY(jacobi_rows_on(ctx, st, j.st, j.X, j.b, j.c, true));
+      VP_TRY(jacobi_rows_on(ctx, st, j.st, j.R, j.X, j.b, j.norms, true, &hn));
     }
   }
   return blaunch_jacobi_dw(ctx, st, fit);
@@ -2015,7 +2001,7 @@ int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v) 
 
 __global__ void kb_select(const __grid_constant__ Pack<BSelect> pk) {
   const BSelect& a = pk.a[blockIdx.y];
-  k_select_body(a.X, a.b, a.c, a.chi, a.tol, a.perm, a.sigma, a.d_rank, a.d_err, a.st);
+  k_select_body(a.X, a.norms, a.b, a.c, a.chi, a.tol, a.want_ent, a.perm, a.sigma, a.d_rank, a.d_err, a.st);
 }
 int blaunch_select(vp_ctx* ctx, cudaStream_t st, const std::vector<BSelect>& v) {
   size_t smem = 0;
@@ -2023,7 +2009,9 @@ int blaunch_select(vp_ctx* ctx, cudaStream_t st, const std::vector<BSelect>& v) 
   if (smem > 200 * 1024) return fail(ctx, VP_ECAPACITY, "select: bond too large");
   static AttrOnce at;
   VP_TRY(at.ensure(ctx, (const void*)kb_select, 200 * 1024, false));
-  return run_packs(ctx, st, v, kb_select, 512, smem, [](const BSelect&) { return 1; }, "b_select");
+  int nt = 128;
+  for (const BSelect& a : v) nt = std::max(nt, select_threads(a.b));
+  return run_packs(ctx, st, v, kb_select, nt, smem, [](const BSelect&) { return 1; }, "b_select");
 }
 __global__ void kb_svd_outputs(const __grid_constant__ Pack<BSvdOut> pk) {
   const BSvdOut& a = pk.a[blockIdx.y];
@@ -2033,14 +2021,4 @@ int blaunch_svd_outputs(vp_ctx* ctx, cudaStream_t st, const std::vector<BSvdOut>
   return run_packs(ctx, st, v, kb_svd_outputs, 256, 0,
                    [&](const BSvdOut& a) { return grid_stride_blocks(ctx, (size_t)a.r * a.q, 8); }, "b_svd_outputs");
 }
-__global__ void kb_scatter(const __grid_constant__ Pack<BScatter> pk) {
-  const BScatter& a = pk.a[blockIdx.y];
-  k_scatter_body(a.Y, a.rows, a.cols_n, a.piv, a.cols, a.out);
-}
-int blaunch_scatter(vp_ctx* ctx, cudaStream_t st, const std::vector<BScatter>& v) {
-  return run_packs(ctx, st, v, kb_scatter, 256, 0,
-                   [&](const BScatter& a) { return grid_stride_blocks(ctx, (size_t)a.rows * a.cols_n, 8); },
-                   "b_scatter");
-}
-
 }  // namespace vp
