@@ -210,6 +210,16 @@ QRPlan qr_plan(const vp_ctx* ctx, int m, int n);
 // Q (m x p, p = min(m,n)) written row-major from the factored A, its row i in row
 // rows[i] of the output (NULL: i).
 int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q, const int* rows = nullptr);
+struct FormQJob {
+  const double* A;
+  int m, n;
+  const double* tau;
+  double* Q;
+  const int* rows;
+  DevBuf* v;        // reflectors as double words
+  DevBuf* scratch;  // columns of more rows than a block holds
+};
+int blaunch_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<FormQJob>& v);
 // Upper-trapezoidal R (p x n) of the factored A, written row-major.
 int launch_qr_getr(vp_ctx* ctx, const double* A, int m, int n, double* R);
 // Output tile and split-K of an FP32 contraction (shape and device only).
@@ -360,7 +370,7 @@ struct BScratch {
   DevBuf wq, wr;                  // wide QR: Q of the square block, R2^T
   DevBuf qrv, qrc;                // grid QR: published reflectors, columns beyond shared memory
   DevBuf fq[kScratchSlots];       // Q formation: double-word reflectors
-  DevBuf qscr[kScratchSlots];     // Q formation: column scratch (m > 512)
+  DevBuf qscr[kScratchSlots];     // Q formation: column scratch (m > 4096)
   DevBuf split[kScratchSlots];    // GEMM split-K partial products
   DevBuf oza[kScratchSlots], ozb[kScratchSlots];  // sliced GEMM: digits of the operands
   DevStatus* st = nullptr;        // status words of the problem (device)

@@ -456,117 +456,8 @@ int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* 
   }
 }
 
-// Q = H_0 ... H_{p-1} [I_p; 0] in double words: the reflectors (below the
-// diagonal of the factored A, leading 1 implicit) and taus are converted
-// once, then one warp per column k of Q applies H_k, ..., H_0 to e_k with
-// double-word dot products and updates (each step would otherwise be a chain
-// of FP64 FMAs at ~400 cycles apiece); Q is stored row-major (m x p).
-__device__ __forceinline__ void k_reflectors_to_dw_body(const double* __restrict__ A, int m, int p, const double* __restrict__ tau,
-                                   dw* __restrict__ V, dw* __restrict__ T) {
-  const size_t total = (size_t)m * p;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
-    const int j = (int)(e / m), i = (int)(e % m);
-    V[e] = i > j ? dw_from_scaled(A[e], 0) : (i == j ? dw{1.0f, 0.0f} : dw{0.0f, 0.0f});
-    if (e < (size_t)p) T[e] = dw_from_scaled(tau[e], 0);
-  }
-}
-__global__ void k_reflectors_to_dw(const double* __restrict__ A, int m, int p, const double* __restrict__ tau,
-                                   dw* __restrict__ V, dw* __restrict__ T) { k_reflectors_to_dw_body(A, m, p, tau, V, T); }
-
-__device__ __forceinline__ void k_qr_formq_dw_body(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T, dw* __restrict__ scratch,
-                              double* __restrict__ Q, const int* __restrict__ rows) {
-  const int lane = threadIdx.x & 31;
-  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (k >= p) return;
-  dw* q = scratch + (size_t)k * m;
-  for (int i = lane; i < m; i += 32) q[i] = (i == k) ? dw{1.0f, 0.0f} : dw{0.0f, 0.0f};
-  __syncwarp();
-  for (int j = k; j >= 0; --j) {
-    const dw t = T[j];
-    if (t.hi == 0.f) continue;
-    const dw* v = V + (size_t)j * m;
-    dw_acc acc;
-    for (int i = j + lane; i < m; i += 32) dw_dot_step(acc, v[i], q[i]);
-    const dw w = dw_mul(dw_warp_sum(dw_acc_value(acc)), t);
-    for (int i = j + lane; i < m; i += 32) q[i] = dw_add(q[i], dw_neg(dw_mul(w, v[i])));
-    __syncwarp();
-  }
-  for (int i = lane; i < m; i += 32) Q[(size_t)(rows ? rows[i] : i) * p + k] = dw_to_scaled(q[i], 0);
-}
-__global__ void k_qr_formq_dw(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T, dw* __restrict__ scratch,
-                              double* __restrict__ Q, const int* __restrict__ rows) { k_qr_formq_dw_body(V, m, p, T, scratch, Q, rows); }
-
-// The same product with column k of Q held in registers (rows lane + 32 u,
-// u < R, for m <= 32 R): per reflector the R reflector entries of a lane are
-// loaded together and the dot product and update run on registers, so the
-// chain of column k costs one L2 round trip per reflector instead of four.
-// Rows above the reflector's start hold zeros in V, which leave the sums and
-// the column unchanged.
-template <int R>
-__device__ __forceinline__ void k_qr_formq_reg_body(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T,
-                               double* __restrict__ Q, const int* __restrict__ rows) {
-  const int lane = threadIdx.x & 31;
-  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (k >= p) return;
-  dw q[R];
-#pragma unroll
-  for (int u = 0; u < R; ++u) q[u] = (lane + 32 * u == k) ? dw{1.0f, 0.0f} : dw{0.0f, 0.0f};
-  for (int j = k; j >= 0; --j) {
-    const float2 t2 = __ldg(reinterpret_cast<const float2*>(T + j));
-    if (t2.x == 0.f) continue;
-    const dw t = {t2.x, t2.y};
-    const dw* v = V + (size_t)j * m;
-    dw vv[R];
-#pragma unroll
-    for (int u = 0; u < R; ++u) {
-      const int i = lane + 32 * u;
-      if (i < m) {
-        const float2 x = __ldg(reinterpret_cast<const float2*>(v + i));
-        vv[u] = {x.x, x.y};
-      } else {
-        vv[u] = {0.f, 0.f};
-      }
-    }
-    dw_acc acc;
-#pragma unroll
-    for (int u = 0; u < R; ++u) dw_dot_step(acc, vv[u], q[u]);
-    const dw w = dw_mul(dw_warp_sum(dw_acc_value(acc)), t);
-#pragma unroll
-    for (int u = 0; u < R; ++u) q[u] = dw_add(q[u], dw_neg(dw_mul(w, vv[u])));
-  }
-#pragma unroll
-  for (int u = 0; u < R; ++u) {
-    const int i = lane + 32 * u;
-    if (i < m) Q[(size_t)(rows ? rows[i] : i) * p + k] = dw_to_scaled(q[u], 0);
-  }
-}
-template <int R>
-__global__ void k_qr_formq_reg(const dw* __restrict__ V, int m, int p, const dw* __restrict__ T,
-                               double* __restrict__ Q, const int* __restrict__ rows) { k_qr_formq_reg_body<R>(V, m, p, T, Q, rows); }
-
 int launch_qr_formq(vp_ctx* ctx, const double* A, int m, int n, const double* tau, double* Q, const int* rows) {
-  const int p = std::min(m, n);
-  if (p <= 0) return VP_OK;
-  VP_TRY(reserve(ctx, ctx->w_q, (size_t)m * p));
-  VP_TRY(reserve(ctx, ctx->w_fq, (size_t)m * p + p + 8));
-  dw* V = reinterpret_cast<dw*>(ctx->w_fq.p);
-  dw* T = V + (size_t)m * p;
-  const size_t total = (size_t)m * p;
-  const int cb = (int)std::min<size_t>((total + 255) / 256, (size_t)ctx->num_sms * 8);
-  ctx->launches += 2;
-  k_reflectors_to_dw<<<cb, 256, 0, ctx->stream>>>(A, m, p, tau, V, T);
-  VP_TRY(check_launch(ctx, "reflectors_to_dw"));
-  if (m <= 512) {  // column of Q in registers
-    const int wpb = 4, blocks = (p + wpb - 1) / wpb;
-    if (m <= 64) k_qr_formq_reg<2><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
-    else if (m <= 128) k_qr_formq_reg<4><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
-    else if (m <= 256) k_qr_formq_reg<8><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
-    else k_qr_formq_reg<16><<<blocks, wpb * 32, 0, ctx->stream>>>(V, m, p, T, Q, rows);
-    return check_launch(ctx, "qr_formq");
-  }
-  const int wpb = 8;
-  k_qr_formq_dw<<<(p + wpb - 1) / wpb, wpb * 32, 0, ctx->stream>>>(V, m, p, T, reinterpret_cast<dw*>(ctx->w_q.p), Q, rows);
-  return check_launch(ctx, "qr_formq");
+  return blaunch_formq(ctx, ctx->stream, {FormQJob{A, m, n, tau, Q, rows, &ctx->w_fq, &ctx->w_q}});
 }
 
 __device__ __forceinline__ void k_qr_getr_body(const double* __restrict__ A, int m, int n, int p, double* __restrict__ R) {
@@ -1783,68 +1674,16 @@ int blaunch_qr_factor(vp_ctx* ctx, cudaStream_t st, const std::vector<BQR>& v) {
   return VP_OK;
 }
 
-struct R2DwArgs {
-  const double* A;
-  int m, p;
-  const double* tau;
-  dw* V;
-  dw* T;
-};
-__global__ void kb_reflectors_to_dw(const __grid_constant__ Pack<R2DwArgs> pk) {
-  const R2DwArgs& a = pk.a[blockIdx.y];
-  k_reflectors_to_dw_body(a.A, a.m, a.p, a.tau, a.V, a.T);
-}
-struct FormQArgs {
-  const dw* V;
-  int m, p;
-  const dw* T;
-  dw* scratch;
-  double* Q;
-  const int* rows;
-};
-template <int R>
-__global__ void kb_qr_formq_reg(const __grid_constant__ Pack<FormQArgs> pk) {
-  const FormQArgs& a = pk.a[blockIdx.y];
-  k_qr_formq_reg_body<R>(a.V, a.m, a.p, a.T, a.Q, a.rows);
-}
-__global__ void kb_qr_formq_dw(const __grid_constant__ Pack<FormQArgs> pk) {
-  const FormQArgs& a = pk.a[blockIdx.y];
-  k_qr_formq_dw_body(a.V, a.m, a.p, a.T, a.scratch, a.Q, a.rows);
-}
-
 int blaunch_qr_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<BFormQ>& v) {
-  std::vector<R2DwArgs> conv;
-  std::vector<FormQArgs> reg[5], gl;
+  std::vector<FormQJob> jobs;
   SlotCounter slots;
   for (const BFormQ& f : v) {
-    const int p = std::min(f.m, f.n);
-    if (p <= 0) continue;
+    if (std::min(f.m, f.n) <= 0) continue;
     int sl = 0;
     VP_TRY(slots.next(ctx, f.s, &sl));
-    VP_TRY(reserve(ctx, f.s->fq[sl], (size_t)f.m * p + p + 8));
-    dw* V = reinterpret_cast<dw*>(f.s->fq[sl].p);
-    dw* T = V + (size_t)f.m * p;
-    conv.push_back({f.A, f.m, p, f.tau, V, T});
-    FormQArgs a{V, f.m, p, T, nullptr, f.Q, f.rows};
-    if (f.m <= 64) reg[1].push_back(a);
-    else if (f.m <= 128) reg[2].push_back(a);
-    else if (f.m <= 256) reg[3].push_back(a);
-    else if (f.m <= 512) reg[4].push_back(a);
-    else {
-      VP_TRY(reserve(ctx, f.s->qscr[sl], (size_t)f.m * p));
-      a.scratch = reinterpret_cast<dw*>(f.s->qscr[sl].p);
-      gl.push_back(a);
-    }
+    jobs.push_back({f.A, f.m, f.n, f.tau, f.Q, f.rows, &f.s->fq[sl], &f.s->qscr[sl]});
   }
-  VP_TRY(run_packs(ctx, st, conv, kb_reflectors_to_dw, 256, 0,
-                   [&](const R2DwArgs& a) { return grid_stride_blocks(ctx, (size_t)a.m * a.p, 8); }, "b_refl_to_dw"));
-  auto blocks4 = [](const FormQArgs& a) { return (a.p + 3) / 4; };
-  VP_TRY(run_packs(ctx, st, reg[1], kb_qr_formq_reg<2>, 128, 0, blocks4, "b_formq"));
-  VP_TRY(run_packs(ctx, st, reg[2], kb_qr_formq_reg<4>, 128, 0, blocks4, "b_formq"));
-  VP_TRY(run_packs(ctx, st, reg[3], kb_qr_formq_reg<8>, 128, 0, blocks4, "b_formq"));
-  VP_TRY(run_packs(ctx, st, reg[4], kb_qr_formq_reg<16>, 128, 0, blocks4, "b_formq"));
-  return run_packs(ctx, st, gl, kb_qr_formq_dw, 256, 0, [](const FormQArgs& a) { return (a.p + 7) / 8; },
-                   "b_formq_dw");
+  return blaunch_formq(ctx, st, jobs);
 }
 
 struct GetRArgs {
