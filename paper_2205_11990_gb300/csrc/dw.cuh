@@ -30,7 +30,7 @@
 
 namespace vp {
 
-struct dw {
+struct __align__(8) dw {
   float hi, lo;
 };
 
