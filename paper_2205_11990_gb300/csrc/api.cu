@@ -773,6 +773,7 @@ static vp_ctx* ctx_child(vp_ctx* parent) {
     return nullptr;
   }
   c->owns_stream = true;
+  c->early = false;  // runs beside the parent's stream
   c->wait_clocks = parent->wait_clocks;
   if (write_wait_limit(c) != VP_OK) {
     vp_ctx_destroy(c);
@@ -1552,6 +1553,8 @@ static int c1_stage(vp_sim* s, int i, const mps_t*& fi, const mps_t*& acc, doubl
     VP_TRY(site_sum_mps(ctx, 1.0, acc, B[i] * dt, &s->L, fi, &s->wa));
     VP_TRY(site_sum_mps(cb, 1.0, &s->f, A[i] * dt, &s->L, fi, &s->wb));
     const int cap0 = ctx->coop_cap;
+    const bool early0 = ctx->early;
+    ctx->early = false;
     ctx->coop_cap = cb->coop_cap = std::max(2, ctx->num_sms / (2 * s->coop_div));
     int stB = VP_OK;
     Flops fB;
@@ -1565,6 +1568,7 @@ static int c1_stage(vp_sim* s, int i, const mps_t*& fi, const mps_t*& acc, doubl
     const int stA = compress(ctx, &s->wa, 1 << 30, s->cfg.tol, nullptr);
     worker.join();
     ctx->coop_cap = cap0;
+    ctx->early = early0;
     if (stA != VP_OK) return stA;
     if (stB != VP_OK) return fail(ctx, stB, cb->err);
     VP_CUDA(ctx, cudaEventRecord(s->evB, cb->stream));

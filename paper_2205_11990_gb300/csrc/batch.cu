@@ -322,6 +322,7 @@ static int make_workers(vp_batch* b) {
     }
     c->owns_stream = true;
     c->coop_cap = std::max(16, parent->num_sms / nw);
+    c->early = nw == 1;
     c->wait_clocks = parent->wait_clocks;
     if (vp::write_wait_limit(c) != VP_OK) {
       vp_ctx_destroy(c);

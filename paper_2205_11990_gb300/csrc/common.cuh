@@ -68,6 +68,7 @@ struct vp_ctx {
   void* user = nullptr;
   std::string err;
   int64_t launches = 0;
+  bool early = true;  // launch_after may start kernels behind the one before
   vp::DevStatus* status = nullptr;  // device
   int* d_small = nullptr;           // device scratch ints (ranks, flags)
   int* h_small = nullptr;           // pinned host mirror
@@ -149,6 +150,46 @@ void release(vp_ctx* ctx, DevBuf& b);
 // Return released blocks whose work has finished (all: wait for every one).
 void drain_pending(vp_ctx* ctx, bool all);
 int check_launch(vp_ctx* ctx, const char* what);
+// Kernels of the sweeps' chains start while the kernel before them in the stream still
+// runs: launched by launch_after, their blocks are in place when it ends, and their
+// first statement waits until it has ended and its writes are visible (without the
+// launch attribute neither does anything).  Every thread calls it first, so that no
+// such kernel ends before the one it follows.
+//
+// It pays where one chain of small kernels is all there is (ctx->early: field solve
+// 211 -> 184 us, a stage of the 128 x 64 initial field 7.6 -> 7.15 ms, 64-point run
+// 40.4 -> 39.0, 1024 x 1024 step 64 -> 55).  Where several chains share the device
+// it costs: two streams 36.7 -> 38.1, three species 39.9 -> 44.0, groups of several
+// runs 117.5 -> 119.7; there the launches are plain ones.  Blocks with much shared
+// memory are not parked on an SM either.
+__device__ __forceinline__ void follow() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// cluster: CTAs of a cluster along x, y, z, or kNoCluster.
+const dim3 kNoCluster(0);
+constexpr size_t kEarlySmem = 32 * 1024;
+template <class... P, class... A>
+int launch_after(vp_ctx* ctx, const char* what, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                 dim3 cluster, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = ctx->early && smem <= kEarlySmem;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster.x;
+  at[1].val.clusterDim.y = cluster.y;
+  at[1].val.clusterDim.z = cluster.z;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster.x > 0 ? 2 : 1;
+  ctx->launches++;
+  if (cudaLaunchKernelEx(&cfg, kern, P(args)...) != cudaSuccess) return check_launch(ctx, what);
+  return VP_OK;
+}
 // Bracket one launch of class `cls` with events when profiling is on.
 void prof_begin(vp_ctx* ctx, int cls);
 void prof_end(vp_ctx* ctx, int cls, double work, int m = 0, int n = 0, int k = 0);

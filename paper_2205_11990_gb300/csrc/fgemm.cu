@@ -128,6 +128,7 @@ __device__ __forceinline__ void fma_tile(const FmaJob& j, int bx, int by, int sl
 // blockIdx.z: job x K slice (the slices of a tile are one cluster)
 template <int KA, int KB, int TILE>
 __global__ void __launch_bounds__(kFT) kb_gemm_fma(const __grid_constant__ Pack<FmaJob> pk, int zs) {
+  follow();
   const FmaJob& j = pk.a[blockIdx.z / zs];
   if ((int)blockIdx.x * TILE >= j.M || (int)blockIdx.y * TILE >= j.N) return;  // the whole cluster
   fma_tile<KA, KB, TILE>(j, blockIdx.x, blockIdx.y, blockIdx.z % zs, zs);
@@ -179,24 +180,8 @@ int launch_group(vp_ctx* ctx, cudaStream_t st, const std::vector<FmaJob>& jobs, 
       gy = std::max(gy, (pk.a[i].N + TILE - 1) / TILE);
     }
     if (gy > 65535) return fail(ctx, VP_ECAPACITY, "gemm: N too large");
-    ctx->launches++;
-    if (zs == 1) {
-      kb_gemm_fma<KA, KB, TILE><<<dim3(gx, gy, nb), kFT, 0, st>>>(pk, zs);
-      VP_TRY(check_launch(ctx, "gemm"));
-      continue;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    cfg.gridDim = dim3(gx, gy, nb * zs);
-    cfg.blockDim = dim3(kFT);
-    cfg.stream = st;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 1;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = zs;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, kb_gemm_fma<KA, KB, TILE>, pk, zs));
+    VP_TRY((launch_after(ctx, "gemm", kb_gemm_fma<KA, KB, TILE>, dim3(gx, gy, nb * zs), dim3(kFT), 0, st,
+                         zs > 1 ? dim3(1, 1, zs) : kNoCluster, pk, zs)));
   }
   return VP_OK;
 }

@@ -46,6 +46,7 @@ __device__ __forceinline__ int panels(int p) { return (p + kFB - 1) / kFB; }
 
 // Panel blockIdx.x of the reflectors as double words, and its T.
 __global__ void __launch_bounds__(256) kb_formq_prep(const __grid_constant__ Pack<FqArgs> pk) {
+  follow();
   const FqArgs& a = pk.a[blockIdx.y];
   __shared__ dw part[8][8];
   const int m = a.m, p = a.p, s = blockIdx.x, j0 = kFB * s;
@@ -107,6 +108,7 @@ __device__ __forceinline__ void copy16(void* dst, const void* src) {
 // Block 0 has the last columns, whose chains are the longest.
 template <int W, int R, int NC>
 __global__ void __launch_bounds__(32 * W * NC, W * NC <= 8 ? 2 : 1) kb_formq(const __grid_constant__ Pack<FqArgs> pk) {
+  follow();
   constexpr int T = 32 * W * NC;
   const FqArgs& a = pk.a[blockIdx.y];
   extern __shared__ double qsm[];
@@ -195,6 +197,7 @@ __global__ void __launch_bounds__(32 * W * NC, W * NC <= 8 ? 2 : 1) kb_formq(con
 // More than kFqMaxRows rows: a warp per column, the column in global memory, one
 // reflector at a time.
 __global__ void kb_formq_long(const __grid_constant__ Pack<FqArgs> pk) {
+  follow();
   const FqArgs& a = pk.a[blockIdx.y];
   const int lane = threadIdx.x & 31, m = a.m;
   const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -230,9 +233,8 @@ int launch_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<FqArgs>& v) {
       gx = std::max(gx, (pk.a[i].p + NC - 1) / NC);
       mm = std::max(mm, pk.a[i].m);
     }
-    ctx->launches++;
-    kb_formq<W, R, NC><<<dim3(gx, nb), 32 * W * NC, shared ? 2 * kFB * (size_t)mm * sizeof(dw) : 0, st>>>(pk);
-    VP_TRY(check_launch(ctx, "formq"));
+    VP_TRY((launch_after(ctx, "formq", kb_formq<W, R, NC>, dim3(gx, nb), dim3(32 * W * NC),
+                         shared ? 2 * kFB * (size_t)mm * sizeof(dw) : 0, st, kNoCluster, pk)));
   }
   return VP_OK;
 }
@@ -265,9 +267,7 @@ int blaunch_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<FormQJob>& v) 
       pk.a[i] = all[i0 + i];
       gx = std::max(gx, (pk.a[i].p + kFB - 1) / kFB);
     }
-    ctx->launches++;
-    kb_formq_prep<<<dim3(gx, nb), 256, 0, st>>>(pk);
-    VP_TRY(check_launch(ctx, "formq_prep"));
+    VP_TRY((launch_after(ctx, "formq_prep", kb_formq_prep, dim3(gx, nb), dim3(256), 0, st, kNoCluster, pk)));
   }
   VP_TRY((launch_formq<1, 1, 4>(ctx, st, by[0])));
   VP_TRY((launch_formq<1, 2, 4>(ctx, st, by[1])));
@@ -285,9 +285,7 @@ int blaunch_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<FormQJob>& v) 
       pk.a[i] = beyond[i0 + i];
       gx = std::max(gx, (pk.a[i].p + 7) / 8);
     }
-    ctx->launches++;
-    kb_formq_long<<<dim3(gx, nb), 256, 0, st>>>(pk);
-    VP_TRY(check_launch(ctx, "formq_long"));
+    VP_TRY((launch_after(ctx, "formq_long", kb_formq_long, dim3(gx, nb), dim3(256), 0, st, kNoCluster, pk)));
   }
   return VP_OK;
 }

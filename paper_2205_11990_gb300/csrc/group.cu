@@ -1042,7 +1042,10 @@ int vp_group_step(vp_group* g, vp_record* records, int* status) {
   g->stat_waits = 0;
   const int64_t l0 = g->ctx->launches;
   const double t0 = wall_ms();
+  const bool early0 = g->ctx->early;
+  if (g->mem.size() > 1) g->ctx->early = false;
   const int st = group_step(g, records);
+  g->ctx->early = early0;
   g->stat_step_ms = wall_ms() - t0;
   g->stat_launches = g->ctx->launches - l0;
   if (st != VP_OK) {

@@ -371,7 +371,10 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
   cl.sync();  // keep every CTA's shared memory alive until all remote accesses are done
 }
 
-__global__ void __launch_bounds__(kJT, 1) kb_jacobi_dw(const __grid_constant__ Pack<JacArgs> pk) { jacobi_body(pk.a[blockIdx.y]); }
+__global__ void __launch_bounds__(kJT, 1) kb_jacobi_dw(const __grid_constant__ Pack<JacArgs> pk) {
+  follow();
+  jacobi_body(pk.a[blockIdx.y]);
+}
 
 struct JacCfg {
   int cs, nb;
@@ -418,20 +421,9 @@ int blaunch_jacobi_dw(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& 
       const int nb = (int)std::min<size_t>(kMaxBatch, grp[cs].size() - i0);
       Pack<JacArgs> pk{};
       for (int i = 0; i < nb; ++i) pk.a[i] = grp[cs][i0 + i];
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute at1[1];
-      cfg.gridDim = dim3(cs, nb);
-      cfg.blockDim = dim3(kJT);
-      cfg.dynamicSmemBytes = std::max<size_t>(smem[cs], 116 * 1024);  // one CTA of the cluster per SM
-      cfg.stream = st;
-      at1[0].id = cudaLaunchAttributeClusterDimension;
-      at1[0].val.clusterDim.x = cs;
-      at1[0].val.clusterDim.y = 1;
-      at1[0].val.clusterDim.z = 1;
-      cfg.attrs = at1;
-      cfg.numAttrs = 1;
-      ctx->launches++;
-      VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, kb_jacobi_dw, pk));
+      VP_TRY(launch_after(ctx, "jacobi_dw", kb_jacobi_dw, dim3(cs, nb), dim3(kJT),
+                          std::max<size_t>(smem[cs], 116 * 1024),  // one CTA of the cluster per SM
+                          st, dim3(cs), pk));
     }
   }
   return VP_OK;

@@ -115,6 +115,7 @@ __device__ __forceinline__ void gather_tile(const QRSrc& s, int m, int n, double
   }
 }
 __global__ void kb_gather(const __grid_constant__ Pack<BGather> pk) {
+  follow();
   const BGather& a = pk.a[blockIdx.z];
   gather_tile(a.src, a.m, a.n, a.A, blockIdx.x, blockIdx.y);
 }
@@ -128,9 +129,7 @@ static int blaunch_gather(vp_ctx* ctx, cudaStream_t st, const std::vector<BGathe
       gx = std::max(gx, (v[i0 + i].n + 31) / 32);
       gy = std::max(gy, (v[i0 + i].m + 31) / 32);
     }
-    ctx->launches++;
-    kb_gather<<<dim3(gx, gy, nb), dim3(32, 8), 0, st>>>(pk);
-    VP_TRY(check_launch(ctx, "gather"));
+    VP_TRY((launch_after(ctx, "gather", kb_gather, dim3(gx, gy, nb), dim3(32, 8), 0, st, kNoCluster, pk)));
   }
   return VP_OK;
 }
@@ -467,16 +466,16 @@ __device__ __forceinline__ void k_qr_getr_body(const double* __restrict__ A, int
     R[e] = (j <= k) ? A[(size_t)k * m + j] : 0.0;
   }
 }
-__global__ void k_qr_getr(const double* __restrict__ A, int m, int n, int p, double* __restrict__ R) { k_qr_getr_body(A, m, n, p, R); }
+__global__ void k_qr_getr(const double* __restrict__ A, int m, int n, int p, double* __restrict__ R) {
+  follow();
+  k_qr_getr_body(A, m, n, p, R); }
 
 int launch_qr_getr(vp_ctx* ctx, const double* A, int m, int n, double* R) {
   const int p = std::min(m, n);
   const size_t total = (size_t)p * n;
   if (total == 0) return VP_OK;
   const int blocks = (int)std::min<size_t>((total + 255) / 256, (size_t)ctx->num_sms * 16);
-  ctx->launches++;
-  k_qr_getr<<<blocks, 256, 0, ctx->stream>>>(A, m, n, p, R);
-  return check_launch(ctx, "qr_getr");
+  return launch_after(ctx, "qr_getr", k_qr_getr, dim3(blocks), dim3(256), 0, ctx->stream, kNoCluster, A, m, n, p, R);
 }
 
 // ------------------------------------------------------------------- GEMM
@@ -608,7 +607,10 @@ __device__ __forceinline__ void k_sum_slices_body(const double* __restrict__ P, 
   }
 }
 __global__ void k_sum_slices(const double* __restrict__ P, int M, int N, int slices, size_t stride, double* C,
-                             int ldc) { k_sum_slices_body(P, M, N, slices, stride, C, ldc); }
+                             int ldc) {
+  follow();
+  k_sum_slices_body(P, M, N, slices, stride, C, ldc);
+}
 
 // The same operands as (row, k) maps for the tensor-core path.
 static TcOperand tc_a(const ARowMajor& a) { return {a.A, a.lda, 0}; }
@@ -653,9 +655,8 @@ static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a
     VP_TRY(blaunch_oz_gemm(ctx, ctx->stream, job));
     if (!split) return VP_OK;
     const int blocks = (int)std::min<size_t>((stride + 255) / 256, (size_t)ctx->num_sms * 8);
-    ctx->launches++;
-    k_sum_slices<<<blocks, 256, 0, ctx->stream>>>(ctx->w_split.p, M, N, oz.slices, stride, C, ldc);
-    return check_launch(ctx, what);
+    return launch_after(ctx, what, k_sum_slices, dim3(blocks), dim3(256), 0, ctx->stream, kNoCluster,
+                        ctx->w_split.p, M, N, oz.slices, stride, C, ldc);
   }
   const GemmPlan pl = gemm_plan(ctx, M, N, K);
   dim3 grid((M + pl.tile - 1) / pl.tile, (N + pl.tile - 1) / pl.tile, 1);
@@ -676,8 +677,8 @@ static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a
   kern<<<grid, 256, 0, ctx->stream>>>(M, N, K, alpha, a, b, ctx->w_split.p, N, kslice, stride);
   VP_TRY(check_launch(ctx, what));
   const int blocks = (int)std::min<size_t>((stride + 255) / 256, (size_t)ctx->num_sms * 8);
-  k_sum_slices<<<blocks, 256, 0, ctx->stream>>>(ctx->w_split.p, M, N, slices, stride, C, ldc);
-  return check_launch(ctx, what);
+  return launch_after(ctx, what, k_sum_slices, dim3(blocks), dim3(256), 0, ctx->stream, kNoCluster, ctx->w_split.p,
+                      M, N, slices, stride, C, ldc);
 }
 
 int launch_gemm(vp_ctx* ctx, int M, int N, int K, double alpha, const double* A, int lda, const double* B,
@@ -1347,6 +1348,7 @@ __device__ __forceinline__ void k_select_body(const double* __restrict__ X, cons
 }
 __global__ void k_select(const double* __restrict__ X, const double* __restrict__ norms, int b, int c, int chi, double tol,
                          int want_ent, int* perm, double* sigma, int* d_rank, double* d_err, DevStatus* st) {
+  follow();
   k_select_body(X, norms, b, c, chi, tol, want_ent, perm, sigma, d_rank, d_err, st);
 }
 // Threads of the selection: one per value up to 512 (the scans take as many steps
@@ -1361,10 +1363,8 @@ int launch_select(vp_ctx* ctx, const double* X, const double* norms, int b, int 
   // 48 KB a block gets without the opt-in
   static AttrOnce sattr;
   VP_TRY(sattr.ensure(ctx, (const void*)k_select, 200 * 1024, false));
-  ctx->launches++;
-  k_select<<<1, select_threads(b), smem, ctx->stream>>>(X, norms, b, c, chi, tol, want_ent, perm, sigma, d_rank, d_err,
-                                                        ctx->status);
-  return check_launch(ctx, "select");
+  return launch_after(ctx, "select", k_select, dim3(1), dim3(select_threads(b)), smem, ctx->stream, kNoCluster, X,
+                      norms, b, c, chi, tol, want_ent, perm, sigma, d_rank, d_err, ctx->status);
 }
 
 __device__ __forceinline__ void k_svd_outputs_body(const double* __restrict__ X, int q, int r, const int* __restrict__ perm,
@@ -1379,15 +1379,15 @@ __device__ __forceinline__ void k_svd_outputs_body(const double* __restrict__ X,
 }
 __global__ void k_svd_outputs(const double* __restrict__ X, int q, int r, const int* __restrict__ perm,
                               const double* __restrict__ sigma, const int* __restrict__ cperm, double* __restrict__ V) {
+  follow();
   k_svd_outputs_body(X, q, r, perm, sigma, cperm, V);
 }
 
 int launch_svd_outputs(vp_ctx* ctx, const double* X, int q, int r, const int* perm, const double* sigma,
                        const int* cperm, double* V) {
   const int blocks = (int)std::min<size_t>(((size_t)r * q + 255) / 256, (size_t)ctx->num_sms * 8);
-  ctx->launches++;
-  k_svd_outputs<<<std::max(1, blocks), 256, 0, ctx->stream>>>(X, q, r, perm, sigma, cperm, V);
-  return check_launch(ctx, "svd_outputs");
+  return launch_after(ctx, "svd_outputs", k_svd_outputs, dim3(std::max(1, blocks)), dim3(256), 0, ctx->stream,
+                      kNoCluster, X, q, r, perm, sigma, cperm, V);
 }
 
 // ------------------------------------------------------ SVD preconditioning
@@ -1464,6 +1464,7 @@ __device__ __forceinline__ void k_norm_order_body(const double* __restrict__ M, 
   }
 }
 __global__ void __launch_bounds__(512) kb_norm_order(const __grid_constant__ Pack<BNormOrder> pk) {
+  follow();
   const BNormOrder& a = pk.a[blockIdx.y];
   k_norm_order_body(a.M, a.ld, a.m, a.c, a.by_cols, a.lower, a.piv);
 }
@@ -1525,9 +1526,7 @@ int run_packs(vp_ctx* ctx, cudaStream_t st, const std::vector<A>& v, void (*kern
       pk.a[i] = v[i0 + i];
       gxm = std::max(gxm, (int)gx(v[i0 + i]));
     }
-    ctx->launches++;
-    kern<<<dim3(gxm, nb), threads, smem, st>>>(pk);
-    VP_TRY(check_launch(ctx, what));
+    VP_TRY(launch_after(ctx, what, kern, dim3(gxm, nb), dim3(threads), smem, st, kNoCluster, pk));
   }
   return VP_OK;
 }
@@ -1692,6 +1691,7 @@ struct GetRArgs {
   double* R;
 };
 __global__ void kb_qr_getr(const __grid_constant__ Pack<GetRArgs> pk) {
+  follow();
   const GetRArgs& a = pk.a[blockIdx.y];
   k_qr_getr_body(a.A, a.m, a.n, a.p, a.R);
 }
@@ -1732,6 +1732,7 @@ struct SumArgs {
   int ldc;
 };
 __global__ void kb_sum_slices(const __grid_constant__ Pack<SumArgs> pk) {
+  follow();
   const SumArgs& a = pk.a[blockIdx.y];
   k_sum_slices_body(a.P, a.M, a.N, a.slices, a.stride, a.C, a.ldc);
 }
@@ -1839,6 +1840,7 @@ int blaunch_jacobi(vp_ctx* ctx, cudaStream_t st, const std::vector<BJacobi>& v, 
 }
 
 __global__ void kb_select(const __grid_constant__ Pack<BSelect> pk) {
+  follow();
   const BSelect& a = pk.a[blockIdx.y];
   k_select_body(a.X, a.norms, a.b, a.c, a.chi, a.tol, a.want_ent, a.perm, a.sigma, a.d_rank, a.d_err, a.st);
 }
@@ -1853,6 +1855,7 @@ int blaunch_select(vp_ctx* ctx, cudaStream_t st, const std::vector<BSelect>& v) 
   return run_packs(ctx, st, v, kb_select, nt, smem, [](const BSelect&) { return 1; }, "b_select");
 }
 __global__ void kb_svd_outputs(const __grid_constant__ Pack<BSvdOut> pk) {
+  follow();
   const BSvdOut& a = pk.a[blockIdx.y];
   k_svd_outputs_body(a.X, a.q, a.r, a.perm, a.sigma, a.cperm, a.V);
 }

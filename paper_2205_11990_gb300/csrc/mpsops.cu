@@ -57,13 +57,15 @@ __device__ __forceinline__ void k_site_sum_body(SiteSum s, double* __restrict__ 
     out[e] = v;
   }
 }
-__global__ void k_site_sum(SiteSum s, double* __restrict__ out, int ol, int orr) { k_site_sum_body(s, out, ol, orr); }
+__global__ void k_site_sum(SiteSum s, double* __restrict__ out, int ol, int orr) {
+  follow();
+  k_site_sum_body(s, out, ol, orr);
+}
 
 int launch_site_sum(vp_ctx* ctx, const SiteSum& s, double* out, int ol, int orr) {
   const size_t total = (size_t)ol * 2 * orr;
-  ctx->launches++;
-  k_site_sum<<<grid_for(ctx, total), 256, 0, ctx->stream>>>(s, out, ol, orr);
-  return check_launch(ctx, "site_sum");
+  return launch_after(ctx, "site_sum", k_site_sum, dim3(grid_for(ctx, total)), dim3(256), 0, ctx->stream,
+                      kNoCluster, s, out, ol, orr);
 }
 
 __device__ __forceinline__ void k_phys_sum_body(const double* __restrict__ core, int rl, int rr, double* __restrict__ T) {
@@ -73,38 +75,43 @@ __device__ __forceinline__ void k_phys_sum_body(const double* __restrict__ core,
     T[e] = core[(l * 2) * rr + r] + core[(l * 2 + 1) * rr + r];
   }
 }
-__global__ void k_phys_sum(const double* __restrict__ core, int rl, int rr, double* __restrict__ T) { k_phys_sum_body(core, rl, rr, T); }
+__global__ void k_phys_sum(const double* __restrict__ core, int rl, int rr, double* __restrict__ T) {
+  follow();
+  k_phys_sum_body(core, rl, rr, T);
+}
 
 int launch_phys_sum(vp_ctx* ctx, const double* core, int rl, int rr, double* T) {
-  ctx->launches++;
-  k_phys_sum<<<grid_for(ctx, (size_t)rl * rr), 256, 0, ctx->stream>>>(core, rl, rr, T);
-  return check_launch(ctx, "phys_sum");
+  return launch_after(ctx, "phys_sum", k_phys_sum, dim3(grid_for(ctx, (size_t)rl * rr)), dim3(256), 0, ctx->stream,
+                      kNoCluster, core, rl, rr, T);
 }
 
 __device__ __forceinline__ void k_copy_body(const double* __restrict__ src, double* __restrict__ dst, size_t n) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
     dst[e] = src[e];
 }
-__global__ void k_copy(const double* __restrict__ src, double* __restrict__ dst, size_t n) { k_copy_body(src, dst, n); }
+__global__ void k_copy(const double* __restrict__ src, double* __restrict__ dst, size_t n) {
+  follow();
+  k_copy_body(src, dst, n);
+}
 
 int launch_copy(vp_ctx* ctx, const double* src, double* dst, size_t n) {
   if (n == 0) return VP_OK;
-  ctx->launches++;
-  k_copy<<<grid_for(ctx, n), 256, 0, ctx->stream>>>(src, dst, n);
-  return check_launch(ctx, "copy");
+  return launch_after(ctx, "copy", k_copy, dim3(grid_for(ctx, n)), dim3(256), 0, ctx->stream, kNoCluster, src, dst,
+                      n);
 }
 
 __device__ __forceinline__ void k_scale_body(double* x, size_t n, double s) {
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
     x[e] *= s;
 }
-__global__ void k_scale(double* x, size_t n, double s) { k_scale_body(x, n, s); }
+__global__ void k_scale(double* x, size_t n, double s) {
+  follow();
+  k_scale_body(x, n, s);
+}
 
 int launch_scale(vp_ctx* ctx, double* x, size_t n, double s) {
   if (n == 0) return VP_OK;
-  ctx->launches++;
-  k_scale<<<grid_for(ctx, n), 256, 0, ctx->stream>>>(x, n, s);
-  return check_launch(ctx, "scale");
+  return launch_after(ctx, "scale", k_scale, dim3(grid_for(ctx, n)), dim3(256), 0, ctx->stream, kNoCluster, x, n, s);
 }
 
 // A core (a, 2, b) read back to front: out (b, 2, a), out[j][s][i] = in[i][s][j]
@@ -184,14 +191,16 @@ __device__ __forceinline__ void k_permute_body(const double* __restrict__ f, int
   }
 }
 __global__ void k_permute(const double* __restrict__ f, int nx, int nv, int mapping, double* __restrict__ out,
-                          int inverse) { k_permute_body(f, nx, nv, mapping, out, inverse); }
+                          int inverse) {
+  follow();
+  k_permute_body(f, nx, nv, mapping, out, inverse);
+}
 
 int launch_permute_to_sites(vp_ctx* ctx, const double* f, int nx, int nv, int mapping, double* out,
                             int inverse) {
   const size_t total = (size_t)1 << (nx + nv);
-  ctx->launches++;
-  k_permute<<<grid_for(ctx, total), 256, 0, ctx->stream>>>(f, nx, nv, mapping, out, inverse);
-  return check_launch(ctx, "permute");
+  return launch_after(ctx, "permute", k_permute, dim3(grid_for(ctx, total)), dim3(256), 0, ctx->stream, kNoCluster,
+                      f, nx, nv, mapping, out, inverse);
 }
 
 // Periodic second-order Poisson on one block.  With s_i = dx^2 (rho_i -
@@ -267,7 +276,10 @@ __device__ __forceinline__ void k_poisson_body(const double* __restrict__ rho, i
   }
 }
 __global__ void k_poisson(const double* __restrict__ rho, int N, double dx, double* __restrict__ E,
-                          double* __restrict__ we) { k_poisson_body(rho, N, dx, E, we); }
+                          double* __restrict__ we) {
+  follow();
+  k_poisson_body(rho, N, dx, E, we);
+}
 
 int launch_poisson(vp_ctx* ctx, const double* rho, int N, double dx, double* E, double* we_dev) {
   const int nt = 256;
@@ -277,9 +289,8 @@ int launch_poisson(vp_ctx* ctx, const double* rho, int N, double dx, double* E, 
     static AttrOnce pattr;  // the largest size once, never lowered under another thread's launch
     VP_TRY(pattr.ensure(ctx, (const void*)k_poisson, 200 * 1024, false));
   }
-  ctx->launches++;
-  k_poisson<<<1, nt, smem, ctx->stream>>>(rho, N, dx, E, we_dev);
-  return check_launch(ctx, "poisson");
+  return launch_after(ctx, "poisson", k_poisson, dim3(1), dim3(nt), smem, ctx->stream, kNoCluster, rho, N, dx, E,
+                      we_dev);
 }
 
 // Net density of several species, net_i = sum_s w_s rho_s[i], and each
@@ -353,14 +364,16 @@ __device__ __forceinline__ void k_assemble_body(const double* __restrict__ U, in
   }
 }
 __global__ void k_assemble(const double* __restrict__ U, int ul, int ur, ETermSite e, int first, int last,
-                           double* __restrict__ out, int ol, int orr) { k_assemble_body(U, ul, ur, e, first, last, out, ol, orr); }
+                           double* __restrict__ out, int ol, int orr) {
+  follow();
+  k_assemble_body(U, ul, ur, e, first, last, out, ol, orr);
+}
 
 int launch_assemble_site(vp_ctx* ctx, const double* U, int ul, int ur, const ETermSite& e, int first, int last,
                          double* out, int ol, int orr) {
   const size_t total = (size_t)ol * 4 * orr;
-  ctx->launches++;
-  k_assemble<<<grid_for(ctx, total), 256, 0, ctx->stream>>>(U, ul, ur, e, first, last, out, ol, orr);
-  return check_launch(ctx, "assemble");
+  return launch_after(ctx, "assemble", k_assemble, dim3(grid_for(ctx, total)), dim3(256), 0, ctx->stream,
+                      kNoCluster, U, ul, ur, e, first, last, out, ol, orr);
 }
 
 // Dense MPO contraction step (tests): T (rows x w) with rows = (out, in)
@@ -401,13 +414,15 @@ __device__ __forceinline__ void k_check_finite_body(const double* __restrict__ x
     bad |= !isfinite(x[e]);
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicCAS(&st->err, 0, 2);
 }
-__global__ void k_check_finite(const double* __restrict__ x, size_t n, DevStatus* st) { k_check_finite_body(x, n, st); }
+__global__ void k_check_finite(const double* __restrict__ x, size_t n, DevStatus* st) {
+  follow();
+  k_check_finite_body(x, n, st);
+}
 
 int launch_check_finite(vp_ctx* ctx, const double* x, size_t n) {
   if (n == 0) return VP_OK;
-  ctx->launches++;
-  k_check_finite<<<grid_for(ctx, n), 256, 0, ctx->stream>>>(x, n, ctx->status);
-  return check_launch(ctx, "check_finite");
+  return launch_after(ctx, "check_finite", k_check_finite, dim3(grid_for(ctx, n)), dim3(256), 0, ctx->stream,
+                      kNoCluster, x, n, ctx->status);
 }
 
 // Sum of squared differences of two vectors, in a fixed order: per-block
@@ -462,15 +477,14 @@ int run_packs(vp_ctx* ctx, cudaStream_t st, const std::vector<A>& v, void (*kern
       pk.a[i] = v[i0 + i];
       gxm = std::max(gxm, (int)gx(v[i0 + i]));
     }
-    ctx->launches++;
-    kern<<<dim3(gxm, nb), threads, smem, st>>>(pk);
-    VP_TRY(check_launch(ctx, what));
+    VP_TRY(launch_after(ctx, what, kern, dim3(gxm, nb), dim3(threads), smem, st, kNoCluster, pk));
   }
   return VP_OK;
 }
 }  // namespace
 
 __global__ void kb_check_finite(const __grid_constant__ Pack<BCheck> pk) {
+  follow();
   const BCheck& a = pk.a[blockIdx.y];
   k_check_finite_body(a.x, a.n, a.st);
 }
@@ -479,6 +493,7 @@ int blaunch_check_finite(vp_ctx* ctx, cudaStream_t st, const std::vector<BCheck>
                    "b_check_finite");
 }
 __global__ void kb_copy(const __grid_constant__ Pack<BCopy> pk) {
+  follow();
   const BCopy& a = pk.a[blockIdx.y];
   k_copy_body(a.src, a.dst, a.n);
 }
@@ -489,6 +504,7 @@ int blaunch_copy(vp_ctx* ctx, cudaStream_t st, const std::vector<BCopy>& v) {
   return run_packs(ctx, st, nz, kb_copy, 256, 0, [&](const BCopy& a) { return grid_for(ctx, a.n); }, "b_copy");
 }
 __global__ void kb_site_sum(const __grid_constant__ Pack<BSiteSum> pk) {
+  follow();
   const BSiteSum& a = pk.a[blockIdx.y];
   k_site_sum_body(a.s, a.out, a.ol, a.orr);
 }
@@ -497,6 +513,7 @@ int blaunch_site_sum(vp_ctx* ctx, cudaStream_t st, const std::vector<BSiteSum>& 
                    [&](const BSiteSum& a) { return grid_for(ctx, (size_t)a.ol * 2 * a.orr); }, "b_site_sum");
 }
 __global__ void kb_phys_sum(const __grid_constant__ Pack<BPhysSum> pk) {
+  follow();
   const BPhysSum& a = pk.a[blockIdx.y];
   k_phys_sum_body(a.core, a.rl, a.rr, a.T);
 }
@@ -505,6 +522,7 @@ int blaunch_phys_sum(vp_ctx* ctx, cudaStream_t st, const std::vector<BPhysSum>& 
                    [&](const BPhysSum& a) { return grid_for(ctx, (size_t)a.rl * a.rr); }, "b_phys_sum");
 }
 __global__ void kb_scale(const __grid_constant__ Pack<BScale> pk) {
+  follow();
   const BScale& a = pk.a[blockIdx.y];
   k_scale_body(a.x, a.n, a.s);
 }
@@ -515,6 +533,7 @@ int blaunch_scale(vp_ctx* ctx, cudaStream_t st, const std::vector<BScale>& v) {
   return run_packs(ctx, st, nz, kb_scale, 256, 0, [&](const BScale& a) { return grid_for(ctx, a.n); }, "b_scale");
 }
 __global__ void kb_poisson(const __grid_constant__ Pack<BPoisson> pk) {
+  follow();
   const BPoisson& a = pk.a[blockIdx.y];
   k_poisson_body(a.rho, a.N, a.dx, a.E, a.we);
 }
@@ -528,6 +547,7 @@ int blaunch_poisson(vp_ctx* ctx, cudaStream_t st, const std::vector<BPoisson>& v
   return run_packs(ctx, st, v, kb_poisson, nt, smem, [](const BPoisson&) { return 1; }, "b_poisson");
 }
 __global__ void kb_assemble(const __grid_constant__ Pack<BAssemble> pk) {
+  follow();
   const BAssemble& a = pk.a[blockIdx.y];
   k_assemble_body(a.U, a.ul, a.ur, a.e, a.first, a.last, a.out, a.ol, a.orr);
 }
@@ -536,6 +556,7 @@ int blaunch_assemble(vp_ctx* ctx, cudaStream_t st, const std::vector<BAssemble>&
                    [&](const BAssemble& a) { return grid_for(ctx, (size_t)a.ol * 4 * a.orr); }, "b_assemble");
 }
 __global__ void kb_permute(const __grid_constant__ Pack<BPermute> pk) {
+  follow();
   const BPermute& a = pk.a[blockIdx.y];
   k_permute_body(a.f, a.nx, a.nv, a.mapping, a.out, a.inverse);
 }

@@ -480,18 +480,21 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
 }
 
 __global__ void __launch_bounds__(kOzThreads) kb_oz_kexp(const __grid_constant__ Pack<OzJob> pk) {
+  follow();
   const OzJob& j = pk.a[blockIdx.y];
   if ((int)blockIdx.x * 8 >= j.K) return;
   oz_kexp_body(j, blockIdx.x);
 }
 // x: 32-row blocks of A, then of B (ablk of A at most); y: K slice; z: job
 __global__ void __launch_bounds__(kOzThreads) kb_oz_pack(const __grid_constant__ Pack<OzJob> pk, int ablk) {
+  follow();
   const OzJob& j = pk.a[blockIdx.z];
   if ((int)blockIdx.y >= j.slices) return;
   const int side = (int)blockIdx.x >= ablk;
   oz_pack_body(j, side, (int)blockIdx.x - (side ? ablk : 0), blockIdx.y);
 }
 __global__ void __launch_bounds__(256, 1) kb_oz_mma(const __grid_constant__ Pack<OzJob> pk, int zs) {
+  follow();
   const OzJob& j = pk.a[blockIdx.z / zs];
   const int slice = blockIdx.z % zs;
   if (slice >= j.slices || (int)blockIdx.x * kOzM >= j.M || (int)blockIdx.y * kOzN >= j.N) return;
@@ -579,11 +582,11 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       gy = std::max(gy, (int)(Np / kOzN));
     }
     if (gy > 65535 || (long long)nb * zs > 65535) return fail(ctx, VP_ECAPACITY, "gemm: too large");
-    ctx->launches += 3;
-    kb_oz_kexp<<<dim3(ks, nb), kOzThreads, 0, st>>>(pk);
-    kb_oz_pack<<<dim3(ablk + bblk, zs, nb), kOzThreads, oz_pack_smem(ksl), st>>>(pk, ablk);
-    kb_oz_mma<<<dim3(gx, gy, nb * zs), 256, kOzSmem, st>>>(pk, zs);
-    VP_TRY(check_launch(ctx, "oz_gemm"));
+    VP_TRY(launch_after(ctx, "oz_kexp", kb_oz_kexp, dim3(ks, nb), dim3(kOzThreads), 0, st, kNoCluster, pk));
+    VP_TRY(launch_after(ctx, "oz_pack", kb_oz_pack, dim3(ablk + bblk, zs, nb), dim3(kOzThreads), oz_pack_smem(ksl),
+                        st, kNoCluster,
+                        pk, ablk));
+    VP_TRY(launch_after(ctx, "oz_mma", kb_oz_mma, dim3(gx, gy, nb * zs), dim3(256), kOzSmem, st, kNoCluster, pk, zs));
   }
   return VP_OK;
 }
