@@ -18,13 +18,17 @@
 // a long update for each of its dependent rounds; here a dependent round is a few
 // operations on a 2 nb x 2 nb matrix.  Rows and rotations are double words, so the
 // rows stay the accurate images of the input; the Gram matrix, recomputed from
-// them every sweep, only steers the rotations.
+// them every sweep, only steers the rotations.  Its diagonal is a double word (two
+// nearly equal norms decide an angle by their difference); what is off it needs only
+// its own digits and is FP32 between two recomputations.
 //
 // Measured on GB300 (event-timed, one problem; before: row-by-row rotations of the
 // same rows, whose every round was a dot product, parameters and an update):
 // a block round of 2 x 4 rows of 128 is ~1300 cycles of products, 650-900 a round
 // of rotations, 1500 for the move and 700 for the cluster barrier; 128 rows 142 us
-// a sweep (243), 64: 51 (83), 44: 40 (82), 16: 13 (19), 212: 334 (519).
+// a sweep (243), 64: 51 (83), 44: 40 (82), 16: 13 (19), 212: 334 (519).  With double
+// words on eight-byte boundaries and the FP32 part: 128 rows 110, 64: 47, 44: 36,
+// 16: 12, 212: 270.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -67,17 +71,17 @@ __device__ __forceinline__ int next_pos(int pos, int CS) {
 // Rotation that zeroes gamma between rows of squared norms alpha, beta: an FP32
 // tangent (the angle need not be exact), its cosine to a double word so that the
 // rotation is orthogonal to 2^-47.  False: the pair is left alone.
-__device__ __forceinline__ bool rotation(dw al, dw be, dw g, float eps, dw& cs, dw& sn) {
+__device__ __forceinline__ bool rotation(dw al, dw be, float g, float eps, dw& cs, dw& sn, float& t) {
   cs = {1.0f, 0.0f};
   sn = {0.0f, 0.0f};
-  if (!(al.hi > kTiny && be.hi > kTiny && fabsf(g.hi) * rsqrt_approx(al.hi) * rsqrt_approx(be.hi) > eps)) return false;
+  if (!(al.hi > kTiny && be.hi > kTiny && fabsf(g) * rsqrt_approx(al.hi) * rsqrt_approx(be.hi) > eps)) return false;
   const float d0 = 0.5f * ((be.hi - al.hi) + (be.lo - al.lo));
   // a power of two brings the larger of the two to [1, 2): no square leaves FP32
-  const int ex = (__float_as_int(fmaxf(fabsf(d0), fabsf(g.hi))) >> 23) & 255;
+  const int ex = (__float_as_int(fmaxf(fabsf(d0), fabsf(g))) >> 23) & 255;
   const float sc = __int_as_float((254 - min(ex, 253)) << 23);
-  const float d = d0 * sc, gs = g.hi * sc;
+  const float d = d0 * sc, gs = g * sc;
   const float x = fmaf(d, d, gs * gs);
-  const float t = copysignf(1.0f, d) * gs * rcp_approx(fabsf(d) + x * rsqrt_approx(x));
+  t = copysignf(1.0f, d) * gs * rcp_approx(fabsf(d) + x * rsqrt_approx(x));
   if (t == 0.f) return false;
   // u = 1 + t^2; y = 1 / sqrt(u) refined in FP32, then with the residual
   // r = 1 - u y^2 in double words: y (1 + r / 2 + 3 r^2 / 8)
@@ -103,11 +107,11 @@ __device__ __forceinline__ dw comb(dw a, dw x, dw b, dw y) {
   return fast_two_sum(s, e);
 }
 
-// Products of row pairs into G (both triangles): warp w takes the pairs w NV ..
-// of tab, then those kJW NV further on.
+// Products of row pairs into G (both triangles; of a row with itself into Dg): warp
+// w takes the pairs w NV .. of tab, then those kJW NV further on.
 template <int NV>
-__device__ __forceinline__ void gram(const dw* rows, int c, int B, const unsigned short* tab, int npair, dw* G, int lane,
-                                     int warp) {
+__device__ __forceinline__ void gram(const dw* rows, int c, int B, const unsigned short* tab, int npair, dw* Dg, float* G,
+                                     int lane, int warp) {
   for (int base = warp * NV; base < npair; base += kJW * NV) {
     dw_acc acc[NV];
     int oi[NV], oj[NV];
@@ -144,8 +148,10 @@ __device__ __forceinline__ void gram(const dw* rows, int c, int B, const unsigne
     const dw s = norm2(warp_sums<NV>(val, lane));
     if (lane % (32 / NV) == 0 && base + v < npair) {
       const int i = mine >> 8, j = mine & 255;
-      G[i * B + j] = s;
-      G[j * B + i] = s;
+      if (i == j)
+        Dg[i] = s;
+      else
+        G[i * B + j] = G[j * B + i] = s.hi;
     }
   }
 }
@@ -157,12 +163,13 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = a.b, c = a.b, nb = a.nb, B = 2 * nb;
   dw* rows = reinterpret_cast<dw*>(smd);  // two sets of B rows: top block, bottom block
-  dw* G2 = rows + 2 * (size_t)B * c;      // two Gram matrices
-  dw* par = G2 + 2 * B * B;  // cosine, sine of pair p of round rd at 2 (16 rd + p)
+  dw* D2 = rows + 2 * (size_t)B * c;      // their squared norms
+  float* G2 = reinterpret_cast<float*>(D2 + 2 * B);  // two Gram matrices (off the diagonal)
+  dw* par = reinterpret_cast<dw*>(G2 + 2 * B * B);   // cosine, sine of pair p of round rd at 2 (16 rd + p)
   unsigned short* tab = reinterpret_cast<unsigned short*>(par + 32 * (2 * nb + 1));  // all pairs of rows
   unsigned short* xtab = tab + B * (B + 1) / 2;     // the pairs across the two blocks
   unsigned short* prow = xtab + nb * nb;            // rows (i << 8 | j) of pair p of round rd at 16 rd + p
-  unsigned short* ptab = prow + 16 * (2 * nb + 1);  // pairs of pairs (P << 8 | Q), P <= Q, of np = nb, then bp
+  unsigned short* ptab = prow + 16 * (2 * nb + 1);  // pairs of pairs (P << 8 | Q), P < Q, of np = nb, then bp
   __shared__ int red[kJW + 1];
   __shared__ unsigned cnt[4];
   __shared__ unsigned rmask[2 * (kJMaxNb + 1)];  // pairs that rotate in each round
@@ -216,12 +223,12 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
     }
     prow[e] = (unsigned short)((i << 8) | j);
   }
-  const int nt0 = nb * (nb + 1) / 2, nt1 = bp * (bp + 1) / 2;
+  const int nt0 = nb * (nb - 1) / 2, nt1 = bp * (bp - 1) / 2;
   if (tid < 2) {
     const int np = tid ? bp : nb;
     unsigned short* o = ptab + (tid ? nt0 : 0);
     for (int P = 0; P < np; ++P)
-      for (int Q = P; Q < np; ++Q) *o++ = (unsigned short)((P << 8) | Q);
+      for (int Q = P + 1; Q < np; ++Q) *o++ = (unsigned short)((P << 8) | Q);
   }
   __syncthreads();
   if (tid == 0) {
@@ -245,19 +252,20 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
     unsigned rotated = 0;
     for (int br = 0; br < brounds; ++br) {
       dw* R = rows + (size_t)cur * B * c;
-      dw* G = G2 + cur * B * B;
+      dw* Dg = D2 + cur * B;
+      float* G = G2 + cur * B * B;
       const unsigned short* tb = br == 0 ? tab : xtab;
       const int ng = br == 0 ? npair : nb * nb, chunk = (ng + kJW - 1) / kJW;
       if (chunk <= 1)
-        gram<1>(R, c, B, tb, ng, G, lane, warp);
+        gram<1>(R, c, B, tb, ng, Dg, G, lane, warp);
       else if (chunk <= 2)
-        gram<2>(R, c, B, tb, ng, G, lane, warp);
+        gram<2>(R, c, B, tb, ng, Dg, G, lane, warp);
       else if (chunk <= 4)
-        gram<4>(R, c, B, tb, ng, G, lane, warp);
+        gram<4>(R, c, B, tb, ng, Dg, G, lane, warp);
       else if (chunk <= 8)
-        gram<8>(R, c, B, tb, ng, G, lane, warp);
+        gram<8>(R, c, B, tb, ng, Dg, G, lane, warp);
       else
-        gram<16>(R, c, B, tb, ng, G, lane, warp);
+        gram<16>(R, c, B, tb, ng, Dg, G, lane, warp);
       __syncthreads();
       const int rd0 = br == 0 ? 0 : inside, rd1 = inside + nb;
       // round rd's rotations applied to the rows: a task is one pair of one column
@@ -285,12 +293,19 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
           const int np = rd < inside ? bp : nb, nt = rd < inside ? nt1 : nt0;
           const unsigned short* pt = ptab + (rd < inside ? nt0 : 0);
           dw cs = {1.0f, 0.0f}, sn = {0.0f, 0.0f};
+          float t = 0.f;
           bool rot = false;
           const int ij = prow[16 * rd + (lane & 15)];
           if (lane < np) {
             const int i = ij >> 8, j = ij & 255;
-            if (i != j) rot = rotation(G[i * B + i], G[j * B + j], G[i * B + j], a.eps, cs, sn);
+            const dw al = Dg[i], be = Dg[j];
+            const float g = G[i * B + j];
+            if (i != j) rot = rotation(al, be, g, a.eps, cs, sn, t);
             if (rot) {
+              const dw tg = two_prod(t, g);
+              Dg[i] = dw_add_fast(al, dw_neg(tg));
+              Dg[j] = dw_add_fast(be, tg);
+              G[i * B + j] = G[j * B + i] = 0.f;
               par[2 * (16 * rd + lane)] = cs;
               par[2 * (16 * rd + lane) + 1] = sn;
               ++rotated;
@@ -298,20 +313,21 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
           }
           const unsigned any = __ballot_sync(0xffffffffu, rot);
           if (lane == 0) rmask[rd] = any;
-          // both sides of the Gram matrix: the 2 x 2 block of pairs P <= Q by one lane
+          // both sides of the Gram matrix: the 2 x 2 block of pairs P < Q by one lane
           for (int e0 = 0; any != 0 && e0 < nt; e0 += 32) {
             const int e = e0 + lane, PQ = pt[min(e, nt - 1)], P = PQ >> 8, Q = PQ & 255;
-            const dw cp = shfl_dw(cs, P), sp = shfl_dw(sn, P), cq = shfl_dw(cs, Q), sq = shfl_dw(sn, Q);
+            const float cp = __shfl_sync(0xffffffffu, cs.hi, P), sp = __shfl_sync(0xffffffffu, sn.hi, P);
+            const float cq = __shfl_sync(0xffffffffu, cs.hi, Q), sq = __shfl_sync(0xffffffffu, sn.hi, Q);
             const int ip = __shfl_sync(0xffffffffu, ij, P), iq = __shfl_sync(0xffffffffu, ij, Q);
             const int i = ip >> 8, j = ip & 255, k = iq >> 8, l = iq & 255;
-            if (e < nt && (sp.hi != 0.f || sq.hi != 0.f)) {
+            if (e < nt && (sp != 0.f || sq != 0.f)) {
               // (a row that sits out: i == j or k == l, with cosine 1 and sine 0 on
               // its side, where both halves of the block are the same numbers)
-              const dw g00 = G[i * B + k], g01 = G[i * B + l], g10 = G[j * B + k], g11 = G[j * B + l];
-              const dw a0 = comb(cp, g00, dw_neg(sp), g10), a1 = comb(sp, g00, cp, g10);
-              const dw b0 = comb(cp, g01, dw_neg(sp), g11), b1 = comb(sp, g01, cp, g11);
-              const dw h00 = comb(cq, a0, dw_neg(sq), b0), h01 = comb(sq, a0, cq, b0);
-              const dw h10 = comb(cq, a1, dw_neg(sq), b1), h11 = comb(sq, a1, cq, b1);
+              const float g00 = G[i * B + k], g01 = G[i * B + l], g10 = G[j * B + k], g11 = G[j * B + l];
+              const float a0 = fmaf(cp, g00, -sp * g10), a1 = fmaf(sp, g00, cp * g10);
+              const float b0 = fmaf(cp, g01, -sp * g11), b1 = fmaf(sp, g01, cp * g11);
+              const float h00 = fmaf(cq, a0, -sq * b0), h01 = fmaf(sq, a0, cq * b0);
+              const float h10 = fmaf(cq, a1, -sq * b1), h11 = fmaf(sq, a1, cq * b1);
               G[i * B + k] = G[k * B + i] = h00;
               G[i * B + l] = G[l * B + i] = h01;
               G[j * B + k] = G[k * B + j] = h10;
@@ -334,7 +350,8 @@ __device__ __forceinline__ void jacobi_body(const JacArgs& a) {
         dw* to = cl.map_shared_rank(rows + (size_t)(cur ^ 1) * B * c + (size_t)ds * nb * c, pos_cta(np, CS));
         const dw* from = R + (size_t)slot * nb * c;
         for (int e = tid; e < nb * c; e += kJT) to[e] = from[e];
-        dw* tg = cl.map_shared_rank(G2 + (cur ^ 1) * B * B, pos_cta(np, CS));
+        float* tg = cl.map_shared_rank(G2 + (cur ^ 1) * B * B, pos_cta(np, CS));
+        if (tid < nb) cl.map_shared_rank(D2 + (cur ^ 1) * B, pos_cta(np, CS))[ds * nb + tid] = Dg[slot * nb + tid];
         for (int e = tid; e < nb * nb; e += kJT) {
           const int i = e / nb, j = e - i * nb;
           tg[(ds * nb + i) * B + ds * nb + j] = G[(slot * nb + i) * B + slot * nb + j];
@@ -389,7 +406,7 @@ JacCfg jac_cfg(int b, int cs_max) {
 }
 size_t jac_smem(const JacCfg& g, int c) {
   const size_t B = 2 * (size_t)g.nb, bp = g.nb + (g.nb & 1);
-  return (2 * B * c + 2 * B * B + 32 * (B + 1)) * sizeof(dw) +
+  return (2 * B * c + 2 * B + 32 * (B + 1)) * sizeof(dw) + 2 * B * B * sizeof(float) +
          (B * (B + 1) / 2 + g.nb * g.nb + 16 * (B + 1) + g.nb * (g.nb + 1) / 2 + bp * (bp + 1) / 2) * sizeof(unsigned short);
 }
 constexpr size_t kJacSmemMax = 216 * 1024;
