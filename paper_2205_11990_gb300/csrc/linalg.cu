@@ -1,9 +1,9 @@
 // FP64 dense linear algebra of the compression sweeps (SI "Canonicalization and
 // Compression"): Householder QR, explicit Q, GEMM, one-sided Jacobi SVD and the
 // truncation rule of the truncation-error equation (main text, "MPS
-// Representation").  All kernels work on one matrix at a time and spread it
-// over every SM: FP64 on GB300 issues about two FMAs per SM per clock, so no
-// factorisation may sit on a single SM.
+// Representation"): the choice between their kernels, the small ones, and the FP64
+// and grid kernels of what the others do not take (panel QR: qrpanel.cu, Q:
+// formq.cu, block Jacobi: jacobi.cu, contractions: fgemm.cu, ozgemm.cu, tcgemm.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -381,14 +381,18 @@ __global__ void __launch_bounds__(kThreads) k_qr_factor_dw(double* A, int m, int
 // block (contiguous in the column-major layout) is factored in place, Q is
 // formed from its reflectors, and the rest of R is one FP64 GEMM, R2 = Q^T A2
 // (stored as R2^T = A2^T Q, which is A2's column-major layout), instead of
-// applying every reflector to all n columns.  Otherwise the panel QR; what has
-// more rows than its panel holds in registers goes to the grid kernel.  The
+// applying every reflector to all n columns.  Not where one block or a cluster
+// applies a panel to all of them in one pass, two columns a warp: those six launches
+// then cost more (us, this way / the panel QR: 4 x 32 53 / 25, 16 x 128 63 / 46, 32 x
+// 384 80 / 51; but 64 x 3392 198 / 355, 128 x 1696 332 / 436).  Otherwise the panel
+// QR; what has more rows than its panel holds in registers goes to the grid kernel.  The
 // choice depends on the shape and the device only, so that results do not depend
 // on the context or on the batch.
 QRPlan qr_plan(const vp_ctx* ctx, int m, int n) {
   if (std::min(m, n) <= 0) return {QR_NONE, {}};
-  if (n > 2 * m && m >= 2) return {QR_WIDE, {}};
   const PanelPlan pl = qr_panel_plan(ctx, m, n);
+  const bool one_pass = pl.kind == PANEL_SOLO || (pl.kind == PANEL_CLUSTER && n <= 32 * (pl.cs - 1));
+  if (n > 2 * m && m >= 2 && !one_pass) return {QR_WIDE, {}};
   if (pl.kind != PANEL_NONE) return {QR_PANEL, pl};
   return {QR_GRID, {}};
 }
