@@ -159,7 +159,7 @@ int check_launch(vp_ctx* ctx, const char* what);
 // It pays where one chain of small kernels is all there is (ctx->early: field solve
 // 211 -> 184 us, a stage of the 128 x 64 initial field 7.6 -> 7.15 ms, 64-point run
 // 40.4 -> 39.0, 1024 x 1024 step 64 -> 55).  Where several chains share the device
-// it costs: two streams 36.7 -> 38.1, three species 39.9 -> 44.0, groups of several
+// it costs: two streams 36.7 -> 38.1, two species 39.9 -> 44.0, groups of several
 // runs 117.5 -> 119.7; there the launches are plain ones.  Blocks with much shared
 // memory are not parked on an SM either.
 __device__ __forceinline__ void follow() {

@@ -1535,32 +1535,6 @@ int run_packs(vp_ctx* ctx, cudaStream_t st, const std::vector<A>& v, void (*kern
   return VP_OK;
 }
 
-// The same for cluster kernels: grid (cs, nb), clusters of cs CTAs along x.
-template <class A>
-int run_cluster_packs(vp_ctx* ctx, cudaStream_t st, const std::vector<A>& v, void (*kern)(const Pack<A>), int cs,
-                      int threads, size_t smem) {
-  for (size_t i0 = 0; i0 < v.size(); i0 += kMaxBatch) {
-    const int nb = (int)std::min<size_t>(kMaxBatch, v.size() - i0);
-    Pack<A> pk{};
-    for (int i = 0; i < nb; ++i) pk.a[i] = v[i0 + i];
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    cfg.gridDim = dim3(cs, nb);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cs;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    ctx->launches++;
-    VP_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, pk));
-  }
-  return VP_OK;
-}
-
 }  // namespace
 
 // --------------------------------------------------------------- QR

@@ -16,7 +16,6 @@ static inline int __clzll(long long x) { return __builtin_clzll((unsigned long l
 static inline float __shfl_xor_sync(unsigned, float v, int) { return v; }
 static inline int max(int a, int b) { return a > b ? a : b; }
 static inline int min(int a, int b) { return a < b ? a : b; }
-static inline float rsqrtf(float x) { return 1.0f / std::sqrt(x); }
 using std::ldexp;
 #include "dw.cuh"
 
