@@ -40,9 +40,9 @@ DTYPE = "f64 storage/contractions, df32 (~2^-48) factorisations"
 PROFILES = os.path.join(ROOT, "profiles")
 # the dominant kernel of each class on the headline path (streams = 0: the
 # batched kernels of a one-member lockstep group) and on the two-stream path
-KERNEL_OF_CLASS = {"qr_factor": "kb_qr_factor_cl", "jacobi": "kb_jacobi_dw", "gemm": "kb_gemm",
-                   "qr_formq": "kb_qr_formq_reg", "apply": "kb_site_sum", "select": "kb_select"}
-KERNEL_OF_CLASS_STREAMS = {k: v[1:] for k, v in KERNEL_OF_CLASS.items()}
+KERNEL_OF_CLASS = {"qr_factor": "kb_qr_cluster", "jacobi": "kb_jacobi_dw", "gemm": "kb_gemm_fma",
+                   "qr_formq": "kb_formq", "apply": "kb_site_sum", "select": "kb_select"}
+KERNEL_OF_CLASS_STREAMS = dict(KERNEL_OF_CLASS, apply="k_site_sum", select="k_select")
 
 
 def profile_traffic(kernel, workload):
