@@ -464,11 +464,11 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
   // V^T enters both cores: FP64 in every contraction mode
   const int prec = ctx->precision;
   ctx->precision = VP_PREC_FP64;
-  const int st = launch_gemm_bt(ctx, r, c, q, ctx->w_a.p, q, ctx->w_q1.p, q, Vt, c);
+  const int st = launch_gemm_bt(ctx, r, c, q, ctx->w_a.p, q, ctx->w_q1.p, q, Vt, c, OZ_ROWS);
   ctx->precision = prec;
   VP_TRY(st);
-  VP_TRY(launch_gemm_bt(ctx, m, r, c, s->core[k].p, c, Vt, c, ctx->w_b.p, r));  // U S = M V
-  VP_TRY(launch_gemm(ctx, pl, r, m, 1.0, s->core[k - 1].p, m, ctx->w_b.p, r, ctx->w_gemm.p, r));
+  VP_TRY(launch_gemm_bt(ctx, m, r, c, s->core[k].p, c, Vt, c, ctx->w_b.p, r, OZ_ROWS));  // U S = M V
+  VP_TRY(launch_gemm(ctx, pl, r, m, 1.0, s->core[k - 1].p, m, ctx->w_b.p, r, ctx->w_gemm.p, r, OZ_COLS));
   const double gem = 2.0 * r * c * q + 2.0 * m * r * c + 2.0 * pl * r * m;
   prof_end(ctx, VP_K_GEMM, gem, q, r, pl);
   std::swap(s->core[k], ctx->w_tmp2);
@@ -524,7 +524,7 @@ static int lq_site(vp_ctx* ctx, mps_t* s, int k) {
   VP_TRY(launch_to_colmajor(ctx, ctx->w_q1.p, m, p, ctx->w_tmp.p));  // Q^T, row-major (p x m)
   VP_TRY(reserve(ctx, ctx->w_gemm, (size_t)rows * p));
   prof_begin(ctx, VP_K_GEMM);
-  VP_TRY(launch_gemm_bt(ctx, rows, p, n, s->core[k - 1].p, n, ctx->w_r.p, n, ctx->w_gemm.p, p));
+  VP_TRY(launch_gemm_bt(ctx, rows, p, n, s->core[k - 1].p, n, ctx->w_r.p, n, ctx->w_gemm.p, p, OZ_COLS_B));
   prof_end(ctx, VP_K_GEMM, 2.0 * rows * p * n, rows, p, n);
   std::swap(s->core[k], ctx->w_tmp);
   std::swap(s->core[k - 1], ctx->w_gemm);

@@ -270,12 +270,21 @@ struct GemmPlan {
   int kslice;  // columns of K per slice
 };
 GemmPlan gemm_plan(const vp_ctx* ctx, int M, int N, int K);
+// How far an FP64 contraction may be off (ozgemm.cu says how each is kept; the FMA
+// kernel is within all of them):
+//   OZ_ELEMENT  every element within the bound of an FP64 sum, K 2^-53 (|A| |B|)_ij;
+//   OZ_ROWS     K 2^-55 max_k|A_ik| max_k|B_kj|: for a factor with orthonormal rows or
+//               columns, known to 1e-14 itself, or one formed column by column;
+//   OZ_COLS     K 2^-55 max_k(max_i|A_ik| |B_kj|): for an A whose columns are each known
+//               to 1e-14 of their largest entry (a QR's R), or a B whose rows are;
+//   OZ_COLS_B   the same with A's and B's parts exchanged.
+enum OzBound { OZ_ELEMENT = 0, OZ_ROWS, OZ_COLS, OZ_COLS_B };
 // C (M x N) = alpha * A (M x K) * B (K x N), all row-major with given leading dims.
 int launch_gemm(vp_ctx* ctx, int M, int N, int K, double alpha, const double* A, int lda,
-                const double* B, int ldb, double* C, int ldc);
+                const double* B, int ldb, double* C, int ldc, OzBound bound = OZ_ELEMENT);
 // C (M x N) = A (M x K) * Bt^T, Bt given row-major (N x K).
 int launch_gemm_bt(vp_ctx* ctx, int M, int N, int K, const double* A, int lda, const double* Bt, int ldbt,
-                   double* C, int ldc);
+                   double* C, int ldc, OzBound bound = OZ_ELEMENT);
 // Decreasing order of the column (by_cols) or row norms of a row-major m x c matrix
 // (row stride ld; lower: entries right of the diagonal count as zero).
 int launch_norm_order(vp_ctx* ctx, const double* M, int ld, int m, int c, int by_cols, int lower, int* piv);
@@ -311,11 +320,12 @@ struct OzGemm {
   DevBuf* wb;
   DevStatus* st;
   OzPlan plan;
+  OzBound bound;
 };
 int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);
 // The same on the FMA pipe (fgemm.cu; neither plan nor scratch are used).
 int blaunch_fma_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);
-// C = alpha * triu(A_colmajor) (M x K) * B: the R factor read in place.
+// C = triu(A_colmajor) (M x K) * B: the R factor read in place (OZ_COLS).
 int launch_gemm_r(vp_ctx* ctx, int M, int N, int K, const double* Acm, int lda, const double* B,
                   int ldb, double* C, int ldc);
 // One-sided Jacobi on the rows of X (b x b, row-major), starting from the upper
@@ -431,6 +441,7 @@ struct BGemm {
   const double* B; int ldb;
   double* C; int ldc;
   BScratch* s;
+  OzBound bound = OZ_ELEMENT;
 };
 struct BNormOrder { const double* M; int ld, m, c, by_cols, lower; int* piv; };
 struct BGather { QRSrc src; int m, n; double* A; };

@@ -447,7 +447,7 @@ int launch_qr_factor(vp_ctx* ctx, double* A, int m, int n, double* tau, double* 
       VP_TRY(reserve(ctx, ctx->w_wr, rest));
       const int prec = ctx->precision;  // R is part of the factorisation: FP64 in every mode
       ctx->precision = VP_PREC_FP64;
-      const int st = launch_gemm(ctx, n - m, m, m, 1.0, A + (size_t)m * m, m, ctx->w_wq.p, m, ctx->w_wr.p, m);
+      const int st = launch_gemm(ctx, n - m, m, m, 1.0, A + (size_t)m * m, m, ctx->w_wq.p, m, ctx->w_wr.p, m, OZ_ROWS);
       ctx->precision = prec;
       VP_TRY(st);
       return launch_copy(ctx, ctx->w_wr.p, A + (size_t)m * m, rest);
@@ -623,7 +623,7 @@ static TcOperand tc_b(const BRowMajor& b) { return {b.B, b.ldb, 1}; }
 static TcOperand tc_b(const BTransposed& b) { return {b.B, b.ldb, 0}; }
 
 static OzGemm oz_job(const TcOperand& a, const TcOperand& b, int M, int N, int K, double alpha, double* C, int ldc,
-                     size_t stride, DevBuf* wa, DevBuf* wb, DevStatus* st, const OzPlan& plan) {
+                     size_t stride, DevBuf* wa, DevBuf* wb, DevStatus* st, const OzPlan& plan, OzBound bound) {
   OzGemm g;
   g.a = a;
   g.b = b;
@@ -638,13 +638,14 @@ static OzGemm oz_job(const TcOperand& a, const TcOperand& b, int M, int N, int K
   g.wb = wb;
   g.st = st;
   g.plan = plan;
+  g.bound = bound;
   return g;
 }
 
 // One GEMM launch (split K per gemm_plan, then the fixed-order slice sum).
 template <class ALoad, class BLoad>
 static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a, BLoad b, double* C, int ldc,
-                         const char* what) {
+                         const char* what, OzBound bound) {
   if (M <= 0 || N <= 0) return VP_OK;
   if (ctx->precision >= VP_PREC_TF32 && K > 0) return launch_tc_gemm(ctx, M, N, K, alpha, tc_a(a), tc_b(b), C, ldc);
   if (ctx->precision == VP_PREC_FP64) {
@@ -654,7 +655,7 @@ static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a
     if (split) VP_TRY(reserve(ctx, ctx->w_split, stride * oz.slices));
     std::vector<OzGemm> job;
     job.push_back(oz_job(tc_a(a), tc_b(b), M, N, K, alpha, split ? ctx->w_split.p : C, split ? N : ldc,
-                         split ? stride : 0, &ctx->w_tca, &ctx->w_tcb, ctx->status, oz));
+                         split ? stride : 0, &ctx->w_tca, &ctx->w_tcb, ctx->status, oz, bound));
     if (!oz.use) return blaunch_fma_gemm(ctx, ctx->stream, job);
     VP_TRY(blaunch_oz_gemm(ctx, ctx->stream, job));
     if (!split) return VP_OK;
@@ -686,18 +687,18 @@ static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a
 }
 
 int launch_gemm(vp_ctx* ctx, int M, int N, int K, double alpha, const double* A, int lda, const double* B,
-                int ldb, double* C, int ldc) {
-  return gemm_dispatch(ctx, M, N, K, alpha, ARowMajor{A, lda}, BRowMajor{B, ldb}, C, ldc, "gemm");
+                int ldb, double* C, int ldc, OzBound bound) {
+  return gemm_dispatch(ctx, M, N, K, alpha, ARowMajor{A, lda}, BRowMajor{B, ldb}, C, ldc, "gemm", bound);
 }
 
 int launch_gemm_bt(vp_ctx* ctx, int M, int N, int K, const double* A, int lda, const double* Bt, int ldbt, double* C,
-                   int ldc) {
-  return gemm_dispatch(ctx, M, N, K, 1.0, ARowMajor{A, lda}, BTransposed{Bt, ldbt}, C, ldc, "gemm_bt");
+                   int ldc, OzBound bound) {
+  return gemm_dispatch(ctx, M, N, K, 1.0, ARowMajor{A, lda}, BTransposed{Bt, ldbt}, C, ldc, "gemm_bt", bound);
 }
 
 int launch_gemm_r(vp_ctx* ctx, int M, int N, int K, const double* Acm, int lda, const double* B, int ldb,
                   double* C, int ldc) {
-  return gemm_dispatch(ctx, M, N, K, 1.0, AUpperColMajor{Acm, lda}, BRowMajor{B, ldb}, C, ldc, "gemm_r");
+  return gemm_dispatch(ctx, M, N, K, 1.0, AUpperColMajor{Acm, lda}, BRowMajor{B, ldb}, C, ldc, "gemm_r", OZ_COLS);
 }
 
 // ------------------------------------------------------------ Jacobi SVD
@@ -1640,7 +1641,7 @@ int blaunch_qr_factor(vp_ctx* ctx, cudaStream_t st, const std::vector<BQR>& v) {
       VP_TRY(reserve(ctx, q.s->wr, rest));
       sq.push_back({q.A, m, m, q.tau, q.vbuf, q.s});
       fq.push_back({q.A, m, m, q.tau, q.s->wq.p, q.s});
-      gm.push_back({BG_AB, 0, q.n - m, m, m, 1.0, q.A + (size_t)m * m, m, q.s->wq.p, m, q.s->wr.p, m, q.s});
+      gm.push_back({BG_AB, 0, q.n - m, m, m, 1.0, q.A + (size_t)m * m, m, q.s->wq.p, m, q.s->wr.p, m, q.s, OZ_ROWS});
       cp.push_back({q.s->wr.p, q.A + (size_t)m * m, rest});
     }
     VP_TRY(blaunch_qr_factor(ctx, st, sq));
@@ -1766,7 +1767,8 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
     if (!g.fp32) {
       const TcOperand ta{g.A, g.lda, g.kind == BG_RB ? 2 : 0}, tb{g.B, g.ldb, g.kind == BG_ABT ? 0 : 1};
       (op.use ? oz : fma).push_back(oz_job(ta, tb, g.M, g.N, g.K, g.alpha, C, ldc, stride, g.s ? &g.s->oza[sl] : nullptr,
-                                           g.s ? &g.s->ozb[sl] : nullptr, g.s && g.s->st ? g.s->st : ctx->status, op));
+                                           g.s ? &g.s->ozb[sl] : nullptr, g.s && g.s->st ? g.s->st : ctx->status, op,
+                                           g.kind == BG_RB ? OZ_COLS : g.bound));
       continue;
     }
     if (g.kind == BG_AB)

@@ -14,22 +14,35 @@
 // exactly (2^24).  The digit products with i + j = l, l = 0..8 (43 of the 64)
 // accumulate into nine 128 x 48 accumulators of tensor memory, and the epilogue
 // adds the nine integers with their weights in 128-bit integer arithmetic and
-// rounds once to FP64.  What is dropped (l > 8) is below 2^-61 of the two
-// scales; the representation error of an element below 2^-56 of its scale.
-// Against 64-bit references the error is about a third of the FMA kernel's
-// (measured for K = 64..1008: 6-9e-17 of the norm, against 1.7-3.1e-16).
+// rounds once to FP64.  What is dropped (l > 8) is below 2^-60.4 of the two
+// scales per product; an element is held to 2^-56 of its scale, and exactly from
+// an eighth of the scale on.
 //
-// The scales only work on rows and columns, so a factor common to column k of A
-// and, inversely, to row k of B would cost digits: kb_oz_kexp balances the
-// largest magnitudes of the two by a power of two per k first (exact).
+// So a product is as accurate as its row's and column's largest elements make it,
+// where an FP64 sum is as accurate as the products that meet in it: a row (1e20, 1,
+// ..) against a column (0, 1, ..) loses every digit.  What the caller needs decides
+// (OzBound):
+//   OZ_ELEMENT  the kernel proves each element of each K slice or forms it again by FP64
+//     FMAs.  Of its products n are nonzero, none off by more than 2^-56 + 2^-60.4 of the
+//     scales' product; where (|A| |B|)_ij is W times that product, an FP64 sum may be off
+//     by n 2^-53 W, so the element passes from W = 2180 / 2^14 = 0.133 on.  W is summed
+//     from 7-bit magnitudes (of the first digits) that kb_oz_pack writes beside the digits
+//     (four products an instruction, by four warps that would wait while the products
+//     run): the first 64 k suffice where sizes are even (standard normal entries: W = 2
+//     there, 0.5 where one outlier each doubles both scales), else all of them are
+//     summed.  An element all of whose products are zero passes as well.
+//   OZ_ROWS     nothing to prove.
+//   OZ_COLS     kb_oz_kexp moves column k of A to one by a power of two, row k of B the
+//     other way (exact), so that columns of A of any size keep their digits.
+// Error against 64-bit references, largest over rows with standard normal entries:
+// 6-9e-17 of the norms for K = 64..1008, the FMA kernel's 1.7-3.1e-16.
 //
-// Passes: kb_oz_kexp (balance exponents), kb_oz_pack (digits, written as the
+// Passes: kb_oz_kexp (OZ_COLS only), kb_oz_pack (digits, written as the
 // 128-byte-swizzled shared-memory images of whole tiles, so that the loads are
 // plain bulk copies), kb_oz_mma (one CTA per 128 x 48 tile and K slice), and with
-// several K slices the fixed-order sum of the FP64 partial products that the FMA
-// kernel uses too.  A row or column that holds a NaN or Inf, or K-scaling that
-// leaves the exponent range, sends its tiles through plain FP64 FMAs inside
-// kb_oz_mma, so non-finite values propagate as they do there.
+// several K slices the fixed-order sum of the FP64 partial products.  The elements of
+// a row or column that holds a NaN or Inf, or that scaling takes out of the exponent
+// range, are FP64 FMAs as well, so non-finite values propagate as they do there.
 //
 // Measured (2048^3): 557 us in kb_oz_mma, 1.33 PFLOP/s of FP16 products, 71 % of
 // the measured 1.88 (the 9-accumulator epilogue is not overlapped: the tile's
@@ -58,13 +71,6 @@ constexpr int kOzPackRows = 32;
 constexpr uint32_t kOzTmem = 512;   // columns allocated (a power of two >= 9 x 48)
 constexpr size_t kOzSmem = 1024 + 2 * (size_t)kOzBBytes + (size_t)kOzAStages * kOzABytes + 256;
 
-// x as an operand element (row r of the operand, index k along the contraction)
-__device__ __forceinline__ double oz_elem(const TcOperand& o, int r, int k) {
-  if (o.kind == 0) return o.p[(size_t)r * o.ld + k];
-  if (o.kind == 1) return o.p[(size_t)k * o.ld + r];
-  return r <= k ? o.p[(size_t)k * o.ld + r] : 0.0;
-}
-
 __device__ __forceinline__ int oz_bexp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
 
 // Exponent of x after the balance shift (0 for a zero, 2047 for a non-finite
@@ -86,9 +92,12 @@ struct OzJob {
   double* C;
   int ldc;
   size_t stride;         // partial products: slice s at C + s * stride
-  int* kexp;             // per k: shift of A (B gets the opposite)
+  int* kexp;             // OZ_COLS: per k, shift of a (b gets the opposite), else NULL
+  int kside;             // the operand whose columns become one
   int* ea;               // slices x Mp exponents, then slices x Np
   int* eb;
+  uint8_t* ma;           // OZ_ELEMENT: per slice and row kslice bytes, |element| in 128ths of
+  uint8_t* mb;           // the scale, at most, + 128 where it is not zero; else NULL
   uint8_t* da;           // digit tiles
   uint8_t* db;
   DevStatus* st;
@@ -96,51 +105,48 @@ struct OzJob {
 
 namespace {
 
-// Shift of column k of A: half the difference of the two largest exponents.
-// One block of 32 warps takes eight k, so that every load of an operand of up
-// to a few hundred rows is in flight at once.
+// Shift of column k that brings its largest element to [1/2, 1).  One block of 32
+// warps takes eight k, so that every load of an operand of up to a few hundred rows
+// is in flight at once.
 constexpr int kOzThreads = 1024;
 __device__ __forceinline__ void oz_kexp_body(const OzJob& j, int kblk) {
-  __shared__ int sa[8], sb[8];
+  __shared__ int s[8];
   const int k0 = kblk * 8;
-  if (threadIdx.x < 8) sa[threadIdx.x] = sb[threadIdx.x] = 0;
+  if (threadIdx.x < 8) s[threadIdx.x] = 0;
   __syncthreads();
-#pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    const TcOperand& o = side ? j.b : j.a;
-    const int R = side ? j.N : j.M;
-    int* s = side ? sb : sa;
-    if (o.kind == 0) {  // k contiguous: eight k per row
-      const int kk = threadIdx.x & 7, k = k0 + kk;
-      int e = 0;
-      if (k < j.K)
+  const TcOperand& o = j.kside ? j.b : j.a;
+  const int R = j.kside ? j.N : j.M;
+  if (o.kind == 0) {  // k contiguous: eight k per row
+    const int kk = threadIdx.x & 7, k = k0 + kk;
+    int e = 0;
+    if (k < j.K)
 #pragma unroll 4
-        for (int r = threadIdx.x >> 3; r < R; r += kOzThreads / 8) e = max(e, oz_bexp(o.p[(size_t)r * o.ld + k]));
-      for (int off = 8; off < 32; off <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
-      if ((threadIdx.x & 31) < 8) atomicMax(&s[kk], e);
-    } else {  // rows contiguous: four warps per k
-      const int kk = threadIdx.x >> 7, k = k0 + kk;
-      int e = 0;
-      if (k < j.K) {
-        const int rend = o.kind == 2 ? min(R, k + 1) : R;
+      for (int r = threadIdx.x >> 3; r < R; r += kOzThreads / 8) e = max(e, oz_bexp(o.p[(size_t)r * o.ld + k]));
+    for (int off = 8; off < 32; off <<= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, off));
+    if ((threadIdx.x & 31) < 8) atomicMax(&s[kk], e);
+  } else {  // rows contiguous: four warps per k
+    const int kk = threadIdx.x >> 7, k = k0 + kk;
+    int e = 0;
+    if (k < j.K) {
+      const int rend = o.kind == 2 ? min(R, k + 1) : R;
 #pragma unroll 8
-        for (int r = threadIdx.x & 127; r < rend; r += 128) e = max(e, oz_bexp(o.p[(size_t)k * o.ld + r]));
-      }
-      e = __reduce_max_sync(0xffffffffu, e);
-      if ((threadIdx.x & 31) == 0) atomicMax(&s[kk], e);
+      for (int r = threadIdx.x & 127; r < rend; r += 128) e = max(e, oz_bexp(o.p[(size_t)k * o.ld + r]));
     }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if ((threadIdx.x & 31) == 0) atomicMax(&s[kk], e);
   }
   __syncthreads();
   if (threadIdx.x < 8 && k0 + threadIdx.x < j.K) {
-    const int a = sa[threadIdx.x], b = sb[threadIdx.x];
-    // a zero row or column (or one with a non-finite value) needs no balance
-    j.kexp[k0 + threadIdx.x] = (a == 0 || b == 0 || a == 2047 || b == 2047) ? 0 : (b - a) >> 1;
+    const int e = s[threadIdx.x], sh = e == 0 || e == 2047 ? 0 : 1022 - e;  // (zero or not finite: none)
+    j.kexp[k0 + threadIdx.x] = j.kside ? -sh : sh;
   }
 }
 
-// Eight consecutive k of one row: eight digits each, one 16-byte store per digit.
+// Eight consecutive k of one row: eight digits each, one 16-byte store per digit, and
+// (mag not NULL) eight bytes of magnitudes: with a first digit d, |x| is at least
+// (|d| - 64 / 127) / 64 of the scale, 2 |d| - 2 of its 128ths.
 __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int (&sh)[8], int emax, uint8_t* tile0,
-                                                size_t digit_stride, int row, int kchunk16) {
+                                                size_t digit_stride, int row, int kchunk16, uint8_t* mag) {
   constexpr long long kBias = 64ll * ((1ll << 49) - 1) / 127;  // 64 * sum_{j<7} 2^(7 j)
   long long X[8];
 #pragma unroll
@@ -154,6 +160,15 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
     else
       m = s <= 54 ? (m + (1ll << (s - 1))) >> s : 0ll;
     X[u] = (bits < 0 ? -m : m) + kBias;
+  }
+  if (mag) {
+    unsigned w[2] = {0, 0};
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int d = abs((int)(X[u] >> 49));
+      w[u / 4] |= ((__double_as_longlong(x[u]) << 1) != 0 ? 128u | (unsigned)max(2 * d - 2, 0) : 0u) << (8 * (u % 4));
+    }
+    *reinterpret_cast<uint2*>(mag) = make_uint2(w[0], w[1]);
   }
   uint8_t* dst = tile0 + row * 128 + ((kchunk16 ^ (row & 7)) << 4);
 #pragma unroll
@@ -236,11 +251,12 @@ __device__ __forceinline__ void oz_pack_body(const OzJob& j, int side, int rblk,
     const int k = kbeg + 8 * (g + 32 * h);
 #pragma unroll
     for (int u = 0; u < 8; ++u)
-      if (k + u < kend) e = max(e, oz_shifted_exp(x[h][u], sgn * j.kexp[k + u]));
+      if (k + u < kend) e = max(e, oz_shifted_exp(x[h][u], j.kexp ? sgn * j.kexp[k + u] : 0));
   }
   e = __reduce_max_sync(0xffffffffu, e);
   if (r >= Rp) return;
   if (g == 0) ex[(size_t)slice * Rp + r] = e;
+  uint8_t* mags = side ? j.mb : j.ma;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int k = kbeg + 8 * (g + 32 * h);
@@ -248,12 +264,12 @@ __device__ __forceinline__ void oz_pack_body(const OzJob& j, int side, int rblk,
     int sh[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      sh[u] = k + u < kend ? sgn * j.kexp[k + u] : 0;
+      sh[u] = j.kexp && k + u < kend ? sgn * j.kexp[k + u] : 0;
       if (e >= 2047) x[h][u] = 0.0;  // the row takes the FP64 path
     }
     oz_store_digits(x[h], sh, e,
                     out + ((size_t)(r / tile_rows) * j.chunks + k / kOzKc) * kOzS * dstride, dstride, r % tile_rows,
-                    (k % kOzKc) >> 3);
+                    (k % kOzKc) >> 3, mags ? mags + ((size_t)slice * Rp + r) * j.kslice + (k - kbeg) : nullptr);
   }
 }
 
@@ -301,8 +317,102 @@ __device__ __forceinline__ double oz_combine(const int (&S)[kOzL], int e2) {
 // stage, double-buffered; the A digits of a stage one by one into their
 // slots); warp 1: per A digit i the products with B digits 0 .. min(7, 8 - i),
 // neighbouring B digits joined into one instruction of up to 240 columns, whose
-// accumulators lie next to each other in tensor memory; then all eight warps
-// read the accumulators, combine and store.
+// accumulators lie next to each other in tensor memory; warps 2 to 5: which elements
+// are FP64 sums instead (oz_unproven); then all eight warps read the accumulators,
+// combine and store.
+// Columns of a tile (a bit each) whose element in the row with magnitudes at ma and
+// exponent er is to be formed again (see OZ_ELEMENT above); mb, eb: the tile's columns,
+// of which nc exist; kn of a slice's kslice magnitudes are there.
+__device__ __forceinline__ unsigned long long oz_unproven(const uint8_t* ma, int er, const uint8_t* mb, const int* eb,
+                                                          int nc, int kslice, int kn) {
+  constexpr int kChunks = kOzMaxK / 64;
+  constexpr unsigned kEnough = 2180, kMag = 0x7f7f7f7fu, kAny = 0x80808080u;
+  unsigned long long bad = 0;
+#pragma unroll 8
+  for (int c = 0; c < kOzN; ++c) bad |= (unsigned long long)(er >= 2047 || eb[c] >= 2047) << c;
+  if (!ma) return bad;
+  const int words = kn / 16;
+  uint4 mine[4 * kChunks];
+  unsigned some = 0;
+#pragma unroll
+  for (int w = 0; w < 4 * kChunks; ++w) {
+    mine[w] = w < words ? reinterpret_cast<const uint4*>(ma)[w] : make_uint4(0, 0, 0, 0);
+    some |= mine[w].x | mine[w].y | mine[w].z | mine[w].w;
+  }
+  // four sums, so that an instruction need not wait for the one before
+  auto add = [&](const uint4& a, const uint4& b, uint4& sum, unsigned& any) {
+    sum.x = __dp4a(a.x & kMag, b.x & kMag, sum.x);
+    sum.y = __dp4a(a.y & kMag, b.y & kMag, sum.y);
+    sum.z = __dp4a(a.z & kMag, b.z & kMag, sum.z);
+    sum.w = __dp4a(a.w & kMag, b.w & kMag, sum.w);
+    any |= (a.x & b.x) | (a.y & b.y) | (a.z & b.z) | (a.w & b.w);
+  };
+  auto little = [&](const uint4& sum) { return sum.x + sum.y + sum.z + sum.w < kEnough; };
+  unsigned long long open = 0;
+#pragma unroll 4
+  for (int c = 0; c < kOzN; ++c) {
+    const uint4* m = reinterpret_cast<const uint4*>(mb + (size_t)c * kslice);
+    uint4 sum = make_uint4(0, 0, 0, 0);
+    unsigned any = 0;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) add(mine[w], m[w], sum, any);
+    open |= (unsigned long long)little(sum) << c;
+  }
+  open &= some == 0 ? 0ull : ~bad & ((1ull << nc) - 1);
+  unsigned long long cols = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)open) |
+                            (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(open >> 32)) << 32;
+  for (; cols; cols &= cols - 1) {
+    const int c = __ffsll((long long)cols) - 1;
+    const uint4* m = reinterpret_cast<const uint4*>(mb + (size_t)c * kslice);
+    uint4 sum = make_uint4(0, 0, 0, 0);
+    unsigned any = 0;
+#pragma unroll
+    for (int w = 0; w < 4 * kChunks; ++w)
+      if (w < words) add(mine[w], m[w], sum, any);
+    bad |= (unsigned long long)(little(sum) && (any & kAny) != 0 && (open >> c & 1)) << c;
+  }
+  return bad;
+}
+
+// Where an operand's row r lies: element k at p[k * step], zero for k < first.
+struct OzRow {
+  const double* p;
+  size_t step;
+  int first;
+};
+__device__ __forceinline__ OzRow oz_row(const TcOperand& o, int r) {
+  if (o.kind == 0) return {o.p + (size_t)r * o.ld, 1, 0};
+  return {o.p + r, (size_t)o.ld, o.kind == 2 ? r : 0};
+}
+// FP64 sums over k in [kb, ke) of one row with columns [col, col + 8) (rows and columns
+// beyond the operands: any value).
+__device__ __forceinline__ void oz_plain(const OzJob& j, int row, int col, int kb, int ke, double (&t)[8]) {
+  const OzRow a = oz_row(j.a, min(row, j.M - 1));
+  OzRow b[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    b[u] = oz_row(j.b, min(col + u, j.N - 1));
+    t[u] = 0.0;
+  }
+#pragma unroll 4
+  for (int k = kb; k < ke; ++k) {
+    const double x = k < a.first ? 0.0 : a.p[k * a.step];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = fma(x, k < b[u].first ? 0.0 : b[u].p[k * b[u].step], t[u]);
+  }
+}
+// One such sum by a warp.
+__device__ __forceinline__ double oz_plain_warp(const OzJob& j, int row, int col, int kb, int ke, int lane) {
+  const OzRow a = oz_row(j.a, row), b = oz_row(j.b, col);
+  double t = 0.0;
+#pragma unroll 4
+  for (int k = kb + lane; k < ke; k += 32)
+    t = fma(k < a.first ? 0.0 : a.p[k * a.step], k < b.first ? 0.0 : b.p[k * b.step], t);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  return t;
+}
+
 __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int slice) {
   extern __shared__ uint8_t oz_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
@@ -314,7 +424,8 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
   uint64_t* emptyB = fullB + 2;
   uint64_t* done = emptyB + 2;
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(done + 1);
-  __shared__ int s_abort, s_plain;
+  __shared__ int s_abort;
+  __shared__ unsigned long long s_bad[kOzM];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = mt * kOzM, n0 = nt * kOzN;
   const int Mp = (j.M + kOzM - 1) / kOzM * kOzM, Np = (j.N + kOzN - 1) / kOzN * kOzN;
@@ -331,24 +442,13 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
     if (i < j.M && col < j.N) C[j.swapped ? (size_t)col * j.ldc + i : (size_t)i * j.ldc + col] = v;
   };
 
-  if (tid == 0) s_abort = s_plain = 0;
-  __syncthreads();
-  if ((tid < kOzM && ea[tid] >= 2047) || (tid < kOzN && eb[tid] >= 2047)) s_plain = 1;
-  __syncthreads();
-  if (s_plain || c0 >= c1) {
-    // non-finite operands (or a K range of exact zeros): plain FP64
-    const int kb = max(slice * j.kslice, c0 * kOzKc), ke = min(j.K, c1 * kOzKc);
-    for (int e = tid; e < kOzM * kOzN; e += 256) {
-      const int i = m0 + (j.swapped ? e % kOzM : e / kOzN), col = n0 + (j.swapped ? e / kOzM : e % kOzN);
-      if (i >= j.M || col >= j.N) continue;
-      double acc = 0.0;
-      for (int k = kb; k < ke; ++k) acc = fma(oz_elem(j.a, i, k), oz_elem(j.b, col, k), acc);
-      store(i, col, j.alpha * acc);
-    }
+  if (c0 >= c1) {  // a K range of exact zeros
+    for (int e = tid; e < kOzM * kOzN; e += 256) store(m0 + e / kOzN, n0 + e % kOzN, 0.0);
     return;
   }
 
   if (tid == 0) {
+    s_abort = 0;
     for (int s = 0; s < kOzAStages; ++s) {
       mbar_init(&fullA[s], 1);
       mbar_init(&emptyA[s], 1);
@@ -440,6 +540,12 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
       if (ok) tc_commit(&emptyB[sb]);
     }
     tc_commit(done);
+  } else if (warp >= 2 && warp < 6) {
+    const int row = tid - 64;
+    const size_t rec = (size_t)j.kslice, ra = (size_t)slice * Mp + m0 + row, rb = (size_t)slice * Np + n0;
+    s_bad[row] = j.ma ? oz_unproven(j.ma + ra * rec, ea[row], j.mb + rb * rec, eb, min(kOzN, j.N - n0), j.kslice,
+                                    min(j.kslice, j.chunks * kOzKc - slice * j.kslice))
+                      : oz_unproven(nullptr, ea[row], nullptr, eb, 0, 0, 0);
   }
   if (!ok) atomicExch(&s_abort, 1);
   __syncwarp();
@@ -451,7 +557,8 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
   if (good) {
     // warp w reads lanes 32 (w mod 4) .., the column groups of 8 with (w / 4)
     const int row = (warp & 3) * 32 + lane;
-    const int er = ea[row];
+    const int er = ea[row], kb = c0 * kOzKc, ke = min(j.K, c1 * kOzKc);
+    const unsigned long long bad = s_bad[row];
 #pragma unroll 1
     for (int g = warp >> 2; g < kOzN / 8; g += 2) {
       uint32_t r[kOzL][8];
@@ -468,7 +575,30 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
         // digit products carry 2^(7 (14 - l)); scales 2^(er - 1022 - 55), 2^(ec - 1022 - 55)
         double v = oz_combine(S, er + eb[col] - 2 * 1077 + 42);
         if (j.alpha != 1.0) v *= j.alpha;
-        store(m0 + row, n0 + col, v);
+        if (!(bad >> col & 1)) store(m0 + row, n0 + col, v);
+      }
+      // the elements that were not proven: few one by one, more as the whole group of
+      // 32 x 8 (the FP64 pipe takes 16 clocks a warp's FMA: at K = 512 the group's 8 per k
+      // cost as much as some 16 elements one by one)
+      const int i0 = m0 + (warp & 3) * 32;
+      const unsigned mine =
+          m0 + row < j.M ? (unsigned)(bad >> (8 * g)) & 255u & ((1u << min(8, max(0, j.N - n0 - 8 * g))) - 1) : 0u;
+      unsigned rows = __ballot_sync(0xffffffffu, mine != 0);
+      if (__reduce_add_sync(0xffffffffu, __popc(mine)) > 16) {
+        double t[8];
+        oz_plain(j, m0 + row, n0 + 8 * g, kb, ke, t);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (mine >> u & 1) store(m0 + row, n0 + 8 * g + u, j.alpha * t[u]);
+        rows = 0;
+      }
+      for (; rows; rows &= rows - 1) {
+        const int l = __ffs(rows) - 1;
+        for (unsigned us = __shfl_sync(0xffffffffu, mine, l); us; us &= us - 1) {
+          const int u = __ffs(us) - 1;
+          const double t = oz_plain_warp(j, i0 + l, n0 + 8 * g + u, kb, ke, lane);
+          if (lane == 0) store(i0 + l, n0 + 8 * g + u, j.alpha * t);
+        }
       }
     }
   }
@@ -482,7 +612,7 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
 __global__ void __launch_bounds__(kOzThreads) kb_oz_kexp(const __grid_constant__ Pack<OzJob> pk) {
   follow();
   const OzJob& j = pk.a[blockIdx.y];
-  if ((int)blockIdx.x * 8 >= j.K) return;
+  if (!j.kexp || (int)blockIdx.x * 8 >= j.K) return;
   oz_kexp_body(j, blockIdx.x);
 }
 // x: 32-row blocks of A, then of B (ablk of A at most); y: K slice; z: job
@@ -544,6 +674,7 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
     const int nb = (int)std::min<size_t>(kMaxBatch, v.size() - i0);
     Pack<OzJob> pk{};
     int ks = 1, ablk = 1, bblk = 1, zs = 1, gx = 1, gy = 1, ksl = kOzKc;
+    bool shifts = false;
     for (int i = 0; i < nb; ++i) {
       const OzGemm& g = v[i0 + i];
       OzJob& j = pk.a[i];
@@ -564,16 +695,24 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       const size_t Mp = (size_t)(j.M + kOzM - 1) / kOzM * kOzM, Np = (size_t)(j.N + kOzN - 1) / kOzN * kOzN;
       const size_t abytes = Mp / kOzM * j.chunks * kOzS * kOzABytes, bbytes = Np / kOzN * j.chunks * (size_t)kOzBBytes;
       const size_t ints = (size_t)j.K + (size_t)j.slices * (Mp + Np);
-      VP_TRY(reserve(ctx, *g.wa, abytes / 8 + ints / 2 + 64));
+      // magnitudes of OZ_ELEMENT, on 16-byte boundaries behind the digits
+      const size_t rec = g.bound == OZ_ELEMENT ? (size_t)j.kslice : 0, mbytes = j.slices * (Mp + Np) * rec;
+      VP_TRY(reserve(ctx, *g.wa, abytes / 8 + mbytes / 8 + ints / 2 + 64));
       VP_TRY(reserve(ctx, *g.wb, bbytes / 8 + 64));
       // bulk copies start on 16-byte boundaries, whatever the allocator's alignment
       auto aligned = [](double* p) { return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 127) & ~uintptr_t(127)); };
       j.da = aligned(g.wa->p);
       j.db = aligned(g.wb->p);
-      j.kexp = reinterpret_cast<int*>(j.da + abytes);
-      j.ea = j.kexp + j.K;
+      j.ma = rec ? j.da + abytes : nullptr;
+      j.mb = rec ? j.ma + j.slices * Mp * rec : nullptr;
+      j.ea = reinterpret_cast<int*>(j.da + abytes + mbytes);
       j.eb = j.ea + (size_t)j.slices * Mp;
-      ks = std::max(ks, (j.K + 7) / 8);
+      if (g.bound == OZ_COLS || g.bound == OZ_COLS_B) {
+        j.kexp = j.eb + (size_t)j.slices * Np;
+        j.kside = (g.bound == OZ_COLS_B) != (j.swapped != 0);
+        ks = std::max(ks, (j.K + 7) / 8);
+        shifts = true;
+      }
       ablk = std::max(ablk, (int)((Mp + kOzPackRows - 1) / kOzPackRows));
       bblk = std::max(bblk, (int)((Np + kOzPackRows - 1) / kOzPackRows));
       zs = std::max(zs, j.slices);
@@ -582,7 +721,8 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       gy = std::max(gy, (int)(Np / kOzN));
     }
     if (gy > 65535 || (long long)nb * zs > 65535) return fail(ctx, VP_ECAPACITY, "gemm: too large");
-    VP_TRY(launch_after(ctx, "oz_kexp", kb_oz_kexp, dim3(ks, nb), dim3(kOzThreads), 0, st, kNoCluster, pk));
+    if (shifts)
+      VP_TRY(launch_after(ctx, "oz_kexp", kb_oz_kexp, dim3(ks, nb), dim3(kOzThreads), 0, st, kNoCluster, pk));
     VP_TRY(launch_after(ctx, "oz_pack", kb_oz_pack, dim3(ablk + bblk, zs, nb), dim3(kOzThreads), oz_pack_smem(ksl),
                         st, kNoCluster,
                         pk, ablk));
