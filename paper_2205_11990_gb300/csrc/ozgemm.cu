@@ -9,12 +9,12 @@
 // number of 56 bits relative to a power of two above its row's (A) or column's
 // (B) largest magnitude within a K slice, cut into eight signed 7-bit digits,
 //   a = 2^(e - 55) sum_i d_i 2^(7 (7 - i)),  -64 <= d_i <= 64,
-// which are exact FP16 integers.  Products of digits are at most 2^12, so the
+// which are exact FP16 integers; -a has the digits -d_i.  Products of digits are at most 2^12, so the
 // FP32 accumulator holds the sum of up to eight digit products over K <= 512
 // exactly (2^24).  The digit products with i + j = l, l = 0..8 (43 of the 64)
 // accumulate into nine 128 x 48 accumulators of tensor memory, and the epilogue
-// adds the nine integers with their weights in 128-bit integer arithmetic and
-// rounds once to FP64.  What is dropped (l > 8) is below 2^-60.4 of the two
+// adds the nine integers with their weights exactly and rounds once to FP64, to
+// nearest.  What is dropped (l > 8) is below 2^-60.4 of the two
 // scales per product; an element is held to 2^-56 of its scale, and exactly from
 // an eighth of the scale on.
 //
@@ -159,7 +159,7 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
       m <<= -s;  // s >= -2: no element exceeds the row's largest
     else
       m = s <= 54 ? (m + (1ll << (s - 1))) >> s : 0ll;
-    X[u] = (bits < 0 ? -m : m) + kBias;
+    X[u] = m + kBias;  // digits of the magnitude; the signs come last
   }
   if (mag) {
     unsigned w[2] = {0, 0};
@@ -171,6 +171,10 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
     *reinterpret_cast<uint2*>(mag) = make_uint2(w[0], w[1]);
   }
   uint8_t* dst = tile0 + row * 128 + ((kchunk16 ^ (row & 7)) << 4);
+  uint32_t sign[4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h)
+    sign[h] = ((uint32_t)__double2hiint(x[2 * h]) >> 16 & 0x8000u) | ((uint32_t)__double2hiint(x[2 * h + 1]) & 0x80000000u);
 #pragma unroll
   for (int i = 0; i < kOzS; ++i) {
     uint32_t w[4];
@@ -187,7 +191,7 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
       }
       const uint32_t raw = 0x64006400u | lo | (hi << 16);
       const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&raw), __float2half2_rn(1088.0f));
-      w[h] = *reinterpret_cast<const uint32_t*>(&d);
+      w[h] = *reinterpret_cast<const uint32_t*>(&d) ^ sign[h];
     }
     *reinterpret_cast<uint4*>(dst + i * digit_stride) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -286,17 +290,20 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "r"(taddr));
 }
 
-// sum_l S_l 2^(7 (8 - l)), |S_l| <= 2^24 exact integers, times 2^e2 as FP64: the
-// sum in two 64-bit integers, its 63 leading positions (what lies below is under
-// the dropped digit products) rounded once.  Integer arithmetic
-// throughout, since the FP64 pipe takes two operations per SM and clock.
+// sum_l S_l 2^(7 (8 - l)), |S_l| <= 2^24 exact integers, times 2^e2 as FP64, rounded
+// once, to nearest: the sum in two 64-bit integers, of which 62 or more leading
+// positions and a bit for all that lies below them (a plain shift would round every sum
+// of 4 and more full-scale products down: up to an ulp, half of one on average) meet in
+// T.  Integer arithmetic throughout, since the FP64 pipe takes two operations per SM
+// and clock.
 __device__ __forceinline__ double oz_combine(const int (&S)[kOzL], int e2) {
   const long long H = ((long long)S[0] << 21) + ((long long)S[1] << 14) + ((long long)S[2] << 7) + S[3];  // times 2^35
   const long long L = ((long long)S[4] << 28) + ((long long)S[5] << 21) + ((long long)S[6] << 14) +
                       ((long long)S[7] << 7) + S[8];
-  // one product of two full-scale elements is 2^68, K <= 512 of them 2^77; |L| < 2^52.1
-  const int sh = (unsigned long long)(H + (1ll << 35)) >> 36 ? 18 : 8;
-  const long long T = (H << (35 - sh)) + (L >> sh);  // |T| < 2^63
+  // one product of two full-scale elements is 2^68, K <= 512 of them 2^77 (|H| < 2^42.1);
+  // |L| < 2^52.1: below 2^27 H leaves room for all of L
+  const int sh = max(0, 64 - __clzll(H < 0 ? -H : H) - 27);
+  const long long T = ((H << (35 - sh)) + (L >> sh)) | ((L & ((1ll << sh) - 1)) != 0);  // |T| < 2^63
   const unsigned long long a = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
   if (a == 0) return 0.0;
   const int lz = __clzll((long long)a);
