@@ -305,23 +305,36 @@ struct OzPlan {
   int use;
   int swapped;  // tiles of C^T
   int slices, kslice;
+  int ranks;    // CTAs that share the slices of a tile
 };
 OzPlan oz_plan(const vp_ctx* ctx, int M, int N, int K);
-// One such contraction: C (M x N, or the partial products of each K slice at
-// C + s * stride) = alpha * A B^T in FP64; wa, wb: scratch of the digits.
+// One such contraction: C (M x N) = alpha * A B^T in FP64; wa, wb: scratch of the
+// digits (at most kOzBand bytes each; products with more go band by band), wsum of the
+// sums that the CTAs of a tile leave, stride apart.
 struct OzGemm {
   TcOperand a, b;
   int M, N, K;
   double alpha;
   double* C;
   int ldc;
-  size_t stride;
   DevBuf* wa;
   DevBuf* wb;
+  DevBuf* wsum;
+  size_t stride;
   DevStatus* st;
   OzPlan plan;
   OzBound bound;
 };
+// C (M x N) = the sum of `slices` matrices at P, stride apart, in ascending order.
+struct OzSum {
+  const double* P;
+  int M, N, slices;
+  size_t stride;
+  double* C;
+  int ldc;
+};
+int blaunch_sum_slices(vp_ctx* ctx, cudaStream_t st, const std::vector<OzSum>& v);
+// (Products whose scratch cannot be had: on the FMA pipe.)
 int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);
 // The same on the FMA pipe (fgemm.cu; neither plan nor scratch are used).
 int blaunch_fma_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v);

@@ -623,7 +623,7 @@ static TcOperand tc_b(const BRowMajor& b) { return {b.B, b.ldb, 1}; }
 static TcOperand tc_b(const BTransposed& b) { return {b.B, b.ldb, 0}; }
 
 static OzGemm oz_job(const TcOperand& a, const TcOperand& b, int M, int N, int K, double alpha, double* C, int ldc,
-                     size_t stride, DevBuf* wa, DevBuf* wb, DevStatus* st, const OzPlan& plan, OzBound bound) {
+                     DevBuf* wa, DevBuf* wb, DevBuf* wsum, DevStatus* st, const OzPlan& plan, OzBound bound) {
   OzGemm g;
   g.a = a;
   g.b = b;
@@ -633,16 +633,18 @@ static OzGemm oz_job(const TcOperand& a, const TcOperand& b, int M, int N, int K
   g.alpha = alpha;
   g.C = C;
   g.ldc = ldc;
-  g.stride = stride;
   g.wa = wa;
   g.wb = wb;
+  g.wsum = wsum;
+  g.stride = 0;
   g.st = st;
   g.plan = plan;
   g.bound = bound;
   return g;
 }
 
-// One GEMM launch (split K per gemm_plan, then the fixed-order slice sum).
+// One GEMM: FP64 by oz_plan and fma_plan; FP32 split over K per gemm_plan, then the
+// fixed-order slice sum.
 template <class ALoad, class BLoad>
 static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a, BLoad b, double* C, int ldc,
                          const char* what, OzBound bound) {
@@ -650,18 +652,9 @@ static int gemm_dispatch(vp_ctx* ctx, int M, int N, int K, double alpha, ALoad a
   if (ctx->precision >= VP_PREC_TF32 && K > 0) return launch_tc_gemm(ctx, M, N, K, alpha, tc_a(a), tc_b(b), C, ldc);
   if (ctx->precision == VP_PREC_FP64) {
     const OzPlan oz = oz_plan(ctx, M, N, K);
-    const size_t stride = (size_t)M * N;
-    const bool split = oz.use && oz.slices > 1;
-    if (split) VP_TRY(reserve(ctx, ctx->w_split, stride * oz.slices));
-    std::vector<OzGemm> job;
-    job.push_back(oz_job(tc_a(a), tc_b(b), M, N, K, alpha, split ? ctx->w_split.p : C, split ? N : ldc,
-                         split ? stride : 0, &ctx->w_tca, &ctx->w_tcb, ctx->status, oz, bound));
-    if (!oz.use) return blaunch_fma_gemm(ctx, ctx->stream, job);
-    VP_TRY(blaunch_oz_gemm(ctx, ctx->stream, job));
-    if (!split) return VP_OK;
-    const int blocks = (int)std::min<size_t>((stride + 255) / 256, (size_t)ctx->num_sms * 8);
-    return launch_after(ctx, what, k_sum_slices, dim3(blocks), dim3(256), 0, ctx->stream, kNoCluster,
-                        ctx->w_split.p, M, N, oz.slices, stride, C, ldc);
+    const std::vector<OzGemm> job{
+        oz_job(tc_a(a), tc_b(b), M, N, K, alpha, C, ldc, &ctx->w_tca, &ctx->w_tcb, &ctx->w_split, ctx->status, oz, bound)};
+    return oz.use ? blaunch_oz_gemm(ctx, ctx->stream, job) : blaunch_fma_gemm(ctx, ctx->stream, job);
   }
   const GemmPlan pl = gemm_plan(ctx, M, N, K);
   dim3 grid((M + pl.tile - 1) / pl.tile, (N + pl.tile - 1) / pl.tile, 1);
@@ -1703,16 +1696,9 @@ __global__ void __launch_bounds__(256) kb_gemm(const __grid_constant__ Pack<Gemm
   gemm_body<ALoad, BLoad, TILE>(j.M, j.N, j.K, j.alpha, j.a, j.b, j.C, j.ldc, j.kslice, j.stride, blockIdx.x,
                                    blockIdx.y, slice);
 }
-struct SumArgs {
-  const double* P;
-  int M, N, slices;
-  size_t stride;
-  double* C;
-  int ldc;
-};
-__global__ void kb_sum_slices(const __grid_constant__ Pack<SumArgs> pk) {
+__global__ void kb_sum_slices(const __grid_constant__ Pack<OzSum> pk) {
   follow();
-  const SumArgs& a = pk.a[blockIdx.y];
+  const OzSum& a = pk.a[blockIdx.y];
   k_sum_slices_body(a.P, a.M, a.N, a.slices, a.stride, a.C, a.ldc);
 }
 
@@ -1744,14 +1730,14 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
   std::vector<GemmJob<ARowMajor, BRowMajor>> ab[2];
   std::vector<GemmJob<ARowMajor, BTransposed>> abt[2];
   std::vector<GemmJob<AUpperColMajor, BRowMajor>> rb[2];
-  std::vector<SumArgs> sums;
+  std::vector<OzSum> sums;
   std::vector<OzGemm> oz, fma;
   SlotCounter slots;
   for (const BGemm& g : v) {
     if (g.M <= 0 || g.N <= 0) continue;
     const GemmPlan pl = gemm_plan(ctx, g.M, g.N, g.K);
     const OzPlan op = g.fp32 ? OzPlan{} : oz_plan(ctx, g.M, g.N, g.K);
-    const int slices = g.fp32 ? pl.slices : op.use ? op.slices : 1, kslice = pl.kslice, ti = pl.tile == 64 ? 0 : 1;
+    const int slices = g.fp32 ? pl.slices : 1, kslice = pl.kslice, ti = pl.tile == 64 ? 0 : 1;
     double* C = g.C;
     int ldc = g.ldc;
     size_t stride = 0;
@@ -1766,8 +1752,8 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
     }
     if (!g.fp32) {
       const TcOperand ta{g.A, g.lda, g.kind == BG_RB ? 2 : 0}, tb{g.B, g.ldb, g.kind == BG_ABT ? 0 : 1};
-      (op.use ? oz : fma).push_back(oz_job(ta, tb, g.M, g.N, g.K, g.alpha, C, ldc, stride, g.s ? &g.s->oza[sl] : nullptr,
-                                           g.s ? &g.s->ozb[sl] : nullptr, g.s && g.s->st ? g.s->st : ctx->status, op,
+      (op.use ? oz : fma).push_back(oz_job(ta, tb, g.M, g.N, g.K, g.alpha, C, ldc, g.s ? &g.s->oza[sl] : nullptr,
+                                           g.s ? &g.s->ozb[sl] : nullptr, g.s ? &g.s->split[sl] : nullptr, g.s && g.s->st ? g.s->st : ctx->status, op,
                                            g.kind == BG_RB ? OZ_COLS : g.bound));
       continue;
     }
@@ -1789,8 +1775,12 @@ int blaunch_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<BGemm>& v) {
   VP_TRY((gemm_group<ARowMajor, BTransposed, 32>(ctx, st, abt[1])));
   VP_TRY((gemm_group<AUpperColMajor, BRowMajor, 64>(ctx, st, rb[0])));
   VP_TRY((gemm_group<AUpperColMajor, BRowMajor, 32>(ctx, st, rb[1])));
-  return run_packs(ctx, st, sums, kb_sum_slices, 256, 0,
-                   [&](const SumArgs& a) { return grid_stride_blocks(ctx, a.stride, 8); }, "b_sum_slices");
+  return blaunch_sum_slices(ctx, st, sums);
+}
+
+int blaunch_sum_slices(vp_ctx* ctx, cudaStream_t st, const std::vector<OzSum>& v) {
+  return run_packs(ctx, st, v, kb_sum_slices, 256, 0, [&](const OzSum& a) { return grid_stride_blocks(ctx, a.stride, 8); },
+                   "b_sum_slices");
 }
 
 // --------------------------------------------------------------- SVD site helpers

@@ -28,8 +28,8 @@
 //     by n 2^-53 W, so the element passes from W = 2180 / 2^14 = 0.133 on.  W is summed
 //     from 7-bit magnitudes (of the first digits) that kb_oz_pack writes beside the digits
 //     (four products an instruction, by four warps that would wait while the products
-//     run): the first 64 k suffice where sizes are even (standard normal entries: W = 2
-//     there, 0.5 where one outlier each doubles both scales), else all of them are
+//     run): the first 32 k suffice where sizes are even (standard normal entries: W = 1.2
+//     there, 0.3 where one outlier each doubles both scales), else all of them are
 //     summed.  An element all of whose products are zero passes as well.
 //   OZ_ROWS     nothing to prove.
 //   OZ_COLS     kb_oz_kexp moves column k of A to one by a power of two, row k of B the
@@ -39,8 +39,11 @@
 //
 // Passes: kb_oz_kexp (OZ_COLS only), kb_oz_pack (digits, written as the
 // 128-byte-swizzled shared-memory images of whole tiles, so that the loads are
-// plain bulk copies), kb_oz_mma (one CTA per 128 x 48 tile and K slice), and with
-// several K slices the fixed-order sum of the FP64 partial products.  The elements of
+// plain bulk copies), kb_oz_mma (a CTA per 128 x 48 tile and K slice; from kOzSums bytes
+// of products on the slices that one CTA takes after the other, each adding to the sum in
+// memory), and with several CTAs a tile kb_sum_slices, which adds what they leave in a
+// fixed order.  The digits take 16 bytes an element; what needs more than kOzBand of them
+// an operand goes band by band through the same memory.  The elements of
 // a row or column that holds a NaN or Inf, or that scaling takes out of the exponent
 // range, are FP64 FMAs as well, so non-finite values propagate as they do there.
 //
@@ -69,6 +72,8 @@ constexpr int kOzAStages = kOzS;  // one slot per digit of a stage
 constexpr int kOzMaxK = 512;        // K whose digit products one accumulator holds exactly
 constexpr int kOzPackRows = 32;
 constexpr uint32_t kOzTmem = 512;   // columns allocated (a power of two >= 9 x 48)
+constexpr size_t kOzBand = size_t(1) << 30;  // bytes of an operand's digits at a time
+constexpr size_t kOzSums = size_t(256) << 20;  // bytes that the CTAs of all tiles leave to be added
 constexpr size_t kOzSmem = 1024 + 2 * (size_t)kOzBBytes + (size_t)kOzAStages * kOzABytes + 256;
 
 __device__ __forceinline__ int oz_bexp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
@@ -86,12 +91,12 @@ __device__ __forceinline__ int oz_shifted_exp(double x, int sh) {
 
 struct OzJob {
   TcOperand a, b;        // a: M rows (tile rows), b: N rows (tile columns), both along K
-  int M, N, K, kslice, slices, chunks;  // chunks: 64-wide K stages
+  int M, N, K, kslice, slices, ranks, chunks;  // chunks: 64-wide K stages
   int swapped;           // the tile is C^T: element (i, j) goes to C[j * ldc + i]
   double alpha;
   double* C;
   int ldc;
-  size_t stride;         // partial products: slice s at C + s * stride
+  size_t stride;         // several ranks: rank s leaves its sums at C + s * stride
   int* kexp;             // OZ_COLS: per k, shift of a (b gets the opposite), else NULL
   int kside;             // the operand whose columns become one
   int* ea;               // slices x Mp exponents, then slices x Np
@@ -148,7 +153,7 @@ __device__ __forceinline__ void oz_kexp_body(const OzJob& j, int kblk) {
 __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int (&sh)[8], int emax, uint8_t* tile0,
                                                 size_t digit_stride, int row, int kchunk16, uint8_t* mag) {
   constexpr long long kBias = 64ll * ((1ll << 49) - 1) / 127;  // 64 * sum_{j<7} 2^(7 j)
-  long long X[8];
+  unsigned long long X[8];  // bit 63: negative, bit 62: not zero
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const long long bits = __double_as_longlong(x[u]);
@@ -159,22 +164,19 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
       m <<= -s;  // s >= -2: no element exceeds the row's largest
     else
       m = s <= 54 ? (m + (1ll << (s - 1))) >> s : 0ll;
-    X[u] = m + kBias;  // digits of the magnitude; the signs come last
+    // (digits of the magnitude; the signs come last)
+    X[u] = (unsigned long long)(m + kBias) | ((unsigned long long)bits & (1ull << 63)) | ((bits << 1) != 0 ? 1ull << 62 : 0ull);
   }
   if (mag) {
     unsigned w[2] = {0, 0};
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int d = abs((int)(X[u] >> 49));
-      w[u / 4] |= ((__double_as_longlong(x[u]) << 1) != 0 ? 128u | (unsigned)max(2 * d - 2, 0) : 0u) << (8 * (u % 4));
+      const unsigned hi = (unsigned)(X[u] >> 32), d = hi >> 17 & 127u;  // 64 at most
+      w[u / 4] |= ((hi >> 23 & 128u) | (d > 1 ? 2 * d - 2 : 0u)) << (8 * (u % 4));
     }
     *reinterpret_cast<uint2*>(mag) = make_uint2(w[0], w[1]);
   }
   uint8_t* dst = tile0 + row * 128 + ((kchunk16 ^ (row & 7)) << 4);
-  uint32_t sign[4];
-#pragma unroll
-  for (int h = 0; h < 4; ++h)
-    sign[h] = ((uint32_t)__double2hiint(x[2 * h]) >> 16 & 0x8000u) | ((uint32_t)__double2hiint(x[2 * h + 1]) & 0x80000000u);
 #pragma unroll
   for (int i = 0; i < kOzS; ++i) {
     uint32_t w[4];
@@ -183,15 +185,16 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
       // 0x6400 | u is the FP16 number 1024 + u (u < 1024); digit = u - 64
       uint32_t lo, hi;
       if (i == 0) {
-        lo = (uint32_t)((int)(X[2 * h] >> 49) + 64);
-        hi = (uint32_t)((int)(X[2 * h + 1] >> 49) + 64);
+        lo = ((uint32_t)(X[2 * h] >> 49) & 127u) + 64;
+        hi = ((uint32_t)(X[2 * h + 1] >> 49) & 127u) + 64;
       } else {
         lo = (uint32_t)(X[2 * h] >> (7 * (7 - i))) & 127u;
         hi = (uint32_t)(X[2 * h + 1] >> (7 * (7 - i))) & 127u;
       }
       const uint32_t raw = 0x64006400u | lo | (hi << 16);
       const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&raw), __float2half2_rn(1088.0f));
-      w[h] = *reinterpret_cast<const uint32_t*>(&d) ^ sign[h];
+      const uint32_t sign = ((uint32_t)(X[2 * h] >> 48) & 0x8000u) | ((uint32_t)(X[2 * h + 1] >> 32) & 0x80000000u);
+      w[h] = *reinterpret_cast<const uint32_t*>(&d) ^ sign;
     }
     *reinterpret_cast<uint4*>(dst + i * digit_stride) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -320,32 +323,29 @@ __device__ __forceinline__ double oz_combine(const int (&S)[kOzL], int e2) {
   return T < 0 ? -v : v;
 }
 
-// One 128 x 48 tile over one K slice.  Warp 0: bulk copies (all digits of a B
+// One 128 x 48 tile over a rank's K slices.  Warp 0: bulk copies (all digits of a B
 // stage, double-buffered; the A digits of a stage one by one into their
 // slots); warp 1: per A digit i the products with B digits 0 .. min(7, 8 - i),
 // neighbouring B digits joined into one instruction of up to 240 columns, whose
 // accumulators lie next to each other in tensor memory; warps 2 to 5: which elements
 // are FP64 sums instead (oz_unproven); then all eight warps read the accumulators,
-// combine and store.
+// combine and add.
 // Columns of a tile (a bit each) whose element in the row with magnitudes at ma and
 // exponent er is to be formed again (see OZ_ELEMENT above); mb, eb: the tile's columns,
 // of which nc exist; kn of a slice's kslice magnitudes are there.
 __device__ __forceinline__ unsigned long long oz_unproven(const uint8_t* ma, int er, const uint8_t* mb, const int* eb,
                                                           int nc, int kslice, int kn) {
-  constexpr int kChunks = kOzMaxK / 64;
   constexpr unsigned kEnough = 2180, kMag = 0x7f7f7f7fu, kAny = 0x80808080u;
-  unsigned long long bad = 0;
-#pragma unroll 8
-  for (int c = 0; c < kOzN; ++c) bad |= (unsigned long long)(er >= 2047 || eb[c] >= 2047) << c;
+  const int lane = threadIdx.x & 31;
+  unsigned long long bad = (unsigned long long)__ballot_sync(0xffffffffu, lane < kOzN - 32 && eb[32 + lane % 16] >= 2047) << 32 |
+                           __ballot_sync(0xffffffffu, eb[lane] >= 2047);
+  if (er >= 2047) bad = (1ull << kOzN) - 1;
   if (!ma) return bad;
-  const int words = kn / 16;
-  uint4 mine[4 * kChunks];
-  unsigned some = 0;
+  // the columns' first 32 k into L1 in one go, for the loop below
+  unsigned touch = 0;
 #pragma unroll
-  for (int w = 0; w < 4 * kChunks; ++w) {
-    mine[w] = w < words ? reinterpret_cast<const uint4*>(ma)[w] : make_uint4(0, 0, 0, 0);
-    some |= mine[w].x | mine[w].y | mine[w].z | mine[w].w;
-  }
+  for (int c = lane; c < kOzN; c += 32) touch |= *reinterpret_cast<const unsigned*>(mb + (size_t)c * kslice);
+  asm volatile("" ::"r"(touch));  // (the loads are for their lines alone)
   // four sums, so that an instruction need not wait for the one before
   auto add = [&](const uint4& a, const uint4& b, uint4& sum, unsigned& any) {
     sum.x = __dp4a(a.x & kMag, b.x & kMag, sum.x);
@@ -355,17 +355,30 @@ __device__ __forceinline__ unsigned long long oz_unproven(const uint8_t* ma, int
     any |= (a.x & b.x) | (a.y & b.y) | (a.z & b.z) | (a.w & b.w);
   };
   auto little = [&](const uint4& sum) { return sum.x + sum.y + sum.z + sum.w < kEnough; };
+  const int words = kn / 16;
+  uint4 mine[kOzMaxK / 16];
+#pragma unroll
+  for (int w = 0; w < 2; ++w) mine[w] = reinterpret_cast<const uint4*>(ma)[w];
   unsigned long long open = 0;
-#pragma unroll 4
+#pragma unroll 8
   for (int c = 0; c < kOzN; ++c) {
     const uint4* m = reinterpret_cast<const uint4*>(mb + (size_t)c * kslice);
     uint4 sum = make_uint4(0, 0, 0, 0);
     unsigned any = 0;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) add(mine[w], m[w], sum, any);
+    for (int w = 0; w < 2; ++w) add(mine[w], m[w], sum, any);
     open |= (unsigned long long)little(sum) << c;
   }
-  open &= some == 0 ? 0ull : ~bad & ((1ull << nc) - 1);
+  open &= ~bad & ((1ull << nc) - 1);
+  if (__all_sync(0xffffffffu, open == 0)) return bad;
+  // all k of the columns that any row has open; a row of zeros has none
+  unsigned some = 0;
+#pragma unroll
+  for (int w = 0; w < kOzMaxK / 16; ++w) {
+    if (w >= 2) mine[w] = w < words ? reinterpret_cast<const uint4*>(ma)[w] : make_uint4(0, 0, 0, 0);
+    some |= mine[w].x | mine[w].y | mine[w].z | mine[w].w;
+  }
+  if (some == 0) open = 0;
   unsigned long long cols = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)open) |
                             (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(open >> 32)) << 32;
   for (; cols; cols &= cols - 1) {
@@ -374,7 +387,7 @@ __device__ __forceinline__ unsigned long long oz_unproven(const uint8_t* ma, int
     uint4 sum = make_uint4(0, 0, 0, 0);
     unsigned any = 0;
 #pragma unroll
-    for (int w = 0; w < 4 * kChunks; ++w)
+    for (int w = 0; w < kOzMaxK / 16; ++w)
       if (w < words) add(mine[w], m[w], sum, any);
     bad |= (unsigned long long)(little(sum) && (any & kAny) != 0 && (open >> c & 1)) << c;
   }
@@ -420,7 +433,7 @@ __device__ __forceinline__ double oz_plain_warp(const OzJob& j, int row, int col
   return t;
 }
 
-__device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int slice) {
+__device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int rank, int ranks) {
   extern __shared__ uint8_t oz_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sB = base;
@@ -436,23 +449,12 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = mt * kOzM, n0 = nt * kOzN;
   const int Mp = (j.M + kOzM - 1) / kOzM * kOzM, Np = (j.N + kOzN - 1) / kOzN * kOzN;
-  const int* ea = j.ea + (size_t)slice * Mp + m0;
-  const int* eb = j.eb + (size_t)slice * Np + n0;
   // an upper-triangular operand is zero for k below its first row
   int kskip = 0;
   if (j.a.kind == 2) kskip = m0;
   if (j.b.kind == 2) kskip = max(kskip, n0);
   const int cper = j.kslice / kOzKc;
-  const int c1 = min(j.chunks, (slice + 1) * cper), c0 = min(c1, max(slice * cper, kskip / kOzKc));
-  double* C = j.C + slice * j.stride;
-  auto store = [&](int i, int col, double v) {
-    if (i < j.M && col < j.N) C[j.swapped ? (size_t)col * j.ldc + i : (size_t)i * j.ldc + col] = v;
-  };
-
-  if (c0 >= c1) {  // a K range of exact zeros
-    for (int e = tid; e < kOzM * kOzN; e += 256) store(m0 + e / kOzN, n0 + e % kOzN, 0.0);
-    return;
-  }
+  const int per = (j.slices + ranks - 1) / ranks, s0 = rank * per, s1 = min(j.slices, s0 + per);
 
   if (tid == 0) {
     s_abort = 0;
@@ -480,88 +482,104 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
   bool ok = true;
-
-  if (warp == 0 && lane == 0) {
-    const uint8_t* ga = j.da + (size_t)mt * j.chunks * kOzS * kOzABytes;
-    const uint8_t* gb = j.db + (size_t)nt * j.chunks * kOzBBytes;
-    int na = 0, nb = 0;  // A digits and B stages issued
-    for (int c = c0; c < c1 && ok; ++c) {
-      const int sb = nb & 1;
-      if (nb >= 2 && !mbar_wait(&emptyB[sb], ((nb >> 1) - 1) & 1)) {
-        ok = false;
-        break;
-      }
-      mbar_expect_tx(&fullB[sb], kOzBBytes);
-      bulk_load(sB + sb * kOzBBytes, gb + (size_t)c * kOzBBytes, kOzBBytes, &fullB[sb]);
-      ++nb;
-      for (int i = 0; i < kOzS; ++i) {
-        const int sa = na % kOzAStages;
-        if (na >= kOzAStages && !mbar_wait(&emptyA[sa], ((na / kOzAStages) - 1) & 1)) {
+  bool first = true;  // (later slices add to what the one before left in C)
+  double* C = j.C + rank * j.stride;
+  auto put = [&](int i, int col, double v) {
+    if (i >= j.M || col >= j.N) return;
+    double* c = C + (j.swapped ? (size_t)col * j.ldc + i : (size_t)i * j.ldc + col);
+    *c = first ? v : *c + v;
+  };
+  int na = 0, nb = 0;  // A digits and B stages issued, or B stages taken (warp 1)
+  int phase = 0;
+  for (int slice = s0; slice < s1; ++slice) {
+    const int c1 = min(j.chunks, (slice + 1) * cper), c0 = min(c1, max(slice * cper, kskip / kOzKc));
+    if (c0 >= c1) continue;  // a K range of exact zeros
+    const int* ea = j.ea + (size_t)slice * Mp + m0;
+    const int* eb = j.eb + (size_t)slice * Np + n0;
+    if (warp == 0 && lane == 0) {
+      const uint8_t* ga = j.da + (size_t)mt * j.chunks * kOzS * kOzABytes;
+      const uint8_t* gb = j.db + (size_t)nt * j.chunks * kOzBBytes;
+      for (int c = c0; c < c1 && ok; ++c) {
+        const int sb = nb & 1;
+        if (nb >= 2 && !mbar_wait(&emptyB[sb], ((nb >> 1) - 1) & 1)) {
           ok = false;
           break;
         }
-        mbar_expect_tx(&fullA[sa], kOzABytes);
-        bulk_load(sA + sa * kOzABytes, ga + ((size_t)c * kOzS + i) * kOzABytes, kOzABytes, &fullA[sa]);
-        ++na;
-      }
-    }
-    // every issued copy lands before the CTA can exit
-    for (int q = max(0, nb - 2); q < nb; ++q)
-      if (!mbar_wait(&fullB[q & 1], (q >> 1) & 1)) ok = false;
-    for (int q = max(0, na - kOzAStages); q < na; ++q)
-      if (!mbar_wait(&fullA[q % kOzAStages], (q / kOzAStages) & 1)) ok = false;
-  } else if (warp == 1 && lane == 0) {
-    // everything but the stage is a constant of the unrolled loops: a descriptor
-    // built at run time costs more issue slots than the smaller products take
-    const uint64_t a_desc = sw128_desc(smem_u32(sA)), b_desc = sw128_desc(smem_u32(sB));
-    for (int c = c0, n = 0; c < c1 && ok; ++c, ++n) {
-      const int sb = n & 1;
-      if (!mbar_wait(&fullB[sb], (n >> 1) & 1)) {
-        ok = false;
-        break;
-      }
-      const uint64_t bd = b_desc + (uint32_t)sb * (kOzBBytes >> 4);
-      const uint32_t later = n > 0 ? 1u : 0u;
-#pragma unroll
-      for (int i = 0; i < kOzS; ++i) {
-        if (ok && !mbar_wait(&fullA[i], n & 1)) ok = false;
-        if (!ok) continue;
-        tc_fence_after();
-        constexpr int kW[kOzS][3] = {{5, 3, 0}, {5, 2, 1}, {5, 2, 0}, {5, 1, 0}, {5, 0, 0}, {4, 0, 0}, {3, 0, 0}, {2, 0, 0}};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          // accumulators are first written by digit 0 (0 .. 7) and by the pair (1, 7) (8)
-          int q = 0;
-#pragma unroll
-          for (int part = 0; part < 3; ++part) {
-            const int w = kW[i][part];
-            if (w == 0) continue;
-            const bool opens = k == 0 && (i == 0 || (i == 1 && part == 2));
-            tc_mma<true>(tmem + (i + q) * kOzN, a_desc + i * (kOzABytes >> 4) + 2 * k, bd + q * (kOzBDigit >> 4) + 2 * k,
-                         tc_idesc(0, w * kOzN), opens ? later : 1u);
-            q += w;
+        mbar_expect_tx(&fullB[sb], kOzBBytes);
+        bulk_load(sB + sb * kOzBBytes, gb + (size_t)c * kOzBBytes, kOzBBytes, &fullB[sb]);
+        ++nb;
+        for (int i = 0; i < kOzS; ++i) {
+          const int sa = na % kOzAStages;
+          if (na >= kOzAStages && !mbar_wait(&emptyA[sa], ((na / kOzAStages) - 1) & 1)) {
+            ok = false;
+            break;
           }
+          mbar_expect_tx(&fullA[sa], kOzABytes);
+          bulk_load(sA + sa * kOzABytes, ga + ((size_t)c * kOzS + i) * kOzABytes, kOzABytes, &fullA[sa]);
+          ++na;
         }
-        tc_commit(&emptyA[i]);
       }
-      if (ok) tc_commit(&emptyB[sb]);
+      // every issued copy lands before the CTA can exit
+      for (int q = max(0, nb - 2); q < nb; ++q)
+        if (!mbar_wait(&fullB[q & 1], (q >> 1) & 1)) ok = false;
+      for (int q = max(0, na - kOzAStages); q < na; ++q)
+        if (!mbar_wait(&fullA[q % kOzAStages], (q / kOzAStages) & 1)) ok = false;
+    } else if (warp == 1 && lane == 0) {
+      // everything but the stage is a constant of the unrolled loops: a descriptor
+      // built at run time costs more issue slots than the smaller products take
+      const uint64_t a_desc = sw128_desc(smem_u32(sA)), b_desc = sw128_desc(smem_u32(sB));
+      for (int c = c0; c < c1 && ok; ++c, ++nb) {
+        const int sb = nb & 1;
+        if (!mbar_wait(&fullB[sb], (nb >> 1) & 1)) {
+          ok = false;
+          break;
+        }
+        const uint64_t bd = b_desc + (uint32_t)sb * (kOzBBytes >> 4);
+        const uint32_t later = c > c0 ? 1u : 0u;
+#pragma unroll
+        for (int i = 0; i < kOzS; ++i) {
+          if (ok && !mbar_wait(&fullA[i], nb & 1)) ok = false;
+          if (!ok) continue;
+          tc_fence_after();
+          constexpr int kW[kOzS][3] = {{5, 3, 0}, {5, 2, 1}, {5, 2, 0}, {5, 1, 0}, {5, 0, 0}, {4, 0, 0}, {3, 0, 0}, {2, 0, 0}};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            // accumulators are first written by digit 0 (0 .. 7) and by the pair (1, 7) (8)
+            int q = 0;
+#pragma unroll
+            for (int part = 0; part < 3; ++part) {
+              const int w = kW[i][part];
+              if (w == 0) continue;
+              const bool opens = k == 0 && (i == 0 || (i == 1 && part == 2));
+              tc_mma<true>(tmem + (i + q) * kOzN, a_desc + i * (kOzABytes >> 4) + 2 * k, bd + q * (kOzBDigit >> 4) + 2 * k,
+                           tc_idesc(0, w * kOzN), opens ? later : 1u);
+              q += w;
+            }
+          }
+          tc_commit(&emptyA[i]);
+        }
+        if (ok) tc_commit(&emptyB[sb]);
+      }
+      tc_commit(done);
+    } else if (warp >= 2 && warp < 6) {
+      const int r = tid - 64;
+      const size_t rec = (size_t)j.kslice, ra = (size_t)slice * Mp + m0 + r, rb = (size_t)slice * Np + n0;
+      s_bad[r] = j.ma ? oz_unproven(j.ma + ra * rec, ea[r], j.mb + rb * rec, eb, min(kOzN, j.N - n0), j.kslice,
+                                      min(j.kslice, j.chunks * kOzKc - slice * j.kslice))
+                        : oz_unproven(nullptr, ea[r], nullptr, eb, 0, 0, 0);
     }
-    tc_commit(done);
-  } else if (warp >= 2 && warp < 6) {
-    const int row = tid - 64;
-    const size_t rec = (size_t)j.kslice, ra = (size_t)slice * Mp + m0 + row, rb = (size_t)slice * Np + n0;
-    s_bad[row] = j.ma ? oz_unproven(j.ma + ra * rec, ea[row], j.mb + rb * rec, eb, min(kOzN, j.N - n0), j.kslice,
-                                    min(j.kslice, j.chunks * kOzKc - slice * j.kslice))
-                      : oz_unproven(nullptr, ea[row], nullptr, eb, 0, 0, 0);
-  }
-  if (!ok) atomicExch(&s_abort, 1);
-  __syncwarp();
-  __syncthreads();
+    if (!ok) atomicExch(&s_abort, 1);
+    __syncwarp();
+    __syncthreads();
 
-  const bool got = mbar_wait(done, 0);
-  const int good = __syncthreads_and(got && s_abort == 0);
-  tc_fence_after();
-  if (good) {
+    const bool got = mbar_wait(done, phase);
+    phase ^= 1;
+    const int good = __syncthreads_and(got && s_abort == 0);
+    tc_fence_after();
+    if (!good) {
+      if (tid == 0) atomicCAS(&j.st->err, 0, 1);
+      break;
+    }
     // warp w reads lanes 32 (w mod 4) .., the column groups of 8 with (w / 4)
     const int row = (warp & 3) * 32 + lane;
     const int er = ea[row], kb = c0 * kOzKc, ke = min(j.K, c1 * kOzKc);
@@ -582,7 +600,7 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
         // digit products carry 2^(7 (14 - l)); scales 2^(er - 1022 - 55), 2^(ec - 1022 - 55)
         double v = oz_combine(S, er + eb[col] - 2 * 1077 + 42);
         if (j.alpha != 1.0) v *= j.alpha;
-        if (!(bad >> col & 1)) store(m0 + row, n0 + col, v);
+        if (!(bad >> col & 1)) put(m0 + row, n0 + col, v);
       }
       // the elements that were not proven: few one by one, more as the whole group of
       // 32 x 8 (the FP64 pipe takes 16 clocks a warp's FMA: at K = 512 the group's 8 per k
@@ -596,7 +614,7 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
         oz_plain(j, m0 + row, n0 + 8 * g, kb, ke, t);
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (mine >> u & 1) store(m0 + row, n0 + 8 * g + u, j.alpha * t[u]);
+          if (mine >> u & 1) put(m0 + row, n0 + 8 * g + u, j.alpha * t[u]);
         rows = 0;
       }
       for (; rows; rows &= rows - 1) {
@@ -604,12 +622,18 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
         for (unsigned us = __shfl_sync(0xffffffffu, mine, l); us; us &= us - 1) {
           const int u = __ffs(us) - 1;
           const double t = oz_plain_warp(j, i0 + l, n0 + 8 * g + u, kb, ke, lane);
-          if (lane == 0) store(i0 + l, n0 + 8 * g + u, j.alpha * t);
+          if (lane == 0) put(i0 + l, n0 + 8 * g + u, j.alpha * t);
         }
       }
     }
+    first = false;
+    tc_fence_before();
+    __syncthreads();  // the accumulators are read
+    tc_fence_after();
   }
-  if (!good && tid == 0) atomicCAS(&j.st->err, 0, 1);
+
+  if (first)  // nothing but slices of exact zeros
+    for (int e = tid; e < kOzM * kOzN; e += 256) put(m0 + e / kOzN, n0 + e % kOzN, 0.0);
   tc_fence_before();
   __syncthreads();
   if (warp == 0)
@@ -630,12 +654,13 @@ __global__ void __launch_bounds__(kOzThreads) kb_oz_pack(const __grid_constant__
   const int side = (int)blockIdx.x >= ablk;
   oz_pack_body(j, side, (int)blockIdx.x - (side ? ablk : 0), blockIdx.y);
 }
+// z: job x rank (of at most zs)
 __global__ void __launch_bounds__(256, 1) kb_oz_mma(const __grid_constant__ Pack<OzJob> pk, int zs) {
   follow();
   const OzJob& j = pk.a[blockIdx.z / zs];
-  const int slice = blockIdx.z % zs;
-  if (slice >= j.slices || (int)blockIdx.x * kOzM >= j.M || (int)blockIdx.y * kOzN >= j.N) return;
-  oz_mma_body(j, blockIdx.x, blockIdx.y, slice);
+  const int rank = blockIdx.z % zs;
+  if (rank >= j.ranks || (int)blockIdx.x * kOzM >= j.M || (int)blockIdx.y * kOzN >= j.N) return;
+  oz_mma_body(j, blockIdx.x, blockIdx.y, rank, j.ranks);
 }
 
 size_t oz_pack_smem(int kslice) { return (size_t)kOzPackRows * (kslice / 8 * 9 + 1) * sizeof(double); }
@@ -643,44 +668,59 @@ long long tiles_of(int M, int N) { return (long long)((M + kOzM - 1) / kOzM) * (
 
 }  // namespace
 
-// Which FP64 contractions are sliced.  Three launches of ~6 + 11 + 17 us at the
-// smallest sizes stand against the FMA kernel's 2 M N K / 1.1 TFLOP/s: whole
-// vp_gemm calls on GB300, sliced / FMA, us: 256^3 (M N K = 1.7e7) 63 / 62,
-// 320 x 256 x 256 (2.1e7) 66 / 86, 300^3 67 / 99, 512 x 324 x 256 (4.3e7) 68 /
-// 135, 341 x 1008 x 503 (1.7e8) 74 / 430, 128 x 6784 x 6147 (5.3e9) 810 / 12300;
+// Which FP64 contractions are sliced.  Two launches of ~14 + 26 us at the smallest
+// sizes stand against the FMA kernel's 2 M N K / 1.1 TFLOP/s: whole vp_gemm calls on
+// GB300, sliced / FMA, us: @FIGURES@;
 // the line is drawn at 2e7.  Below K = 64 (one stage) or 16 rows or columns most
 // of a tile would be padding; so would a shape that fills less than a quarter of
-// its tiles in the better of the two orientations.  K is cut into slices until
-// the tiles fill the SMs once (at least 128 of K each, two stages), and always at
-// 512, where the accumulators stop being exact.
+// its tiles in the better of the two orientations; and from K = 524288 on a band of one
+// tile's rows would take more than kOzBand.  K is cut into slices of at most 512, where
+// the accumulators stop being exact, and into at least as many as fill the SMs with tiles
+// once (128 of K each, two stages); a CTA takes one, while what they leave to be added
+// stays below kOzSums.  (Slices added in registers, or over the CTAs of a cluster, took 5
+// to 15 us longer a product than a CTA each and the launch that adds.)
 OzPlan oz_plan(const vp_ctx* ctx, int M, int N, int K) {
-  OzPlan p{0, 0, 1, 0};
-  if (K < 64 || std::min(M, N) < 16 || (double)M * N * K < 2e7) return p;
+  OzPlan p{0, 0, 1, 0, 1};
+  if (K < 64 || K >= 1 << 19 || std::min(M, N) < 16 || (double)M * N * K < 2e7) return p;
   const long long t = tiles_of(M, N), ts = tiles_of(N, M);
   p.swapped = ts < t;
   const long long tiles = std::min(t, ts);
   // partial tiles compute their padding: not worth it where most of it is
   if ((double)tiles * kOzM * kOzN > 4.0 * M * N) return p;
-  if (tiles > 2000000) return p;
-  const int chunks = (K + kOzKc - 1) / kOzKc;
+  const int chunks = (K + kOzKc - 1) / kOzKc, most = kOzMaxK / kOzKc;
   int sl = (K + kOzMaxK - 1) / kOzMaxK;
   sl = std::max<long long>(sl, std::min<long long>(ctx->num_sms / tiles, (chunks + 1) / 2));
-  const int per = std::min(kOzMaxK / kOzKc, (chunks + sl - 1) / sl);
+  const int per = std::min(most, (chunks + sl - 1) / sl);
   p.use = 1;
   p.kslice = per * kOzKc;
   p.slices = (chunks + per - 1) / per;
+  const long long held = std::max(1ll, (long long)kOzSums / (8ll * M * N));
+  const int rounds = (int)((p.slices + held - 1) / held);  // slices a CTA
+  p.ranks = (p.slices + rounds - 1) / rounds;
   return p;
 }
 
-int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
-  if (v.empty()) return VP_OK;
+namespace {
+
+// Scratch of a product in doubles: A's digits, the magnitudes, exponents and shifts;
+// B's digits.
+void oz_scratch(const OzGemm& g, size_t& wa, size_t& wb) {
+  const size_t M = g.plan.swapped ? g.N : g.M, N = g.plan.swapped ? g.M : g.N;
+  const size_t Mp = (M + kOzM - 1) / kOzM * kOzM, Np = (N + kOzN - 1) / kOzN * kOzN;
+  const size_t chunks = (g.K + kOzKc - 1) / kOzKc, rec = g.bound == OZ_ELEMENT ? g.plan.kslice : 0;
+  const size_t ints = (size_t)g.K + g.plan.slices * (Mp + Np);
+  wa = (Mp / kOzM * chunks * kOzS * kOzABytes + g.plan.slices * (Mp + Np) * rec) / 8 + ints / 2 + 64;
+  wb = Np / kOzN * chunks * kOzBBytes / 8 + 64;
+}
+
+int launch_oz(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
   static AttrOnce attr, pattr;
   VP_TRY(attr.ensure(ctx, (const void*)kb_oz_mma, (int)kOzSmem, false));
   VP_TRY(pattr.ensure(ctx, (const void*)kb_oz_pack, (int)oz_pack_smem(kOzMaxK), false));
   for (size_t i0 = 0; i0 < v.size(); i0 += kMaxBatch) {
     const int nb = (int)std::min<size_t>(kMaxBatch, v.size() - i0);
     Pack<OzJob> pk{};
-    int ks = 1, ablk = 1, bblk = 1, zs = 1, gx = 1, gy = 1, ksl = kOzKc;
+    int ks = 1, ablk = 1, bblk = 1, slices = 1, zs = 1, gx = 1, gy = 1, ksl = kOzKc;
     bool shifts = false;
     for (int i = 0; i < nb; ++i) {
       const OzGemm& g = v[i0 + i];
@@ -692,6 +732,7 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       j.K = g.K;
       j.kslice = g.plan.kslice;
       j.slices = g.plan.slices;
+      j.ranks = g.plan.ranks;
       j.chunks = (g.K + kOzKc - 1) / kOzKc;
       j.swapped = g.plan.swapped;
       j.alpha = g.alpha;
@@ -700,12 +741,9 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       j.stride = g.stride;
       j.st = g.st;
       const size_t Mp = (size_t)(j.M + kOzM - 1) / kOzM * kOzM, Np = (size_t)(j.N + kOzN - 1) / kOzN * kOzN;
-      const size_t abytes = Mp / kOzM * j.chunks * kOzS * kOzABytes, bbytes = Np / kOzN * j.chunks * (size_t)kOzBBytes;
-      const size_t ints = (size_t)j.K + (size_t)j.slices * (Mp + Np);
+      const size_t abytes = Mp / kOzM * j.chunks * kOzS * kOzABytes;
       // magnitudes of OZ_ELEMENT, on 16-byte boundaries behind the digits
       const size_t rec = g.bound == OZ_ELEMENT ? (size_t)j.kslice : 0, mbytes = j.slices * (Mp + Np) * rec;
-      VP_TRY(reserve(ctx, *g.wa, abytes / 8 + mbytes / 8 + ints / 2 + 64));
-      VP_TRY(reserve(ctx, *g.wb, bbytes / 8 + 64));
       // bulk copies start on 16-byte boundaries, whatever the allocator's alignment
       auto aligned = [](double* p) { return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 127) & ~uintptr_t(127)); };
       j.da = aligned(g.wa->p);
@@ -722,20 +760,80 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       }
       ablk = std::max(ablk, (int)((Mp + kOzPackRows - 1) / kOzPackRows));
       bblk = std::max(bblk, (int)((Np + kOzPackRows - 1) / kOzPackRows));
-      zs = std::max(zs, j.slices);
+      slices = std::max(slices, j.slices);
+      zs = std::max(zs, j.ranks);
       ksl = std::max(ksl, j.kslice);
       gx = std::max(gx, (int)(Mp / kOzM));
       gy = std::max(gy, (int)(Np / kOzN));
     }
-    if (gy > 65535 || (long long)nb * zs > 65535) return fail(ctx, VP_ECAPACITY, "gemm: too large");
+    if (gy > 65535) return fail(ctx, VP_ECAPACITY, "gemm: too large");
     if (shifts)
       VP_TRY(launch_after(ctx, "oz_kexp", kb_oz_kexp, dim3(ks, nb), dim3(kOzThreads), 0, st, kNoCluster, pk));
-    VP_TRY(launch_after(ctx, "oz_pack", kb_oz_pack, dim3(ablk + bblk, zs, nb), dim3(kOzThreads), oz_pack_smem(ksl),
+    VP_TRY(launch_after(ctx, "oz_pack", kb_oz_pack, dim3(ablk + bblk, slices, nb), dim3(kOzThreads), oz_pack_smem(ksl),
                         st, kNoCluster,
                         pk, ablk));
     VP_TRY(launch_after(ctx, "oz_mma", kb_oz_mma, dim3(gx, gy, nb * zs), dim3(256), kOzSmem, st, kNoCluster, pk, zs));
   }
   return VP_OK;
+}
+
+}  // namespace
+
+int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
+  std::vector<OzGemm> sliced, fma;
+  for (const OzGemm& g : v) {
+    if (!g.plan.use) {
+      fma.push_back(g);
+      continue;
+    }
+    // rows of A and of B in bands whose digits fit
+    const long long fit = (long long)(kOzBand / 16) / ((g.K + kOzKc - 1) / kOzKc * kOzKc) / kOzM * kOzM;
+    if (g.M > fit || g.N > fit) {
+      const int mb = (int)((g.M + fit - 1) / fit), nb = (int)((g.N + fit - 1) / fit);
+      const int mr = ((g.M + mb - 1) / mb + kOzM - 1) / kOzM * kOzM, nr = ((g.N + nb - 1) / nb + kOzM - 1) / kOzM * kOzM;
+      for (int m0 = 0; m0 < g.M; m0 += mr)
+        for (int n0 = 0; n0 < g.N; n0 += nr) {
+          OzGemm s = g;
+          s.M = std::min(mr, g.M - m0);
+          s.N = std::min(nr, g.N - n0);
+          s.C = g.C + (size_t)m0 * g.ldc + n0;
+          const int k0 = g.a.kind == 2 ? m0 : 0;  // a triangle below row m0: from its column m0 on
+          s.K = g.K - k0;
+          s.a.p += g.a.kind == 0 ? (size_t)m0 * g.a.ld : (size_t)k0 * g.a.ld + m0;
+          s.b.p += g.b.kind == 0 ? (size_t)n0 * g.b.ld + k0 : (size_t)k0 * g.b.ld + n0;
+          s.plan = oz_plan(ctx, s.M, s.N, s.K);
+          VP_TRY(blaunch_oz_gemm(ctx, st, {s}));  // in turn: the bands share the scratch
+        }
+      continue;
+    }
+    sliced.push_back(g);
+  }
+  // scratch of every product before the first launch; without it: FMAs
+  const std::string err = ctx->err;
+  std::vector<OzSum> sums;
+  size_t n = 0;
+  for (OzGemm g : sliced) {
+    size_t wa, wb;
+    oz_scratch(g, wa, wb);
+    const size_t stride = (size_t)g.M * g.N;
+    if (reserve(ctx, *g.wa, wa) != VP_OK || reserve(ctx, *g.wb, wb) != VP_OK ||
+        (g.plan.ranks > 1 && reserve(ctx, *g.wsum, stride * g.plan.ranks) != VP_OK)) {
+      ctx->err = err;
+      fma.push_back(g);
+      continue;
+    }
+    if (g.plan.ranks > 1) {
+      sums.push_back({g.wsum->p, g.M, g.N, g.plan.ranks, stride, g.C, g.ldc});
+      g.C = g.wsum->p;
+      g.ldc = g.N;
+      g.stride = stride;
+    }
+    sliced[n++] = g;
+  }
+  sliced.resize(n);
+  VP_TRY(launch_oz(ctx, st, sliced));
+  VP_TRY(blaunch_sum_slices(ctx, st, sums));
+  return blaunch_fma_gemm(ctx, st, fma);
 }
 
 }  // namespace vp
