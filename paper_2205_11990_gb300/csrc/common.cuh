@@ -270,6 +270,7 @@ struct GemmPlan {
   int kslice;  // columns of K per slice
 };
 GemmPlan gemm_plan(const vp_ctx* ctx, int M, int N, int K);
+constexpr int kGemmMaxN = 64 * 65535;  // columns of a contraction in any mode
 // How far an FP64 contraction may be off (ozgemm.cu says how each is kept; the FMA
 // kernel is within all of them):
 //   OZ_ELEMENT  every element within the bound of an FP64 sum, K 2^-53 (|A| |B|)_ij;

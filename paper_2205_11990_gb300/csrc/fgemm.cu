@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include <cooperative_groups.h>
@@ -125,13 +126,16 @@ __device__ __forceinline__ void fma_tile(const FmaJob& j, int bx, int by, int sl
   }
 }
 
-// blockIdx.z: job x K slice (the slices of a tile are one cluster)
+// blockIdx.x: tile, down a column of tiles first (as one number: along y there would be
+// too few blocks for 16-wide tiles of a million columns); blockIdx.z: job x K slice (the
+// slices of a tile are one cluster)
 template <int KA, int KB, int TILE>
 __global__ void __launch_bounds__(kFT) kb_gemm_fma(const __grid_constant__ Pack<FmaJob> pk, int zs) {
   follow();
   const FmaJob& j = pk.a[blockIdx.z / zs];
-  if ((int)blockIdx.x * TILE >= j.M || (int)blockIdx.y * TILE >= j.N) return;  // the whole cluster
-  fma_tile<KA, KB, TILE>(j, blockIdx.x, blockIdx.y, blockIdx.z % zs, zs);
+  const int down = (j.M + TILE - 1) / TILE, bx = blockIdx.x % down, by = blockIdx.x / down;
+  if (by >= (j.N + TILE - 1) / TILE) return;  // the whole cluster
+  fma_tile<KA, KB, TILE>(j, bx, by, blockIdx.z % zs, zs);
 }
 
 struct FmaPlan {
@@ -173,14 +177,13 @@ int launch_group(vp_ctx* ctx, cudaStream_t st, const std::vector<FmaJob>& jobs, 
   for (size_t i0 = 0; i0 < jobs.size(); i0 += kMaxBatch) {
     const int nb = (int)std::min<size_t>(kMaxBatch, jobs.size() - i0);
     Pack<FmaJob> pk{};
-    int gx = 1, gy = 1;
+    long long tiles = 1;
     for (int i = 0; i < nb; ++i) {
       pk.a[i] = jobs[i0 + i];
-      gx = std::max(gx, (pk.a[i].M + TILE - 1) / TILE);
-      gy = std::max(gy, (pk.a[i].N + TILE - 1) / TILE);
+      tiles = std::max(tiles, (long long)((pk.a[i].M + TILE - 1) / TILE) * ((pk.a[i].N + TILE - 1) / TILE));
     }
-    if (gy > 65535) return fail(ctx, VP_ECAPACITY, "gemm: N too large");
-    VP_TRY((launch_after(ctx, "gemm", kb_gemm_fma<KA, KB, TILE>, dim3(gx, gy, nb * zs), dim3(kFT), 0, st,
+    if (tiles > INT_MAX) return fail(ctx, VP_ECAPACITY, "gemm: too large");
+    VP_TRY((launch_after(ctx, "gemm", kb_gemm_fma<KA, KB, TILE>, dim3((unsigned)tiles, 1, nb * zs), dim3(kFT), 0, st,
                          zs > 1 ? dim3(1, 1, zs) : kNoCluster, pk, zs)));
   }
   return VP_OK;
@@ -198,6 +201,7 @@ int launch_kind(vp_ctx* ctx, cudaStream_t st, const std::vector<FmaJob>& jobs, i
 int blaunch_fma_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
   std::vector<FmaJob> jobs[3][3][4];  // [layout][tile 16 / 32 / 64][1, 2, 4, 8 slices]
   for (const OzGemm& g : v) {
+    if (g.N > kGemmMaxN) return fail(ctx, VP_ECAPACITY, "gemm: N too large");
     const FmaPlan pl = fma_plan(ctx, g.M, g.N, g.K);
     const int kind = g.a.kind == 2 ? 2 : g.b.kind == 0 ? 1 : 0;
     const int ti = pl.tile == 64 ? 2 : pl.tile == 32 ? 1 : 0;

@@ -766,7 +766,6 @@ int launch_oz(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
       gx = std::max(gx, (int)(Mp / kOzM));
       gy = std::max(gy, (int)(Np / kOzN));
     }
-    if (gy > 65535) return fail(ctx, VP_ECAPACITY, "gemm: too large");
     if (shifts)
       VP_TRY(launch_after(ctx, "oz_kexp", kb_oz_kexp, dim3(ks, nb), dim3(kOzThreads), 0, st, kNoCluster, pk));
     VP_TRY(launch_after(ctx, "oz_pack", kb_oz_pack, dim3(ablk + bblk, slices, nb), dim3(kOzThreads), oz_pack_smem(ksl),
@@ -786,7 +785,8 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       fma.push_back(g);
       continue;
     }
-    // rows of A and of B in bands whose digits fit
+    if (g.N > kGemmMaxN) return fail(ctx, VP_ECAPACITY, "gemm: N too large");
+    // rows of A and of B in bands whose digits fit (a million of them at K = 64: 22000 tiles)
     const long long fit = (long long)(kOzBand / 16) / ((g.K + kOzKc - 1) / kOzKc * kOzKc) / kOzM * kOzM;
     if (g.M > fit || g.N > fit) {
       const int mb = (int)((g.M + fit - 1) / fit), nb = (int)((g.N + fit - 1) / fit);
