@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdint>
 
 #include "common.cuh"
 #include "dw.cuh"
@@ -218,6 +219,8 @@ __global__ void kb_formq_long(const __grid_constant__ Pack<FqArgs> pk) {
   for (int i = lane; i < m; i += 32) a.Q[(size_t)(a.rows ? a.rows[i] : i) * a.p + k] = dw_to_scaled(q[i], 0);
 }
 
+dw* align16(double* p) { return reinterpret_cast<dw*>((reinterpret_cast<uintptr_t>(p) + 15) & ~uintptr_t(15)); }
+
 template <int W, int R, int NC>
 int launch_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<FqArgs>& v) {
   constexpr bool shared = 32 * W * R <= kFqShared;
@@ -247,9 +250,11 @@ int blaunch_formq(vp_ctx* ctx, cudaStream_t st, const std::vector<FormQJob>& v) 
     const int p = std::min(j.m, j.n);
     if (p <= 0) continue;
     const size_t np = (p + kFB - 1) / kFB;
-    VP_TRY(reserve(ctx, *j.v, (size_t)j.m * kFB * np + 16 * np));
-    FqArgs a{j.A, j.tau, j.m, p, nullptr, reinterpret_cast<dw*>(j.v->p), nullptr, j.Q, j.rows};
-    a.V = a.T + 16 * np;  // (both on 16-byte boundaries)
+    // T and V on 16-byte boundaries, as their asynchronous copies need, whatever the
+    // allocator's alignment
+    VP_TRY(reserve(ctx, *j.v, (size_t)j.m * kFB * np + 16 * np + 1));
+    FqArgs a{j.A, j.tau, j.m, p, nullptr, align16(j.v->p), nullptr, j.Q, j.rows};
+    a.V = a.T + 16 * np;
     if (j.m > kFqMaxRows) {
       VP_TRY(reserve(ctx, *j.scratch, (size_t)j.m * p));
       a.scratch = reinterpret_cast<dw*>(j.scratch->p);
