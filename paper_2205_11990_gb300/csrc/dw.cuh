@@ -90,7 +90,7 @@ __device__ __forceinline__ double dw_to(dw x) { return (double)x.hi + (double)x.
 // The same through integer and FP32 operations: a conversion, product or sum on the
 // FP64 pipe costs one of the two slots an SM has per clock, and a split or a
 // recombination four of them.  x 2^-e split to hi = RN24, lo = RN24 of the rest
-// (|x 2^-e| below 2^127; what lies below the FP32 range becomes zero).
+// (|x 2^-e| below 2^127; below 2^-126 hi, and below 2^-102 lo, becomes zero).
 __device__ __forceinline__ float pow2f(int e) { return e < -126 ? 0.0f : __int_as_float((e + 127) << 23); }
 __device__ __forceinline__ dw dw_from_scaled(double x, int e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
@@ -102,9 +102,10 @@ __device__ __forceinline__ dw dw_from_scaled(double x, int e) {
   unsigned top = (unsigned)(m >> 29);
   const unsigned up = (rest + (1u << 28) - 1 + (top & 1u)) >> 29;  // to nearest, ties to even
   top += up;
-  const int s = ex - 1075 - e;  // x 2^-e = m 2^s
+  const int s = ex - 1023 - e;  // x 2^-e is 1.f 2^s
   const float sg = (b >> 63) ? -1.0f : 1.0f;
-  return {sg * __uint2float_rn(top) * pow2f(s + 29), sg * __int2float_rn((int)rest - (int)(up << 29)) * pow2f(s)};
+  return {sg * (__uint2float_rn(top) * 0x1p-23f) * pow2f(s),
+          sg * (__int2float_rn((int)rest - (int)(up << 29)) * 0x1p-28f) * pow2f(s - 24)};
 }
 // (hi + lo) 2^e as FP64, rounded to nearest.
 __device__ __forceinline__ double dw_to_scaled(dw v, int e) {
