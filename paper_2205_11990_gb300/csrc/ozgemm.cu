@@ -177,6 +177,9 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
     *reinterpret_cast<uint2*>(mag) = make_uint2(w[0], w[1]);
   }
   uint8_t* dst = tile0 + row * 128 + ((kchunk16 ^ (row & 7)) << 4);
+  uint32_t sign[4];  // bits 15 and 31
+#pragma unroll
+  for (int h = 0; h < 4; ++h) sign[h] = __byte_perm((uint32_t)(X[2 * h] >> 32), (uint32_t)(X[2 * h + 1] >> 32), 0x7030) & 0x80008000u;
 #pragma unroll
   for (int i = 0; i < kOzS; ++i) {
     uint32_t w[4];
@@ -193,8 +196,7 @@ __device__ __forceinline__ void oz_store_digits(const double (&x)[8], const int 
       }
       const uint32_t raw = 0x64006400u | lo | (hi << 16);
       const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&raw), __float2half2_rn(1088.0f));
-      const uint32_t sign = ((uint32_t)(X[2 * h] >> 48) & 0x8000u) | ((uint32_t)(X[2 * h + 1] >> 32) & 0x80000000u);
-      w[h] = *reinterpret_cast<const uint32_t*>(&d) ^ sign;
+      w[h] = *reinterpret_cast<const uint32_t*>(&d) ^ sign[h];
     }
     *reinterpret_cast<uint4*>(dst + i * digit_stride) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -433,6 +435,8 @@ __device__ __forceinline__ double oz_plain_warp(const OzJob& j, int row, int col
   return t;
 }
 
+// MORE: a rank has several slices.
+template <bool MORE>
 __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int rank, int ranks) {
   extern __shared__ uint8_t oz_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
@@ -454,7 +458,7 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
   if (j.a.kind == 2) kskip = m0;
   if (j.b.kind == 2) kskip = max(kskip, n0);
   const int cper = j.kslice / kOzKc;
-  const int per = (j.slices + ranks - 1) / ranks, s0 = rank * per, s1 = min(j.slices, s0 + per);
+  const int per = MORE ? (j.slices + ranks - 1) / ranks : 1, s0 = rank * per, s1 = MORE ? min(j.slices, s0 + per) : s0 + 1;
 
   if (tid == 0) {
     s_abort = 0;
@@ -487,7 +491,7 @@ __device__ __forceinline__ void oz_mma_body(const OzJob& j, int mt, int nt, int 
   auto put = [&](int i, int col, double v) {
     if (i >= j.M || col >= j.N) return;
     double* c = C + (j.swapped ? (size_t)col * j.ldc + i : (size_t)i * j.ldc + col);
-    *c = first ? v : *c + v;
+    *c = !MORE || first ? v : *c + v;
   };
   int na = 0, nb = 0;  // A digits and B stages issued, or B stages taken (warp 1)
   int phase = 0;
@@ -655,12 +659,13 @@ __global__ void __launch_bounds__(kOzThreads) kb_oz_pack(const __grid_constant__
   oz_pack_body(j, side, (int)blockIdx.x - (side ? ablk : 0), blockIdx.y);
 }
 // z: job x rank (of at most zs)
+template <bool MORE>
 __global__ void __launch_bounds__(256, 1) kb_oz_mma(const __grid_constant__ Pack<OzJob> pk, int zs) {
   follow();
   const OzJob& j = pk.a[blockIdx.z / zs];
   const int rank = blockIdx.z % zs;
   if (rank >= j.ranks || (int)blockIdx.x * kOzM >= j.M || (int)blockIdx.y * kOzN >= j.N) return;
-  oz_mma_body(j, blockIdx.x, blockIdx.y, rank, j.ranks);
+  oz_mma_body<MORE>(j, blockIdx.x, blockIdx.y, rank, j.ranks);
 }
 
 size_t oz_pack_smem(int kslice) { return (size_t)kOzPackRows * (kslice / 8 * 9 + 1) * sizeof(double); }
@@ -713,9 +718,10 @@ void oz_scratch(const OzGemm& g, size_t& wa, size_t& wb) {
   wb = Np / kOzN * chunks * kOzBBytes / 8 + 64;
 }
 
+template <bool MORE>
 int launch_oz(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
   static AttrOnce attr, pattr;
-  VP_TRY(attr.ensure(ctx, (const void*)kb_oz_mma, (int)kOzSmem, false));
+  VP_TRY(attr.ensure(ctx, (const void*)kb_oz_mma<MORE>, (int)kOzSmem, false));
   VP_TRY(pattr.ensure(ctx, (const void*)kb_oz_pack, (int)oz_pack_smem(kOzMaxK), false));
   for (size_t i0 = 0; i0 < v.size(); i0 += kMaxBatch) {
     const int nb = (int)std::min<size_t>(kMaxBatch, v.size() - i0);
@@ -771,7 +777,7 @@ int launch_oz(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
     VP_TRY(launch_after(ctx, "oz_pack", kb_oz_pack, dim3(ablk + bblk, slices, nb), dim3(kOzThreads), oz_pack_smem(ksl),
                         st, kNoCluster,
                         pk, ablk));
-    VP_TRY(launch_after(ctx, "oz_mma", kb_oz_mma, dim3(gx, gy, nb * zs), dim3(256), kOzSmem, st, kNoCluster, pk, zs));
+    VP_TRY(launch_after(ctx, "oz_mma", kb_oz_mma<MORE>, dim3(gx, gy, nb * zs), dim3(256), kOzSmem, st, kNoCluster, pk, zs));
   }
   return VP_OK;
 }
@@ -779,7 +785,7 @@ int launch_oz(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
 }  // namespace
 
 int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) {
-  std::vector<OzGemm> sliced, fma;
+  std::vector<OzGemm> sliced, one, more, fma;  // a slice a CTA, or several
   for (const OzGemm& g : v) {
     if (!g.plan.use) {
       fma.push_back(g);
@@ -811,7 +817,6 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
   // scratch of every product before the first launch; without it: FMAs
   const std::string err = ctx->err;
   std::vector<OzSum> sums;
-  size_t n = 0;
   for (OzGemm g : sliced) {
     size_t wa, wb;
     oz_scratch(g, wa, wb);
@@ -828,10 +833,10 @@ int blaunch_oz_gemm(vp_ctx* ctx, cudaStream_t st, const std::vector<OzGemm>& v) 
       g.ldc = g.N;
       g.stride = stride;
     }
-    sliced[n++] = g;
+    (g.plan.slices > g.plan.ranks ? more : one).push_back(g);
   }
-  sliced.resize(n);
-  VP_TRY(launch_oz(ctx, st, sliced));
+  VP_TRY(launch_oz<false>(ctx, st, one));
+  VP_TRY(launch_oz<true>(ctx, st, more));
   VP_TRY(blaunch_sum_slices(ctx, st, sums));
   return blaunch_fma_gemm(ctx, st, fma);
 }
