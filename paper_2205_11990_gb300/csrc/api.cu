@@ -461,13 +461,14 @@ static int svd_site(vp_ctx* ctx, mps_t* s, int k, int chi, double tol, double* e
   prof_begin(ctx, VP_K_GEMM);
   double* Vt = ctx->w_tmp2.p;  // the new core k (r x c)
   VP_TRY(launch_svd_outputs(ctx, X, q, r, perm, sigma, piv2, ctx->w_a.p));
-  // V^T enters both cores: FP64 in every contraction mode
+  // V^T enters both cores, and M V (= U S) carries the whole state's norm in every
+  // column: FP64 in every contraction mode
   const int prec = ctx->precision;
   ctx->precision = VP_PREC_FP64;
-  const int st = launch_gemm_bt(ctx, r, c, q, ctx->w_a.p, q, ctx->w_q1.p, q, Vt, c, OZ_ROWS);
+  int st = launch_gemm_bt(ctx, r, c, q, ctx->w_a.p, q, ctx->w_q1.p, q, Vt, c, OZ_ROWS);
+  if (st == VP_OK) st = launch_gemm_bt(ctx, m, r, c, s->core[k].p, c, Vt, c, ctx->w_b.p, r, OZ_ROWS);
   ctx->precision = prec;
   VP_TRY(st);
-  VP_TRY(launch_gemm_bt(ctx, m, r, c, s->core[k].p, c, Vt, c, ctx->w_b.p, r, OZ_ROWS));  // U S = M V
   VP_TRY(launch_gemm(ctx, pl, r, m, 1.0, s->core[k - 1].p, m, ctx->w_b.p, r, ctx->w_gemm.p, r, OZ_COLS));
   const double gem = 2.0 * r * c * q + 2.0 * m * r * c + 2.0 * pl * r * m;
   prof_end(ctx, VP_K_GEMM, gem, q, r, pl);

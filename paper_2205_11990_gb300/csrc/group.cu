@@ -440,11 +440,11 @@ int svd_sweep(vp_group* g, const Tasks& all) {
       int* perm = (int*)w.vec.p;
       double* sigma = w.vec.p + (q + 1) / 2 + 4;
       const int* piv2 = (const int*)w.piv.p + q;
-      // core_k <- V^T (in tmp2, swapped in below; FP64 in every mode, as it enters
-      // both cores); core_{k-1} <- core_{k-1} (M V)
+      // core_k <- V^T (in tmp2, swapped in below); core_{k-1} <- core_{k-1} (M V); V^T and
+      // M V in FP64 in every mode (api.cu's svd_site)
       so.push_back({w.tmp.p, q, r, perm, sigma, piv2, w.a.p});
       g2.push_back({BG_ABT, 0, r, c, q, 1.0, w.a.p, q, w.q1.p, q, w.tmp2.p, c, &w.main, OZ_ROWS});
-      g3.push_back({BG_ABT, t->fp32, m, r, c, 1.0, s->core[k].p, c, w.tmp2.p, c, w.b.p, r, &w.main, OZ_ROWS});
+      g3.push_back({BG_ABT, 0, m, r, c, 1.0, s->core[k].p, c, w.tmp2.p, c, w.b.p, r, &w.main, OZ_ROWS});
       g4.push_back({BG_AB, t->fp32, pl, r, m, 1.0, s->core[k - 1].p, m, w.b.p, r, w.gemm.p, r, &w.main, OZ_COLS});
     }
     double wo = 0.0;

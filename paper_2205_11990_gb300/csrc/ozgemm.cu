@@ -675,7 +675,10 @@ long long tiles_of(int M, int N) { return (long long)((M + kOzM - 1) / kOzM) * (
 
 // Which FP64 contractions are sliced.  Two launches of ~14 + 26 us at the smallest
 // sizes stand against the FMA kernel's 2 M N K / 1.1 TFLOP/s: whole vp_gemm calls on
-// GB300, sliced / FMA, us: @FIGURES@;
+// GB300, sliced / FMA, us: 256^3 (M N K = 1.7e7) 61 / 61, 320 x 256 x 256 (2.1e7) 56 / 86, 300^3 59 / 99,
+// 512 x 324 x 256 (4.3e7) 62 / 135, 341 x 1008 x 503 (1.7e8) 65 / 430, 128 x 6784 x
+// 6147 (5.3e9) 870 / 12300 (operands whose elements the proof leaves open: 300^3 320,
+// 341 x 1008 x 503 560, 128 x 6784 x 6147 15300);
 // the line is drawn at 2e7.  Below K = 64 (one stage) or 16 rows or columns most
 // of a tile would be padding; so would a shape that fills less than a quarter of
 // its tiles in the better of the two orientations; and from K = 524288 on a band of one
