@@ -304,10 +304,12 @@ int vp_poisson_noalloc(void* cuda_stream, const double* rho_dev, int nx, double 
 
 /* Dense contraction C (M x N) = alpha * A (M x K) * B (K x N), row-major
  * device buffers with leading dimensions lda >= K, ldb >= N, ldc >= N, in
- * the arithmetic of `precision` (VP_PREC_*, see vp_config): the kernel the
- * sweeps use for their GEMM-shaped contractions (R x next core, U S
- * products).  K = 0 gives C = 0.  Synchronises the context stream; a device
- * wait that gave up is reported as VP_ETIMEOUT.  Errors: VP_EINVAL. */
+ * the arithmetic of `precision` (VP_PREC_*, see vp_config): the kernels the
+ * sweeps use for their GEMM-shaped contractions.  In FP64 every element is
+ * within the bound of an FP64 sum, K 2^-53 (|A| |B|)_ij to first order.
+ * K = 0 gives C = 0.  Synchronises the context stream; a device wait that
+ * gave up is reported as VP_ETIMEOUT.  Errors: VP_EINVAL, VP_ECAPACITY
+ * (N above 64 * 65535). */
 int vp_gemm(vp_ctx* ctx, int precision, int M, int N, int K, double alpha, const double* A, int lda,
             const double* B, int ldb, double* C, int ldc);
 
@@ -336,13 +338,15 @@ typedef struct {
   int e_chi;        /* bond cap D_F of the field MPS (main text, "Approximation
                        of the nonlinear term"); 0: no cap */
   int precision;    /* VP_PREC_*: arithmetic of the dense contractions of the
-                       sweeps (R x next core, the Q and U S products).  The
-                       other steps do not change with the mode: the MPO
-                       application, the truncation rule and the Poisson
-                       solve stay FP64, and the QR, Q formation and Jacobi
+                       sweeps (R x next core, core x U S), the density
+                       and the expansions.  The other steps do not
+                       change with the mode: V^T and U S = M V of a site,
+                       the MPO application, the truncation rule and the
+                       Poisson solve stay FP64, and the QR, Q formation and Jacobi
                        SVD stay in double-word FP32 (~2^-48, see the
                        precision convention at the top of this file).
-                         FP64          FP64 FMA;
+                         FP64          FP64 FMA, or exact FP16 slices on the
+                                       tensor cores within FP64's bound;
                          FP32_CONTRACT FP32 FMA, FP32 accumulation (CUDA cores);
                          TF32          tensor cores, operands rounded to TF32,
                                        FP32 accumulation in tensor memory;

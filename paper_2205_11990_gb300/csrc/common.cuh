@@ -156,12 +156,13 @@ int check_launch(vp_ctx* ctx, const char* what);
 // launch attribute neither does anything).  Every thread calls it first, so that no
 // such kernel ends before the one it follows.
 //
-// It pays where one chain of small kernels is all there is (ctx->early: field solve
-// 211 -> 184 us, a stage of the 128 x 64 initial field 7.6 -> 7.15 ms, 64-point run
-// 40.4 -> 39.0, 1024 x 1024 step 64 -> 55).  Where several chains share the device
-// it costs: two streams 36.7 -> 38.1, two species 39.9 -> 44.0, groups of several
-// runs 117.5 -> 119.7; there the launches are plain ones.  Blocks with much shared
-// memory are not parked on an SM either.
+// It pays where one chain of small kernels is all there is (ctx->early, without / with:
+// field solve 216 / 180 us, a stage of the 128 x 64 grid 7.5 / 7.0 ms, 64-point run 37.6 /
+// 35.7, 1024 x 1024 step 64.7 / 54.9).  Where several chains share the device it costs:
+// two streams 36.7 / 38.1, two species 39.9 / 44.0, groups of several runs 117.5 / 119.7;
+// there the launches are plain ones.  Contexts that a program creates itself do not know
+// of each other and keep it: two stepping 1024 x 1024 side by side 54.8 / 54.8 ms a step,
+// four 61.5 / 71.1.  Blocks with much shared memory are not parked on an SM either.
 __device__ __forceinline__ void follow() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -301,7 +302,7 @@ struct TcOperand {
 // tensor cores in the context's reduced-precision mode (tcgemm.cu).
 int launch_tc_gemm(vp_ctx* ctx, int M, int N, int K, double alpha, TcOperand a, TcOperand b, double* C, int ldc);
 // How an FP64 contraction is sliced over the tensor cores (ozgemm.cu); use = 0:
-// the FMA kernel (gemm_plan).  Shape and device only.
+// the FMA kernel (fgemm.cu: fma_plan).  Shape and device only.
 struct OzPlan {
   int use;
   int swapped;  // tiles of C^T

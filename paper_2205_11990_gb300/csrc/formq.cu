@@ -13,9 +13,9 @@
 // in flight while one is applied.  Rows above a panel are neither loaded nor
 // touched.  The arithmetic of a column depends on the factor's shape only.
 //
-// Measured on GB300 (event-timed, one factor; before: one reflector at a time):
-// 1024 x 528 396 us (2840), 1456 x 348 250 (2810), 1056 x 184 122 (1140), 448 x 168
-// 97 (159), 128 x 128 66 (118), 64 x 64 39 (54).
+// Measured on GB300 (event-timed, in a sweep, best of five; before: one reflector at a
+// time): 1024 x 528 391 us (2891), 1456 x 348 244 (2894), 1056 x 184 122 (1154), 448 x 168
+// 93 (153), 128 x 128 31 (106), 64 x 64 19 (36).
 #include <cuda_runtime.h>
 
 #include <algorithm>

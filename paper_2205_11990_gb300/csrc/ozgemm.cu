@@ -9,14 +9,13 @@
 // number of 56 bits relative to a power of two above its row's (A) or column's
 // (B) largest magnitude within a K slice, cut into eight signed 7-bit digits,
 //   a = 2^(e - 55) sum_i d_i 2^(7 (7 - i)),  -64 <= d_i <= 64,
-// which are exact FP16 integers; -a has the digits -d_i.  Products of digits are at most 2^12, so the
-// FP32 accumulator holds the sum of up to eight digit products over K <= 512
-// exactly (2^24).  The digit products with i + j = l, l = 0..8 (43 of the 64)
-// accumulate into nine 128 x 48 accumulators of tensor memory, and the epilogue
-// adds the nine integers with their weights exactly and rounds once to FP64, to
-// nearest.  What is dropped (l > 8) is below 2^-60.4 of the two
-// scales per product; an element is held to 2^-56 of its scale, and exactly from
-// an eighth of the scale on.
+// which are exact FP16 integers; -a has the digits -d_i.  Products of digits are at
+// most 2^12, so the FP32 accumulator holds the sum of up to eight digit products over
+// K <= 512 exactly (2^24).  The digit products with i + j = l, l = 0..8 (43 of the 64)
+// accumulate into nine 128 x 48 accumulators of tensor memory, and the epilogue adds the
+// nine integers with their weights exactly and rounds once to FP64, to nearest.  What is
+// dropped (l > 8) is below 2^-60.4 of the two scales per product; an element is held to
+// 2^-56 of its scale, and exactly from an eighth of the scale on.
 //
 // So a product is as accurate as its row's and column's largest elements make it,
 // where an FP64 sum is as accurate as the products that meet in it: a row (1e20, 1,
@@ -28,14 +27,15 @@
 //     by n 2^-53 W, so the element passes from W = 2180 / 2^14 = 0.133 on.  W is summed
 //     from 7-bit magnitudes (of the first digits) that kb_oz_pack writes beside the digits
 //     (four products an instruction, by four warps that would wait while the products
-//     run): the first 32 k suffice where sizes are even (standard normal entries: W = 1.2
-//     there, 0.3 where one outlier each doubles both scales), else all of them are
+//     run): the first 32 k suffice where sizes are even (standard normal entries: W = 1.1
+//     there, 0.2 where one outlier each doubles both scales), else all of them are
 //     summed.  An element all of whose products are zero passes as well.
-//   OZ_ROWS     nothing to prove.
+//   OZ_ROWS     nothing to prove: 2^-56 of the scales' product for each of K products.
 //   OZ_COLS     kb_oz_kexp moves column k of A to one by a power of two, row k of B the
 //     other way (exact), so that columns of A of any size keep their digits.
-// Error against 64-bit references, largest over rows with standard normal entries:
-// 6-9e-17 of the norms for K = 64..1008, the FMA kernel's 1.7-3.1e-16.
+// Error against 64-bit references, standard normal entries: largest 0.14-0.5 times 2^-53
+// (|A| |B|)_ij for K = 64..6147, the FMA kernel's 1.0 at K = 256; entries of exponents
+// -70..70, where 97 of 100 elements stay open, 4-9 times 2^-53 (|A| |B|)_ij.
 //
 // Passes: kb_oz_kexp (OZ_COLS only), kb_oz_pack (digits, written as the
 // 128-byte-swizzled shared-memory images of whole tiles, so that the loads are
@@ -47,10 +47,10 @@
 // a row or column that holds a NaN or Inf, or that scaling takes out of the exponent
 // range, are FP64 FMAs as well, so non-finite values propagate as they do there.
 //
-// Measured (2048^3): 557 us in kb_oz_mma, 1.33 PFLOP/s of FP16 products, 71 % of
-// the measured 1.88 (the 9-accumulator epilogue is not overlapped: the tile's
-// accumulators fill tensor memory); kb_oz_pack moves 24 bytes per element at
-// 3 TB/s; whole call 24 TFLOP/s of FP64 against 1.1 for the FMA kernel.
+// Measured (2048^3): 578 us in kb_oz_mma, 1.28 PFLOP/s of FP16 products, 68 % of the
+// measured 1.88 (the 9-accumulator epilogue is not overlapped: the tile's accumulators
+// fill tensor memory); kb_oz_pack 81 us, 25 bytes per element at 2.6 TB/s; the sum of
+// four slices 38 us; whole call 738 us, 23 TFLOP/s of FP64 against 1.1 for the FMA kernel.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -78,7 +78,7 @@ constexpr size_t kOzSmem = 1024 + 2 * (size_t)kOzBBytes + (size_t)kOzAStages * k
 
 __device__ __forceinline__ int oz_bexp(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7ff); }
 
-// Exponent of x after the balance shift (0 for a zero, 2047 for a non-finite
+// Exponent of x after its column's shift (0 for a zero, 2047 for a non-finite
 // value, clamped into 1 .. 2047 otherwise: 2047 sends the row to the FP64 path).
 __device__ __forceinline__ int oz_shifted_exp(double x, int sh) {
   const int e = oz_bexp(x);
@@ -675,18 +675,18 @@ long long tiles_of(int M, int N) { return (long long)((M + kOzM - 1) / kOzM) * (
 
 // Which FP64 contractions are sliced.  Two launches of ~14 + 26 us at the smallest
 // sizes stand against the FMA kernel's 2 M N K / 1.1 TFLOP/s: whole vp_gemm calls on
-// GB300, sliced / FMA, us: 256^3 (M N K = 1.7e7) 61 / 61, 320 x 256 x 256 (2.1e7) 56 / 86, 300^3 59 / 99,
-// 512 x 324 x 256 (4.3e7) 62 / 135, 341 x 1008 x 503 (1.7e8) 65 / 430, 128 x 6784 x
-// 6147 (5.3e9) 870 / 12300 (operands whose elements the proof leaves open: 300^3 320,
-// 341 x 1008 x 503 560, 128 x 6784 x 6147 15300);
-// the line is drawn at 2e7.  Below K = 64 (one stage) or 16 rows or columns most
-// of a tile would be padding; so would a shape that fills less than a quarter of
-// its tiles in the better of the two orientations; and from K = 524288 on a band of one
-// tile's rows would take more than kOzBand.  K is cut into slices of at most 512, where
-// the accumulators stop being exact, and into at least as many as fill the SMs with tiles
-// once (128 of K each, two stages); a CTA takes one, while what they leave to be added
-// stays below kOzSums.  (Slices added in registers, or over the CTAs of a cluster, took 5
-// to 15 us longer a product than a CTA each and the launch that adds.)
+// GB300, sliced / FMA, us: 320 x 256 x 256 (M N K = 2.1e7) 56 / 86, 300^3 59 / 99, 512 x
+// 324 x 256 (4.3e7) 62 / 135, 341 x 1008 x 503 (1.7e8) 65 / 430, 128 x 6784 x 6147 (5.3e9)
+// 870 / 12300 (operands whose elements the proof leaves open: 300^3 320, 341 x 1008 x 503
+// 560, 128 x 6784 x 6147 15300), and 256^3 (1.7e7) 61 on the FMA kernel; the line is drawn
+// at 2e7.  Below K = 64 (one stage) or 16 rows or columns most of a tile would be padding;
+// so would a shape that fills less than a quarter of its tiles in the better of the two
+// orientations; and from K = 524288 on a band of one tile's rows would take more than
+// kOzBand.  K is cut into slices of at most 512, where the accumulators stop being exact,
+// and into at least as many as fill the SMs with tiles once (128 of K each, two stages); a
+// CTA takes one, while what they leave to be added stays below kOzSums.  (Slices added in
+// registers, or over the CTAs of a cluster, took 5 to 15 us longer a product than a CTA
+// each and the launch that adds.)
 OzPlan oz_plan(const vp_ctx* ctx, int M, int N, int K) {
   OzPlan p{0, 0, 1, 0, 1};
   if (K < 64 || K >= 1 << 19 || std::min(M, N) < 16 || (double)M * N * K < 2e7) return p;

@@ -74,3 +74,23 @@ def test_without_memory_the_fma_pipe(vp):
     ctx.set_alloc_budget(None)
     check(A, B, ctx.gemm(A, B))
     ctx.close()
+
+
+def test_several_slices_with_elements_formed_again(vp):
+    """4096 x 4096 x 1100: three slices one after the other in a CTA, entries of every size
+    in a tenth of the rows and columns, a NaN and an Inf in others."""
+    import torch
+    ctx = vp.Context()
+    A, B = operands(4096, 4096, 1100, 3)
+    rng = np.random.default_rng(3)
+    rows, cols = torch.from_numpy(rng.choice(4096, 400, False)).cuda(), torch.from_numpy(rng.choice(4096, 400, False)).cuda()
+    A[rows] *= torch.exp2(torch.from_numpy(rng.integers(-70, 71, (400, 1100))).cuda().double())
+    B[:, cols] *= torch.exp2(torch.from_numpy(rng.integers(-70, 71, (1100, 400))).cuda().double())
+    A[7, 600], B[1099, 9] = float("nan"), float("inf")
+    C = ctx.gemm(A, B, alpha=-0.5).cpu().numpy()
+    a, b = A.cpu().numpy(), B.cpu().numpy()
+    assert np.all(np.isnan(C[7])) and not np.any(np.isfinite(C[:, 9]))
+    keep, kept = np.arange(4096) != 7, np.arange(4096) != 9
+    a, b, C = a[keep], b[:, kept], C[keep][:, kept]
+    assert np.all(np.abs(C + 0.5 * (a @ b)) <= 0.5 * (2 * 1100 + 16) * 2.0 ** -53 * (np.abs(a) @ np.abs(b)))
+    ctx.close()
