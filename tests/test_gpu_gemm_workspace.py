@@ -35,9 +35,9 @@ def check(A, B, C):
 
 
 # several K slices a CTA, a cluster of CTAs, both; swapped tiles; more than a band of digits
-# in A, in B, in both (from K x rows = 2^26 on)
+# in A, in B, in both (from K x rows = 2^26 on); the FMA pipe from K = 2^19 on
 SHAPES = [(900, 1100, 2100), (260, 200, 5000), (48, 128, 9000), (128, 600, 6147), (40000, 64, 2048), (64, 40000, 2048),
-          (200, 130, 300000)]
+          (200, 130, 300000), (48, 40, 600000)]
 
 
 @pytest.mark.parametrize("shape", SHAPES)
